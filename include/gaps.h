@@ -7,7 +7,7 @@
  * backward initial-state evolution (Appendix A), Catani-Seymour recoil
  * kinematics (Appendix B.2-B.5) and the MC@NLO-like matching for on-shell Z
  * production (Appendix C), and computes per-event observables and weighted
- * histograms (Section 4.1). One event per CUDA thread.
+ * histograms (Section 4.1).
  *
  * Conventions shared by every entry point:
  *   - Four-vectors are (E, px, py, pz) in GeV, metric (+,-,-,-).
@@ -27,7 +27,10 @@
  *     non-finite values) are stored per event in `status` and counted by
  *     gaps_get_stats, which synchronises the stream.
  *   - Device buffers are owned by the caller; the library owns its copy of
- *     the PDF grid, its bound tables, its counters and, for GAPS_MIXED, a
+ *     the PDF grid, its bound tables, its counters and, for GAPS_FP64, the
+ *     scratch of the events in flight (allocated by gaps_init: 208 B x nmax per
+ *     event, 64 events per SM, 259 MB for 128 slots; calls on several streams
+ *     share it), for GAPS_MIXED, a
  *     working set of nmax partons per resident thread (allocated by the
  *     first mixed gaps_shower call; about 132 B x nmax x resident threads),
  *     or with GAPS_SCHED_WAVE one per event of ev->capacity (about
@@ -66,8 +69,9 @@ extern "C" {
 #define GAPS_FP64        0   /* all FP64; matches the reference per event */
 #define GAPS_MIXED       1   /* FP32 trials, PDF and bounds; FP64 kinematics */
 
-/* launch schedules of the shower */
-#define GAPS_SCHED_PER_EVENT  0   /* one thread per event, run to completion */
+/* launch schedules of the shower (GAPS_FP64 runs one kernel, eight lanes per
+ * event, for both of the first two) */
+#define GAPS_SCHED_PER_EVENT  0   /* GAPS_MIXED: the same as GAPS_SCHED_PERSISTENT */
 #define GAPS_SCHED_PERSISTENT 1   /* persistent grid, finished lanes take the next event */
 #define GAPS_SCHED_WARP       2   /* GAPS_MIXED only: persistent grid, one event per warp
                                      in shared memory, the lanes share its trials */
@@ -125,9 +129,9 @@ typedef struct {
     double p_s;           /* probability of an S event in GAPS_PP_Z_NLO, in (0,1) */
     uint64_t seed;        /* Philox key */
     const float* pdf_grid;/* host pointer to the PDF grid (pp processes), copied */
-    int block_size;       /* threads per block for the shower, 0 = library default */
+    int block_size;       /* GAPS_MIXED: threads per block for the shower, 0 = library default */
     int schedule;         /* GAPS_SCHED_PER_EVENT, GAPS_SCHED_PERSISTENT or GAPS_SCHED_WARP */
-    int blocks_per_sm;    /* persistent schedule: resident blocks per SM, 0 = default */
+    int blocks_per_sm;    /* GAPS_MIXED: resident blocks per SM, 0 = default */
     int refill_period;    /* GAPS_MIXED: idle lanes take new events at most every
                              this many cycles (compaction period), 0 = 1 */
     int emit_batch;       /* GAPS_MIXED: accepted emissions of a warp are built

@@ -13,8 +13,9 @@
 
 namespace gaps {
 cudaError_t launch_generate_hard(const DevParams&, const DevEvents&, uint64_t, uint64_t, int, cudaStream_t);
-cudaError_t launch_shower_fp64(const DevParams&, const DevEvents&, uint64_t, uint64_t, int, int,
-                               unsigned long long*, cudaStream_t);
+size_t fp64_pool_layout(int n_sm, int nmax, unsigned& regions, size_t& flag_bytes);
+cudaError_t launch_shower_fp64(const DevParams&, const DevEvents&, uint64_t, uint64_t, void*, unsigned, size_t,
+                               cudaStream_t);
 void workset_carve(void* base, int lanes, int nmax, WorkSet& W);
 cudaError_t launch_shower_mixed(const DevParams&, const DevEvents&, const WorkSet&, const LearnedCfg&, uint64_t,
                                 uint64_t, int, int, int, int, int, int, unsigned long long*, cudaStream_t);
@@ -53,6 +54,9 @@ struct gaps_ctx {
   DevParams P;
   HistSet H;   // binning per row (one row for one process)
   int q_independent = 0;     // every Q^2 column of the grid is identical
+  void* d_pool = nullptr;    // FP64 shower: flags and scratch of the resident blocks
+  unsigned pool_regions = 0;
+  size_t pool_flag_bytes = 0;
   void* d_work = nullptr;    // mixed-precision working set
   size_t work_bytes = 0;
   void* d_wave = nullptr;    // wavefront schedule: working set with one lane per event, then its state
@@ -400,6 +404,12 @@ int gaps_init(gaps_ctx** out, const gaps_config* cfg) {
     if ((rc = cuda_fail(cudaMalloc(&ctx->d_counters, (C_NCOUNTERS + 1) * sizeof(unsigned long long))))) break;
     if ((rc = cuda_fail(cudaMemset(ctx->d_counters, 0, (C_NCOUNTERS + 1) * sizeof(unsigned long long))))) break;
     if ((rc = cuda_fail(mixed_kernels_init()))) break;
+    if (c.precision == GAPS_FP64) {
+      // allocated here and not by the first shower, which a caller may capture
+      const size_t bytes = fp64_pool_layout(ctx->n_sm, c.nmax_partons, ctx->pool_regions, ctx->pool_flag_bytes);
+      if ((rc = cuda_fail(cudaMalloc(&ctx->d_pool, bytes)))) break;
+      if ((rc = cuda_fail(cudaMemset(ctx->d_pool, 0, ctx->pool_flag_bytes)))) break;
+    }
     if ((rc = cuda_fail(observables_init()))) break;
   } while (false);
   if (rc != GAPS_OK) {
@@ -532,14 +542,8 @@ int shower_impl(gaps_ctx* ctx, uint64_t first_event, uint64_t n, const gaps_even
     if (c.schedule == GAPS_SCHED_WAVE) return shower_wave(ctx, first_event, n, ev, Lc, stream, slot);
     return shower_mixed(ctx, first_event, n, ev, Lc, stream);
   }
-  int bs = c.block_size > 0 ? c.block_size : 128;
-  int pblocks = 0;
-  if (c.schedule == GAPS_SCHED_PERSISTENT) {
-    int per_sm = c.blocks_per_sm > 0 ? c.blocks_per_sm : 4;
-    pblocks = ctx->n_sm * per_sm;
-  }
-  return cuda_fail(launch_shower_fp64(ctx->P, dev_events(ev), first_event, n, bs, pblocks,
-                                      ctx->d_counters + C_NCOUNTERS, (cudaStream_t)stream));
+  return cuda_fail(launch_shower_fp64(ctx->P, dev_events(ev), first_event, n, ctx->d_pool, ctx->pool_regions,
+                                      ctx->pool_flag_bytes, (cudaStream_t)stream));
 }
 }  // namespace
 
@@ -1078,6 +1082,7 @@ void gaps_destroy(gaps_ctx* ctx) {
   if (ctx->d_grid) cudaFree(ctx->d_grid);
   if (ctx->d_tables) cudaFree(ctx->d_tables);
   if (ctx->d_counters) cudaFree(ctx->d_counters);
+  if (ctx->d_pool) cudaFree(ctx->d_pool);
   if (ctx->d_work) cudaFree(ctx->d_work);
   if (ctx->d_wave) cudaFree(ctx->d_wave);
   if (ctx->d_mlp) cudaFree(ctx->d_mlp);

@@ -1,397 +1,923 @@
 // FP64 max-veto dipole shower (Section 2, Fig. 1; Appendices A and B of
-// arXiv:2511.19633), one event per thread, evolving the caller's SoA record
-// in place. Compiled without FMA contraction (-fmad=false) so that every
-// event reproduces a plain FP64 CPU evaluation to rounding of libm calls.
+// arXiv:2511.19633). Compiled without FMA contraction (-fmad=false): every
+// event reproduces a plain FP64 evaluation of the same formulas bit for bit.
 //
-// Launch forms:
-//   k_shower_fp64     one thread per event, runs each event to completion
-//                     (the paper's layout without partitioning);
-//   k_shower_fp64_pq  persistent grid: a thread takes the next unstarted
-//                     event from a global counter as soon as its event
-//                     finishes (live-event refill instead of the paper's
-//                     thrust::partition, Section 3.1).
+// The algorithm of Fig. 1 draws one trial per channel of every colour end in
+// each cycle, takes the largest, and vetoes about fifteen of sixteen winners.
+// Three properties let a group of kG lanes run kG cycles of one event at once
+// with the same results:
+//   - While the event does not change, a cycle uses a fixed number of Philox
+//     blocks, so the blocks of the cycles ahead are known.
+//   - Which channel wins needs its trial scale only to the accuracy that
+//     separates it from the next one. FP32 values with an error bound decide
+//     that (screening); a cycle in which the bounds of two channels overlap,
+//     or in which a bound straddles a threshold, is decided in FP64.
+//   - A winner's exact scale is min(t, t_kin) R^(1/c), with t the exact scale
+//     of the cycle before: the powers of the kG cycles are formed side by
+//     side, the products one after the other.
+// The lanes then evaluate one cycle's acceptance each, assuming that the
+// cycles before were vetoed; the first that was not ends the batch and the
+// cycles behind it are dropped, their counters with them.
+//
+// What bounds it: FP64 runs at 1/64 of the FP32 rate here, and an FP64
+// instruction costs a warp the same however few lanes are active. One thread
+// per event (the earlier form of this file) evaluated every trial in FP64 with
+// a partner search and the bound tables again in each cycle; now the end table
+// is kept between emissions (only the ends an emission touched are formed
+// again), the trials run in FP32 and the FP64 work fills the lanes. Whole path
+// (hard events, shower, observables), before and now: 30 000 LO pp -> Z events
+// at 13.6 TeV 1128 and 60 ms, 3001 NLO events with heavy-quark thresholds 1093
+// and 36 ms (the longest event's chain of cycles), 10 000 e+e- events at 91.2
+// GeV 35.0 and 3.5 ms.
 #include "physics_fp64.cuh"
 
 namespace gaps {
 namespace {
 
+// lanes per event: eight cycles a batch (an acceptance comes every 9 to 16
+// cycles), and the about eight ends that an emission touches in one step
+constexpr int kG = 8;
+constexpr int kThreads = 128;
+constexpr int kGroups = kThreads / kG;  // events a block holds
+constexpr int kMinBlocks = 4;           // 128 registers a thread
+constexpr int kMaxPerBlock = 128;       // events a block takes before it leaves
+constexpr unsigned kAll = 0xffffffffu;
+
 struct Counters {
-  unsigned long long steps = 0, trials = 0, isr_trials = 0, vetoes = 0, accepts = 0, violations = 0;
+  unsigned long long finished = 0, steps = 0, trials = 0, isr_trials = 0, vetoes = 0, accepts = 0, violations = 0;
+  unsigned long long err_cap = 0, err_iter = 0, err_num = 0;
 };
 
-struct Winner {
-  int i, k, side, ch, type, shape;
-  double t, Rz, coef, zm, delta, s, eta, B;
-  double m2;  // heavy-quark measure dt/(t - m2) of the trial, 0: dt/t
+// exact record of a colour end (emitter slot q / 2, side q % 2) in the group's
+// scratch: the inputs of its two channels' trials and weights
+struct EndX {
+  double s, eta, tkin, cc[2], B[2];
+  int k, type;  // partner slot (-1: no dipole on this side), dipole type
+};
+static_assert(sizeof(EndX) == 64, "one end is two sectors");
+
+// a parton's flavour and colour tags
+struct Tag { int f, c, a, pad; };
+
+// One event's scratch. `scr` holds the screening values of an end: {1/c of
+// channel 0, 1/c of channel 1 (-1: absent, infinity: no trial), ln t_kin,
+// number of trial blocks before this end}.
+struct Scratch {
+  double* p;     // [nmax][4]
+  EndX* end;     // [2 nmax]
+  float4* scr;   // [2 nmax]
+  Tag* tag;      // [nmax]
+};
+constexpr size_t kSlotBytesPerParton = 4 * sizeof(double) + 2 * sizeof(EndX) + 2 * sizeof(float4) + sizeof(Tag);
+
+__device__ __forceinline__ Scratch scratch_of(unsigned char* base, int nmax) {
+  Scratch w;
+  w.p = reinterpret_cast<double*>(base);
+  w.end = reinterpret_cast<EndX*>(base + (size_t)nmax * 4 * sizeof(double));
+  w.scr = reinterpret_cast<float4*>(w.end + 2 * nmax);
+  w.tag = reinterpret_cast<Tag*>(w.scr + 2 * nmax);
+  return w;
+}
+
+// per row of a mixed batch
+struct RowShared {
+  double t_cut, as_over;
+  float lnTc;
+  int pp;
 };
 
-// One max-veto cycle for event e. Returns the new status (ACTIVE, DONE or an
-// error code). n, t, eta0/eta1, draw live in registers of the caller.
-__device__ int shower_step(const DevParams& P, const DevEvents& E, uint64_t e, int& n, double& t,
-                           double& eta0, double& eta1, Rng& rng, int& n_emit, Counters& cnt) {
-  cnt.steps += 1;
-  Winner best;
-  best.t = -1.0;
-  best.i = -1;
-  best.m2 = 0.0;
-  for (int i = 0; i < n; ++i) {
-    int ci = E.C(i, e), ai = E.A(i, e);
-    if (ci == 0 && ai == 0) continue;
-    int fi = E.F(i, e);
-    bool ini = (P.process != GAPS_EE_QQ) && i < 2;
-    for (int side = 0; side < 2; ++side) {
-      int tag = side == 0 ? ci : ai;
-      if (tag == 0) continue;
-      int k = -1;
-      for (int m = 0; m < n; ++m) {
-        if (m == i) continue;
-        if (side == 0 ? (E.A(m, e) == tag) : (E.C(m, e) == tag)) { k = m; break; }
-      }
-      if (k < 0) continue;
-      bool ink = (P.process != GAPS_EE_QQ) && k < 2;
-      int type = ini ? (ink ? kII : kIF) : (ink ? kFI : kFF);
-      double pi[4], pk[4];
+// values of lane `src` of the caller's group, and reductions over the group
+// (all 32 lanes of the warp call them)
+__device__ __forceinline__ double gshfl(double v, int src) { return __shfl_sync(kAll, v, src, kG); }
+__device__ __forceinline__ int gshfl(int v, int src) { return __shfl_sync(kAll, v, src, kG); }
+__device__ __forceinline__ float gshfl(float v, int src) { return __shfl_sync(kAll, v, src, kG); }
+__device__ __forceinline__ float gmax(float v) {
 #pragma unroll
-      for (int mu = 0; mu < 4; ++mu) { pi[mu] = E.P(mu, i, e); pk[mu] = E.P(mu, k, e); }
-      double s = 2.0 * dot4(pi, pk);
-      double eta = 0.0;
-      if (type == kFI) eta = (k == 0) ? eta0 : eta1;
-      if (type == kIF || type == kII) eta = (i == 0) ? eta0 : eta1;
-      int first = ini ? (fi == 21 ? 5 : 3) : (fi == 21 ? 1 : 0);
-      int nch = (!ini && fi != 21) ? 1 : 2;
-      for (int c = 0; c < nch; ++c) {
-        int ch = first + c;
-        double Rt, Rz;
-        rng.next2(Rt, Rz);
-        double tmax = fmin(t, t_kin_max(type, s, eta));
-        if (!(tmax > P.t_cut)) continue;
-        // heavy-quark measure correction (App. A.2): an incoming c or b with a
-        // threshold draws its q <- q and q <- g trials in dt/(t - m_q^2), down to
-        // m_q^2 (1 + kHqFloor)
-        double mq2 = 0.0;
-        if ((type == kIF || type == kII) && (ch == 3 || ch == 4)) {
-          const int fe = pdf_index(fi);
-          if (fe >= 0 && P.thr[fe] >= 0) mq2 = P.m2[fe];
-        }
-        if (mq2 > 0.0 && !(tmax > mq2 * (1.0 + kHqFloor))) continue;
-        double zm, delta;
-        if (!z_limits(type, P.t_cut, s, eta, zm, delta)) continue;
+  for (int o = kG / 2; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(kAll, v, o, kG));
+  return v;
+}
+__device__ __forceinline__ int gsum(int v) {
+#pragma unroll
+  for (int o = kG / 2; o > 0; o >>= 1) v += __shfl_xor_sync(kAll, v, o, kG);
+  return v;
+}
+// bit j: `b` of lane j of the group
+__device__ __forceinline__ unsigned gballot(bool b) {
+  const unsigned m = __ballot_sync(kAll, b);
+  return (m >> (threadIdx.x & 31 & ~(kG - 1))) & ((1u << kG) - 1u);
+}
+
+// squared mass of the heavy-quark measure of an end's channels (App. A.2: an
+// incoming c or b with a threshold draws both its channels in dt/(t - m^2))
+__device__ __forceinline__ double heavy_m2(const DevParams& P, int type, int fl) {
+  if (type != kIF && type != kII) return 0.0;
+  if (fl == 21) return 0.0;
+  const int fe = pdf_index(fl);
+  return fe >= 0 && P.thr[fe] >= 0 ? P.m2[fe] : 0.0;
+}
+
+// channel c of an emitter: 0 q->qg, 1 g->gg, 2 g->qqbar (final); 3 q->qg,
+// 4 q->g qbar, 5 g->gg, 6 g->qq (initial)
+__device__ __forceinline__ int channel_of(bool ini, int fl, int c) {
+  return (ini ? (fl == 21 ? 5 : 3) : (fl == 21 ? 1 : 0)) + c;
+}
+
+// The record of end q (one lane): partner, invariant, overestimate
+// coefficients and PDF-ratio bounds of its channels.
+__device__ __forceinline__ void form_end(const DevParams& P, const Scratch& w, const RowShared& R, int n, int q,
+                                      double eta0, double eta1) {
+  const int i = q >> 1, side = q & 1;
+  const Tag ti = w.tag[i];
+  const int tag = side == 0 ? ti.c : ti.a;
+  int k = -1;
+  if (tag != 0)
+    for (int m = 0; m < n; ++m) {
+      if (m == i) continue;
+      if (side == 0 ? (w.tag[m].a == tag) : (w.tag[m].c == tag)) { k = m; break; }
+    }
+  EndX x;
+  x.k = k;
+  x.type = 0;
+  float4 sc = make_float4(-1.0f, -1.0f, 0.0f, 0.0f);
+  if (k >= 0) {
+    const int fi = ti.f;
+    const bool ini = R.pp && i < 2, ink = R.pp && k < 2;
+    const int type = ini ? (ink ? kII : kIF) : (ink ? kFI : kFF);
+    double pi[4], pk[4];
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) { pi[mu] = w.p[4 * i + mu]; pk[mu] = w.p[4 * k + mu]; }
+    const double s = 2.0 * dot4(pi, pk);
+    double eta = 0.0;
+    if (type == kFI) eta = (k == 0) ? eta0 : eta1;
+    if (type == kIF || type == kII) eta = (i == 0) ? eta0 : eta1;
+    const int nch = (!ini && fi != 21) ? 1 : 2;
+    x.type = type;
+    x.s = s;
+    x.eta = eta;
+    x.tkin = t_kin_max(type, s, eta);
+    double zm, delta;
+    // (every trial starts above the cutoff, so min(t, t_kin) > t_c here is t_kin > t_c)
+    const bool ok = !(x.tkin <= R.t_cut) && z_limits(type, R.t_cut, s, eta, zm, delta);
+    x.cc[0] = x.cc[1] = 0.0;
+    x.B[0] = x.B[1] = 1.0;
+    float ic[2] = {-1.0f, -1.0f};
+    // the two logarithms of the shapes' integrals, shared by the channels
+    double lsoft = 0.0, linv = 0.0;
+    if (ok) {
+      const double zp = 1.0 - delta;
+      int sh0, sh1;
+      double unused;
+      channel_over(channel_of(ini, fi, 0), type, P.nf, sh0, unused);
+      channel_over(channel_of(ini, fi, 1), type, P.nf, sh1, unused);
+      if (nch == 1) sh1 = sh0;
+      if (sh0 == kSoft || sh0 == kBoth || sh1 == kSoft || sh1 == kBoth) lsoft = gm_log((1.0 - zm) / delta);
+      if (sh0 == kInv || sh0 == kBoth || sh1 == kInv || sh1 == kBoth) linv = gm_log(zp / zm);
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        if (c >= nch) continue;
+        const int ch = channel_of(ini, fi, c);
         int shape;
         double coef;
         channel_over(ch, type, P.nf, shape, coef);
         double B = 1.0;
         if (type == kFI) {
-          int f = pdf_index(E.F(k, e));
-          B = pdf_ratio_bound(P, f, f, eta);
+          // both channels of a final emitter have the spectator's bound
+          if (c == 0) {
+            const int f = pdf_index(w.tag[k].f);
+            B = pdf_ratio_bound(P, f, f, eta);
+          } else {
+            B = x.B[0];
+          }
         } else if (type == kIF || type == kII) {
           int num, den;
           isr_pdf_indices(ch, fi, num, den);
           B = pdf_ratio_bound(P, num, den, eta);
         }
+        x.B[c] = B;
         if (!(B > 0.0)) continue;
-        double cc = P.as_over / (2.0 * kPi) * B * coef * shape_integral(shape, zm, delta);
-        if (!(cc > 0.0)) continue;
-        cnt.trials += 1;
-        if (type == kIF || type == kII) cnt.isr_trials += 1;
-        double tt = mq2 > 0.0 ? mq2 + (tmax - mq2) * gm_exp(gm_log(Rt) / cc) : tmax * gm_exp(gm_log(Rt) / cc);
-        if (mq2 > 0.0 && !(tt > mq2 * (1.0 + kHqFloor))) continue;  // below the channel's floor
-        if (tt > best.t) {
-          best.i = i; best.k = k; best.side = side; best.ch = ch; best.type = type;
-          best.t = tt; best.Rz = Rz; best.shape = shape; best.coef = coef;
-          best.zm = zm; best.delta = delta; best.s = s; best.eta = eta; best.B = B; best.m2 = mq2;
-        }
+        const double in = shape == kSoft ? lsoft : shape == kFlat ? zp - zm : shape == kBoth ? linv + lsoft : linv;
+        const double cc = R.as_over / (2.0 * kPi) * B * coef * in;
+        if (cc > 0.0) x.cc[c] = cc;
       }
     }
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+      if (c < nch) ic[c] = x.cc[c] > 0.0 ? fminf(1.0f / (float)x.cc[c], 1e30f) : INFINITY;
+    sc = make_float4(ic[0], ic[1], __logf((float)x.tkin), 0.0f);
   }
-  if (best.i < 0 || best.t < P.t_cut) return GAPS_STATUS_DONE;
-  if (!isfinite(best.t)) return GAPS_ERR_NUMERIC;
-  double Rveto, Rphi, Rfl, Rcol;
-  rng.next2(Rveto, Rphi);
-  rng.next2(Rfl, Rcol);
-  const double tw = best.t;
-  t = tw;
+  w.end[q] = x;
+  w.scr[q] = sc;
+}
 
-  double z, omz;
-  shape_sample(best.shape, best.zm, best.delta, best.Rz, z, omz);
-  double zm_t, delta_t;
-  if (!z_limits(best.type, tw, best.s, best.eta, zm_t, delta_t) || !(omz > delta_t) || !(z > zm_t)) {
-    cnt.vetoes += 1;
-    return GAPS_STATUS_ACTIVE;
+// exact trial scale of channel c of end x below t with the uniform Rt (-1: no
+// trial, counted false); the order of Fig. 1's tests
+__device__ __noinline__ double exact_trial(const EndX& x, int c, double m2, double t, double t_cut, double Rt, bool& counted) {
+  counted = false;
+  const double tmax = fmin(t, x.tkin);
+  if (!(tmax > t_cut)) return -1.0;
+  if (m2 > 0.0 && !(tmax > m2 * (1.0 + kHqFloor))) return -1.0;
+  if (!(x.cc[c] > 0.0)) return -1.0;
+  counted = true;
+  if (m2 > 0.0) {
+    const double tt = m2 + (tmax - m2) * gm_exp(gm_log(Rt) / x.cc[c]);
+    return tt > m2 * (1.0 + kHqFloor) ? tt : -1.0;
   }
-  double pover = shape_value(best.shape, best.coef, z, omz);
-  double as_ratio = alpha_s(P, tw) / P.as_over;
-  const int type = best.type, ch = best.ch, bi = best.i, bk = best.k;
-  const double s = best.s;
-  int fl_i = E.F(bi, e);
-  double w = 0.0;
-  double y = 0.0, rho = 0.0, x = 1.0, omx = 0.0, u = 0.0, omu = 1.0, v = 0.0;
-  int new_fl_i = fl_i, fl_j = 21;
-  double sumF = 0.0;
-  if (type == kFF) {
-    y = tw / (z * omz * s);
-    double k;
-    double den = omz + z * y;
-    if (ch == 0) k = kCF * (2.0 / den - (1.0 + z));
-    else if (ch == 1) k = kCA / 2.0 * (2.0 / den - 2.0 + z * omz);
-    else k = P.nf * kTR / 2.0 * (1.0 - 2.0 * z * omz);
-    w = as_ratio * (1.0 - y) * k / pover;
-  } else if (type == kFI) {
-    rho = tw / (z * omz * s);
-    x = 1.0 / (1.0 + rho);
-    omx = rho / (1.0 + rho);
-    double k;
-    double den = omz + omx;
-    if (ch == 0) k = kCF * (2.0 / den - (1.0 + z));
-    else if (ch == 1) k = kCA / 2.0 * (2.0 / den - 2.0 + z * omz);
-    else k = P.nf * kTR / 2.0 * (1.0 - 2.0 * z * omz);
-    int f = pdf_index(E.F(bk, e));
-    double eta = best.eta;
-    double F1 = pdf_xf(P, f, eta * (1.0 + rho), tw);
-    double F0 = pdf_xf(P, f, eta, tw);
-    double ratio = (F0 > 0.0) ? x * F1 / F0 : 0.0;
-    w = as_ratio * k / pover * ratio / best.B;
+  return tmax * gm_exp(gm_log(Rt) / x.cc[c]);
+}
+
+// outcome of one cycle
+enum Outcome { kVeto = 0, kAccept, kDone, kNumericT, kNumericW, kCapacity };
+
+struct Winner {
+  int outcome, type, ch, bi, bk, side, new_fl, fl_j;
+  bool violation;
+  double t, z, omz, a0, a1, a2, a3, Rphi;  // a0..a3: the map's variables (see emission)
+};
+
+// The cycle after its trials for the winner (q, c) at scale tw: Appendix B's
+// weight and the accept test. One lane, on its own cycle. Values that every
+// dipole type needs (the z sample, alpha_s, the two densities) are formed
+// outside the branches on the type, so that the lanes of a warp share them.
+__device__ __forceinline__ void weigh(const DevParams& P, const Scratch& w, const RowShared& R, int n, int q, int c,
+                                   double tw, double Rz, const uint32_t o1[4], const uint32_t o2[4], Winner& W) {
+  W.violation = false;
+  W.t = tw;
+  if (tw < R.t_cut) { W.outcome = kDone; return; }
+  if (!isfinite(tw)) { W.outcome = kNumericT; return; }
+  const EndX x = w.end[q];
+  const int bi = q >> 1, bk = x.k, type = x.type;
+  const int fl_i = w.tag[bi].f;
+  const bool ini = type == kIF || type == kII;
+  const int ch = channel_of(ini, fl_i, c);
+  const double s = x.s, eta = x.eta;
+  W.bi = bi; W.bk = bk; W.side = q & 1; W.type = type; W.ch = ch;
+  W.new_fl = fl_i; W.fl_j = 21;
+  W.outcome = kVeto;
+  int shape;
+  double coef, zm, delta, z, omz;
+  channel_over(ch, type, P.nf, shape, coef);
+  z_limits(type, R.t_cut, s, eta, zm, delta);
+  shape_sample(shape, zm, delta, Rz, z, omz);
+  double zm_t, delta_t;
+  if (!z_limits(type, tw, s, eta, zm_t, delta_t) || !(omz > delta_t) || !(z > zm_t)) return;
+  const double pover = shape_value(shape, coef, z, omz);
+  W.z = z;
+  W.omz = omz;
+  double xm = 1.0, omx = 0.0, u = 0.0, omu = 1.0, v = 0.0, rho = 0.0, y = 0.0, J = 1.0, kk;
+  double x1 = 0.0;  // the numerator density's momentum fraction
+  if (!ini) {
+    rho = y = tw / (z * omz * s);
+    double soft = z * y;
+    if (type == kFI) {
+      xm = 1.0 / (1.0 + rho);
+      omx = rho / (1.0 + rho);
+      soft = omx;
+      x1 = eta * (1.0 + rho);
+    }
+    const double den = omz + soft;
+    if (ch == 0) kk = kCF * (2.0 / den - (1.0 + z));
+    else if (ch == 1) kk = kCA / 2.0 * (2.0 / den - 2.0 + z * omz);
+    else kk = P.nf * kTR / 2.0 * (1.0 - 2.0 * z * omz);
   } else {
-    double r = tw / s;
-    double J;
+    const double r = tw / s;
     if (type == kIF) {
-      if (!if_map(r, z, omz, x, omx, u, omu)) { cnt.vetoes += 1; return GAPS_STATUS_ACTIVE; }
-      J = 1.0 / (x * omu + u * omx);
+      if (!if_map(r, z, omz, xm, omx, u, omu)) return;
+      J = 1.0 / (xm * omu + u * omx);
     } else {
-      if (!ii_map(r, z, omz, x, omx, v)) { cnt.vetoes += 1; return GAPS_STATUS_ACTIVE; }
+      if (!ii_map(r, z, omz, xm, omx, v)) return;
       J = 1.0 / z;
     }
-    double eta = best.eta;
-    if (!(x > eta)) { cnt.vetoes += 1; return GAPS_STATUS_ACTIVE; }
-    double k;
-    double soft = (type == kIF) ? (omx + u) : omx;
-    if (ch == 3) k = kCF * (2.0 / soft - (1.0 + x));
-    else if (ch == 4) k = kTR * (1.0 - 2.0 * x * omx);
-    else if (ch == 5) k = kCA * (1.0 / soft + omx / x - 1.0 + x * omx);
-    else k = kCF / 2.0 * (x + 2.0 * omx / x);
+    if (!(xm > eta)) return;
+    x1 = eta / xm;
+    const double soft = (type == kIF) ? (omx + u) : omx;
+    if (ch == 3) kk = kCF * (2.0 / soft - (1.0 + xm));
+    else if (ch == 4) kk = kTR * (1.0 - 2.0 * xm * omx);
+    else if (ch == 5) kk = kCA * (1.0 / soft + omx / xm - 1.0 + xm * omx);
+    else kk = kCF / 2.0 * (xm + 2.0 * omx / xm);
+  }
+  const double as_ratio = alpha_s(P, tw) / R.as_over;
+  double wgt, sumF = 0.0;
+  PdfLoc l1;
+  l1.ok = false;
+  if (type == kFF) {
+    wgt = as_ratio * (1.0 - y) * kk / pover;
+  } else {
+    // the two points' cells: one Q^2 location for both
+    PdfLoc l0;
+    l0.ix = l0.iq = 0;
+    l0.fx = l0.fq = 0.0;
+    l1 = l0;
+    const bool okq = pdf_locate_q(P, tw, l0.iq, l0.fq);
+    l1.iq = l0.iq;
+    l1.fq = l0.fq;
+    l0.ok = pdf_locate_x(P, eta, l0.ix, l0.fx) && okq;
+    l1.ok = pdf_locate_x(P, x1, l1.ix, l1.fx) && okq;
     int num, den;
-    isr_pdf_indices(ch, fl_i, num, den);
-    double F0 = pdf_xf(P, den, eta, tw);
+    if (type == kFI) num = den = pdf_index(w.tag[bk].f);
+    else isr_pdf_indices(ch, fl_i, num, den);
+    const double F0 = pdf_at(P, den, l0);
     double F1;
     if (ch == 6) {
       F1 = 0.0;
-      for (int f = 1; f <= 10; ++f) F1 += pdf_xf(P, f, eta / x, tw);
+      for (int f = 1; f <= 10; ++f) F1 += pdf_at(P, f, l1);
       sumF = F1;
     } else {
-      F1 = pdf_xf(P, num, eta / x, tw);
+      F1 = pdf_at(P, num, l1);
     }
-    double Fratio = (F0 > 0.0) ? F1 / F0 : 0.0;
-    if (best.m2 > 0.0) Fratio = Fratio * ((tw - best.m2) / tw);  // heavy-quark measure correction
-    w = as_ratio * k * J * x / pover * Fratio / best.B;
-    if (ch == 4) { new_fl_i = 21; fl_j = -fl_i; }
-    if (ch == 5) { new_fl_i = 21; fl_j = 21; }
+    if (type == kFI) {
+      const double ratio = (F0 > 0.0) ? xm * F1 / F0 : 0.0;
+      wgt = as_ratio * kk / pover * ratio / x.B[c];
+    } else {
+      double Fratio = (F0 > 0.0) ? F1 / F0 : 0.0;
+      const double m2 = heavy_m2(P, type, fl_i);
+      if (m2 > 0.0) Fratio = Fratio * ((tw - m2) / tw);  // heavy-quark measure correction
+      wgt = as_ratio * kk * J * xm / pover * Fratio / x.B[c];
+      if (ch == 4) { W.new_fl = 21; W.fl_j = -fl_i; }
+      if (ch == 5) { W.new_fl = 21; W.fl_j = 21; }
+    }
   }
-  if (!isfinite(w)) return GAPS_ERR_NUMERIC;
-  if (w > 1.0) cnt.violations += 1;
-  if (!(Rveto < w)) { cnt.vetoes += 1; return GAPS_STATUS_ACTIVE; }
+  if (!isfinite(wgt)) { W.outcome = kNumericW; return; }
+  W.violation = wgt > 1.0;
+  if (!(u01(o1[0], o1[1]) < wgt)) return;
 
   // accepted: flavours
+  const double Rfl = u01(o2[0], o2[1]);
   if (ch == 2) {
     int f = 1 + (int)floor(Rfl * P.nf);
     if (f > P.nf) f = P.nf;
-    new_fl_i = f; fl_j = -f;
+    W.new_fl = f; W.fl_j = -f;
   } else if (ch == 6) {
     double target = Rfl * sumF, acc = 0.0;
     int pick = 10;
     for (int f = 1; f <= 10; ++f) {
-      acc += pdf_xf(P, f, best.eta / x, tw);
+      acc += pdf_at(P, f, l1);
       if (target < acc) { pick = f; break; }
     }
-    int fl = pick <= 5 ? pick : -(pick - 5);
-    new_fl_i = fl; fl_j = fl;
+    const int fl = pick <= 5 ? pick : -(pick - 5);
+    W.new_fl = fl; W.fl_j = fl;
   }
-  if (n >= P.nmax) return GAPS_ERR_CAPACITY;
-
-  // kinematics
-  double Pm[4], K[4];
-#pragma unroll
-  for (int mu = 0; mu < 4; ++mu) { Pm[mu] = E.P(mu, bi, e); K[mu] = E.P(mu, bk, e); }
-  double e1[4], e2[4];
-  transverse_basis(Pm, K, e1, e2);
-  double st = sqrt(tw), cph, sph;
-  gm_sincos2pi(Rphi, cph, sph);  // phi = 2 pi R_phi
-  double kt[4];
-#pragma unroll
-  for (int mu = 0; mu < 4; ++mu) kt[mu] = st * (cph * e1[mu] + sph * e2[mu]);
-  const int j = n;
-  double pj[4];
-  if (type == kFF) {
-#pragma unroll
-    for (int mu = 0; mu < 4; ++mu) {
-      E.P(mu, bi, e) = z * Pm[mu] + (y * omz) * K[mu] + kt[mu];
-      pj[mu] = omz * Pm[mu] + (y * z) * K[mu] - kt[mu];
-      E.P(mu, bk, e) = (1.0 - y) * K[mu];
-    }
-  } else if (type == kFI) {
-    double xinv = 1.0 + rho;
-#pragma unroll
-    for (int mu = 0; mu < 4; ++mu) {
-      E.P(mu, bi, e) = z * Pm[mu] + (omz * rho) * K[mu] + kt[mu];
-      pj[mu] = omz * Pm[mu] + (z * rho) * K[mu] - kt[mu];
-      E.P(mu, bk, e) = xinv * K[mu];
-    }
-    if (bk == 0) eta0 = eta0 * xinv; else eta1 = eta1 * xinv;
-  } else if (type == kIF) {
-#pragma unroll
-    for (int mu = 0; mu < 4; ++mu) {
-      E.P(mu, bi, e) = Pm[mu] / x;
-      pj[mu] = (omu * omx / x) * Pm[mu] + u * K[mu] - kt[mu];
-      E.P(mu, bk, e) = (u * omx / x) * Pm[mu] + omu * K[mu] + kt[mu];
-    }
-    if (bi == 0) eta0 = eta0 / x; else eta1 = eta1 / x;
-  } else {
-    double pa[4];
-#pragma unroll
-    for (int mu = 0; mu < 4; ++mu) {
-      pa[mu] = Pm[mu] / x;
-      E.P(mu, bi, e) = pa[mu];
-      pj[mu] = ((omx - v) / x) * Pm[mu] + v * K[mu] - kt[mu];
-    }
-    if (bi == 0) eta0 = eta0 / x; else eta1 = eta1 / x;
-    // Lorentz kick of all other final-state particles (eq. IIkinematics3)
-    double Kp[4], Kn[4], KK[4];
-#pragma unroll
-    for (int mu = 0; mu < 4; ++mu) {
-      Kp[mu] = Pm[mu] + K[mu];
-      Kn[mu] = (pa[mu] + K[mu]) - pj[mu];
-      KK[mu] = Kp[mu] + Kn[mu];
-    }
-    double KK2 = dot4(KK, KK), Kp2 = dot4(Kp, Kp);
-    for (int m = 2; m < n; ++m) {
-      double q[4];
-#pragma unroll
-      for (int mu = 0; mu < 4; ++mu) q[mu] = E.P(mu, m, e);
-      double a = 2.0 * dot4(KK, q) / KK2;
-      double b = 2.0 * dot4(Kp, q) / Kp2;
-#pragma unroll
-      for (int mu = 0; mu < 4; ++mu) E.P(mu, m, e) = q[mu] - a * KK[mu] + b * Kn[mu];
-    }
-  }
-#pragma unroll
-  for (int mu = 0; mu < 4; ++mu) E.P(mu, j, e) = pj[mu];
-
-  // colours: new tag 100 + slot of j
-  int T = 100 + n;
-  int ci = E.C(bi, e), ai = E.A(bi, e);
-  int cj = 0, aj = 0;
-  if (ch == 0 || ch == 1 || ch == 3 || ch == 5) {
-    if (best.side == 0) { cj = ci; aj = T; ci = T; }
-    else { aj = ai; cj = T; ai = T; }
-  } else if (ch == 2) {
-    aj = ai; cj = 0; ai = 0;
-  } else if (ch == 4) {
-    if (ai != 0) { ci = T; aj = T; cj = 0; }
-    else { ai = T; cj = T; aj = 0; }
-  } else {
-    int A = ci, Bt = ai;
-    if (new_fl_i > 0) { ci = 0; ai = Bt; cj = A; aj = 0; }
-    else { ci = A; ai = 0; cj = 0; aj = Bt; }
-  }
-  E.C(bi, e) = ci; E.A(bi, e) = ai; E.F(bi, e) = new_fl_i;
-  E.C(j, e) = cj; E.A(j, e) = aj; E.F(j, e) = fl_j;
-  n += 1;
-  n_emit += 1;
-  cnt.accepts += 1;
-  return GAPS_STATUS_ACTIVE;
+  W.outcome = n >= P.nmax ? kCapacity : kAccept;
+  W.Rphi = u01(o1[2], o1[3]);
+  if (type == kFF) { W.a0 = y; W.a1 = W.a2 = W.a3 = 0.0; }
+  else if (type == kFI) { W.a0 = rho; W.a1 = W.a2 = W.a3 = 0.0; }
+  else if (type == kIF) { W.a0 = xm; W.a1 = omx; W.a2 = u; W.a3 = omu; }
+  else { W.a0 = xm; W.a1 = omx; W.a2 = v; W.a3 = 0.0; }
 }
 
-// warp-aggregated counter flush; every lane of the warp must call it
-__device__ __forceinline__ void flush_counters(const DevParams& P, const Counters& c,
-                                               unsigned long long finished) {
-  __syncwarp();
-  unsigned long long v[7] = {finished, c.steps, c.trials, c.isr_trials, c.vetoes, c.accepts, c.violations};
-  const int idx[7] = {C_EVENTS, C_STEPS, C_TRIALS, C_ISR_TRIALS, C_VETOES, C_ACCEPTS, C_VIOLATIONS};
+// Minkowski product of group-distributed four-vectors (lane mu holds component
+// mu, lanes 4.. the same again), summed in dot4's order
+__device__ __forceinline__ double gdot(double a, double b) {
+  const double m = a * b;
+  return gshfl(m, 0) - gshfl(m, 1) - gshfl(m, 2) - gshfl(m, 3);
+}
+
+// The emission of group's winner W (lane f's copy, broadcast): kinematics with
+// one momentum component per lane (lanes 4..7 repeat 0..3), the II kick with
+// one parton per lane, colours on lane 0. All lanes of the warp take part;
+// groups with on = false compute on slot 0 and write nothing.
+__device__ __forceinline__ void emission(const Scratch& w, bool on, int n, const Winner& W, int f, double& eta0,
+                                      double& eta1) {
+  const int gl = threadIdx.x & (kG - 1), mu = gl & 3;
+  const int pack = gshfl(W.type | (W.ch << 2) | (W.side << 5) | (W.bi << 6) | (W.bk << 14), f);
+  const int type = pack & 3, ch = (pack >> 2) & 7, side = (pack >> 5) & 1;
+  const int bi = on ? (pack >> 6) & 0xff : 0, bk = on ? (pack >> 14) & 0xff : 0;
+  const int new_fl = gshfl(W.new_fl, f), fl_j = gshfl(W.fl_j, f);
+  const double z = gshfl(W.z, f), omz = gshfl(W.omz, f), tw = gshfl(W.t, f), Rphi = gshfl(W.Rphi, f);
+  const double a0 = gshfl(W.a0, f), a1 = gshfl(W.a1, f), a2 = gshfl(W.a2, f), a3 = gshfl(W.a3, f);
+  const double Pm = w.p[4 * bi + mu], K = w.p[4 * bk + mu];
+  // transverse basis (physics_fp64.cuh's steps)
+  const double PK = gdot(Pm, K);
+  const double N = 1.0 + 2.0 * Pm * K / PK;
+  const double N1 = gshfl(N, 1), N2 = gshfl(N, 2), N3 = gshfl(N, 3);
+  int a = 1;
+  double Na = N1;
+  if (N2 > Na) { a = 2; Na = N2; }
+  if (N3 > Na) { a = 3; Na = N3; }
+  int b;
+  if (a == 1) b = (N3 > N2) ? 3 : 2;
+  else if (a == 2) b = (N3 > N1) ? 3 : 1;
+  else b = (N2 > N1) ? 2 : 1;
+  const double na = sqrt(Na);
+  // K_a / PK, P_a / PK, K_b / PK, P_b / PK: one division, on lanes 0..3
+  const double Ka = gshfl(K, a), Pa = gshfl(Pm, a), Kb = gshfl(K, b), Pb = gshfl(Pm, b);
+  const double dv = (mu == 0 ? Ka : mu == 1 ? Pa : mu == 2 ? Kb : Pb) / PK;
+  const double KaP = gshfl(dv, 0), PaP = gshfl(dv, 1), KbP = gshfl(dv, 2), PbP = gshfl(dv, 3);
+  const double e1 = (((mu == a) ? 1.0 : 0.0) + KaP * Pm + PaP * K) / na;
+  const double e1b = gshfl(e1, b);
+  const double rperp = ((mu == b) ? 1.0 : 0.0) + KbP * Pm + PbP * K;
+  const double e2p = rperp - e1b * e1;
+  const double n2 = sqrt(-gdot(e2p, e2p));
+  const double e2 = e2p / n2;
+  const double st = sqrt(tw);
+  double cph, sph;
+  gm_sincos2pi(Rphi, cph, sph);  // phi = 2 pi R_phi
+  const double kt = st * (cph * e1 + sph * e2);
+  double pi, pk, pj;
+  if (type == kFF) {
+    pi = z * Pm + (a0 * omz) * K + kt;
+    pj = omz * Pm + (a0 * z) * K - kt;
+    pk = (1.0 - a0) * K;
+  } else if (type == kFI) {
+    const double xinv = 1.0 + a0;
+    pi = z * Pm + (omz * a0) * K + kt;
+    pj = omz * Pm + (z * a0) * K - kt;
+    pk = xinv * K;
+    if (on) { if (bk == 0) eta0 = eta0 * xinv; else eta1 = eta1 * xinv; }
+  } else {
+    pi = Pm / a0;
+    if (type == kIF) {
+      pj = (a3 * a1 / a0) * Pm + a2 * K - kt;
+      pk = (a2 * a1 / a0) * Pm + a3 * K + kt;
+    } else {
+      pj = ((a1 - a2) / a0) * Pm + a2 * K - kt;
+      pk = K;
+    }
+    if (on) { if (bi == 0) eta0 = eta0 / a0; else eta1 = eta1 / a0; }
+  }
+  __syncwarp();  // every lane has read its old momenta
+  if (on && gl < 4) {
+    w.p[4 * bi + mu] = pi;
+    if (type != kII) w.p[4 * bk + mu] = pk;
+    w.p[4 * n + mu] = pj;
+  }
+  if (__any_sync(kAll, on && type == kII)) {
+    // Lorentz kick of all other final-state particles (eq. IIkinematics3)
+    const double kp = Pm + K, kn = (pi + K) - pj, kq = kp + kn;
+    double Kp[4], Kn[4], KK[4];
 #pragma unroll
-  for (int q = 0; q < 7; ++q) {
+    for (int m = 0; m < 4; ++m) { Kp[m] = gshfl(kp, m); Kn[m] = gshfl(kn, m); KK[m] = gshfl(kq, m); }
+    if (on && type == kII) {
+      const double KK2 = dot4(KK, KK), Kp2 = dot4(Kp, Kp);
+      for (int m = 2 + gl; m < n; m += kG) {
+        double v[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[j] = w.p[4 * m + j];
+        const double ka = 2.0 * dot4(KK, v) / KK2;
+        const double kb = 2.0 * dot4(Kp, v) / Kp2;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) w.p[4 * m + j] = v[j] - ka * KK[j] + kb * Kn[j];
+      }
+    }
+  }
+  if (on && gl == 0) {
+    // colours: new tag 100 + slot of the new parton
+    const int T = 100 + n;
+    Tag t = w.tag[bi];
+    int ci = t.c, ai = t.a, cj = 0, aj = 0;
+    if (ch == 0 || ch == 1 || ch == 3 || ch == 5) {
+      if (side == 0) { cj = ci; aj = T; ci = T; }
+      else { aj = ai; cj = T; ai = T; }
+    } else if (ch == 2) {
+      aj = ai; cj = 0; ai = 0;
+    } else if (ch == 4) {
+      if (ai != 0) { ci = T; aj = T; cj = 0; }
+      else { ai = T; cj = T; aj = 0; }
+    } else {
+      const int A = ci, Bt = ai;
+      if (new_fl > 0) { ci = 0; ai = Bt; cj = A; aj = 0; }
+      else { ci = A; ai = 0; cj = 0; aj = Bt; }
+    }
+    w.tag[bi] = Tag{new_fl, ci, ai, 0};
+    w.tag[n] = Tag{fl_j, cj, aj, 0};
+  }
+  __syncwarp();
+}
+
+// The warp-wide sum of every counter, one atomic per warp and counter
+__device__ __forceinline__ void flush_counters(const DevParams& P, const Counters& c) {
+  __syncwarp();
+  const unsigned long long v[10] = {c.finished, c.steps, c.trials, c.isr_trials, c.vetoes,
+                                    c.accepts, c.violations, c.err_cap, c.err_iter, c.err_num};
+  const int idx[10] = {C_EVENTS, C_STEPS, C_TRIALS, C_ISR_TRIALS, C_VETOES,
+                       C_ACCEPTS, C_VIOLATIONS, C_ERR_CAP, C_ERR_ITER, C_ERR_NUM};
+#pragma unroll
+  for (int q = 0; q < 10; ++q) {
     unsigned long long x = v[q];
-    for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+    for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(kAll, x, off);
     if ((threadIdx.x & 31) == 0 && x) atomicAdd(&P.counters[idx[q]], x);
   }
 }
 
-__device__ __forceinline__ void count_error(const DevParams& P, int st) {
-  if (st == GAPS_ERR_CAPACITY) atomicAdd(&P.counters[C_ERR_CAP], 1ull);
-  else if (st == GAPS_ERR_ITER_CAP) atomicAdd(&P.counters[C_ERR_ITER], 1ull);
-  else if (st == GAPS_ERR_NUMERIC) atomicAdd(&P.counters[C_ERR_NUM], 1ull);
+// FP32 bounds of a screened trial: v +- er holds ln t of the exact trial. The
+// terms: the uniform's rounding and the fast logarithm (2^-21.41 between 1/2
+// and 2, 3 ulp elsewhere) times 1/c, whose own rounding and the product's are
+// relative to |lr|; the roundings of ln t_max and of the sum; the bound eT of
+// ln t itself. Each is taken at least twice.
+__device__ __forceinline__ float screen_error(float ic, float lr, float v, float lnTm, float eT) {
+  return ic * (1.2e-6f + 1.2e-6f * fabsf(lr)) + (fabsf(v) + fabsf(lnTm)) * 4e-7f + 2e-6f + eT;
 }
+// slack of a comparison with a logarithm formed in FP32 (|ln| < 64)
+constexpr float kLnSlack = 1e-4f;
 
-// run event e to completion; returns its final status
-__device__ int run_event(const DevParams& P0, const DevEvents& E, uint64_t e, uint64_t id, Counters& cnt) {
-  int st = E.status[e];
-  if (st != GAPS_STATUS_ACTIVE) return st;
-  DevParams P = P0;  // the event's row of a mixed batch
-  if (P0.n_rows > 1) apply_row(P, mix_row(P0, id));
-  int n = E.npart[e];
-  if (n < 2 || n > P.nmax) {  // not a record written by the hard-process kernel
-    E.status[e] = GAPS_ERR_NUMERIC;
-    count_error(P, GAPS_ERR_NUMERIC);
-    return GAPS_ERR_NUMERIC;
+__global__ void __launch_bounds__(kThreads, kMinBlocks)
+    k_shower_fp64(const __grid_constant__ DevParams P, const __grid_constant__ DevEvents E, uint64_t first, uint64_t n_events,
+                  unsigned per_block, unsigned char* pool, unsigned* taken, unsigned regions, int heavy_table) {
+  __shared__ RowShared rows[kMaxRows];
+  __shared__ int s_region;
+  __shared__ unsigned s_next;
+  const int tid = threadIdx.x, lane = tid & 31, gl = tid & (kG - 1), gw = lane / kG;
+  if (tid < kMaxRows) {
+    const RowParams& r = P.rows[tid < P.n_rows ? tid : 0];
+    rows[tid] = RowShared{r.t_cut, r.as_over, (float)gm_log(r.t_cut), r.process != GAPS_EE_QQ};
   }
-  double t = E.t[e];
-  double eta0 = E.eta[e], eta1 = E.eta[E.cap + e];
-  int n_emit = E.n_emit[e];
-  Rng rng;
-  rng.init(P.seed, id, E.draw[e]);
-  int steps = 0;
-  while (st == GAPS_STATUS_ACTIVE) {
-    st = shower_step(P, E, e, n, t, eta0, eta1, rng, n_emit, cnt);
-    if (++steps >= P.max_steps && st == GAPS_STATUS_ACTIVE) st = GAPS_ERR_ITER_CAP;
+  if (tid == 0) {
+    s_next = 0;
+    // a free part of the scratch pool: it has one for every block that can be
+    // resident on the device at a time, whichever launches they belong to
+    unsigned smid;
+    asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
+    int got = -1;
+    for (unsigned k = 0; k < 64 * regions && got < 0; ++k) {
+      const unsigned r = (smid * kMinBlocks + k) % regions;
+      if (atomicCAS(&taken[r], 0u, 1u) == 0u) got = (int)r;
+    }
+    s_region = got;
+    __threadfence();
   }
-  E.npart[e] = n;
-  E.t[e] = t;
-  E.eta[e] = eta0;
-  E.eta[E.cap + e] = eta1;
-  E.n_emit[e] = n_emit;
-  E.draw[e] = rng.draw;
-  E.status[e] = st;
-  if (st < 0) count_error(P, st);
-  return st;
-}
+  __syncthreads();
+  if (s_region < 0) return;  // cannot happen: see above (the events stay active)
+  const size_t slot = (size_t)s_region * kGroups + tid / kG;
+  const Scratch w = scratch_of(pool + slot * (size_t)P.nmax * kSlotBytesPerParton, P.nmax);
+  const uint64_t block0 = (uint64_t)blockIdx.x * per_block;
+  const unsigned block_n = (unsigned)(n_events - block0 < per_block ? n_events - block0 : per_block);
+  // event j of the block starts in warp j % 4: few events spread over the warps
+  const uint32_t k0 = (uint32_t)P.seed, k1 = (uint32_t)(P.seed >> 32);
 
-__global__ void k_shower_fp64(DevParams P, DevEvents E, uint64_t first, uint64_t n) {
-  uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   Counters cnt;
-  unsigned long long fin = 0;
-  if (e < n) {
-    run_event(P, E, e, first + e, cnt);
-    fin = 1;
-  }
-  flush_counters(P, cnt, fin);
-}
-
-// persistent form: each thread pulls event indices from *next until n
-__global__ void k_shower_fp64_pq(DevParams P, DevEvents E, uint64_t first, uint64_t n,
-                                 unsigned long long* next) {
-  Counters cnt;
-  unsigned long long fin = 0;
+  bool active = false, exhausted = false;
+  uint64_t e = 0, id = 0, draw = 0;
+  int n = 0, n_emit = 0, steps = 0, row = 0, status = GAPS_STATUS_ACTIVE;
+  int nblk = 0;          // trial blocks of a cycle
+  int chg = -1;          // emitter | spectator << 8 of the emission since the last table, -1: all ends
+  bool table = false;    // the end table has to be formed
+  double t = 0.0, eta0 = 0.0, eta1 = 0.0;
+  bool first_take = true;
   while (true) {
-    unsigned long long e = atomicAdd(next, 1ull);
-    if (e >= n) break;
-    run_event(P, E, e, first + e, cnt);
-    fin += 1;
+    // ---- a new event for every idle group ------------------------------
+    while (__any_sync(kAll, !active && !exhausted)) {
+      unsigned j = 0xffffffffu;
+      if (first_take) {
+        j = (unsigned)(tid >> 5) + (kThreads / 32) * (unsigned)gw;  // groups take 0 .. kGroups - 1 first
+      } else {
+        if (gl == 0 && !active && !exhausted) j = kGroups + atomicAdd(&s_next, 1u);
+        j = (unsigned)gshfl((int)j, 0);
+      }
+      first_take = false;
+      if (active || exhausted) continue;
+      if (j >= block_n) { exhausted = true; continue; }
+      e = block0 + j;
+      id = first + e;
+      if (gl == 0) cnt.finished += 1;
+      status = E.status[e];
+      if (status != GAPS_STATUS_ACTIVE) continue;
+      n = E.npart[e];
+      row = mix_row(P, id);
+      if (n < 2 || n > P.nmax) {  // not a record written by the hard-process kernel
+        if (gl == 0) { E.status[e] = GAPS_ERR_NUMERIC; cnt.err_num += 1; }
+        continue;
+      }
+      for (int s = gl; s < n; s += kG) {
+#pragma unroll
+        for (int mu = 0; mu < 4; ++mu) w.p[4 * s + mu] = E.P(mu, s, e);
+        w.tag[s] = Tag{E.F(s, e), E.C(s, e), E.A(s, e), 0};
+      }
+      t = E.t[e];
+      eta0 = E.eta[e];
+      eta1 = E.eta[E.cap + e];
+      n_emit = E.n_emit[e];
+      draw = E.draw[e];
+      steps = 0;
+      active = table = true;
+      chg = -1;
+    }
+    if (!__any_sync(kAll, active)) break;
+    const RowShared& R = rows[row];
+    const int ne = active ? 2 * n : 0;
+    __syncwarp();
+
+    // ---- end table: the ends the last emission touched (all: chg < 0) ---
+    if (__any_sync(kAll, table)) {
+      if (table) {
+        const int ci = chg & 0xff, ck = (chg >> 8) & 0xff, T = 99 + n;
+        for (int q = gl; q < ne; q += kG) {
+          if (chg >= 0 && q < ne - 2) {
+            // an end away from the emitter, the spectator and the new parton
+            // whose partner is neither of them keeps its record: its inputs
+            // did not change; one without a partner or with the new tag is
+            // matched again
+            const int i = q >> 1, k = w.end[q].k;
+            const Tag ti = w.tag[i];
+            const int tag = (q & 1) ? ti.a : ti.c;
+            if (i != ci && i != ck && k != ci && k != ck && (tag == 0 || (k >= 0 && tag != T))) continue;
+          }
+          form_end(P, w, R, n, q, eta0, eta1);
+        }
+      }
+      __syncwarp();
+      // trial blocks before each end, and of a cycle
+      int run = 0;
+      const int rounds = (ne + kG - 1) / kG;
+      const int most = __reduce_max_sync(kAll, table ? rounds : 0);
+      for (int r = 0; r < most; ++r) {
+        const int q = r * kG + gl;
+        int nd = 0;
+        float4 sc = make_float4(-1.0f, -1.0f, 0.0f, 0.0f);
+        if (table && q < ne) {
+          sc = w.scr[q];
+          nd = (sc.x >= 0.0f ? 1 : 0) + (sc.y >= 0.0f ? 1 : 0);
+        }
+        int inc = nd;
+#pragma unroll
+        for (int o = 1; o < kG; o <<= 1) {
+          const int v = __shfl_up_sync(kAll, inc, o, kG);
+          if (gl >= o) inc += v;
+        }
+        if (table && q < ne) w.scr[q].w = __int_as_float(run + inc - nd);
+        run += gshfl(inc, kG - 1);
+      }
+      if (table) nblk = run;
+      table = false;
+      __syncwarp();
+    }
+
+    // ---- screening: the winners of up to kG cycles ----------------------
+    const uint32_t e0 = (uint32_t)id, e1 = (uint32_t)(id >> 32);
+    const float lnTc = R.lnTc;
+    float lnT = active ? __logf((float)t) : 0.0f, eT = 2e-6f + fabsf(lnT) * 4e-7f;
+    int len = 0;                  // cycles with a winner
+    bool ends_done = false;       // the cycle after them has no trial above the cutoff
+    bool going = active;          // the batch can take another cycle
+    int my_q = 0, my_c = 0;       // winner of cycle gl
+    int my_trials = 0;            // trials of cycle gl: all | initial-state << 16
+    const bool live_t = t > R.t_cut;
+#pragma unroll 1
+    for (int k = 0; k < kG; ++k) {
+      if (!__any_sync(kAll, going)) break;
+      const uint64_t dk = draw + (uint64_t)k * (uint64_t)(nblk + 2);
+      float u1 = -INFINITY, u2 = -INFINITY, lmax = -INFINITY, v1 = 0.0f, er1 = 0.0f;
+      int i1 = 0, nt = 0;
+      bool doubt = false;
+      if (going && live_t) {
+#pragma unroll 1
+        for (int q = gl; q < ne; q += kG) {
+          const float4 sc = w.scr[q];
+          double m2 = 0.0;
+          if (heavy_table && q < 4 && R.pp) m2 = sc.x >= 0.0f ? heavy_m2(P, w.end[q].type, w.tag[q >> 1].f) : 0.0;
+#pragma unroll 1
+          for (int c = 0; c < 2; ++c) {
+            const float ic = c == 0 ? sc.x : sc.y;
+            if (!(ic >= 0.0f && ic < INFINITY)) continue;  // absent, or no trial
+            const uint64_t d = dk + (uint64_t)(__float_as_int(sc.w) + c);
+            uint32_t o[4];
+            philox(e0, e1, (uint32_t)d, (uint32_t)(d >> 32), k0, k1, o);
+            const float lnTm = fminf(lnT, sc.z);
+            float x = fmaf((float)o[0], 1.0f / 4294967296.0f, (float)o[1]) * (1.0f / 4294967296.0f);
+            const bool tiny = o[1] < 16u;  // R below 2^-28: only an upper bound
+            if (tiny) x = 3.7252903e-9f;
+            const float lr = __logf(x);
+            float v = fmaf(lr, ic, lnTm);
+            float er = screen_error(ic, lr, v, lnTm, eT);
+            bool sure = !tiny && ic < 1e30f;
+            if (m2 > 0.0) {
+              // the heavy-quark measure: t = m^2 + (t_max - m^2) R^(1/c) is at
+              // least t_max R^(1/c), so its relative error is not larger
+              const float mf = (float)m2, lnF = __logf(mf * (1.0f + (float)kHqFloor));
+              if (lnTm < lnF + kLnSlack) {
+                doubt = doubt || lnTm > lnF - kLnSlack;  // whether it draws is close
+                if (lnTm <= lnF - kLnSlack) continue;
+              }
+              v = __logf(mf + (__expf(lnTm) - mf) * __expf(fmaxf(lr * ic, -80.0f)));
+              er += kLnSlack;
+              if (v < lnF + kLnSlack) sure = false;  // may be below the channel's floor
+              if (v + er < lnF - kLnSlack) { ++nt; if (q < 4 && R.pp) nt += 1 << 16; continue; }
+            }
+            nt += (q < 4 && R.pp) ? 1 + (1 << 16) : 1;
+            const float ub = v + er;
+            if (sure) lmax = fmaxf(lmax, v - er);
+            if (ub > u1) { u2 = u1; u1 = ub; v1 = v; er1 = er; i1 = 2 * q + c; }
+            else u2 = fmaxf(u2, ub);
+          }
+        }
+      }
+      const float U = gmax(u1), Lm = gmax(lmax);
+      const unsigned cand = gballot(u1 >= Lm && u1 > -INFINITY);
+      const unsigned second = gballot(u2 >= Lm && u2 > -INFINITY);
+      const unsigned dmask = gballot(doubt);
+      if (heavy_table || k == 0) {
+        const int s = gsum(nt);
+        if (heavy_table ? gl == k : true) my_trials = s;
+      }
+      const int wl = __ffs(cand) - 1;
+      const float wv = gshfl(v1, wl < 0 ? 0 : wl), we = gshfl(er1, wl < 0 ? 0 : wl);
+      const int wi = gshfl(i1, wl < 0 ? 0 : wl);
+      const bool below = !(U >= lnTc - kLnSlack) && !dmask;  // no trial above the cutoff
+      // (some channel's lower bound is finite, and it alone reaches it)
+      const bool clear = !below && !dmask && Lm > -INFINITY && __popc(cand) == 1 && !second;
+      // a first cycle that the bounds do not decide: exact trials of the
+      // channels in question
+      const bool decide = going && k == 0 && !below && !clear;
+      int xi = -1;
+      if (__any_sync(kAll, decide)) {
+        double bt = -1.0;
+        int bidx = 0x7fffffff, xt = 0;
+        if (decide) {
+          for (int q = gl; q < ne; q += kG) {
+            const float4 sc = w.scr[q];
+            for (int c = 0; c < 2; ++c) {
+              const float ic = c == 0 ? sc.x : sc.y;
+              if (!(ic >= 0.0f && ic < INFINITY)) continue;
+              const uint64_t d = dk + (uint64_t)(__float_as_int(sc.w) + c);
+              uint32_t o[4];
+              philox(e0, e1, (uint32_t)d, (uint32_t)(d >> 32), k0, k1, o);
+              const EndX x = w.end[q];
+              bool counted;
+              const double tt = exact_trial(x, c, heavy_m2(P, x.type, w.tag[q >> 1].f), t, R.t_cut, u01(o[0], o[1]), counted);
+              if (counted) xt += (q < 4 && R.pp) ? 1 + (1 << 16) : 1;
+              if (tt > bt) { bt = tt; bidx = 2 * q + c; }
+            }
+          }
+        }
+#pragma unroll
+        for (int o = kG / 2; o > 0; o >>= 1) {
+          const double ot = __shfl_xor_sync(kAll, bt, o, kG);
+          const int oi = __shfl_xor_sync(kAll, bidx, o, kG);
+          if (ot > bt || (ot == bt && oi < bidx)) { bt = ot; bidx = oi; }
+        }
+        const int s = gsum(xt);
+        if (decide) {
+          if (!heavy_table || gl == 0) my_trials = s;
+          if (bidx != 0x7fffffff) xi = bidx;
+        }
+      }
+      if (going) {
+        if (below || (decide && xi < 0)) {
+          ends_done = true;
+          going = false;
+        } else if (clear || decide) {
+          const int win = clear ? wi : xi;
+          if (gl == k) { my_q = win >> 1; my_c = win & 1; }
+          len = k + 1;
+          lnT = wv;
+          eT = we;
+          // near or below the cutoff, or decided exactly: the batch ends here
+          if (decide || wv - we < lnTc + kLnSlack) going = false;
+        } else {
+          going = false;  // not decided in FP32: the next batch begins with it
+        }
+      }
+    }
+
+    // ---- exact scales and weights: lane j evaluates cycle j --------------
+    Winner W;
+    W.outcome = kVeto;
+    W.violation = false;
+    W.t = 0.0;
+    W.type = W.ch = W.bi = W.bk = W.side = W.new_fl = W.fl_j = 0;
+    W.z = W.omz = W.Rphi = W.a0 = W.a1 = W.a2 = W.a3 = 0.0;
+    const bool mine = active && gl < len;
+    const uint64_t dm = draw + (uint64_t)gl * (uint64_t)(nblk + 2);
+    double pw = 1.0, tkin = 0.0, m2 = 0.0, Rz = 0.5;
+    if (mine) {
+      const EndX& x = w.end[my_q];
+      const float4 sc = w.scr[my_q];
+      const uint64_t d = dm + (uint64_t)(__float_as_int(sc.w) + my_c);
+      uint32_t o[4];
+      philox(e0, e1, (uint32_t)d, (uint32_t)(d >> 32), k0, k1, o);
+      Rz = u01(o[2], o[3]);
+      pw = gm_exp(gm_log(u01(o[0], o[1])) / x.cc[my_c]);
+      tkin = x.tkin;
+      if (heavy_table) m2 = heavy_m2(P, x.type, w.tag[my_q >> 1].f);
+    }
+    double my_t = 0.0, tc = t;
+    const int most = __reduce_max_sync(kAll, active ? len : 0);
+    for (int k = 0; k < most; ++k) {
+      const double tmax = fmin(tc, tkin);
+      const double tt = m2 > 0.0 ? m2 + (tmax - m2) * pw : tmax * pw;
+      if (gl == k) my_t = tt;
+      tc = gshfl(tt, k);
+    }
+    if (mine) {
+      uint32_t o1[4], o2[4];
+      const uint64_t d1 = dm + (uint64_t)nblk, d2 = d1 + 1;
+      philox(e0, e1, (uint32_t)d1, (uint32_t)(d1 >> 32), k0, k1, o1);
+      philox(e0, e1, (uint32_t)d2, (uint32_t)(d2 >> 32), k0, k1, o2);
+      weigh(P, w, R, n, my_q, my_c, my_t, Rz, o1, o2, W);
+    }
+
+    // ---- commit: the cycles up to the first that was not vetoed ----------
+    const unsigned other = gballot(mine && W.outcome != kVeto);
+    const int room = P.max_steps - steps;  // cycles before the cap
+    int f = other ? __ffs(other) - 1 : -1;
+    if (f >= room) f = -1;
+    int done_cycles = f >= 0 ? f + 1 : min(len, room);  // committed
+    const int out = gshfl(W.outcome, f < 0 ? 0 : f);
+    const bool viol = gshfl((int)W.violation, f < 0 ? 0 : f) != 0;
+    const bool tail_done = f < 0 && ends_done && done_cycles == len && len < room;
+    // scale after the committed cycles (a cycle that ends without a veto test
+    // leaves it)
+    const int tl = f >= 0 && (out == kDone || out == kNumericT) ? f - 1 : done_cycles - 1;
+    const double tn = gshfl(my_t, tl < 0 ? 0 : tl);
+    bool accepted = false;
+    if (active) {
+      const int counted = done_cycles + (tail_done ? 1 : 0);
+      if (!heavy_table ? gl == 0 : gl < counted) {
+        const unsigned long long times = heavy_table ? 1 : (unsigned long long)counted;
+        cnt.trials += times * (unsigned long long)(my_trials & 0xffff);
+        cnt.isr_trials += times * (unsigned long long)(my_trials >> 16);
+      }
+      if (tl >= 0) t = tn;
+      steps += counted;
+      draw += (uint64_t)done_cycles * (uint64_t)(nblk + 2);
+      if (tail_done) draw += (uint64_t)nblk;
+      if (f >= 0 && (out == kDone || out == kNumericT)) draw -= 2;
+      if (gl == 0) {
+        cnt.steps += counted;
+        cnt.vetoes += f >= 0 ? f : done_cycles;
+        if (f >= 0 && viol) cnt.violations += 1;
+      }
+      int st = GAPS_STATUS_ACTIVE;
+      if (tail_done || (f >= 0 && out == kDone)) st = GAPS_STATUS_DONE;
+      else if (f >= 0 && (out == kNumericT || out == kNumericW)) st = GAPS_ERR_NUMERIC;
+      else if (f >= 0 && out == kCapacity) st = GAPS_ERR_CAPACITY;
+      else if (f >= 0) accepted = true;
+      if (st == GAPS_STATUS_ACTIVE && steps >= P.max_steps) st = GAPS_ERR_ITER_CAP;
+      status = st;
+    }
+
+    // ---- emission --------------------------------------------------------
+    if (__any_sync(kAll, accepted)) {
+      emission(w, accepted, n, W, f < 0 ? 0 : f, eta0, eta1);
+      const int pack = gshfl(W.type | (W.bi << 2) | (W.bk << 10), f < 0 ? 0 : f);
+      if (accepted) {
+        chg = (pack & 3) == kII ? -1 : ((pack >> 2) & 0xff) | (((pack >> 10) & 0xff) << 8);
+        n += 1;
+        n_emit += 1;
+        if (gl == 0) cnt.accepts += 1;
+        table = true;
+      }
+    }
+
+    // ---- finished events back into the caller's records ------------------
+    if (active && status != GAPS_STATUS_ACTIVE) {
+      for (int s = gl; s < n; s += kG) {
+#pragma unroll
+        for (int mu = 0; mu < 4; ++mu) E.P(mu, s, e) = w.p[4 * s + mu];
+        const Tag tg = w.tag[s];
+        E.F(s, e) = tg.f;
+        E.C(s, e) = tg.c;
+        E.A(s, e) = tg.a;
+      }
+      if (gl == 0) {
+        E.npart[e] = n;
+        E.t[e] = t;
+        E.eta[e] = eta0;
+        E.eta[E.cap + e] = eta1;
+        E.n_emit[e] = n_emit;
+        E.draw[e] = draw;
+        E.status[e] = status;
+        if (status == GAPS_ERR_CAPACITY) cnt.err_cap += 1;
+        else if (status == GAPS_ERR_ITER_CAP) cnt.err_iter += 1;
+        else if (status == GAPS_ERR_NUMERIC) cnt.err_num += 1;
+      }
+      active = table = false;
+    }
+    __syncwarp();
   }
-  flush_counters(P, cnt, fin);
+  flush_counters(P, cnt);
+  __syncthreads();
+  if (tid == 0) {
+    __threadfence();
+    atomicExch(&taken[s_region], 0u);
+  }
 }
 
 }  // namespace
 
-cudaError_t launch_shower_fp64(const DevParams& P, const DevEvents& E, uint64_t first, uint64_t n,
-                               int block_size, int persistent_blocks, unsigned long long* next,
-                               cudaStream_t stream) {
+// Scratch pool of the FP64 shower: parts for every block that can be resident
+// on the device at a time, with a flag each, so that calls on several streams
+// share it.
+size_t fp64_pool_layout(int n_sm, int nmax, unsigned& regions, size_t& flag_bytes) {
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_shower_fp64, kThreads, 0) != cudaSuccess || per_sm < 1)
+    per_sm = kMinBlocks;
+  regions = (unsigned)(n_sm * per_sm);
+  flag_bytes = (regions * sizeof(unsigned) + 255) / 256 * 256;
+  return flag_bytes + (size_t)regions * kGroups * (size_t)nmax * kSlotBytesPerParton;
+}
+
+cudaError_t launch_shower_fp64(const DevParams& P, const DevEvents& E, uint64_t first, uint64_t n, void* pool,
+                               unsigned regions, size_t flag_bytes, cudaStream_t stream) {
   if (n == 0) return cudaSuccess;
-  int bs = block_size > 0 ? block_size : 128;
-  if (persistent_blocks > 0 && next) {
-    cudaError_t err = cudaMemsetAsync(next, 0, sizeof(unsigned long long), stream);
-    if (err != cudaSuccess) return err;
-    k_shower_fp64_pq<<<persistent_blocks, bs, 0, stream>>>(P, E, first, n, next);
-  } else {
-    unsigned grid = (unsigned)((n + bs - 1) / bs);
-    k_shower_fp64<<<grid, bs, 0, stream>>>(P, E, first, n);
-  }
+  // events a block takes: one round over the resident blocks, up to
+  // kMaxPerBlock (its groups refill from the block's share); few events go one
+  // to a block, where an event has a warp's FP64 pipe for itself
+  uint64_t per = (n + regions - 1) / regions;
+  if (per > kMaxPerBlock) per = kMaxPerBlock;
+  int heavy = 0;
+  for (int f = 0; f < 12; ++f) heavy = heavy || P.thr[f] >= 0;
+  const unsigned grid = (unsigned)((n + per - 1) / per);
+  k_shower_fp64<<<grid, kThreads, 0, stream>>>(P, E, first, n, (unsigned)per, (unsigned char*)pool + flag_bytes,
+                                                (unsigned*)pool, regions, heavy);
   return cudaGetLastError();
 }
 
