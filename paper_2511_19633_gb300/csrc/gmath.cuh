@@ -13,6 +13,14 @@
 
 #include <cmath>
 
+// a unit whose kernel is bound by its instruction fetches defines
+// GAPS_GM_OUT_OF_LINE before including this file: one copy of each function
+#ifdef GAPS_GM_OUT_OF_LINE
+#define GAPS_GM_FN static __noinline__
+#else
+#define GAPS_GM_FN inline
+#endif
+
 namespace gaps {
 
 constexpr double kGmLn2Hi = 0x1.62e42fee00000p-1;
@@ -21,7 +29,12 @@ constexpr double kGmInvLn2 = 0x1.71547652b82fep+0;
 constexpr double kGmTwoPi = 0x1.921fb54442d18p+2;
 constexpr double kGmSqrtHalf = 0x1.6a09e667f3bcdp-1;
 
-__host__ __device__ inline double gm_exp(double x) {
+// IEEE division and square root, a call each in such a unit (inlined, an FP64
+// division is a long sequence here)
+__host__ __device__ GAPS_GM_FN double gm_div(double a, double b) { return a / b; }
+__host__ __device__ GAPS_GM_FN double gm_sqrt(double a) { return sqrt(a); }
+
+__host__ __device__ GAPS_GM_FN double gm_exp(double x) {
   if (!(x == x)) return x;
   if (x > 709.8) return HUGE_VAL;
   if (x < -745.2) return 0.0;
@@ -46,7 +59,7 @@ __host__ __device__ inline double gm_exp(double x) {
   return ldexp(p, (int)k);
 }
 
-__host__ __device__ inline double gm_log(double x) {
+__host__ __device__ GAPS_GM_FN double gm_log(double x) {
   if (!(x == x) || x < 0.0) return NAN;
   if (x == 0.0) return -HUGE_VAL;
   if (x > 1.7976931348623157e308) return x;
@@ -56,7 +69,7 @@ __host__ __device__ inline double gm_log(double x) {
     m = m * 2.0;
     e -= 1;
   }
-  double s = (m - 1.0) / (m + 1.0);
+  double s = gm_div(m - 1.0, m + 1.0);
   double z = s * s;
   // 1/(2j+1) for j = 11 down to 1, then 1
   double p = 1.0 / 23.0;

@@ -22,7 +22,7 @@ __device__ __forceinline__ double pdf_node(const DevParams& P, int f, int ix, in
 
 __device__ __forceinline__ bool pdf_locate_x(const DevParams& P, double x, int& ix, double& fx) {
   if (!(x >= kXMin && x <= kXMax)) return false;
-  double u = (gm_log(x) - P.lxmin) / P.dlx;
+  double u = gm_div(gm_log(x) - P.lxmin, P.dlx);
   ix = (int)floor(u);
   if (ix < 0) ix = 0;
   if (ix > kNX - 2) ix = kNX - 2;
@@ -32,7 +32,7 @@ __device__ __forceinline__ bool pdf_locate_x(const DevParams& P, double x, int& 
 
 __device__ __forceinline__ bool pdf_locate_q(const DevParams& P, double q2, int& iq, double& fq) {
   if (!(q2 >= kQ2Min && q2 <= kQ2Max)) return false;
-  double u = (gm_log(q2) - P.lqmin) / P.dlq;
+  double u = gm_div(gm_log(q2) - P.lqmin, P.dlq);
   iq = (int)floor(u);
   if (iq < 0) iq = 0;
   if (iq > kNQ - 2) iq = kNQ - 2;
@@ -73,12 +73,9 @@ __device__ __forceinline__ double pdf_xf(const DevParams& P, int f, double x, do
 
 // Upper bound of x' f_num(x', Q^2) / (eta f_den(eta, Q^2)) for all Q^2 and all
 // x' >= eta, from per-node extrema over Q^2 (the interpolant is linear in
-// ln x inside a cell at fixed Q^2). 0 when eta is off the grid.
-__device__ __forceinline__ double pdf_ratio_bound(const DevParams& P, int num, int den, double eta) {
-  int ix;
-  double fx;
+// ln x inside a cell at fixed Q^2), with eta in cell ix at fraction fx.
+__device__ __forceinline__ double pdf_ratio_bound_at(const DevParams& P, int num, int den, int ix, double fx) {
   if (num < 0 || num > 11 || den < 0 || den > 11) return 0.0;
-  if (!pdf_locate_x(P, eta, ix, fx)) return 0.0;
   double uin = (1.0 - fx) * __ldg(&P.umax[num * kNX + ix]) + fx * __ldg(&P.umax[num * kNX + ix + 1]);
   double un = fmax(uin, __ldg(&P.sufmax[num * (kNX + 1) + ix + 1]));
   double ld = (1.0 - fx) * __ldg(&P.lmin[den * kNX + ix]) + fx * __ldg(&P.lmin[den * kNX + ix + 1]);
@@ -89,14 +86,14 @@ __device__ __forceinline__ double pdf_ratio_bound(const DevParams& P, int num, i
     // numerator / lmin above it (App. A.2)
     double fd = (1.0 - fx) * __ldg(&P.first[den * kNX + ix]) + fx * __ldg(&P.first[den * kNX + ix + 1]);
     if (!(fd > 0.0)) return 0.0;
-    return un * fmax(P.dlq / fd, 1.0 / ld);
+    return un * fmax(gm_div(P.dlq, fd), gm_div(1.0, ld));
   }
-  return un / ld;
+  return gm_div(un, ld);
 }
 
 // one-loop alpha_s(t) from alpha_s(m_Z^2)
 __device__ __forceinline__ double alpha_s(const DevParams& P, double t) {
-  return P.as_mz / (1.0 + P.as_mz * P.beta0 * gm_log(t / (kMZ * kMZ)));
+  return gm_div(P.as_mz, 1.0 + P.as_mz * P.beta0 * gm_log(gm_div(t, kMZ * kMZ)));
 }
 
 // --- dipole types, channels and overestimates -----------------------------
@@ -121,74 +118,67 @@ __device__ __forceinline__ void channel_over(int ch, int type, int nf, int& shap
 // rationalised: 1 - sqrt(D) = (1 - D)/(1 + sqrt(D))); false above the limit
 __device__ __forceinline__ bool z_limits(int type, double t, double s, double eta, double& zm,
                                          double& delta) {
-  double e;
-  if (type == kFF) e = 4.0 * t / s;
-  else if (type == kFI) e = 4.0 * t / s * eta / (1.0 - eta);
-  else if (type == kIF) e = 4.0 * t * eta / (s * (1.0 - eta));
-  else e = 4.0 * t * eta / (s * (1.0 - eta) * (1.0 - eta));
+  // 4 t / s (FF), 4 t / s eta / (1 - eta) (FI), 4 t eta / (s (1 - eta)) (IF),
+  // 4 t eta / (s (1 - eta) (1 - eta)) (II); one division for all four, so that
+  // the lanes of a warp share it whatever their types
+  const bool fin = type == kFF || type == kFI;
+  double num = 4.0 * t, den = s;
+  if (!fin) {
+    num = num * eta;
+    den = den * (1.0 - eta);
+    if (type == kII) den = den * (1.0 - eta);
+  }
+  double e = gm_div(num, den);
+  if (type == kFI) e = gm_div(e * eta, 1.0 - eta);
   double D = 1.0 - e;
   if (!(D > 0.0)) return false;
-  double sq = sqrt(D);
-  if (type == kFF || type == kFI) {
-    delta = 0.5 * e / (1.0 + sq);
-    zm = delta;
-  } else {
-    delta = 0.5 * (1.0 - eta) * e / (1.0 + sq);
-    zm = eta + delta;
-  }
+  double sq = gm_sqrt(D);
+  delta = gm_div(fin ? 0.5 * e : 0.5 * (1.0 - eta) * e, 1.0 + sq);
+  zm = fin ? delta : eta + delta;
   return true;
 }
 
 __device__ __forceinline__ double t_kin_max(int type, double s, double eta) {
   if (type == kFF) return s / 4.0;
-  if (type == kFI || type == kIF) return s / 4.0 * (1.0 - eta) / eta;
-  return s / 4.0 * (1.0 - eta) * (1.0 - eta) / eta;
+  const double a = s / 4.0 * (1.0 - eta);
+  return gm_div(type == kFI || type == kIF ? a : a * (1.0 - eta), eta);
 }
 
-__device__ __forceinline__ double shape_integral(int sh, double zm, double delta) {
-  double zp = 1.0 - delta;
-  switch (sh) {
-    case kSoft: return gm_log((1.0 - zm) / delta);
-    case kFlat: return zp - zm;
-    case kBoth: return gm_log(zp / zm) + gm_log((1.0 - zm) / delta);
-    default: return gm_log(zp / zm);
-  }
-}
-
+// z with cumulative R of the shape between the limits, and 1 - z. In logarithms
+// (1 - z) = (1 - zm) (delta / (1 - zm))^R for kSoft, z = zm (zp / zm)^R for
+// kInv, the logit of z linear in R for kBoth; the logarithm and the power are
+// formed once for all shapes, so that the lanes of a warp share them.
 __device__ __forceinline__ void shape_sample(int sh, double zm, double delta, double R, double& z,
                                              double& omz) {
   double zp = 1.0 - delta;
-  switch (sh) {
-    case kSoft:
-      omz = (1.0 - zm) * gm_exp(R * gm_log(delta / (1.0 - zm)));
-      z = 1.0 - omz;
-      break;
-    case kFlat:
-      z = zm + R * (zp - zm);
-      omz = 1.0 - z;
-      break;
-    case kBoth: {
-      double lm = gm_log(zm / (1.0 - zm)), lp = gm_log(zp / delta);
-      double L = lm + R * (lp - lm);
-      double em = gm_exp(-L);
-      z = 1.0 / (1.0 + em);
-      omz = em / (1.0 + em);
-      break;
-    }
-    default:
-      z = zm * gm_exp(R * gm_log(zp / zm));
-      omz = 1.0 - z;
-      break;
+  if (sh == kFlat) {
+    z = zm + R * (zp - zm);
+    omz = 1.0 - z;
+    return;
+  }
+  const double omm = 1.0 - zm;
+  const double la = gm_log(gm_div(sh == kSoft ? delta : sh == kBoth ? zm : zp, sh == kInv ? zm : omm));
+  double L = R * la;
+  if (sh == kBoth) {
+    double lp = gm_log(gm_div(zp, delta));
+    L = -(la + R * (lp - la));
+  }
+  const double ex = gm_exp(L);
+  if (sh == kSoft) {
+    omz = omm * ex;
+    z = 1.0 - omz;
+  } else if (sh == kBoth) {
+    z = gm_div(1.0, 1.0 + ex);
+    omz = gm_div(ex, 1.0 + ex);
+  } else {
+    z = zm * ex;
+    omz = 1.0 - z;
   }
 }
 
 __device__ __forceinline__ double shape_value(int sh, double coef, double z, double omz) {
-  switch (sh) {
-    case kSoft: return coef / omz;
-    case kFlat: return coef;
-    case kBoth: return coef / (z * omz);
-    default: return coef / z;
-  }
+  if (sh == kFlat) return coef;
+  return gm_div(coef, sh == kSoft ? omz : sh == kBoth ? z * omz : z);
 }
 
 // initial-state PDF-ratio flavours: numerator = new incoming parton,
@@ -207,22 +197,22 @@ __device__ __forceinline__ void isr_pdf_indices(int ch, int fl_emitter, int& num
 __device__ __forceinline__ bool if_map(double r, double z, double omz, double& x, double& omx,
                                        double& u, double& omu) {
   double q = omz + r;
-  double disc = 1.0 - 4.0 * r * z * omz / (q * q);
+  double disc = 1.0 - gm_div(4.0 * r * z * omz, q * q);
   if (!(disc >= 0.0)) return false;
-  x = 2.0 * z * omz / (q * (1.0 + sqrt(disc)));
-  u = x * r / omz;
+  x = gm_div(2.0 * z * omz, q * (1.0 + gm_sqrt(disc)));
+  u = gm_div(x * r, omz);
   omu = 1.0 - u;
   if (!(omu > 0.0)) return false;
-  omx = omz / omu;
+  omx = gm_div(omz, omu);
   return true;
 }
 
 // eq. ii-jacobian map (t, z) -> (x, v)
 __device__ __forceinline__ bool ii_map(double r, double z, double omz, double& x, double& omx,
                                        double& v) {
-  x = z * omz / (omz + r);
-  omx = (omz * omz + r) / (omz + r);
-  v = x * r / omz;
+  x = gm_div(z * omz, omz + r);
+  omx = gm_div(omz * omz + r, omz + r);
+  v = gm_div(x * r, omz);
   return omx - v > 0.0;
 }
 

@@ -24,22 +24,42 @@
 // per event (the earlier form of this file) evaluated every trial in FP64 with
 // a partner search and the bound tables again in each cycle; now the end table
 // is kept between emissions (only the ends an emission touched are formed
-// again), the trials run in FP32 and the FP64 work fills the lanes. Whole path
-// (hard events, shower, observables), before and now: 30 000 LO pp -> Z events
-// at 13.6 TeV 1128 and 60 ms, 3001 NLO events with heavy-quark thresholds 1093
-// and 36 ms (the longest event's chain of cycles), 10 000 e+e- events at 91.2
-// GeV 35.0 and 3.5 ms.
+// again), the trials run in FP32 and the FP64 work fills the lanes. The warps
+// are in different phases, so the next limit was the instruction cache: with
+// every logarithm, division and density inlined the kernel was 376 KB, its
+// fetches hit in 48 % and 36 of 55 stall cycles had no instruction; with one
+// copy of each it is 154 KB and half the time. An FP64 instruction in the
+// screening loop, even a comparison, waits behind the other warps' FP64 work.
+// Whole path (hard events, shower, observables), one thread per event and now:
+// 30 000 LO pp -> Z events at 13.6 TeV 1128 and 26 ms, 3001 NLO events with
+// heavy-quark thresholds 1093 and 17 ms (the longest event's chain of cycles),
+// 10 000 e+e- events at 91.2 GeV 35.0 and 1.9 ms, 500 of them 22.2 and 0.7 ms.
+#define GAPS_GM_OUT_OF_LINE
 #include "physics_fp64.cuh"
 
 namespace gaps {
 namespace {
 
+// One copy of a Philox block outside the screening loop (see
+// GAPS_GM_OUT_OF_LINE)
+__device__ __noinline__ uint4 block_of(uint64_t event, uint64_t draw, uint32_t k0, uint32_t k1) {
+  uint32_t o[4];
+  philox((uint32_t)event, (uint32_t)(event >> 32), (uint32_t)draw, (uint32_t)(draw >> 32), k0, k1, o);
+  return make_uint4(o[0], o[1], o[2], o[3]);
+}
+
 // lanes per event: eight cycles a batch (an acceptance comes every 9 to 16
 // cycles), and the about eight ends that an emission touches in one step
 constexpr int kG = 8;
+// cycles of a batch when a warp has one event left and gives it all its lanes
+// (3001 NLO events: 33 ms with 8 lanes to the end, 28 ms with 32; 8, 16 or 32
+// cycles a batch made no difference beyond the runs' spread)
+constexpr int kWideBatch = 16;
 constexpr int kThreads = 128;
 constexpr int kGroups = kThreads / kG;  // events a block holds
-constexpr int kMinBlocks = 4;           // 128 registers a thread
+// 128 registers a thread (5, 6 and 8 blocks, with more spills, were level to
+// 10 % slower; so were blocks of 256 and 512 threads that begin a batch together)
+constexpr int kMinBlocks = 4;
 constexpr int kMaxPerBlock = 128;       // events a block takes before it leaves
 constexpr unsigned kAll = 0xffffffffu;
 
@@ -81,31 +101,36 @@ __device__ __forceinline__ Scratch scratch_of(unsigned char* base, int nmax) {
 
 // per row of a mixed batch
 struct RowShared {
-  double t_cut, as_over;
+  double t_cut, as_over, as_2pi;  // as_2pi: as_over / 2 pi
   float lnTc;
   int pp;
 };
 
-// values of lane `src` of the caller's group, and reductions over the group
-// (all 32 lanes of the warp call them)
-__device__ __forceinline__ double gshfl(double v, int src) { return __shfl_sync(kAll, v, src, kG); }
-__device__ __forceinline__ int gshfl(int v, int src) { return __shfl_sync(kAll, v, src, kG); }
-__device__ __forceinline__ float gshfl(float v, int src) { return __shfl_sync(kAll, v, src, kG); }
-__device__ __forceinline__ float gmax(float v) {
-#pragma unroll
-  for (int o = kG / 2; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(kAll, v, o, kG));
-  return v;
-}
-__device__ __forceinline__ int gsum(int v) {
-#pragma unroll
-  for (int o = kG / 2; o > 0; o >>= 1) v += __shfl_xor_sync(kAll, v, o, kG);
-  return v;
-}
-// bit j: `b` of lane j of the group
-__device__ __forceinline__ unsigned gballot(bool b) {
-  const unsigned m = __ballot_sync(kAll, b);
-  return (m >> (threadIdx.x & 31 & ~(kG - 1))) & ((1u << kG) - 1u);
-}
+// A group of G consecutive lanes of a warp (G = kG or 32, one copy of the code
+// for both): values of lane `src` of the caller's group and reductions over it
+// (all 32 lanes of the warp call them).
+struct Group {
+  int G;
+  __device__ __forceinline__ int lane() const { return threadIdx.x & (G - 1); }
+  template <class T>
+  __device__ __forceinline__ T get(T v, int src) const { return __shfl_sync(kAll, v, src, G); }
+  template <class T>
+  __device__ __forceinline__ T xchg(T v, int o) const { return __shfl_xor_sync(kAll, v, o); }
+  __device__ __forceinline__ float max(float v) const {
+#pragma unroll 1
+    for (int o = G >> 1; o > 0; o >>= 1) v = fmaxf(v, xchg(v, o));
+    return v;
+  }
+  __device__ __forceinline__ int sum(int v) const {
+#pragma unroll 1
+    for (int o = G >> 1; o > 0; o >>= 1) v += xchg(v, o);
+    return v;
+  }
+  // bit j: `b` of lane j of the group
+  __device__ __forceinline__ unsigned ballot(bool b) const {
+    return (__ballot_sync(kAll, b) >> (threadIdx.x & 31 & ~(G - 1))) & (kAll >> (32 - G));
+  }
+};
 
 // squared mass of the heavy-quark measure of an end's channels (App. A.2: an
 // incoming c or b with a threshold draws both its channels in dt/(t - m^2))
@@ -170,11 +195,14 @@ __device__ __forceinline__ void form_end(const DevParams& P, const Scratch& w, c
       channel_over(channel_of(ini, fi, 0), type, P.nf, sh0, unused);
       channel_over(channel_of(ini, fi, 1), type, P.nf, sh1, unused);
       if (nch == 1) sh1 = sh0;
-      if (sh0 == kSoft || sh0 == kBoth || sh1 == kSoft || sh1 == kBoth) lsoft = gm_log((1.0 - zm) / delta);
-      if (sh0 == kInv || sh0 == kBoth || sh1 == kInv || sh1 == kBoth) linv = gm_log(zp / zm);
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        if (c >= nch) continue;
+      if (sh0 == kSoft || sh0 == kBoth || sh1 == kSoft || sh1 == kBoth) lsoft = gm_log(gm_div(1.0 - zm, delta));
+      if (sh0 == kInv || sh0 == kBoth || sh1 == kInv || sh1 == kBoth) linv = gm_log(gm_div(zp, zm));
+      // the grid cell of eta, for every channel's bound
+      int ix = 0;
+      double fx = 0.0;
+      const bool on_grid = type != kFF && pdf_locate_x(P, eta, ix, fx);
+#pragma unroll 1
+      for (int c = 0; c < nch; ++c) {
         const int ch = channel_of(ini, fi, c);
         int shape;
         double coef;
@@ -184,19 +212,19 @@ __device__ __forceinline__ void form_end(const DevParams& P, const Scratch& w, c
           // both channels of a final emitter have the spectator's bound
           if (c == 0) {
             const int f = pdf_index(w.tag[k].f);
-            B = pdf_ratio_bound(P, f, f, eta);
+            B = on_grid ? pdf_ratio_bound_at(P, f, f, ix, fx) : 0.0;
           } else {
             B = x.B[0];
           }
         } else if (type == kIF || type == kII) {
           int num, den;
           isr_pdf_indices(ch, fi, num, den);
-          B = pdf_ratio_bound(P, num, den, eta);
+          B = on_grid ? pdf_ratio_bound_at(P, num, den, ix, fx) : 0.0;
         }
         x.B[c] = B;
         if (!(B > 0.0)) continue;
         const double in = shape == kSoft ? lsoft : shape == kFlat ? zp - zm : shape == kBoth ? linv + lsoft : linv;
-        const double cc = R.as_over / (2.0 * kPi) * B * coef * in;
+        const double cc = R.as_2pi * B * coef * in;
         if (cc > 0.0) x.cc[c] = cc;
       }
     }
@@ -209,6 +237,15 @@ __device__ __forceinline__ void form_end(const DevParams& P, const Scratch& w, c
   w.scr[q] = sc;
 }
 
+// pdf_at of one flavour (0..10; 0 for any other), one copy
+__device__ __noinline__ double xf_at(const DevParams& P, int f, const PdfLoc& L) {
+  if (f < 0 || f > 10 || !L.ok) return 0.0;
+  const float* g = P.grid + ((size_t)f * kNX + L.ix) * kNQ + L.iq;
+  const double lo = (1.0 - L.fx) * (double)__ldg(g) + L.fx * (double)__ldg(g + kNQ);
+  const double hi = (1.0 - L.fx) * (double)__ldg(g + 1) + L.fx * (double)__ldg(g + kNQ + 1);
+  return lo * (1.0 - L.fq) + hi * L.fq;
+}
+
 // exact trial scale of channel c of end x below t with the uniform Rt (-1: no
 // trial, counted false); the order of Fig. 1's tests
 __device__ __noinline__ double exact_trial(const EndX& x, int c, double m2, double t, double t_cut, double Rt, bool& counted) {
@@ -219,10 +256,10 @@ __device__ __noinline__ double exact_trial(const EndX& x, int c, double m2, doub
   if (!(x.cc[c] > 0.0)) return -1.0;
   counted = true;
   if (m2 > 0.0) {
-    const double tt = m2 + (tmax - m2) * gm_exp(gm_log(Rt) / x.cc[c]);
+    const double tt = m2 + (tmax - m2) * gm_exp(gm_div(gm_log(Rt), x.cc[c]));
     return tt > m2 * (1.0 + kHqFloor) ? tt : -1.0;
   }
-  return tmax * gm_exp(gm_log(Rt) / x.cc[c]);
+  return tmax * gm_exp(gm_div(gm_log(Rt), x.cc[c]));
 }
 
 // outcome of one cycle
@@ -239,7 +276,7 @@ struct Winner {
 // dipole type needs (the z sample, alpha_s, the two densities) are formed
 // outside the branches on the type, so that the lanes of a warp share them.
 __device__ __forceinline__ void weigh(const DevParams& P, const Scratch& w, const RowShared& R, int n, int q, int c,
-                                   double tw, double Rz, const uint32_t o1[4], const uint32_t o2[4], Winner& W) {
+                                   double tw, double Rz, const uint4& o1, const uint4& o2, Winner& W) {
   W.violation = false;
   W.t = tw;
   if (tw < R.t_cut) { W.outcome = kDone; return; }
@@ -263,44 +300,46 @@ __device__ __forceinline__ void weigh(const DevParams& P, const Scratch& w, cons
   const double pover = shape_value(shape, coef, z, omz);
   W.z = z;
   W.omz = omz;
-  double xm = 1.0, omx = 0.0, u = 0.0, omu = 1.0, v = 0.0, rho = 0.0, y = 0.0, J = 1.0, kk;
+  double xm = 1.0, omx = 0.0, u = 0.0, omu = 1.0, v = 0.0, rho = 0.0, y = 0.0, J = 1.0, den = 1.0, kk;
   double x1 = 0.0;  // the numerator density's momentum fraction
   if (!ini) {
-    rho = y = tw / (z * omz * s);
+    rho = y = gm_div(tw, z * omz * s);
     double soft = z * y;
     if (type == kFI) {
-      xm = 1.0 / (1.0 + rho);
-      omx = rho / (1.0 + rho);
+      xm = gm_div(1.0, 1.0 + rho);
+      omx = gm_div(rho, 1.0 + rho);
       soft = omx;
       x1 = eta * (1.0 + rho);
     }
-    const double den = omz + soft;
-    if (ch == 0) kk = kCF * (2.0 / den - (1.0 + z));
-    else if (ch == 1) kk = kCA / 2.0 * (2.0 / den - 2.0 + z * omz);
-    else kk = P.nf * kTR / 2.0 * (1.0 - 2.0 * z * omz);
+    den = omz + soft;
   } else {
-    const double r = tw / s;
+    const double r = gm_div(tw, s);
     if (type == kIF) {
       if (!if_map(r, z, omz, xm, omx, u, omu)) return;
-      J = 1.0 / (xm * omu + u * omx);
+      J = gm_div(1.0, xm * omu + u * omx);
     } else {
       if (!ii_map(r, z, omz, xm, omx, v)) return;
-      J = 1.0 / z;
+      J = gm_div(1.0, z);
     }
     if (!(xm > eta)) return;
-    x1 = eta / xm;
-    const double soft = (type == kIF) ? (omx + u) : omx;
-    if (ch == 3) kk = kCF * (2.0 / soft - (1.0 + xm));
-    else if (ch == 4) kk = kTR * (1.0 - 2.0 * xm * omx);
-    else if (ch == 5) kk = kCA * (1.0 / soft + omx / xm - 1.0 + xm * omx);
-    else kk = kCF / 2.0 * (xm + 2.0 * omx / xm);
+    x1 = gm_div(eta, xm);
+    den = (type == kIF) ? (omx + u) : omx;
   }
-  const double as_ratio = alpha_s(P, tw) / R.as_over;
+  // the kernels' soft poles, one division for all channels
+  const double pole = gm_div(ch == 5 ? 1.0 : 2.0, den);
+  if (ch == 0) kk = kCF * (pole - (1.0 + z));
+  else if (ch == 1) kk = kCA / 2.0 * (pole - 2.0 + z * omz);
+  else if (ch == 2) kk = P.nf * kTR / 2.0 * (1.0 - 2.0 * z * omz);
+  else if (ch == 3) kk = kCF * (pole - (1.0 + xm));
+  else if (ch == 4) kk = kTR * (1.0 - 2.0 * xm * omx);
+  else if (ch == 5) kk = kCA * (pole + gm_div(omx, xm) - 1.0 + xm * omx);
+  else kk = kCF / 2.0 * (xm + gm_div(2.0 * omx, xm));
+  const double as_ratio = gm_div(alpha_s(P, tw), R.as_over);
   double wgt, sumF = 0.0;
   PdfLoc l1;
   l1.ok = false;
   if (type == kFF) {
-    wgt = as_ratio * (1.0 - y) * kk / pover;
+    wgt = gm_div(as_ratio * (1.0 - y) * kk, pover);
   } else {
     // the two points' cells: one Q^2 location for both
     PdfLoc l0;
@@ -315,33 +354,34 @@ __device__ __forceinline__ void weigh(const DevParams& P, const Scratch& w, cons
     int num, den;
     if (type == kFI) num = den = pdf_index(w.tag[bk].f);
     else isr_pdf_indices(ch, fl_i, num, den);
-    const double F0 = pdf_at(P, den, l0);
+    const double F0 = xf_at(P, den, l0);
     double F1;
     if (ch == 6) {
       F1 = 0.0;
-      for (int f = 1; f <= 10; ++f) F1 += pdf_at(P, f, l1);
+#pragma unroll 1
+      for (int f = 1; f <= 10; ++f) F1 += xf_at(P, f, l1);
       sumF = F1;
     } else {
-      F1 = pdf_at(P, num, l1);
+      F1 = xf_at(P, num, l1);
     }
     if (type == kFI) {
-      const double ratio = (F0 > 0.0) ? xm * F1 / F0 : 0.0;
-      wgt = as_ratio * kk / pover * ratio / x.B[c];
+      const double ratio = (F0 > 0.0) ? gm_div(xm * F1, F0) : 0.0;
+      wgt = gm_div(gm_div(as_ratio * kk, pover) * ratio, x.B[c]);
     } else {
-      double Fratio = (F0 > 0.0) ? F1 / F0 : 0.0;
+      double Fratio = (F0 > 0.0) ? gm_div(F1, F0) : 0.0;
       const double m2 = heavy_m2(P, type, fl_i);
-      if (m2 > 0.0) Fratio = Fratio * ((tw - m2) / tw);  // heavy-quark measure correction
-      wgt = as_ratio * kk * J * xm / pover * Fratio / x.B[c];
+      if (m2 > 0.0) Fratio = Fratio * gm_div(tw - m2, tw);  // heavy-quark measure correction
+      wgt = gm_div(gm_div(as_ratio * kk * J * xm, pover) * Fratio, x.B[c]);
       if (ch == 4) { W.new_fl = 21; W.fl_j = -fl_i; }
       if (ch == 5) { W.new_fl = 21; W.fl_j = 21; }
     }
   }
   if (!isfinite(wgt)) { W.outcome = kNumericW; return; }
   W.violation = wgt > 1.0;
-  if (!(u01(o1[0], o1[1]) < wgt)) return;
+  if (!(u01(o1.x, o1.y) < wgt)) return;
 
   // accepted: flavours
-  const double Rfl = u01(o2[0], o2[1]);
+  const double Rfl = u01(o2.x, o2.y);
   if (ch == 2) {
     int f = 1 + (int)floor(Rfl * P.nf);
     if (f > P.nf) f = P.nf;
@@ -349,15 +389,16 @@ __device__ __forceinline__ void weigh(const DevParams& P, const Scratch& w, cons
   } else if (ch == 6) {
     double target = Rfl * sumF, acc = 0.0;
     int pick = 10;
+#pragma unroll 1
     for (int f = 1; f <= 10; ++f) {
-      acc += pdf_at(P, f, l1);
+      acc += xf_at(P, f, l1);
       if (target < acc) { pick = f; break; }
     }
     const int fl = pick <= 5 ? pick : -(pick - 5);
     W.new_fl = fl; W.fl_j = fl;
   }
   W.outcome = n >= P.nmax ? kCapacity : kAccept;
-  W.Rphi = u01(o1[2], o1[3]);
+  W.Rphi = u01(o1.z, o1.w);
   if (type == kFF) { W.a0 = y; W.a1 = W.a2 = W.a3 = 0.0; }
   else if (type == kFI) { W.a0 = rho; W.a1 = W.a2 = W.a3 = 0.0; }
   else if (type == kIF) { W.a0 = xm; W.a1 = omx; W.a2 = u; W.a3 = omu; }
@@ -366,29 +407,29 @@ __device__ __forceinline__ void weigh(const DevParams& P, const Scratch& w, cons
 
 // Minkowski product of group-distributed four-vectors (lane mu holds component
 // mu, lanes 4.. the same again), summed in dot4's order
-__device__ __forceinline__ double gdot(double a, double b) {
+__device__ __forceinline__ double gdot(const Group& g, double a, double b) {
   const double m = a * b;
-  return gshfl(m, 0) - gshfl(m, 1) - gshfl(m, 2) - gshfl(m, 3);
+  return g.get(m, 0) - g.get(m, 1) - g.get(m, 2) - g.get(m, 3);
 }
 
-// The emission of group's winner W (lane f's copy, broadcast): kinematics with
-// one momentum component per lane (lanes 4..7 repeat 0..3), the II kick with
+// The emission of the group's winner W (lane f's copy, broadcast): kinematics with
+// one momentum component per lane (lanes 4.. repeat 0..3), the II kick with
 // one parton per lane, colours on lane 0. All lanes of the warp take part;
 // groups with on = false compute on slot 0 and write nothing.
-__device__ __forceinline__ void emission(const Scratch& w, bool on, int n, const Winner& W, int f, double& eta0,
+__device__ __forceinline__ void emission(const Group& g, const Scratch& w, bool on, int n, const Winner& W, int f, double& eta0,
                                       double& eta1) {
-  const int gl = threadIdx.x & (kG - 1), mu = gl & 3;
-  const int pack = gshfl(W.type | (W.ch << 2) | (W.side << 5) | (W.bi << 6) | (W.bk << 14), f);
+  const int gl = g.lane(), mu = gl & 3;
+  const int pack = g.get(W.type | (W.ch << 2) | (W.side << 5) | (W.bi << 6) | (W.bk << 14), f);
   const int type = pack & 3, ch = (pack >> 2) & 7, side = (pack >> 5) & 1;
   const int bi = on ? (pack >> 6) & 0xff : 0, bk = on ? (pack >> 14) & 0xff : 0;
-  const int new_fl = gshfl(W.new_fl, f), fl_j = gshfl(W.fl_j, f);
-  const double z = gshfl(W.z, f), omz = gshfl(W.omz, f), tw = gshfl(W.t, f), Rphi = gshfl(W.Rphi, f);
-  const double a0 = gshfl(W.a0, f), a1 = gshfl(W.a1, f), a2 = gshfl(W.a2, f), a3 = gshfl(W.a3, f);
+  const int new_fl = g.get(W.new_fl, f), fl_j = g.get(W.fl_j, f);
+  const double z = g.get(W.z, f), omz = g.get(W.omz, f), tw = g.get(W.t, f), Rphi = g.get(W.Rphi, f);
+  const double a0 = g.get(W.a0, f), a1 = g.get(W.a1, f), a2 = g.get(W.a2, f), a3 = g.get(W.a3, f);
   const double Pm = w.p[4 * bi + mu], K = w.p[4 * bk + mu];
   // transverse basis (physics_fp64.cuh's steps)
-  const double PK = gdot(Pm, K);
-  const double N = 1.0 + 2.0 * Pm * K / PK;
-  const double N1 = gshfl(N, 1), N2 = gshfl(N, 2), N3 = gshfl(N, 3);
+  const double PK = gdot(g, Pm, K);
+  const double N = 1.0 + gm_div(2.0 * Pm * K, PK);
+  const double N1 = g.get(N, 1), N2 = g.get(N, 2), N3 = g.get(N, 3);
   int a = 1;
   double Na = N1;
   if (N2 > Na) { a = 2; Na = N2; }
@@ -397,18 +438,18 @@ __device__ __forceinline__ void emission(const Scratch& w, bool on, int n, const
   if (a == 1) b = (N3 > N2) ? 3 : 2;
   else if (a == 2) b = (N3 > N1) ? 3 : 1;
   else b = (N2 > N1) ? 2 : 1;
-  const double na = sqrt(Na);
+  const double na = gm_sqrt(Na);
   // K_a / PK, P_a / PK, K_b / PK, P_b / PK: one division, on lanes 0..3
-  const double Ka = gshfl(K, a), Pa = gshfl(Pm, a), Kb = gshfl(K, b), Pb = gshfl(Pm, b);
-  const double dv = (mu == 0 ? Ka : mu == 1 ? Pa : mu == 2 ? Kb : Pb) / PK;
-  const double KaP = gshfl(dv, 0), PaP = gshfl(dv, 1), KbP = gshfl(dv, 2), PbP = gshfl(dv, 3);
-  const double e1 = (((mu == a) ? 1.0 : 0.0) + KaP * Pm + PaP * K) / na;
-  const double e1b = gshfl(e1, b);
+  const double Ka = g.get(K, a), Pa = g.get(Pm, a), Kb = g.get(K, b), Pb = g.get(Pm, b);
+  const double dv = gm_div(mu == 0 ? Ka : mu == 1 ? Pa : mu == 2 ? Kb : Pb, PK);
+  const double KaP = g.get(dv, 0), PaP = g.get(dv, 1), KbP = g.get(dv, 2), PbP = g.get(dv, 3);
+  const double e1 = gm_div(((mu == a) ? 1.0 : 0.0) + KaP * Pm + PaP * K, na);
+  const double e1b = g.get(e1, b);
   const double rperp = ((mu == b) ? 1.0 : 0.0) + KbP * Pm + PbP * K;
   const double e2p = rperp - e1b * e1;
-  const double n2 = sqrt(-gdot(e2p, e2p));
-  const double e2 = e2p / n2;
-  const double st = sqrt(tw);
+  const double n2 = gm_sqrt(-gdot(g, e2p, e2p));
+  const double e2 = gm_div(e2p, n2);
+  const double st = gm_sqrt(tw);
   double cph, sph;
   gm_sincos2pi(Rphi, cph, sph);  // phi = 2 pi R_phi
   const double kt = st * (cph * e1 + sph * e2);
@@ -424,15 +465,15 @@ __device__ __forceinline__ void emission(const Scratch& w, bool on, int n, const
     pk = xinv * K;
     if (on) { if (bk == 0) eta0 = eta0 * xinv; else eta1 = eta1 * xinv; }
   } else {
-    pi = Pm / a0;
+    pi = gm_div(Pm, a0);
     if (type == kIF) {
-      pj = (a3 * a1 / a0) * Pm + a2 * K - kt;
-      pk = (a2 * a1 / a0) * Pm + a3 * K + kt;
+      pj = gm_div(a3 * a1, a0) * Pm + a2 * K - kt;
+      pk = gm_div(a2 * a1, a0) * Pm + a3 * K + kt;
     } else {
-      pj = ((a1 - a2) / a0) * Pm + a2 * K - kt;
+      pj = gm_div(a1 - a2, a0) * Pm + a2 * K - kt;
       pk = K;
     }
-    if (on) { if (bi == 0) eta0 = eta0 / a0; else eta1 = eta1 / a0; }
+    if (on) { const double en = gm_div(bi == 0 ? eta0 : eta1, a0); if (bi == 0) eta0 = en; else eta1 = en; }
   }
   __syncwarp();  // every lane has read its old momenta
   if (on && gl < 4) {
@@ -445,15 +486,15 @@ __device__ __forceinline__ void emission(const Scratch& w, bool on, int n, const
     const double kp = Pm + K, kn = (pi + K) - pj, kq = kp + kn;
     double Kp[4], Kn[4], KK[4];
 #pragma unroll
-    for (int m = 0; m < 4; ++m) { Kp[m] = gshfl(kp, m); Kn[m] = gshfl(kn, m); KK[m] = gshfl(kq, m); }
+    for (int m = 0; m < 4; ++m) { Kp[m] = g.get(kp, m); Kn[m] = g.get(kn, m); KK[m] = g.get(kq, m); }
     if (on && type == kII) {
       const double KK2 = dot4(KK, KK), Kp2 = dot4(Kp, Kp);
-      for (int m = 2 + gl; m < n; m += kG) {
+      for (int m = 2 + gl; m < n; m += g.G) {
         double v[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) v[j] = w.p[4 * m + j];
-        const double ka = 2.0 * dot4(KK, v) / KK2;
-        const double kb = 2.0 * dot4(Kp, v) / Kp2;
+        const double ka = gm_div(2.0 * dot4(KK, v), KK2);
+        const double kb = gm_div(2.0 * dot4(Kp, v), Kp2);
 #pragma unroll
         for (int j = 0; j < 4; ++j) w.p[4 * m + j] = v[j] - ka * KK[j] + kb * Kn[j];
       }
@@ -509,17 +550,340 @@ __device__ __forceinline__ float screen_error(float ic, float lr, float v, float
 // slack of a comparison with a logarithm formed in FP32 (|ln| < 64)
 constexpr float kLnSlack = 1e-4f;
 
+// An event in flight, the same in every lane of its group
+struct Event {
+  bool active = false, table = false;  // table: the end table has to be formed
+  uint64_t e = 0, id = 0, draw = 0;
+  int n = 0, n_emit = 0, steps = 0, row = 0, status = GAPS_STATUS_ACTIVE;
+  int nblk = 0;  // trial blocks of a cycle
+  int chg = -1;  // emitter | spectator << 8 of the emission since the last table, -1: all ends
+  double t = 0.0, eta0 = 0.0, eta1 = 0.0;
+};
+
+// One batch of up to K <= g.G cycles of every group's event, with the end table
+// before and the emission after it. All lanes of the warp call it.
+__device__ __forceinline__ void batch(const Group g, int K, const DevParams& P, const DevEvents& E, const Scratch& w, const RowShared* rows,
+                                      const float* m2f, unsigned char* list, Event& S, Counters& cnt, bool heavy_table) {
+  const int G = g.G, gl = g.lane();
+  const uint32_t k0 = (uint32_t)P.seed, k1 = (uint32_t)(P.seed >> 32);
+  const RowShared& R = rows[S.row];
+  const int ne = S.active ? 2 * S.n : 0;
+  __syncwarp();
+
+  // ---- end table: the ends the last emission touched (all: chg < 0) ----
+  if (__any_sync(kAll, S.table)) {
+    // the ends to form, gathered first so that they fill the group's lanes
+    const int ci = S.chg & 0xff, ck = (S.chg >> 8) & 0xff, T = 99 + S.n;
+    int todo = 0;
+    const int scans = __reduce_max_sync(kAll, S.table ? (ne + G - 1) / G : 0);
+    for (int r = 0; r < scans; ++r) {
+      const int q = r * G + gl;
+      bool form = S.table && q < ne;
+      if (form && S.chg >= 0 && q < ne - 2) {
+        // an end away from the emitter, the spectator and the new parton
+        // whose partner is neither of them keeps its record: its inputs did
+        // not change; one without a partner or with the new tag is matched
+        // again
+        const int i = q >> 1, k = w.end[q].k;
+        const Tag ti = w.tag[i];
+        const int tag = (q & 1) ? ti.a : ti.c;
+        form = !(i != ci && i != ck && k != ci && k != ck && (tag == 0 || (k >= 0 && tag != T)));
+      }
+      const unsigned m = g.ballot(form);
+      if (form) list[todo + __popc(m & ((1u << gl) - 1u))] = (unsigned char)q;
+      todo += __popc(m);
+    }
+    __syncwarp();
+    for (int j = gl; j < todo; j += G) form_end(P, w, R, S.n, list[j], S.eta0, S.eta1);
+    __syncwarp();
+    // trial blocks before each end, and of a cycle
+    int run = 0;
+    for (int r = 0; r < scans; ++r) {
+      const int q = r * G + gl;
+      int nd = 0;
+      float4 sc = make_float4(-1.0f, -1.0f, 0.0f, 0.0f);
+      if (S.table && q < ne) {
+        sc = w.scr[q];
+        nd = (sc.x >= 0.0f ? 1 : 0) + (sc.y >= 0.0f ? 1 : 0);
+      }
+      int inc = nd;
+#pragma unroll 1
+      for (int o = 1; o < G; o <<= 1) {
+        const int v = __shfl_up_sync(kAll, inc, o, G);
+        if (gl >= o) inc += v;
+      }
+      if (S.table && q < ne) w.scr[q].w = __int_as_float(run + inc - nd);
+      run += g.get(inc, G - 1);
+    }
+    if (S.table) S.nblk = run;
+    S.table = false;
+    __syncwarp();
+  }
+
+  // ---- screening: the winners of up to K cycles ----------------------
+  const uint32_t e0 = (uint32_t)S.id, e1 = (uint32_t)(S.id >> 32);
+  const float lnTc = R.lnTc;
+  float lnT = S.active ? __logf((float)S.t) : 0.0f, eT = 2e-6f + fabsf(lnT) * 4e-7f;
+  int len = 0;                  // cycles with a winner
+  bool ends_done = false;       // the cycle after them has no trial above the cutoff
+  bool going = S.active;        // the batch can take another cycle
+  int my_q = 0, my_c = 0;       // winner of cycle gl
+  int my_trials = 0;            // trials of cycle gl: all | initial-state << 16
+  const bool live_t = S.t > R.t_cut;
+#pragma unroll 1
+  for (int k = 0; k < K; ++k) {
+    if (!__any_sync(kAll, going)) break;
+    const uint64_t dk = S.draw + (uint64_t)k * (uint64_t)(S.nblk + 2);
+    float u1 = -INFINITY, u2 = -INFINITY, lmax = -INFINITY, v1 = 0.0f, er1 = 0.0f;
+    int i1 = 0, nt = 0;
+    bool doubt = false;
+    if (going && live_t) {
+#pragma unroll 1
+      for (int q = gl; q < ne; q += G) {
+        const float4 sc = w.scr[q];
+        // (no FP64 instruction in this loop: it would wait for the other warps')
+        float mf = 0.0f;
+        if (heavy_table && q < 4 && R.pp && sc.x >= 0.0f) {
+          const int fe = pdf_index(w.tag[q >> 1].f);
+          mf = fe > 0 ? m2f[fe] : 0.0f;
+        }
+        // the blocks of both channels side by side (two chains of products)
+        uint32_t oc[2][4];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          const uint64_t d = dk + (uint64_t)(__float_as_int(sc.w) + c);
+          philox(e0, e1, (uint32_t)d, (uint32_t)(d >> 32), k0, k1, oc[c]);
+        }
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          const float ic = c == 0 ? sc.x : sc.y;
+          if (!(ic >= 0.0f && ic < INFINITY)) continue;  // absent, or no trial
+          const uint32_t* o = oc[c];
+          const float lnTm = fminf(lnT, sc.z);
+          float x = fmaf((float)o[0], 1.0f / 4294967296.0f, (float)o[1]) * (1.0f / 4294967296.0f);
+          const bool tiny = o[1] < 16u;  // R below 2^-28: only an upper bound
+          if (tiny) x = 3.7252903e-9f;
+          const float lr = __logf(x);
+          float v = fmaf(lr, ic, lnTm);
+          float er = screen_error(ic, lr, v, lnTm, eT);
+          bool sure = !tiny && ic < 1e30f;
+          if (mf > 0.0f) {
+            // the heavy-quark measure: t = m^2 + (t_max - m^2) R^(1/c) is at
+            // least t_max R^(1/c), so its relative error is not larger
+            const float lnF = __logf(mf * (1.0f + (float)kHqFloor));
+            if (lnTm < lnF + kLnSlack) {
+              doubt = doubt || lnTm > lnF - kLnSlack;  // whether it draws is close
+              if (lnTm <= lnF - kLnSlack) continue;
+            }
+            v = __logf(mf + (__expf(lnTm) - mf) * __expf(fmaxf(lr * ic, -80.0f)));
+            er += kLnSlack;
+            if (v < lnF + kLnSlack) sure = false;  // may be below the channel's floor
+            if (v + er < lnF - kLnSlack) { ++nt; if (q < 4 && R.pp) nt += 1 << 16; continue; }
+          }
+          nt += (q < 4 && R.pp) ? 1 + (1 << 16) : 1;
+          const float ub = v + er;
+          if (sure) lmax = fmaxf(lmax, v - er);
+          if (ub > u1) { u2 = u1; u1 = ub; v1 = v; er1 = er; i1 = 2 * q + c; }
+          else u2 = fmaxf(u2, ub);
+        }
+      }
+    }
+    const float Lm = g.max(lmax);
+    const unsigned cand = g.ballot(u1 >= Lm && u1 > -INFINITY);
+    const unsigned second = g.ballot((u2 >= Lm && u2 > -INFINITY) || doubt);
+    // no trial above the cutoff
+    const bool below = !g.ballot(u1 >= lnTc - kLnSlack || doubt);
+    if (heavy_table || k == 0) {
+      const int s = g.sum(nt);
+      if (heavy_table ? gl == k : true) my_trials = s;
+    }
+    const int wl = __ffs(cand) - 1;
+    const float wv = g.get(v1, wl < 0 ? 0 : wl), we = g.get(er1, wl < 0 ? 0 : wl);
+    const int wi = g.get(i1, wl < 0 ? 0 : wl);
+    // (some channel's lower bound is finite, and it alone reaches it)
+    const bool clear = !below && Lm > -INFINITY && __popc(cand) == 1 && !second;
+    // a first cycle that the bounds do not decide: exact trials of the
+    // channels in question
+    const bool decide = going && k == 0 && !below && !clear;
+    int xi = -1;
+    if (__any_sync(kAll, decide)) {
+      double bt = -1.0;
+      int bidx = 0x7fffffff, xt = 0;
+      if (decide) {
+        for (int q = gl; q < ne; q += G) {
+          const float4 sc = w.scr[q];
+          for (int c = 0; c < 2; ++c) {
+            const float ic = c == 0 ? sc.x : sc.y;
+            if (!(ic >= 0.0f && ic < INFINITY)) continue;
+            const uint64_t d = dk + (uint64_t)(__float_as_int(sc.w) + c);
+            const uint4 o = block_of(S.id, d, k0, k1);
+            const EndX& x = w.end[q];
+            bool counted;
+            const double tt = exact_trial(x, c, heavy_m2(P, x.type, w.tag[q >> 1].f), S.t, R.t_cut, u01(o.x, o.y),
+                                          counted);
+            if (counted) xt += (q < 4 && R.pp) ? 1 + (1 << 16) : 1;
+            if (tt > bt) { bt = tt; bidx = 2 * q + c; }
+          }
+        }
+      }
+#pragma unroll 1
+      for (int o = G / 2; o > 0; o >>= 1) {
+        const double ot = g.xchg(bt, o);
+        const int oi = g.xchg(bidx, o);
+        if (ot > bt || (ot == bt && oi < bidx)) { bt = ot; bidx = oi; }
+      }
+      const int s = g.sum(xt);
+      if (decide) {
+        if (!heavy_table || gl == 0) my_trials = s;
+        if (bidx != 0x7fffffff) xi = bidx;
+      }
+    }
+    if (going) {
+      if (below || (decide && xi < 0)) {
+        ends_done = true;
+        going = false;
+      } else if (clear || decide) {
+        const int win = clear ? wi : xi;
+        if (gl == k) { my_q = win >> 1; my_c = win & 1; }
+        len = k + 1;
+        lnT = wv;
+        eT = we;
+        // near or below the cutoff, or decided exactly: the batch ends here
+        if (decide || wv - we < lnTc + kLnSlack) going = false;
+      } else {
+        going = false;  // not decided in FP32: the next batch begins with it
+      }
+    }
+  }
+
+  // ---- exact scales and weights: lane j evaluates cycle j --------------
+  Winner W;
+  W.outcome = kVeto;
+  W.violation = false;
+  W.t = 0.0;
+  W.type = W.ch = W.bi = W.bk = W.side = W.new_fl = W.fl_j = 0;
+  W.z = W.omz = W.Rphi = W.a0 = W.a1 = W.a2 = W.a3 = 0.0;
+  const bool mine = S.active && gl < len;
+  const uint64_t dm = S.draw + (uint64_t)gl * (uint64_t)(S.nblk + 2);
+  double pw = 1.0, tkin = 0.0, m2 = 0.0, Rz = 0.5;
+  if (mine) {
+    const EndX& x = w.end[my_q];
+    const float4 sc = w.scr[my_q];
+    const uint64_t d = dm + (uint64_t)(__float_as_int(sc.w) + my_c);
+    const uint4 o = block_of(S.id, d, k0, k1);
+    Rz = u01(o.z, o.w);
+    pw = gm_exp(gm_div(gm_log(u01(o.x, o.y)), x.cc[my_c]));
+    tkin = x.tkin;
+    if (heavy_table) m2 = heavy_m2(P, x.type, w.tag[my_q >> 1].f);
+  }
+  double my_t = 0.0, tc = S.t;
+  const int most = __reduce_max_sync(kAll, S.active ? len : 0);
+  for (int k = 0; k < most; ++k) {
+    const double tmax = fmin(tc, tkin);
+    const double tt = m2 > 0.0 ? m2 + (tmax - m2) * pw : tmax * pw;
+    if (gl == k) my_t = tt;
+    tc = g.get(tt, k);
+  }
+  if (mine) {
+    const uint64_t d1 = dm + (uint64_t)S.nblk;
+    const uint4 o1 = block_of(S.id, d1, k0, k1), o2 = block_of(S.id, d1 + 1, k0, k1);
+    weigh(P, w, R, S.n, my_q, my_c, my_t, Rz, o1, o2, W);
+  }
+
+  // ---- commit: the cycles up to the first that was not vetoed ----------
+  const unsigned other = g.ballot(mine && W.outcome != kVeto);
+  const int room = P.max_steps - S.steps;  // cycles before the cap
+  int f = other ? __ffs(other) - 1 : -1;
+  if (f >= room) f = -1;
+  int done_cycles = f >= 0 ? f + 1 : min(len, room);  // committed
+  const int out = g.get(W.outcome, f < 0 ? 0 : f);
+  const bool viol = g.get((int)W.violation, f < 0 ? 0 : f) != 0;
+  const bool tail_done = f < 0 && ends_done && done_cycles == len && len < room;
+  // scale after the committed cycles (a cycle that ends without a veto test
+  // leaves it)
+  const int tl = f >= 0 && (out == kDone || out == kNumericT) ? f - 1 : done_cycles - 1;
+  const double tn = g.get(my_t, tl < 0 ? 0 : tl);
+  bool accepted = false;
+  if (S.active) {
+    const int counted = done_cycles + (tail_done ? 1 : 0);
+    if (!heavy_table ? gl == 0 : gl < counted) {
+      const unsigned long long times = heavy_table ? 1 : (unsigned long long)counted;
+      cnt.trials += times * (unsigned long long)(my_trials & 0xffff);
+      cnt.isr_trials += times * (unsigned long long)(my_trials >> 16);
+    }
+    if (tl >= 0) S.t = tn;
+    S.steps += counted;
+    S.draw += (uint64_t)done_cycles * (uint64_t)(S.nblk + 2);
+    if (tail_done) S.draw += (uint64_t)S.nblk;
+    if (f >= 0 && (out == kDone || out == kNumericT)) S.draw -= 2;
+    if (gl == 0) {
+      cnt.steps += counted;
+      cnt.vetoes += f >= 0 ? f : done_cycles;
+      if (f >= 0 && viol) cnt.violations += 1;
+    }
+    int st = GAPS_STATUS_ACTIVE;
+    if (tail_done || (f >= 0 && out == kDone)) st = GAPS_STATUS_DONE;
+    else if (f >= 0 && (out == kNumericT || out == kNumericW)) st = GAPS_ERR_NUMERIC;
+    else if (f >= 0 && out == kCapacity) st = GAPS_ERR_CAPACITY;
+    else if (f >= 0) accepted = true;
+    if (st == GAPS_STATUS_ACTIVE && S.steps >= P.max_steps) st = GAPS_ERR_ITER_CAP;
+    S.status = st;
+  }
+
+  // ---- emission --------------------------------------------------------
+  if (__any_sync(kAll, accepted)) {
+    emission(g, w, accepted, S.n, W, f < 0 ? 0 : f, S.eta0, S.eta1);
+    const int pack = g.get(W.type | (W.bi << 2) | (W.bk << 10), f < 0 ? 0 : f);
+    if (accepted) {
+      S.chg = (pack & 3) == kII ? -1 : ((pack >> 2) & 0xff) | (((pack >> 10) & 0xff) << 8);
+      S.n += 1;
+      S.n_emit += 1;
+      if (gl == 0) cnt.accepts += 1;
+      S.table = true;
+    }
+  }
+
+  // ---- finished events back into the caller's records ------------------
+  if (S.active && S.status != GAPS_STATUS_ACTIVE) {
+    for (int s = gl; s < S.n; s += G) {
+#pragma unroll
+      for (int mu = 0; mu < 4; ++mu) E.P(mu, s, S.e) = w.p[4 * s + mu];
+      const Tag tg = w.tag[s];
+      E.F(s, S.e) = tg.f;
+      E.C(s, S.e) = tg.c;
+      E.A(s, S.e) = tg.a;
+    }
+    if (gl == 0) {
+      E.npart[S.e] = S.n;
+      E.t[S.e] = S.t;
+      E.eta[S.e] = S.eta0;
+      E.eta[E.cap + S.e] = S.eta1;
+      E.n_emit[S.e] = S.n_emit;
+      E.draw[S.e] = S.draw;
+      E.status[S.e] = S.status;
+      if (S.status == GAPS_ERR_CAPACITY) cnt.err_cap += 1;
+      else if (S.status == GAPS_ERR_ITER_CAP) cnt.err_iter += 1;
+      else if (S.status == GAPS_ERR_NUMERIC) cnt.err_num += 1;
+    }
+    S.active = S.table = false;
+  }
+  __syncwarp();
+}
+
 __global__ void __launch_bounds__(kThreads, kMinBlocks)
     k_shower_fp64(const __grid_constant__ DevParams P, const __grid_constant__ DevEvents E, uint64_t first, uint64_t n_events,
                   unsigned per_block, unsigned char* pool, unsigned* taken, unsigned regions, int heavy_table) {
   __shared__ RowShared rows[kMaxRows];
+  __shared__ float m2f[12];
+  __shared__ unsigned char s_list[kGroups][256];
   __shared__ int s_region;
   __shared__ unsigned s_next;
-  const int tid = threadIdx.x, lane = tid & 31, gl = tid & (kG - 1), gw = lane / kG;
+  const int tid = threadIdx.x, lane = tid & 31, gl = tid & (kG - 1);
   if (tid < kMaxRows) {
     const RowParams& r = P.rows[tid < P.n_rows ? tid : 0];
-    rows[tid] = RowShared{r.t_cut, r.as_over, (float)gm_log(r.t_cut), r.process != GAPS_EE_QQ};
+    rows[tid] = RowShared{r.t_cut, r.as_over, r.as_over / (2.0 * kPi), (float)gm_log(r.t_cut), r.process != GAPS_EE_QQ};
   }
+  if (tid < 12) m2f[tid] = (float)P.m2[tid];
   if (tid == 0) {
     s_next = 0;
     // a free part of the scratch pool: it has one for every block that can be
@@ -537,351 +901,78 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
   __syncthreads();
   if (s_region < 0) return;  // cannot happen: see above (the events stay active)
   const size_t slot = (size_t)s_region * kGroups + tid / kG;
-  const Scratch w = scratch_of(pool + slot * (size_t)P.nmax * kSlotBytesPerParton, P.nmax);
+  Scratch w = scratch_of(pool + slot * (size_t)P.nmax * kSlotBytesPerParton, P.nmax);
   const uint64_t block0 = (uint64_t)blockIdx.x * per_block;
   const unsigned block_n = (unsigned)(n_events - block0 < per_block ? n_events - block0 : per_block);
-  // event j of the block starts in warp j % 4: few events spread over the warps
-  const uint32_t k0 = (uint32_t)P.seed, k1 = (uint32_t)(P.seed >> 32);
 
   Counters cnt;
-  bool active = false, exhausted = false;
-  uint64_t e = 0, id = 0, draw = 0;
-  int n = 0, n_emit = 0, steps = 0, row = 0, status = GAPS_STATUS_ACTIVE;
-  int nblk = 0;          // trial blocks of a cycle
-  int chg = -1;          // emitter | spectator << 8 of the emission since the last table, -1: all ends
-  bool table = false;    // the end table has to be formed
-  double t = 0.0, eta0 = 0.0, eta1 = 0.0;
-  bool first_take = true;
+  Event S;
+  Group g{kG};
+  bool exhausted = false, first_take = true;
   while (true) {
     // ---- a new event for every idle group ------------------------------
-    while (__any_sync(kAll, !active && !exhausted)) {
-      unsigned j = 0xffffffffu;
-      if (first_take) {
-        j = (unsigned)(tid >> 5) + (kThreads / 32) * (unsigned)gw;  // groups take 0 .. kGroups - 1 first
-      } else {
-        if (gl == 0 && !active && !exhausted) j = kGroups + atomicAdd(&s_next, 1u);
-        j = (unsigned)gshfl((int)j, 0);
+    while (__any_sync(kAll, !S.active && !exhausted)) {
+      // the block's first events one to a group, spread over the warps first
+      unsigned j = (unsigned)(tid >> 5) + (kThreads / 32) * (unsigned)(lane / kG);
+      if (!first_take) {
+        if (gl == 0 && !S.active && !exhausted) j = kGroups + atomicAdd(&s_next, 1u);
+        j = __shfl_sync(kAll, j, 0, kG);
       }
       first_take = false;
-      if (active || exhausted) continue;
+      if (S.active || exhausted) continue;
       if (j >= block_n) { exhausted = true; continue; }
-      e = block0 + j;
-      id = first + e;
+      const uint64_t e = block0 + j;
+      S.e = e;
+      S.id = first + e;
       if (gl == 0) cnt.finished += 1;
-      status = E.status[e];
-      if (status != GAPS_STATUS_ACTIVE) continue;
-      n = E.npart[e];
-      row = mix_row(P, id);
-      if (n < 2 || n > P.nmax) {  // not a record written by the hard-process kernel
+      S.status = E.status[e];
+      if (S.status != GAPS_STATUS_ACTIVE) continue;
+      S.n = E.npart[e];
+      S.row = mix_row(P, S.id);
+      if (S.n < 2 || S.n > P.nmax) {  // not a record written by the hard-process kernel
         if (gl == 0) { E.status[e] = GAPS_ERR_NUMERIC; cnt.err_num += 1; }
         continue;
       }
-      for (int s = gl; s < n; s += kG) {
+      for (int s = gl; s < S.n; s += kG) {
 #pragma unroll
         for (int mu = 0; mu < 4; ++mu) w.p[4 * s + mu] = E.P(mu, s, e);
         w.tag[s] = Tag{E.F(s, e), E.C(s, e), E.A(s, e), 0};
       }
-      t = E.t[e];
-      eta0 = E.eta[e];
-      eta1 = E.eta[E.cap + e];
-      n_emit = E.n_emit[e];
-      draw = E.draw[e];
-      steps = 0;
-      active = table = true;
-      chg = -1;
+      S.t = E.t[e];
+      S.eta0 = E.eta[e];
+      S.eta1 = E.eta[E.cap + e];
+      S.n_emit = E.n_emit[e];
+      S.draw = E.draw[e];
+      S.steps = 0;
+      S.active = S.table = true;
+      S.chg = -1;
     }
-    if (!__any_sync(kAll, active)) break;
-    const RowShared& R = rows[row];
-    const int ne = active ? 2 * n : 0;
-    __syncwarp();
-
-    // ---- end table: the ends the last emission touched (all: chg < 0) ---
-    if (__any_sync(kAll, table)) {
-      if (table) {
-        const int ci = chg & 0xff, ck = (chg >> 8) & 0xff, T = 99 + n;
-        for (int q = gl; q < ne; q += kG) {
-          if (chg >= 0 && q < ne - 2) {
-            // an end away from the emitter, the spectator and the new parton
-            // whose partner is neither of them keeps its record: its inputs
-            // did not change; one without a partner or with the new tag is
-            // matched again
-            const int i = q >> 1, k = w.end[q].k;
-            const Tag ti = w.tag[i];
-            const int tag = (q & 1) ? ti.a : ti.c;
-            if (i != ci && i != ck && k != ci && k != ck && (tag == 0 || (k >= 0 && tag != T))) continue;
-          }
-          form_end(P, w, R, n, q, eta0, eta1);
-        }
-      }
-      __syncwarp();
-      // trial blocks before each end, and of a cycle
-      int run = 0;
-      const int rounds = (ne + kG - 1) / kG;
-      const int most = __reduce_max_sync(kAll, table ? rounds : 0);
-      for (int r = 0; r < most; ++r) {
-        const int q = r * kG + gl;
-        int nd = 0;
-        float4 sc = make_float4(-1.0f, -1.0f, 0.0f, 0.0f);
-        if (table && q < ne) {
-          sc = w.scr[q];
-          nd = (sc.x >= 0.0f ? 1 : 0) + (sc.y >= 0.0f ? 1 : 0);
-        }
-        int inc = nd;
-#pragma unroll
-        for (int o = 1; o < kG; o <<= 1) {
-          const int v = __shfl_up_sync(kAll, inc, o, kG);
-          if (gl >= o) inc += v;
-        }
-        if (table && q < ne) w.scr[q].w = __int_as_float(run + inc - nd);
-        run += gshfl(inc, kG - 1);
-      }
-      if (table) nblk = run;
-      table = false;
-      __syncwarp();
+    const unsigned act = __ballot_sync(kAll, S.active);
+    if (!act) break;
+    if (g.G == kG && __popc(act) == kG && __all_sync(kAll, S.active || exhausted)) {
+      // the warp's last event: all 32 lanes take it to its end
+      const int src = __ffs(act) - 1;
+      S.active = true;
+      S.table = __shfl_sync(kAll, (int)S.table, src) != 0;
+      S.e = __shfl_sync(kAll, S.e, src);
+      S.id = __shfl_sync(kAll, S.id, src);
+      S.draw = __shfl_sync(kAll, S.draw, src);
+      S.n = __shfl_sync(kAll, S.n, src);
+      S.n_emit = __shfl_sync(kAll, S.n_emit, src);
+      S.steps = __shfl_sync(kAll, S.steps, src);
+      S.row = __shfl_sync(kAll, S.row, src);
+      S.status = GAPS_STATUS_ACTIVE;
+      S.nblk = __shfl_sync(kAll, S.nblk, src);
+      S.chg = __shfl_sync(kAll, S.chg, src);
+      S.t = __shfl_sync(kAll, S.t, src);
+      S.eta0 = __shfl_sync(kAll, S.eta0, src);
+      S.eta1 = __shfl_sync(kAll, S.eta1, src);
+      w = scratch_of(reinterpret_cast<unsigned char*>(
+                         __shfl_sync(kAll, reinterpret_cast<unsigned long long>(w.p), src)), P.nmax);
+      exhausted = true;
+      g.G = 32;
     }
-
-    // ---- screening: the winners of up to kG cycles ----------------------
-    const uint32_t e0 = (uint32_t)id, e1 = (uint32_t)(id >> 32);
-    const float lnTc = R.lnTc;
-    float lnT = active ? __logf((float)t) : 0.0f, eT = 2e-6f + fabsf(lnT) * 4e-7f;
-    int len = 0;                  // cycles with a winner
-    bool ends_done = false;       // the cycle after them has no trial above the cutoff
-    bool going = active;          // the batch can take another cycle
-    int my_q = 0, my_c = 0;       // winner of cycle gl
-    int my_trials = 0;            // trials of cycle gl: all | initial-state << 16
-    const bool live_t = t > R.t_cut;
-#pragma unroll 1
-    for (int k = 0; k < kG; ++k) {
-      if (!__any_sync(kAll, going)) break;
-      const uint64_t dk = draw + (uint64_t)k * (uint64_t)(nblk + 2);
-      float u1 = -INFINITY, u2 = -INFINITY, lmax = -INFINITY, v1 = 0.0f, er1 = 0.0f;
-      int i1 = 0, nt = 0;
-      bool doubt = false;
-      if (going && live_t) {
-#pragma unroll 1
-        for (int q = gl; q < ne; q += kG) {
-          const float4 sc = w.scr[q];
-          double m2 = 0.0;
-          if (heavy_table && q < 4 && R.pp) m2 = sc.x >= 0.0f ? heavy_m2(P, w.end[q].type, w.tag[q >> 1].f) : 0.0;
-#pragma unroll 1
-          for (int c = 0; c < 2; ++c) {
-            const float ic = c == 0 ? sc.x : sc.y;
-            if (!(ic >= 0.0f && ic < INFINITY)) continue;  // absent, or no trial
-            const uint64_t d = dk + (uint64_t)(__float_as_int(sc.w) + c);
-            uint32_t o[4];
-            philox(e0, e1, (uint32_t)d, (uint32_t)(d >> 32), k0, k1, o);
-            const float lnTm = fminf(lnT, sc.z);
-            float x = fmaf((float)o[0], 1.0f / 4294967296.0f, (float)o[1]) * (1.0f / 4294967296.0f);
-            const bool tiny = o[1] < 16u;  // R below 2^-28: only an upper bound
-            if (tiny) x = 3.7252903e-9f;
-            const float lr = __logf(x);
-            float v = fmaf(lr, ic, lnTm);
-            float er = screen_error(ic, lr, v, lnTm, eT);
-            bool sure = !tiny && ic < 1e30f;
-            if (m2 > 0.0) {
-              // the heavy-quark measure: t = m^2 + (t_max - m^2) R^(1/c) is at
-              // least t_max R^(1/c), so its relative error is not larger
-              const float mf = (float)m2, lnF = __logf(mf * (1.0f + (float)kHqFloor));
-              if (lnTm < lnF + kLnSlack) {
-                doubt = doubt || lnTm > lnF - kLnSlack;  // whether it draws is close
-                if (lnTm <= lnF - kLnSlack) continue;
-              }
-              v = __logf(mf + (__expf(lnTm) - mf) * __expf(fmaxf(lr * ic, -80.0f)));
-              er += kLnSlack;
-              if (v < lnF + kLnSlack) sure = false;  // may be below the channel's floor
-              if (v + er < lnF - kLnSlack) { ++nt; if (q < 4 && R.pp) nt += 1 << 16; continue; }
-            }
-            nt += (q < 4 && R.pp) ? 1 + (1 << 16) : 1;
-            const float ub = v + er;
-            if (sure) lmax = fmaxf(lmax, v - er);
-            if (ub > u1) { u2 = u1; u1 = ub; v1 = v; er1 = er; i1 = 2 * q + c; }
-            else u2 = fmaxf(u2, ub);
-          }
-        }
-      }
-      const float U = gmax(u1), Lm = gmax(lmax);
-      const unsigned cand = gballot(u1 >= Lm && u1 > -INFINITY);
-      const unsigned second = gballot(u2 >= Lm && u2 > -INFINITY);
-      const unsigned dmask = gballot(doubt);
-      if (heavy_table || k == 0) {
-        const int s = gsum(nt);
-        if (heavy_table ? gl == k : true) my_trials = s;
-      }
-      const int wl = __ffs(cand) - 1;
-      const float wv = gshfl(v1, wl < 0 ? 0 : wl), we = gshfl(er1, wl < 0 ? 0 : wl);
-      const int wi = gshfl(i1, wl < 0 ? 0 : wl);
-      const bool below = !(U >= lnTc - kLnSlack) && !dmask;  // no trial above the cutoff
-      // (some channel's lower bound is finite, and it alone reaches it)
-      const bool clear = !below && !dmask && Lm > -INFINITY && __popc(cand) == 1 && !second;
-      // a first cycle that the bounds do not decide: exact trials of the
-      // channels in question
-      const bool decide = going && k == 0 && !below && !clear;
-      int xi = -1;
-      if (__any_sync(kAll, decide)) {
-        double bt = -1.0;
-        int bidx = 0x7fffffff, xt = 0;
-        if (decide) {
-          for (int q = gl; q < ne; q += kG) {
-            const float4 sc = w.scr[q];
-            for (int c = 0; c < 2; ++c) {
-              const float ic = c == 0 ? sc.x : sc.y;
-              if (!(ic >= 0.0f && ic < INFINITY)) continue;
-              const uint64_t d = dk + (uint64_t)(__float_as_int(sc.w) + c);
-              uint32_t o[4];
-              philox(e0, e1, (uint32_t)d, (uint32_t)(d >> 32), k0, k1, o);
-              const EndX x = w.end[q];
-              bool counted;
-              const double tt = exact_trial(x, c, heavy_m2(P, x.type, w.tag[q >> 1].f), t, R.t_cut, u01(o[0], o[1]), counted);
-              if (counted) xt += (q < 4 && R.pp) ? 1 + (1 << 16) : 1;
-              if (tt > bt) { bt = tt; bidx = 2 * q + c; }
-            }
-          }
-        }
-#pragma unroll
-        for (int o = kG / 2; o > 0; o >>= 1) {
-          const double ot = __shfl_xor_sync(kAll, bt, o, kG);
-          const int oi = __shfl_xor_sync(kAll, bidx, o, kG);
-          if (ot > bt || (ot == bt && oi < bidx)) { bt = ot; bidx = oi; }
-        }
-        const int s = gsum(xt);
-        if (decide) {
-          if (!heavy_table || gl == 0) my_trials = s;
-          if (bidx != 0x7fffffff) xi = bidx;
-        }
-      }
-      if (going) {
-        if (below || (decide && xi < 0)) {
-          ends_done = true;
-          going = false;
-        } else if (clear || decide) {
-          const int win = clear ? wi : xi;
-          if (gl == k) { my_q = win >> 1; my_c = win & 1; }
-          len = k + 1;
-          lnT = wv;
-          eT = we;
-          // near or below the cutoff, or decided exactly: the batch ends here
-          if (decide || wv - we < lnTc + kLnSlack) going = false;
-        } else {
-          going = false;  // not decided in FP32: the next batch begins with it
-        }
-      }
-    }
-
-    // ---- exact scales and weights: lane j evaluates cycle j --------------
-    Winner W;
-    W.outcome = kVeto;
-    W.violation = false;
-    W.t = 0.0;
-    W.type = W.ch = W.bi = W.bk = W.side = W.new_fl = W.fl_j = 0;
-    W.z = W.omz = W.Rphi = W.a0 = W.a1 = W.a2 = W.a3 = 0.0;
-    const bool mine = active && gl < len;
-    const uint64_t dm = draw + (uint64_t)gl * (uint64_t)(nblk + 2);
-    double pw = 1.0, tkin = 0.0, m2 = 0.0, Rz = 0.5;
-    if (mine) {
-      const EndX& x = w.end[my_q];
-      const float4 sc = w.scr[my_q];
-      const uint64_t d = dm + (uint64_t)(__float_as_int(sc.w) + my_c);
-      uint32_t o[4];
-      philox(e0, e1, (uint32_t)d, (uint32_t)(d >> 32), k0, k1, o);
-      Rz = u01(o[2], o[3]);
-      pw = gm_exp(gm_log(u01(o[0], o[1])) / x.cc[my_c]);
-      tkin = x.tkin;
-      if (heavy_table) m2 = heavy_m2(P, x.type, w.tag[my_q >> 1].f);
-    }
-    double my_t = 0.0, tc = t;
-    const int most = __reduce_max_sync(kAll, active ? len : 0);
-    for (int k = 0; k < most; ++k) {
-      const double tmax = fmin(tc, tkin);
-      const double tt = m2 > 0.0 ? m2 + (tmax - m2) * pw : tmax * pw;
-      if (gl == k) my_t = tt;
-      tc = gshfl(tt, k);
-    }
-    if (mine) {
-      uint32_t o1[4], o2[4];
-      const uint64_t d1 = dm + (uint64_t)nblk, d2 = d1 + 1;
-      philox(e0, e1, (uint32_t)d1, (uint32_t)(d1 >> 32), k0, k1, o1);
-      philox(e0, e1, (uint32_t)d2, (uint32_t)(d2 >> 32), k0, k1, o2);
-      weigh(P, w, R, n, my_q, my_c, my_t, Rz, o1, o2, W);
-    }
-
-    // ---- commit: the cycles up to the first that was not vetoed ----------
-    const unsigned other = gballot(mine && W.outcome != kVeto);
-    const int room = P.max_steps - steps;  // cycles before the cap
-    int f = other ? __ffs(other) - 1 : -1;
-    if (f >= room) f = -1;
-    int done_cycles = f >= 0 ? f + 1 : min(len, room);  // committed
-    const int out = gshfl(W.outcome, f < 0 ? 0 : f);
-    const bool viol = gshfl((int)W.violation, f < 0 ? 0 : f) != 0;
-    const bool tail_done = f < 0 && ends_done && done_cycles == len && len < room;
-    // scale after the committed cycles (a cycle that ends without a veto test
-    // leaves it)
-    const int tl = f >= 0 && (out == kDone || out == kNumericT) ? f - 1 : done_cycles - 1;
-    const double tn = gshfl(my_t, tl < 0 ? 0 : tl);
-    bool accepted = false;
-    if (active) {
-      const int counted = done_cycles + (tail_done ? 1 : 0);
-      if (!heavy_table ? gl == 0 : gl < counted) {
-        const unsigned long long times = heavy_table ? 1 : (unsigned long long)counted;
-        cnt.trials += times * (unsigned long long)(my_trials & 0xffff);
-        cnt.isr_trials += times * (unsigned long long)(my_trials >> 16);
-      }
-      if (tl >= 0) t = tn;
-      steps += counted;
-      draw += (uint64_t)done_cycles * (uint64_t)(nblk + 2);
-      if (tail_done) draw += (uint64_t)nblk;
-      if (f >= 0 && (out == kDone || out == kNumericT)) draw -= 2;
-      if (gl == 0) {
-        cnt.steps += counted;
-        cnt.vetoes += f >= 0 ? f : done_cycles;
-        if (f >= 0 && viol) cnt.violations += 1;
-      }
-      int st = GAPS_STATUS_ACTIVE;
-      if (tail_done || (f >= 0 && out == kDone)) st = GAPS_STATUS_DONE;
-      else if (f >= 0 && (out == kNumericT || out == kNumericW)) st = GAPS_ERR_NUMERIC;
-      else if (f >= 0 && out == kCapacity) st = GAPS_ERR_CAPACITY;
-      else if (f >= 0) accepted = true;
-      if (st == GAPS_STATUS_ACTIVE && steps >= P.max_steps) st = GAPS_ERR_ITER_CAP;
-      status = st;
-    }
-
-    // ---- emission --------------------------------------------------------
-    if (__any_sync(kAll, accepted)) {
-      emission(w, accepted, n, W, f < 0 ? 0 : f, eta0, eta1);
-      const int pack = gshfl(W.type | (W.bi << 2) | (W.bk << 10), f < 0 ? 0 : f);
-      if (accepted) {
-        chg = (pack & 3) == kII ? -1 : ((pack >> 2) & 0xff) | (((pack >> 10) & 0xff) << 8);
-        n += 1;
-        n_emit += 1;
-        if (gl == 0) cnt.accepts += 1;
-        table = true;
-      }
-    }
-
-    // ---- finished events back into the caller's records ------------------
-    if (active && status != GAPS_STATUS_ACTIVE) {
-      for (int s = gl; s < n; s += kG) {
-#pragma unroll
-        for (int mu = 0; mu < 4; ++mu) E.P(mu, s, e) = w.p[4 * s + mu];
-        const Tag tg = w.tag[s];
-        E.F(s, e) = tg.f;
-        E.C(s, e) = tg.c;
-        E.A(s, e) = tg.a;
-      }
-      if (gl == 0) {
-        E.npart[e] = n;
-        E.t[e] = t;
-        E.eta[e] = eta0;
-        E.eta[E.cap + e] = eta1;
-        E.n_emit[e] = n_emit;
-        E.draw[e] = draw;
-        E.status[e] = status;
-        if (status == GAPS_ERR_CAPACITY) cnt.err_cap += 1;
-        else if (status == GAPS_ERR_ITER_CAP) cnt.err_iter += 1;
-        else if (status == GAPS_ERR_NUMERIC) cnt.err_num += 1;
-      }
-      active = table = false;
-    }
-    __syncwarp();
+    batch(g, g.G == kG ? kG : kWideBatch, P, E, w, rows, m2f, s_list[tid / g.G * (g.G / kG)], S, cnt, heavy_table != 0);
   }
   flush_counters(P, cnt);
   __syncthreads();
