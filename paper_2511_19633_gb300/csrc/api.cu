@@ -19,6 +19,14 @@ cudaError_t launch_shower_fp64(const DevParams&, const DevEvents&, uint64_t, uin
 void workset_carve(void* base, int lanes, int nmax, WorkSet& W);
 cudaError_t launch_shower_mixed(const DevParams&, const DevEvents&, const WorkSet&, const LearnedCfg&, uint64_t,
                                 uint64_t, int, int, int, int, int, int, unsigned long long*, cudaStream_t);
+int groups_blocks(int sm_count);
+int groups_lanes(int blocks);
+cudaError_t launch_shower_groups(const DevParams&, const DevEvents&, const WorkSet&, const LearnedCfg&, uint64_t,
+                                 uint64_t, int, int, int, const void*, unsigned long long*, cudaStream_t);
+size_t groups_bytes(int lanes, int nmax);
+void groups_carve(void* base, int lanes, int nmax, WorkSet& W);
+size_t groups_tables_bytes();
+cudaError_t launch_groups_tables(const DevParams&, void*, cudaStream_t);
 cudaError_t launch_isr_targets(const DevParams&, int, const float4*, uint64_t, float*, float*, cudaStream_t);
 cudaError_t mixed_kernels_init();
 cudaError_t launch_mlp_image(const float* params, void* image, cudaStream_t stream);
@@ -44,13 +52,15 @@ cudaError_t calibration_stats(const float*, const float*, const float*, uint64_t
 
 using namespace gaps;
 
+constexpr int kCounterWords = C_NCOUNTERS + 2;
+
 struct gaps_ctx {
   gaps_config cfg;
   int device = 0;
   int n_sm = 0;
   float* d_grid = nullptr;
   double* d_tables = nullptr;  // umax [12][100], sufmax [12][101], lmin [12][100]
-  unsigned long long* d_counters = nullptr;  // C_NCOUNTERS + 1 (work counter)
+  unsigned long long* d_counters = nullptr;  // the counters, then the work counters of the two slots
   DevParams P;
   HistSet H;   // binning per row (one row for one process)
   int q_independent = 0;     // every Q^2 column of the grid is identical
@@ -59,6 +69,11 @@ struct gaps_ctx {
   size_t pool_flag_bytes = 0;
   void* d_work = nullptr;    // mixed-precision working set
   size_t work_bytes = 0;
+  // kept trials: the working sets of the events in flight (the second one for
+  // gaps_process's second slot)
+  int group_blocks = 0;
+  void* d_groups[2] = {nullptr, nullptr};
+  void* d_tables32 = nullptr;  // the FP32 tables of the kept-trial shower
   void* d_wave = nullptr;    // wavefront schedule: working set with one lane per event, then its state
   size_t wave_bytes = 0;
   uint64_t wave_cap = 0;
@@ -401,8 +416,8 @@ int gaps_init(gaps_ctx** out, const gaps_config* cfg) {
     if ((rc = cuda_fail(cudaMalloc(&ctx->d_tables, tables.size() * sizeof(double))))) break;
     if ((rc = cuda_fail(cudaMemcpy(ctx->d_tables, tables.data(), tables.size() * sizeof(double),
                                    cudaMemcpyHostToDevice)))) break;
-    if ((rc = cuda_fail(cudaMalloc(&ctx->d_counters, (C_NCOUNTERS + 1) * sizeof(unsigned long long))))) break;
-    if ((rc = cuda_fail(cudaMemset(ctx->d_counters, 0, (C_NCOUNTERS + 1) * sizeof(unsigned long long))))) break;
+    if ((rc = cuda_fail(cudaMalloc(&ctx->d_counters, kCounterWords * sizeof(unsigned long long))))) break;
+    if ((rc = cuda_fail(cudaMemset(ctx->d_counters, 0, kCounterWords * sizeof(unsigned long long))))) break;
     if ((rc = cuda_fail(mixed_kernels_init()))) break;
     if (c.precision == GAPS_FP64) {
       // allocated here and not by the first shower, which a caller may capture
@@ -422,6 +437,13 @@ int gaps_init(gaps_ctx** out, const gaps_config* cfg) {
   set_bound_tables(P, ctx->d_tables, c.pdf_grid);
   P.counters = ctx->d_counters;
   for (int r = 0; r < P.n_rows; ++r) set_hist_defs(P.rows[r].process, ctx->H.h[r]);
+  if (c.precision == GAPS_MIXED &&
+      (cudaMalloc(&ctx->d_tables32, groups_tables_bytes()) != cudaSuccess ||
+       launch_groups_tables(P, ctx->d_tables32, nullptr) != cudaSuccess || cudaStreamSynchronize(nullptr) != cudaSuccess)) {
+    cudaGetLastError();
+    gaps_destroy(ctx);
+    return GAPS_ERR_CUDA;
+  }
   *out = ctx;
   return GAPS_OK;
 }
@@ -460,10 +482,14 @@ int ensure_workset(gaps_ctx* ctx, int& blocks, int& bs, WorkSet& W) {
 // (allocated on first use, grown when a larger capacity comes)
 constexpr int kWavePassesDefault = 24;
 constexpr int kWaveCyclesDefault = 64;  // veto cycles of one event in one pass
+// the largest capacity of the wavefront schedule
+bool wave_capacity_ok(uint64_t cap, int nmax) {
+  return cap * 4 * (uint64_t)nmax < ((uint64_t)1 << 32) && cap < ((uint64_t)1 << 31);
+}
 int ensure_wave(gaps_ctx* ctx, uint64_t cap, WorkSet& W, WaveSet& V, int slot = 0) {
   const int nmax = ctx->cfg.nmax_partons;
   // the kernels index the working set with unsigned 32-bit element offsets
-  if (cap * 4 * (uint64_t)nmax >= ((uint64_t)1 << 32) || cap >= ((uint64_t)1 << 31)) return GAPS_ERR_INVALID_ARG;
+  if (!wave_capacity_ok(cap, nmax)) return GAPS_ERR_INVALID_ARG;
   void*& mem = slot ? ctx->d_wave2 : ctx->d_wave;
   size_t& bytes = slot ? ctx->wave_bytes2 : ctx->wave_bytes;
   uint64_t& have = slot ? ctx->wave_cap2 : ctx->wave_cap;
@@ -504,6 +530,37 @@ int shower_wave(gaps_ctx* ctx, uint64_t first_event, uint64_t n, const gaps_even
                                       c.emit_batch, ctx->q_independent, (cudaStream_t)stream));
 }
 
+// whether a shower of the context runs the kept-trial kernel
+bool keeps_trials(const gaps_ctx* ctx) {
+  const gaps_config& c = ctx->cfg;
+  return c.precision == GAPS_MIXED && c.trial_mode == GAPS_TRIALS_KEEP && c.schedule != GAPS_SCHED_WARP;
+}
+
+// its working set (allocated on first use; the same for every capacity)
+int ensure_groups(gaps_ctx* ctx, int slot, WorkSet& W) {
+  const int nmax = ctx->cfg.nmax_partons;
+  if (ctx->group_blocks == 0) ctx->group_blocks = groups_blocks(ctx->n_sm);
+  const int lanes = groups_lanes(ctx->group_blocks);
+  void*& mem = ctx->d_groups[slot];
+  if (!mem && cudaMalloc(&mem, groups_bytes(lanes, nmax)) != cudaSuccess) {
+    cudaGetLastError();
+    mem = nullptr;
+    return GAPS_ERR_CUDA;
+  }
+  groups_carve(mem, lanes, nmax, W);
+  return GAPS_OK;
+}
+
+int shower_groups(gaps_ctx* ctx, uint64_t first_event, uint64_t n, const gaps_events* ev, const LearnedCfg& Lc,
+                  void* stream, int slot) {
+  WorkSet W;
+  const int rc = ensure_groups(ctx, slot, W);
+  if (rc != GAPS_OK) return rc;
+  return cuda_fail(launch_shower_groups(ctx->P, dev_events(ev), W, Lc, first_event, n, ctx->group_blocks,
+                                        ctx->cfg.schedule == GAPS_SCHED_WAVE, ctx->q_independent, ctx->d_tables32,
+                                        ctx->d_counters + C_NCOUNTERS + slot, (cudaStream_t)stream));
+}
+
 int shower_mixed(gaps_ctx* ctx, uint64_t first_event, uint64_t n, const gaps_events* ev, const LearnedCfg& Lc,
                  void* stream) {
   const gaps_config& c = ctx->cfg;
@@ -538,6 +595,10 @@ int shower_impl(gaps_ctx* ctx, uint64_t first_event, uint64_t n, const gaps_even
       return cuda_fail(launch_shower_warp(ctx->P, dev_events(ev), Lc, first_event, n, ctx->n_sm * per_sm, bs,
                                           per_sm, ctx->q_independent, ctx->d_counters + C_NCOUNTERS,
                                           (cudaStream_t)stream));
+    }
+    if (keeps_trials(ctx)) {
+      if (c.schedule == GAPS_SCHED_WAVE && !wave_capacity_ok(ev->capacity, c.nmax_partons)) return GAPS_ERR_INVALID_ARG;
+      return shower_groups(ctx, first_event, n, ev, Lc, stream, slot);
     }
     if (c.schedule == GAPS_SCHED_WAVE) return shower_wave(ctx, first_event, n, ev, Lc, stream, slot);
     return shower_mixed(ctx, first_event, n, ev, Lc, stream);
@@ -879,6 +940,8 @@ namespace {
 void free_slot2(gaps_ctx* ctx) {
   if (ctx->d_slot2) cudaFree(ctx->d_slot2);
   if (ctx->d_wave2) cudaFree(ctx->d_wave2);
+  if (ctx->d_groups[1]) cudaFree(ctx->d_groups[1]);
+  ctx->d_groups[1] = nullptr;
   ctx->d_slot2 = ctx->d_wave2 = nullptr;
   ctx->slot2_bytes = ctx->wave_bytes2 = 0;
   ctx->wave_cap2 = 0;
@@ -925,7 +988,7 @@ bool ensure_slot2(gaps_ctx* ctx, const gaps_events* ev) {
   }
   WorkSet W;
   WaveSet V;
-  if (ensure_wave(ctx, cap, W, V, 1) != GAPS_OK) {
+  if ((keeps_trials(ctx) ? ensure_groups(ctx, 1, W) : ensure_wave(ctx, cap, W, V, 1)) != GAPS_OK) {
     free_slot2(ctx);
     return false;
   }
@@ -948,16 +1011,20 @@ int gaps_process(gaps_ctx* ctx, uint64_t first_event, uint64_t n, const gaps_eve
   const uint64_t cap = ev->capacity;
   if (!events_ok(ctx, ev, n < cap ? n : cap)) return GAPS_ERR_INVALID_ARG;
   // everything the launches need is allocated before the capture
-  if (ctx->cfg.precision == GAPS_MIXED && ctx->cfg.schedule == GAPS_SCHED_PERSISTENT) {
-    int blocks, bs;
+  if (keeps_trials(ctx)) {
+    if (ctx->cfg.schedule == GAPS_SCHED_WAVE && !wave_capacity_ok(cap, ctx->cfg.nmax_partons)) return GAPS_ERR_INVALID_ARG;
     WorkSet W;
-    const int rc = ensure_workset(ctx, blocks, bs, W);
+    const int rc = ensure_groups(ctx, 0, W);
     if (rc != GAPS_OK) return rc;
-  }
-  if (ctx->cfg.precision == GAPS_MIXED && ctx->cfg.schedule == GAPS_SCHED_WAVE) {
+  } else if (ctx->cfg.precision == GAPS_MIXED && ctx->cfg.schedule == GAPS_SCHED_WAVE) {
     WorkSet W;
     WaveSet V;
     const int rc = ensure_wave(ctx, cap, W, V);
+    if (rc != GAPS_OK) return rc;
+  } else if (ctx->cfg.precision == GAPS_MIXED && ctx->cfg.schedule == GAPS_SCHED_PERSISTENT) {
+    int blocks, bs;
+    WorkSet W;
+    const int rc = ensure_workset(ctx, blocks, bs, W);
     if (rc != GAPS_OK) return rc;
   }
   if (!ctx->cap_stream && cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking) != cudaSuccess)
@@ -1084,6 +1151,8 @@ void gaps_destroy(gaps_ctx* ctx) {
   if (ctx->d_counters) cudaFree(ctx->d_counters);
   if (ctx->d_pool) cudaFree(ctx->d_pool);
   if (ctx->d_work) cudaFree(ctx->d_work);
+  if (ctx->d_groups[0]) cudaFree(ctx->d_groups[0]);
+  if (ctx->d_tables32) cudaFree(ctx->d_tables32);
   if (ctx->d_wave) cudaFree(ctx->d_wave);
   if (ctx->d_mlp) cudaFree(ctx->d_mlp);
   if (ctx->d_mlp_image) cudaFree(ctx->d_mlp_image);

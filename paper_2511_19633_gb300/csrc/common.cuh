@@ -69,6 +69,7 @@ struct WorkSet {
   float4* end;
   float4* trial;         // kept trials {ln t, R_z} of both channels per end [lanes][2 nmax]
   float4* aux;           // the veto's inputs per end {s, eta, emitter tag, partner tag} [lanes][2 nmax]
+  float4* bnd;           // the veto's per-end constants [lanes][2 nmax] (kept trials only)
   float* tmx;            // per end the larger of its two kept trials' ln t (NaN: draws next cycle),
                          // [lanes][tmx_stride(nmax)]: the scan of a veto cycle reads only these
   float4* lkey;          // learned proposal: network inputs of the last evaluation [lanes][4 ends]
@@ -98,23 +99,15 @@ struct WaveSet {
   int* flags;               // [cap] bit 0: learned bounds active; bit 1: write the record
                             // back; bit 2: write the status back only; bit 3: an emission
                             // is parked; bits 8..15: mix row
-  int* keep;                // [cap] ends that may keep their trials at the next rebuild (-1: none)
-  int* chg;                 // [cap] slots the last emission changed, emitter | spectator << 8 |
-                            // new << 16, or -1: the next rebuild recomputes every end
   double* eta;              // [2][cap] momentum fractions of slots 0 and 1
   uint64_t* draw;           // [cap] next Philox block of the event's stream
   unsigned char* pend;      // [cap][kWavePendBytes] the parked emission of the pass
   uint32_t* list;           // [4][cap] live events of even / odd passes, (unused), rebuilds
-  float4* mlpq;             // [cap][4 ends][3] initial-state ends for the dense network pass
-  uint32_t* mlpi;           // [4 cap] the pass's queue of those ends: 4 event + end
   unsigned long long* ctl;  // [8] lengths of the lists, work counter of the veto pass
   uint64_t cap;
 };
 constexpr int kWavePendBytes = 64;
-enum WaveList { WL_LIVE0 = 0, WL_LIVE1 = 1, WL_REBUILD = 3, WL_GRAB = 4, WL_MLP = 5, WL_NCTL = 8 };
-// entries of a rebuild warp's network-queue buffer in shared memory (one
-// atomic on the queue length per flush)
-constexpr int kMlpBuf = 64;
+enum WaveList { WL_LIVE0 = 0, WL_LIVE1 = 1, WL_REBUILD = 3, WL_GRAB = 4, WL_NCTL = 8 };
 // WaveSet::flags bits
 constexpr int kWaveParked = 8;
 // events of the live list a veto warp takes with one atomic on the work counter

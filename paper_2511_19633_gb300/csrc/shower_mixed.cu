@@ -88,7 +88,30 @@ struct MixedCtx {
   WaveSet V;
   int wave_par;
   int wave_budget;
+  // the kept-trial shower: events a block holds, wavefront schedule asked for,
+  // some density has a heavy-quark threshold, the FP32 tables (SmemPdf) in
+  // global memory
+  int slots, wave, heavy;
+  const void* tables;
 };
+
+// the block's PDF tables (the caller synchronises)
+__device__ __forceinline__ void load_tables(SmemPdf& S, const MixedCtx& M) {
+  for (int q = threadIdx.x; q < 12 * kSmNX; q += blockDim.x) {
+    int f = q / kSmNX, ix = q % kSmNX;
+    S.umax[f][ix] = (float)M.P.umax[q];
+    S.lmin[f][ix] = (float)M.P.lmin[q];
+    float xf = 0.0f;
+    if (f < 11) xf = M.P.grid[((size_t)f * kNX + ix) * kNQ];
+    else for (int k = 1; k <= 10; ++k) xf += M.P.grid[((size_t)k * kNX + ix) * kNQ];
+    S.xf[f][ix] = xf;
+  }
+  for (int q = threadIdx.x; q < 12 * (kSmNX + 1); q += blockDim.x)
+    S.sufmax[q / (kSmNX + 1)][q % (kSmNX + 1)] = (float)M.P.sufmax[q];
+  for (int q = threadIdx.x; q < 12 * kSmNX; q += blockDim.x) S.first[q / kSmNX][q % kSmNX] = (float)M.P.first[q];
+  if (threadIdx.x < 12) S.m2[threadIdx.x] = (float)M.P.m2[threadIdx.x];
+  load_rows(S, M.P);
+}
 
 __device__ __forceinline__ float u24(uint32_t w) { return ((float)(w >> 8) + 0.5f) * (1.0f / 16777216.0f); }
 
@@ -282,6 +305,11 @@ struct WS {
   __device__ __forceinline__ float4& Aux(int q) const {
     return W.aux[(unsigned)lane * (unsigned)(2 * nmax) + (unsigned)q];
   }
+  // of end q: the PDF-ratio bounds of its channels, the density under them (a
+  // table that does not depend on Q^2) and delta of the z limits at t_c
+  __device__ __forceinline__ float4& Bnd(int q) const {
+    return W.bnd[(unsigned)lane * (unsigned)(2 * nmax) + (unsigned)q];
+  }
   // the larger ln t of end q's two kept trials (NaN with the mark above)
   __device__ __forceinline__ float& Tmx(int q) const {
     return W.tmx[(unsigned)lane * tmx_stride(nmax) + (unsigned)q];
@@ -328,6 +356,23 @@ __host__ __device__ constexpr size_t tag_stage_bytes(int warps, int nmax) {
 // bytes of one warp's event in shared memory
 __host__ __device__ constexpr size_t wss_bytes(int nmax) {
   return (size_t)nmax * (4 * sizeof(double) + sizeof(uint32_t) + 4 * sizeof(float4));
+}
+
+// the same from tags in global memory: eight loads at a time (one after the
+// other, each would wait for its own)
+__device__ __forceinline__ int find_partner_global(const uint32_t* tg, int n, int i, int side, int tag) {
+  const int sh = side == 0 ? 16 : 8;  // the other side's tag
+  for (int b = 0; b < n; b += 8) {
+    uint32_t t[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) t[j] = tg[min(b + j, n - 1)];
+    int m = -1;
+#pragma unroll
+    for (int j = 7; j >= 0; --j)
+      if (b + j < n && b + j != i && (int)((t[j] >> sh) & 0xffu) == tag) m = b + j;
+    if (m >= 0) return m;
+  }
+  return -1;
 }
 
 // colour partner of end (i, side) among the event's tags (shared memory)
@@ -456,25 +501,36 @@ __device__ IsrEval isr_eval32(const MixedCtx& M, const SmemPdf& S, int type, int
 
 // Cached record of colour end q = 2 slot + side of an event: {1/c0, 1/c1,
 // ln t_kin, partner} (partner -1: no dipole on this side), and in aux_out the
-// veto's inputs {s, eta, emitter tag, partner tag}.
-template <class W>
-__device__ float4 end_record(const MixedCtx& M, const SmemPdf& S, const W& w, const uint32_t* tg,
+// veto's inputs {s, eta, emitter tag, partner tag}; with BND also the values of
+// WS::Bnd.
+template <bool BND, class W>
+__device__ float4 end_record_impl(const MixedCtx& M, const SmemPdf& S, const W& w, const uint32_t* tg,
                              const unsigned char* own, int n, float eta0, float eta1, int row, int q,
-                             float& s_out, float& eta_out, int& type_out, float4& aux_out) {
+                             float& s_out, float& eta_out, int& type_out, float4& aux_out, float4& bnd) {
   type_out = -1;
   aux_out = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   const bool pp = S.pp[row] != 0;
   const int i = q >> 1, side = q & 1;
   const uint32_t ti = tg[i];
   const int tag = side == 0 ? tag_col(ti) : tag_acol(ti);
-  const int k = !tag ? -1 : (own ? partner_from_table(own, i, side, tag) : find_partner_tags(tg, n, i, side, tag));
+  double pi[4], pk[4];
+  if (BND) {  // (on their way during the search)
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) pi[mu] = w.P(mu, i);
+  }
+  const int k = !tag  ? -1
+                : BND ? find_partner_global(tg, n, i, side, tag)
+                : own ? partner_from_table(own, i, side, tag)
+                      : find_partner_tags(tg, n, i, side, tag);
   if (k < 0) return make_float4(-1.0f, -1.0f, 0.0f, __int_as_float(-1));
   const int fi = tag_fl(ti);
   const bool ini = pp && i < 2, ink = pp && k < 2;
   const int type = ini ? (ink ? kII : kIF) : (ink ? kFI : kFF);
-  double pi[4], pk[4];
 #pragma unroll
-  for (int mu = 0; mu < 4; ++mu) { pi[mu] = w.P(mu, i); pk[mu] = w.P(mu, k); }
+  for (int mu = 0; mu < 4; ++mu) {
+    if (!BND) pi[mu] = w.P(mu, i);
+    pk[mu] = w.P(mu, k);
+  }
   const float s = (float)(2.0 * dot4(pi, pk));  // FP64: near-collinear invariant
   float eta = 0.0f;
   if (type == kFI) eta = k == 0 ? eta0 : eta1;
@@ -490,6 +546,7 @@ __device__ float4 end_record(const MixedCtx& M, const SmemPdf& S, const W& w, co
   float zm, delta;
   const bool ok = tk > tc && zlim32(type, tc, s, eta, zm, delta);
   float ic[2] = {0.0f, -1.0f};
+  if (BND) bnd = make_float4(1.0f, 1.0f, 0.0f, ok ? delta : 0.0f);
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
     if (c >= nch) continue;
@@ -500,7 +557,22 @@ __device__ float4 end_record(const MixedCtx& M, const SmemPdf& S, const W& w, co
     float coefd;
     channel_over32(ch, type, M.P.nf, shape, coefd);
     float B = 1.0f;
-    if (type == kFI) {
+    if (BND) {
+      // one call site for every type (a warp's lanes hold all of them)
+      if (type != kFF) {
+        if (type == kFI && c == 1) {
+          B = bnd.x;  // both channels have the spectator's bound
+        } else {
+          int num, den;
+          if (type == kFI) num = den = pdf_index(tag_fl(tg[k]));
+          else isr_pdf_indices(ch, fi, num, den);
+          B = bound32(M, S, num, den, eta);
+          if (c == 0 && M.q_independent) bnd.z = pdf32(M, S, den, eta, 1.0f);
+        }
+      }
+      if (c == 0) bnd.x = B;
+      else bnd.y = B;
+    } else if (type == kFI) {
       const int f = pdf_index(tag_fl(tg[k]));
       B = bound32(M, S, f, f, eta);
     } else if (type == kIF || type == kII) {
@@ -512,6 +584,13 @@ __device__ float4 end_record(const MixedCtx& M, const SmemPdf& S, const W& w, co
     ic[c] = cc > 0.0f ? 1.0f / cc : 0.0f;
   }
   return make_float4(ic[0], ic[1], __logf(tk), __int_as_float(k));
+}
+template <class W>
+__device__ __forceinline__ float4 end_record(const MixedCtx& M, const SmemPdf& S, const W& w, const uint32_t* tg,
+                                             const unsigned char* own, int n, float eta0, float eta1, int row, int q,
+                                             float& s_out, float& eta_out, int& type_out, float4& aux_out) {
+  float4 unused;
+  return end_record_impl<false>(M, S, w, tg, own, n, eta0, eta1, row, q, s_out, eta_out, type_out, aux_out, unused);
 }
 
 // Learned bin heights of an event slot, 8-bit codes: height = 2^(-k/16)
@@ -566,7 +645,8 @@ __device__ __forceinline__ void set_end(const W& w, int q, const float4& rec, in
 // ends to evaluate. Rows r = lane and lane + 32 of the staging hold end r / 16,
 // channel (r / 8) % 2, bin r % 8: one 16-row tensor-core tile per end. Writes
 // the ends' 8-bit height codes and keys and returns on lane j the coefficient
-// scales of end j's two channels, 8 / the sum of its heights.
+// scales of end j's two channels, 8 / the sum of its heights. `four`: all four
+// tiles, two at a time, which then share the reads of the weight fragments.
 __device__ __noinline__ void learned_heights(const MixedCtx& M, const MlpSmem& mlp, const LearnedSmem& ls,
                                              float (*stage)[4], float* ustage, unsigned eval, float tc,
                                              float isr_eta, float isr_s, int isr_type, int fl_i, int slot_j, int q_j,
@@ -605,7 +685,7 @@ __device__ __noinline__ void learned_heights(const MixedCtx& M, const MlpSmem& m
   }
   __syncwarp();
   if (four) {
-    // all four tiles, two at a time (rows of unselected ends are unused)
+    // (rows of an unselected end are unused)
     mlp_tiles<2>(mlp, stage, ustage);
     mlp_tiles<2>(mlp, stage + 32, ustage + 32);
   } else {
@@ -665,9 +745,7 @@ __device__ __forceinline__ int rebuild_body(const MixedCtx& M, const SmemPdf& S,
                                             const LearnedSmem& ls, float (*stage)[4], float* ustage,
                                             const W& w, uint32_t* tg, bool stage_tags, int slot, uint64_t ev_src,
                                             int n, double eta0, double eta1, int row, bool learned_src,
-                                            int keep_ends, int lane_id, bool defer = false,
-                                            unsigned* defer_mask = nullptr, float4* deferred = nullptr,
-                                            float4* isr_plain = nullptr, int chg = -1) {
+                                            int keep_ends, int lane_id) {
   // the event's tags in shared memory, and (lane kernels) the table of the
   // slot owning each colour and anticolour tag, so that an end finds its
   // partner in one lookup; with a tag held by two partons (not a leading-
@@ -706,23 +784,6 @@ __device__ __forceinline__ int rebuild_body(const MixedCtx& M, const SmemPdf& S,
   float isr_s = 0.0f, isr_eta = 0.0f;
   int isr_type = -1;
   for (int q = lane_id; q < 2 * n; q += 32) {
-    if (chg >= 0 && !(pp && q < 4) && q < keep_ends) {
-      // an end whose parton and colour partner the last emission left alone
-      // keeps its record (the same bits a recomputation gives): its inputs
-      // are the two momenta, the tags and the momentum fraction of an
-      // initial-state parton among them, and the emission changed only the
-      // emitter, the spectator and the new parton, whose ends and partners'
-      // ends take the new colour line
-      const int ci = chg & 0xff, ck = (chg >> 8) & 0xff, cj = (chg >> 16) & 0xff;
-      const int a = q >> 1;
-      if (a != ci && a != ck && a != cj) {
-        const int side = q & 1;
-        const uint32_t ta = tg[a];
-        const int tag = side == 0 ? tag_col(ta) : tag_acol(ta);
-        const int p = !tag ? -1 : (own ? partner_from_table(own, a, side, tag) : find_partner_tags(tg, n, a, side, tag));
-        if (p != ci && p != ck && p != cj) continue;
-      }
-    }
     float s_, eta_;
     int type_;
     float4 aux;
@@ -758,12 +819,7 @@ __device__ __forceinline__ int rebuild_body(const MixedCtx& M, const SmemPdf& S,
   const bool need = use && !(key.x == isr_eta && key.y == isr_s && key.z == code);
   const unsigned eval = __ballot_sync(0xffffffffu, need) & 0xFu;
   float scale0 = 0.0f, scale1 = 0.0f;  // 8 / sum of the new heights (lanes 0..3)
-  if (defer) *defer_mask = eval;
-  if (eval && defer) {
-    // the wavefront's dense network pass evaluates these ends; their records
-    // and trials are finished there
-    if (need) *deferred = make_float4(isr_eta, isr_s, __int_as_float(isr_type), __int_as_float(fl_i));
-  } else if (eval) {
+  if (eval) {
     learned_heights(M, mlp, ls, stage, ustage, eval, __expf(S.lnTc[row]), isr_eta, isr_s, isr_type, fl_i, slot,
                     lane_id, lane_id, scale0, scale1);
   }
@@ -771,9 +827,7 @@ __device__ __forceinline__ int rebuild_body(const MixedCtx& M, const SmemPdf& S,
     if (use) {
       // the coefficient scale c * mean(U): new heights, or the unchanged
       // inputs' record of the last evaluation (the same product)
-      if (need && defer) {
-        *isr_plain = isr_rec;  // scaled by the dense pass
-      } else if (need) {
+      if (need) {
         isr_rec.x *= scale0;
         isr_rec.y *= scale1;
       } else {
@@ -791,7 +845,7 @@ __device__ __forceinline__ int rebuild_body(const MixedCtx& M, const SmemPdf& S,
     set_end(w, lane_id, isr_rec, (need && keep_ends >= 0) ? 0 : keep_ends);
   }
   __syncwarp();
-  return defer ? 0 : __popc(eval);
+  return __popc(eval);
 }
 
 template <class W>
@@ -1633,20 +1687,7 @@ __device__ __forceinline__ void mixed_prologue(const MixedCtx& M, SmemPdf& S, un
       D.ustage = reinterpret_cast<float(*)[64]>(st + (size_t)nw * 64 * 4 * sizeof(float));
     }
   }
-  for (int q = threadIdx.x; q < 12 * kSmNX; q += blockDim.x) {
-    int f = q / kSmNX, ix = q % kSmNX;
-    S.umax[f][ix] = (float)M.P.umax[q];
-    S.lmin[f][ix] = (float)M.P.lmin[q];
-    float xf = 0.0f;
-    if (f < 11) xf = M.P.grid[((size_t)f * kNX + ix) * kNQ];
-    else for (int k = 1; k <= 10; ++k) xf += M.P.grid[((size_t)k * kNX + ix) * kNQ];
-    S.xf[f][ix] = xf;
-  }
-  for (int q = threadIdx.x; q < 12 * (kSmNX + 1); q += blockDim.x)
-    S.sufmax[q / (kSmNX + 1)][q % (kSmNX + 1)] = (float)M.P.sufmax[q];
-  for (int q = threadIdx.x; q < 12 * kSmNX; q += blockDim.x) S.first[q / kSmNX][q % kSmNX] = (float)M.P.first[q];
-  if (threadIdx.x < 12) S.m2[threadIdx.x] = (float)M.P.m2[threadIdx.x];
-  load_rows(S, M.P);
+  load_tables(S, M);
 }
 
 // dynamic shared memory of a mixed-precision block of `block_size` threads
@@ -1915,7 +1956,6 @@ __global__ void k_wave_init(const __grid_constant__ MixedCtx M) {
   ls.key = M.Lc.learned ? M.W.lkey : nullptr;
   ls.dec = nullptr;
   const int lane_id = threadIdx.x & 31;
-  const bool cache = M.P.trial_mode == GAPS_TRIALS_KEEP;
   unsigned long long finished = 0, err_num = 0;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   // whole warps iterate together (the appends are warp-collective)
@@ -1931,8 +1971,6 @@ __global__ void k_wave_init(const __grid_constant__ MixedCtx M) {
       // status changed (a record that could not be read)
       const int wb = live ? 2 : (L.status != M.E.status[e] ? 4 : 0);
       M.V.flags[e] = 1 | wb | (L.row << 8);
-      M.V.keep[e] = cache ? 0 : -1;
-      M.V.chg[e] = -1;
       wave_store(M, L);
       if (!live) {
         finished += 1;
@@ -1944,75 +1982,6 @@ __global__ void k_wave_init(const __grid_constant__ MixedCtx M) {
   }
   Counters32 cnt;
   flush_counters(M, cnt, finished, 0, 0, err_num, 0, 0, 0, 0, lane_id);
-}
-
-// The trials of the ends a rebuild marked (kept-trial scheme), drawn by the
-// warp together, one end per lane: the same Philox blocks, in the same
-// canonical order, as the first cycle's trial loop would draw them one by one
-// (each end's first counter is the event's counter plus a warp prefix sum of
-// the draws of the marked ends before it), so the events are unchanged and
-// the cycle that follows only scans. Returns the event's counter after the
-// draws (every lane).
-__device__ __forceinline__ uint64_t draw_marked_ends(const MixedCtx& M, const SmemPdf& S, const WS& w, uint64_t id,
-                                                     int n, int row, float lnT, uint64_t d, int lane_id,
-                                                     Counters32& cnt, unsigned defer_mask, uint64_t& defer_off) {
-  const unsigned full = 0xffffffffu;
-  const bool pp = S.pp[row] != 0;
-  const float lnTc = S.lnTc[row];
-  const uint32_t k0 = (uint32_t)M.P.seed, k1 = (uint32_t)(M.P.seed >> 32);
-  const uint32_t e0 = (uint32_t)id, e1 = (uint32_t)(id >> 32);
-  const int ne = 2 * n;
-  for (int q0 = 0; q0 < ne; q0 += 32) {
-    const int q = q0 + lane_id;
-    bool marked = false;
-    float4 rec = make_float4(-1.0f, -1.0f, 0.0f, __int_as_float(-1));
-    int nd = 0;  // Philox blocks of this end: one per channel present
-    if (q < ne) {
-      marked = isnan(w.Tmx(q));
-      if (marked) {
-        rec = w.End(q);
-        if (__float_as_int(rec.w) >= 0) nd = (rec.x >= 0.0f ? 1 : 0) + (rec.y >= 0.0f ? 1 : 0);
-      }
-    }
-    int inc = nd;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const int t = __shfl_up_sync(full, inc, off);
-      if (lane_id >= off) inc += t;
-    }
-    const int tot = __shfl_sync(full, inc, 31);
-    if (marked && q < 4 && ((defer_mask >> q) & 1u)) {
-      // the dense network pass draws this end's trials from here
-      defer_off = d + (uint64_t)(inc - nd);
-      marked = false;
-    }
-    if (marked) {
-      float4 tr = make_float4(-INFINITY, 0.5f, -INFINITY, 0.5f);
-      if (__float_as_int(rec.w) >= 0) {
-        uint64_t dd = d + (uint64_t)(inc - nd);
-        const float lnTmax = fminf(lnT, rec.z);
-        const bool live = lnTmax > lnTc;
-        const float m2 = q < 4 ? end_m2(S, w.Aux(q), q, row) : 0.0f;
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          const float ic = c == 0 ? rec.x : rec.y;  // 1/c
-          if (ic < 0.0f) continue;                  // channel absent for this emitter
-          const uint64_t dc = dd++;
-          if (!(live && ic > 0.0f)) continue;
-          uint32_t out[4];
-          philox(e0, e1, (uint32_t)dc, (uint32_t)(dc >> 32), k0, k1, out);
-          cnt.trials += 1;
-          if (pp && q < 4) cnt.isr_trials += 1;
-          const float lt = trial_lnt(lnTmax, ic, __logf(u24(out[1])), m2);
-          if (c == 0) { tr.x = lt; tr.y = u24(out[3]); }
-          else { tr.z = lt; tr.w = u24(out[3]); }
-        }
-      }
-      w.SetTrial(q, tr);
-    }
-    d += (uint64_t)tot;
-  }
-  return d;
 }
 
 // L2 prefetch of the rows a rebuild reads (one line per lane): the event's
@@ -2028,8 +1997,6 @@ __device__ __forceinline__ void prefetch_event_rows(const MixedCtx& M, uint32_t 
   switch (lane_id) {
     case 0: a = (const char*)(V.flags + e); break;
     case 1: a = (const char*)(V.n + e); break;
-    case 2: a = (const char*)(V.keep + e); break;
-    case 3: a = (const char*)(V.chg + e); break;
     case 4: a = (const char*)(V.eta + e); break;
     case 5: a = (const char*)(V.eta + V.cap + e); break;
     case 6: a = (const char*)(V.lnT + e); break;
@@ -2050,9 +2017,8 @@ __device__ __forceinline__ void prefetch_event_rows(const MixedCtx& M, uint32_t 
   if (a) asm volatile("prefetch.global.L2 [%0];" ::"l"(a));
 }
 
-// One warp per event of the rebuild list: the end table, then (kept trials)
-// the trials of the ends it marked. Also clears, for the passes after it, the
-// lists this pass's later kernels fill.
+// One warp per event of the rebuild list: the end table. Also clears, for the
+// passes after it, the lists this pass's later kernels fill.
 template <int MINB>
 __global__ void __launch_bounds__(256, MINB) k_wave_ends(const __grid_constant__ MixedCtx M) {
   __shared__ SmemPdf S;
@@ -2065,28 +2031,11 @@ __global__ void __launch_bounds__(256, MINB) k_wave_ends(const __grid_constant__
   // blocks past the list's last warp leave before loading their tables
   if ((uint64_t)blockIdx.x * (blockDim.x >> 5) >= count) return;
   MixedSmem D;
-  const bool with_stage = M.P.trial_mode != GAPS_TRIALS_KEEP;
-  mixed_prologue(M, S, dyn_lane_smem, D, with_stage);
+  mixed_prologue(M, S, dyn_lane_smem, D, true);
   const MlpSmem& mlp_s = *reinterpret_cast<const MlpSmem*>(M.Lc.image);
   __syncthreads();
   const int lane_id = threadIdx.x & 31, warp_id = threadIdx.x >> 5;
   const uint64_t nw = (uint64_t)gridDim.x * (blockDim.x >> 5);
-  const bool cache = M.P.trial_mode == GAPS_TRIALS_KEEP;
-  // the warp's buffer of initial-state ends for the network pass (with the
-  // learned proposal and kept trials), after the prologue's shared memory
-  uint32_t* mbuf = reinterpret_cast<uint32_t*>(
-                       dyn_lane_smem + mixed_dyn_bytes(blockDim.x, M.P.nmax, M.Lc.learned != 0, with_stage)) +
-                   warp_id * kMlpBuf;
-  int mfill = 0;  // warp-uniform
-  auto mflush = [&]() {
-    __syncwarp();
-    unsigned long long base = 0;
-    if (lane_id == 0) base = atomicAdd(&M.V.ctl[WL_MLP], (unsigned long long)mfill);
-    base = __shfl_sync(0xffffffffu, base, 0);
-    for (int j = lane_id; j < mfill; j += 32) M.V.mlpi[base + j] = mbuf[j];
-    __syncwarp();
-    mfill = 0;
-  };
   unsigned long long rebuilds = 0, mlp_tiles = 0;
   Counters32 cnt;
   // the list two events ahead, so that the next event's rows can be brought
@@ -2102,133 +2051,13 @@ __global__ void __launch_bounds__(256, MINB) k_wave_ends(const __grid_constant__
     if (i + nw < count) prefetch_event_rows(M, e_a, lane_id);
     const int flags = M.V.flags[e], n = M.V.n[e], row = (flags >> 8) & 0xff;
     const WS w{M.W, (int)e, M.P.nmax};
-    unsigned defer_mask = 0;
-    float4 deferred = make_float4(0.0f, 0.0f, 0.0f, 0.0f), plain = deferred;
     mlp_tiles += rebuild_body(M, S, mlp_s, D.ls, D.stage[warp_id], D.ustage[warp_id], w,
                               D.tag_stage + warp_id * tag_stage_words(M.P.nmax), true, (int)e, e, n, M.V.eta[e],
-                              M.V.eta[M.V.cap + e], row, (flags & 1) != 0, M.V.keep[e], lane_id, cache, &defer_mask,
-                              &deferred, &plain, M.V.chg[e]);
+                              M.V.eta[M.V.cap + e], row, (flags & 1) != 0, -1, lane_id);
     rebuilds += 1;
-    if (cache) {
-      uint64_t off = 0;
-      const uint64_t d = draw_marked_ends(M, S, w, M.first + e, n, row, M.V.lnT[e], M.V.draw[e], lane_id, cnt,
-                                          defer_mask, off);
-      __syncwarp();  // every lane has read the old counter
-      if (lane_id == 0) M.V.draw[e] = d;
-      // initial-state ends whose network inputs changed: their inputs in the
-      // event's own slots, their index to the warp's buffer for the network
-      // pass's queue
-      const bool mine = lane_id < 4 && ((defer_mask >> lane_id) & 1u);
-      const unsigned m = __ballot_sync(0xffffffffu, mine) & 0xFu;
-      if (mine) {
-        float4* q = M.V.mlpq + 3 * (4 * e + lane_id);
-        q[0] = plain;
-        q[1] = deferred;
-        q[2] = make_float4(__uint_as_float((uint32_t)e), __int_as_float(lane_id | (row << 8)),
-                           __uint_as_float((uint32_t)off), __uint_as_float((uint32_t)(off >> 32)));
-      }
-      if (m) {
-        const int k = __popc(m);
-        if (mfill + k > kMlpBuf) mflush();
-        if (mine) mbuf[mfill + __popc(m & ((1u << lane_id) - 1u))] = (uint32_t)(4 * e + lane_id);
-        mfill += k;
-      }
-    }
   }
-  if (mfill) mflush();
   flush_counters(M, cnt, 0, 0, 0, 0, 0, 0, lane_id == 0 ? rebuilds : 0ull, lane_id == 0 ? mlp_tiles : 0ull,
                  lane_id);
-}
-
-// The dense network pass of the learned proposal: four queued initial-state
-// ends per warp iteration (one 16-row tile each), from whatever events the
-// rebuild pass queued them. Each end gets its height codes and key, its
-// record scaled by c * mean(U), and its two trials drawn at the Philox
-// counters the rebuild pass reserved for it, as the persistent kernel's
-// inline evaluation and first trial loop would give them.
-__global__ void __launch_bounds__(256, 2) k_wave_mlp(const __grid_constant__ MixedCtx M) {
-  // the pass's queue of initial-state ends, four per warp step
-  const uint64_t count = M.V.ctl[WL_MLP];
-  if ((uint64_t)blockIdx.x * (blockDim.x >> 5) * 4 >= count) return;  // nothing queued for this block
-  __shared__ float dec[256];
-  __shared__ __align__(16) float stage_s[8][64][4];
-  __shared__ float ustage_s[8][64];
-  __shared__ float lnTc[kMaxRows];
-  __shared__ __align__(16) unsigned char wimg[kMlpSmemBytes];  // the network's BF16 image
-  {
-    const uint4* src = reinterpret_cast<const uint4*>(M.Lc.image);
-    uint4* dst = reinterpret_cast<uint4*>(wimg);
-    for (int k = threadIdx.x; k < (int)(kMlpSmemBytes / 16); k += blockDim.x) dst[k] = src[k];
-  }
-  for (int k = threadIdx.x; k < 256; k += blockDim.x) dec[k] = k < 255 ? exp2f(-(float)k * 0.0625f) : 0.0f;
-  if (threadIdx.x < kMaxRows) {
-    const RowParams& R = M.P.rows[threadIdx.x < M.P.n_rows ? threadIdx.x : 0];
-    lnTc[threadIdx.x] = (float)gm_log(R.t_cut);
-  }
-  __syncthreads();
-  LearnedSmem ls;
-  ls.code = M.W.lcode;
-  ls.key = M.W.lkey;
-  ls.dec = dec;
-  const MlpSmem& mlp_s = *reinterpret_cast<const MlpSmem*>(wimg);
-  const int lane_id = threadIdx.x & 31, warp_id = threadIdx.x >> 5;
-  const uint64_t nw = (uint64_t)gridDim.x * (blockDim.x >> 5);
-  const uint32_t k0 = (uint32_t)M.P.seed, k1 = (uint32_t)(M.P.seed >> 32);
-  Counters32 cnt;
-  unsigned long long tiles = 0;
-  for (uint64_t g = (uint64_t)blockIdx.x * (blockDim.x >> 5) + warp_id; 4 * g < count; g += nw) {
-    const uint64_t j = 4 * g + lane_id;
-    const bool have = lane_id < 4 && j < count;
-    float4 plain = make_float4(0.0f, 0.0f, 0.0f, 0.0f), in = plain, tag = plain;
-    if (have) {
-      const uint32_t idx = M.V.mlpi[j];
-      const float4* qe = M.V.mlpq + 3 * (uint64_t)idx;  // slot (event idx / 4, end idx % 4)
-      plain = qe[0];
-      in = qe[1];
-      tag = qe[2];
-    }
-    const unsigned eval = __ballot_sync(0xffffffffu, have) & 0xFu;
-    const int e = (int)__float_as_uint(tag.x), qq = __float_as_int(tag.y) & 0xff, row = __float_as_int(tag.y) >> 8;
-    const float tc = have ? __expf(lnTc[row]) : 1.0f;
-    float scale0 = 0.0f, scale1 = 0.0f;
-    learned_heights(M, mlp_s, ls, stage_s[warp_id], ustage_s[warp_id], eval, tc, in.x, in.y, __float_as_int(in.z),
-                    __float_as_int(in.w), e, qq, lane_id, scale0, scale1, true);
-    tiles += __popc(eval);
-    if (have) {
-      const WS w{M.W, e, M.P.nmax};
-      float4 rec = plain;
-      rec.x *= scale0;
-      rec.y *= scale1;
-      w.End(qq) = rec;
-      // the end's trials, channel by channel, from its reserved counter
-      uint64_t dd = ((uint64_t)__float_as_uint(tag.w) << 32) | (uint64_t)__float_as_uint(tag.z);
-      const uint64_t id = M.first + (uint64_t)e;
-      const uint32_t e0 = (uint32_t)id, e1 = (uint32_t)(id >> 32);
-      const float lnTmax = fminf(M.V.lnT[e], rec.z);
-      const bool live = lnTmax > lnTc[row];
-      // heavy-quark measure of an incoming c or b (its two channels)
-      const int fe = pdf_index(tag_fl(__float_as_uint(w.Aux(qq).z)));
-      const float m2 = fe > 0 ? (float)M.P.m2[fe] : 0.0f;
-      float4 tr = make_float4(-INFINITY, 0.5f, -INFINITY, 0.5f);
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        const float ic = c == 0 ? rec.x : rec.y;
-        if (ic < 0.0f) continue;
-        const uint64_t dc = dd++;
-        if (!(live && ic > 0.0f)) continue;
-        uint32_t out[4];
-        philox(e0, e1, (uint32_t)dc, (uint32_t)(dc >> 32), k0, k1, out);
-        cnt.trials += 1;
-        cnt.isr_trials += 1;
-        const float lt = trial_lnt(lnTmax, ic, __logf(u24(out[1])), m2);
-        if (c == 0) { tr.x = lt; tr.y = u24(out[3]); }
-        else { tr.z = lt; tr.w = u24(out[3]); }
-      }
-      w.SetTrial(qq, tr);
-    }
-    __syncwarp();
-  }
-  flush_counters(M, cnt, 0, 0, 0, 0, 0, 0, 0, lane_id == 0 ? tiles : 0ull, lane_id);
 }
 
 // Persistent lanes over the live list: each lane runs max-veto cycles of one
@@ -2241,7 +2070,6 @@ __global__ void __launch_bounds__(256, MINB) k_wave_veto(const __grid_constant__
   const uint64_t n_work = M.V.ctl[M.wave_par];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     M.V.ctl[WL_REBUILD] = 0;  // filled by this pass's emissions
-    M.V.ctl[WL_MLP] = 0;      // filled by the next pass's rebuilds
   }
   // blocks with more lanes than the list has events leave before loading their tables
   if ((uint64_t)blockIdx.x * blockDim.x >= n_work) return;
@@ -2343,7 +2171,6 @@ __global__ void __launch_bounds__(128) k_wave_emit(const __grid_constant__ Mixed
   const uint32_t* live = M.V.list + (size_t)M.wave_par * M.V.cap;
   if ((uint64_t)blockIdx.x * blockDim.x >= count) return;
   const int lane_id = threadIdx.x & 31;
-  const bool cache = M.P.trial_mode == GAPS_TRIALS_KEEP;
   const int next_live = WL_LIVE0 + (M.wave_par ^ 1);
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   Counters32 cnt;
@@ -2361,23 +2188,14 @@ __global__ void __launch_bounds__(128) k_wave_emit(const __grid_constant__ Mixed
       Lane L;
       wave_load(M, L, e);
       const Emission em = *reinterpret_cast<const Emission*>(M.V.pend + e * kWavePendBytes);
-      int keep = -1, chg = -1;
       if (em.kind == 1) {
         rebuild = true;
-        keep = cache ? 0 : -1;
       } else if (emit(M, WS{M.W, (int)e, M.P.nmax}, L, em)) {
         cnt.accepts += 1;
         rebuild = true;
-        keep = cache ? 2 * (L.n - 1) : -1;
-        // the partons the emission moved: emitter, spectator and the new one
-        // (an initial-initial emission kicks every final parton: all ends)
-        if (em.type != kII) chg = em.bi | (em.k << 8) | ((L.n - 1) << 16);
       } else {
-        cnt.vetoes += 1;  // the map failed: the winner's end draws again
-        if (cache) WS{M.W, (int)e, M.P.nmax}.MarkTrial(2 * em.bi + em.bside);
+        cnt.vetoes += 1;  // the map failed
       }
-      M.V.keep[e] = keep;
-      M.V.chg[e] = chg;
       wave_store(M, L);
     }
     wave_append(M, WL_REBUILD, rebuild, e, lane_id);
@@ -2398,6 +2216,1090 @@ __global__ void k_wave_final(const __grid_constant__ MixedCtx M) {
   }
 }
 
+
+// ---------------------------------------------------------------------------
+// The kept-trial shower (GAPS_TRIALS_KEEP, the persistent and the wavefront
+// schedule): one block per SM holds kSlots events in flight and takes them
+// through the phases of an emission together, each phase's work items spread
+// over the lanes whatever event they belong to.
+//
+//   touch   lists the ends that the slots' last emissions touched (eight lanes
+//           per slot)
+//   form    one lane per listed end: its record; ends whose record changed are
+//           marked, with the number of Philox blocks that their trials use
+//   draw    one lane per marked end: its trials, at the counter that the marks
+//           below it give (the canonical order); at the same time one lane per
+//           slot and cycle: the uniforms of the next trials of eight cycles
+//   net     the learned proposal's tiles of the changed initial-state ends,
+//           four a warp step, and their trials
+//   chain   four lanes per slot: eight cycles under the assumption of vetoes
+//           (the largest kept trial wins and its channel draws again)
+//   weigh   one lane per cycle, sorted by dipole type: the acceptance weight
+//   commit  one lane per slot: the cycles up to the first that was not vetoed;
+//           the trials that the cycles behind it replaced are put back
+//   emit    four more warps, beside all of the above, on the last round's
+//           results: the FP64 kinematics of its emissions, one lane each; its
+//           ended events are written back and the next ones loaded, eight
+//           lanes per slot
+//
+// The chain may run ahead because a vetoed cycle uses exactly three Philox
+// blocks (two of the veto, one of the winner's next trial). Every cycle uses
+// the numbers that one lane per event would use, so the events are the same
+// bits.
+//
+// Why this shape. The bound is instruction fetch and the latency of serial
+// steps, not arithmetic or memory: an event is 32 000 instructions a lane of
+// phases that have little code in common. With one lane per event 7 of 32 lanes
+// were active in the veto cycles and 12 in the rebuilds (53 000 instructions an
+// event), and with independent warps the phases' code (160 KB) evicted itself
+// from the instruction cache (two thirds of the stalls). In lockstep all warps
+// of the SM run one phase's code, and lists keep the lanes full; what is left is
+// a round of 66 000 clocks (touch 7 000, form 18 000, draw 5 000, chain 17 000,
+// list 3 000, weigh 11 000, commit 5 000; net 24 000 where it runs), most of it
+// the latency of one event's chain of loads and trials. The events in flight
+// (about 3 KB each) stay in L2 where a pass over a whole chunk per phase moved
+// 71 KB an event through DRAM. An emission's FP64 runs at 1/64 of the FP32 rate
+// and costs a warp the same for 1 or 32 lanes, so it needs a list of many
+// events, and warps of its own to hide behind the other phases.
+//
+// kSlots: a round's time is mostly latency, so more events a round are nearly
+// free until the chain's four lanes per slot leave the worker warps (224). 96
+// and 128 slots are slower, 168 and 200 alike; 168 leaves shared memory for the
+// network image. Measured, one GPU, before (a warp of events, then a pass per
+// phase over all events) and now: 32 768 p p events with matrix-element
+// corrections and the plain bound 47.2 -> 23.9 ms, 65 536 with the learned
+// proposal 116.8 -> 82 ms, 10 240 leading-order p p events 24.4 -> 7.1 ms, 200
+// events 14.4 -> 3.9 ms, 32 768 events of a beam and process mix 58.8 -> 35.3 ms.
+// ---------------------------------------------------------------------------
+constexpr int kSlots = 168;
+constexpr int kWorkers = 896;               // 28 warps
+constexpr int kEmitters = 128;              // four warps, one per scheduler
+constexpr int kGThreads = kWorkers + kEmitters;
+constexpr int kCyc = 8;                     // cycles of a round
+constexpr int kEndList = 4096;              // ends formed in a round (the slots beyond wait for the next)
+constexpr int kTmx = 64;                    // ends whose larger kept trial is in shared memory
+static_assert(4 * kSlots <= kWorkers && 4 * kSlots % 32 == 0 && kSlots <= 256, "the phases' lane mappings");
+static_assert(kEndList >= 256, "one event always fits");
+static_assert(kCyc * kSlots <= 2 * kWorkers, "two cycles a thread in phase_list");
+
+// a thread's counters of one launch (32 bits: a lane sees a small share of the
+// launch's events)
+struct GCount {
+  unsigned steps = 0, trials = 0, isr_trials = 0, vetoes = 0, accepts = 0, violations = 0, rebuilds = 0, tiles = 0;
+  unsigned lane_steps = 0, warp_steps = 0;  // lanes that weighed a cycle, lanes of their warps
+  unsigned finished = 0, err_cap = 0, err_iter = 0, err_num = 0;
+};
+
+// cycle of the chain: its winner (bits 0 .. 8: 2 end + channel; 9: its next trial
+// was drawn, 10: by an initial-state end; 12 and 13: dipole type), its ln t and z
+// draw; before the chain the ln of the uniform and the z draw of the next trial
+struct GCycle {
+  int win;
+  float best, Rz;
+  __device__ __forceinline__ int end() const { return (win & 0x1ff) >> 1; }
+  __device__ __forceinline__ int channel() const { return win & 1; }
+  __device__ __forceinline__ int type() const { return (win >> 12) & 3; }
+};
+// weight of a cycle: z and 1 - z (a violation: z and zeta), the weight, and
+// outcome | new emitter flavour << 8 | new parton's flavour (a violation: the
+// bin) << 16
+struct GWeight { float z, omz, w; int what; };
+enum CycleOutcome { kCycVeto = 0, kCycAccept, kCycViolation, kCycNumeric, kCycCapacity };
+
+struct GSmem {
+  SmemPdf S;
+  // per slot
+  uint64_t ev[kSlots], draw[kSlots];
+  double eta0[kSlots], eta1[kSlots];
+  float lnT[kSlots];
+  int n[kSlots], n_emit[kSlots], steps[kSlots], row[kSlots];
+  int live[kSlots];    // the slot holds an event: 1, on the plain bounds after a violation: 3
+  int end[kSlots];     // its status once it ended (GAPS_STATUS_ACTIVE before)
+  int busy[kSlots];    // 1: an emission is parked or being built, 2: it is built
+  int ready[kSlots];   // takes part in this round's chain
+  int table[kSlots];   // 1: form the touched ends, 2: only end chg draws again
+  int keep[kSlots];    // ends that may keep their trials
+  int chg[kSlots];     // emitter | spectator << 8, or -1: every end
+  unsigned defer[kSlots];        // initial-state ends in the network's queue
+  int tot[kSlots];               // Philox blocks of this round's marked ends
+  uint32_t mk1[kSlots][8], mk2[kSlots][8];  // marked ends with one and with two channels
+  int len[kSlots], done[kSlots]; // cycles of the chain; the one after them has no trial above the cutoff
+  unsigned nv[kSlots];           // cycles that were not vetoed
+  GCycle park[kSlots];           // the parked emission: its cycle
+  GWeight pw[kSlots];            // and weight
+  alignas(16) float tmx[kSlots][kTmx + 4];  // the larger kept trial of ends 0 .. kTmx - 1 (the rest: WS::Tmx)
+  int n_ends, n_ends_ok, n_q, n_items[4], n_tables[2], n_park[2], n_ended[2];
+  unsigned ends[kEndList];       // slot << 8 | end; bit 16: draw only, then: marked
+  unsigned short q[4 * kSlots];  // 4 slot + end of the network's queue
+  unsigned short items[4][kCyc * kSlots];  // 8 slot + cycle, by dipole type
+  // slots with ends to form, with a parked emission, ended; by the round's parity
+  unsigned char tables[2][kSlots], parked[2][kSlots], ended[2][kSlots];
+  float dec[256];
+  alignas(16) unsigned char image[kMlpSmemBytes];  // the network's BF16 image
+  GCycle cyc[kCyc][kSlots];
+  union {
+    GWeight wt[kCyc][kSlots];
+    struct {
+      alignas(16) float stage[kWorkers / 32][64][4];  // (float4 rows)
+      float ustage[kWorkers / 32][64];
+    } m;
+  };
+};
+
+static_assert(sizeof(GSmem) <= 227 * 1024, "one block per SM");
+
+__device__ __forceinline__ void workers_sync() { asm volatile("bar.sync 1, 896;" ::: "memory"); }
+static_assert(kWorkers == 896, "workers_sync");
+
+// Philox block d of event id, one copy for all phases
+__device__ __noinline__ uint4 block_of(uint64_t seed, uint64_t id, uint64_t d) {
+  uint32_t o[4];
+  philox((uint32_t)id, (uint32_t)(id >> 32), (uint32_t)d, (uint32_t)(d >> 32), (uint32_t)seed, (uint32_t)(seed >> 32), o);
+  return make_uint4(o[0], o[1], o[2], o[3]);
+}
+
+// The veto of cycle cy (its first block: draw) of an event: the arithmetic of
+// step_veto and isr_eval32 for dipole type `type`, with the end's constants read
+// from the table.
+__device__ __forceinline__ GWeight weigh_cycle(const MixedCtx& M, const SmemPdf& S, const LearnedSmem& ls, const WS& w,
+                                               int n, int row, bool learned_ok, uint64_t id, uint64_t draw, int type,
+                                               const GCycle& cy) {
+  const int bq = cy.end(), bch = cy.channel();
+  const float bRz = cy.Rz;
+  GWeight out{0.0f, 0.0f, 0.0f, kCycVeto};
+  const float tw = __expf(cy.best);
+  // the winner's dipole as the last table stored it
+  const float4 ax = w.Aux(bq), bn = w.Bnd(bq);
+  const uint32_t ti = __float_as_uint(ax.z);
+  const int fl_i = tag_fl(ti);
+  const bool ini = type == kIF || type == kII;
+  const int ch = (ini ? (fl_i == 21 ? 5 : 3) : (fl_i == 21 ? 1 : 0)) + bch;
+  const float s = ax.x;
+  const float eta = ax.y;
+  int shape;
+  float coef;
+  channel_over32(ch, type, M.P.nf, shape, coef);
+  // the z limits at the cutoff (a winner's end has them)
+  const float delta = bn.w, zm = ini ? eta + delta : delta;
+  // learned bounds: pick the bin from R_z, then zeta inside it
+  const bool learned_end = M.Lc.learned && learned_ok && ini;
+  float zeta = bRz, Um = 1.0f;
+  int mbin = -1;
+  if (learned_end) {
+    float U[8], tot = 0.0f;
+    const uint2 kc = *reinterpret_cast<const uint2*>(ls.at(bq, bch, w.lane));
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+      U[m] = ls.dec[((m < 4 ? kc.x : kc.y) >> (8 * (m & 3))) & 0xffu];
+      tot += U[m];
+    }
+    const float target = bRz * tot;
+    float acc = 0.0f, Up = U[7];
+    int mb = 7;  // when no earlier bin is reached, acc = U[0] + ... + U[6]
+    bool found = false;
+#pragma unroll
+    for (int m = 0; m < 7; ++m) {
+      if (!found) {
+        if (target < acc + U[m]) { mb = m; Up = U[m]; found = true; }
+        else acc += U[m];
+      }
+    }
+    Um = Up;
+    mbin = mb;
+    float frac = Um > 0.0f ? (target - acc) / Um : 0.5f;
+    frac = fminf(fmaxf(frac, 0.0f), 0.99999994f);
+    zeta = ((float)mb + frac) * 0.125f;
+  }
+  // shape_sample32 and shape_val32 with one logarithm, power and quotient for
+  // the shapes that have them (the lanes of a warp hold all of them)
+  float z, omz, pover = coef;
+  if (shape == kFlat) {
+    const float zp = 1.0f - delta;
+    z = zm + zeta * (zp - zm);
+    omz = 1.0f - z;
+  } else {
+    const float zp = 1.0f - delta, omm = 1.0f - zm;
+    const float la = __logf((shape == kSoft ? delta : shape == kBoth ? zm : zp) / (shape == kInv ? zm : omm));
+    float arg;
+    if (shape == kBoth) {
+      const float lp = __logf(zp / delta);
+      arg = -(la + zeta * (lp - la));
+    } else {
+      arg = zeta * la;
+    }
+    const float ex = __expf(arg);
+    if (shape == kSoft) {
+      omz = omm * ex;
+      z = 1.0f - omz;
+    } else if (shape == kBoth) {
+      z = 1.0f / (1.0f + ex);
+      omz = ex / (1.0f + ex);
+    } else {
+      z = zm * ex;
+      omz = 1.0f - z;
+    }
+    pover = coef / (shape == kSoft ? omz : shape == kBoth ? z * omz : z);
+  }
+  float zm_t, delta_t;
+  if (!zlim32(type, tw, s, eta, zm_t, delta_t) || !(omz > delta_t) || !(z > zm_t)) return out;
+  const float as_t = (float)M.P.as_mz / (1.0f + (float)M.P.as_mz * (float)M.P.beta0 * __logf(tw / (float)(kMZ * kMZ)));
+  const float as_ratio = as_t / (S.asOver2pi[row] * 2.0f * (float)kPi);
+  float w8 = 0.0f, x = 1.0f, J = 1.0f, kk, x1 = 0.0f, F1 = 0.0f;
+  int new_fl_i = fl_i, fl_j = 21, num = 0, den_i = 0;
+  // (each kernel in one expression with its pole, as in step_veto: FP32
+  // quotients are products with a reciprocal here, so a quotient taken out of a
+  // branch would be contracted differently and change the last bit)
+  if (type == kFF) {
+    const float y = tw / (z * omz * s);
+    const float den = omz + z * y;
+    if (ch == 0) kk = (float)kCF * (2.0f / den - (1.0f + z));
+    else if (ch == 1) kk = (float)kCA * 0.5f * (2.0f / den - 2.0f + z * omz);
+    else kk = M.P.nf * (float)kTR * 0.5f * (1.0f - 2.0f * z * omz);
+    w8 = as_ratio * (1.0f - y) * kk / pover;
+  } else if (type == kFI) {
+    const float rho = tw / (z * omz * s);
+    x = 1.0f / (1.0f + rho);
+    const float omx = rho / (1.0f + rho);
+    const float den = omz + omx;
+    if (ch == 0) kk = (float)kCF * (2.0f / den - (1.0f + z));
+    else if (ch == 1) kk = (float)kCA * 0.5f * (2.0f / den - 2.0f + z * omz);
+    else kk = M.P.nf * (float)kTR * 0.5f * (1.0f - 2.0f * z * omz);
+    x1 = eta * (1.0f + rho);
+    num = den_i = pdf_index(tag_fl(__float_as_uint(ax.w)));
+  } else {
+    // the maps of isr_eval32
+    const float r = tw / s;
+    float omx, soft;
+    if (type == kIF) {
+      const float q = omz + r;
+      const float disc = 1.0f - 4.0f * r * z * omz / (q * q);
+      if (!(disc >= 0.0f)) return out;
+      x = 2.0f * z * omz / (q * (1.0f + sqrtf(disc)));
+      const float u = x * r / omz;
+      const float omu = 1.0f - u;
+      if (!(omu > 0.0f)) return out;
+      omx = omz / omu;
+      J = 1.0f / (x * omu + u * omx);
+      soft = omx + u;
+    } else {
+      x = z * omz / (omz + r);
+      omx = (omz * omz + r) / (omz + r);
+      const float v = x * r / omz;
+      if (!(omx - v > 0.0f)) return out;
+      J = 1.0f / z;
+      soft = omx;
+    }
+    if (!(x > eta)) return out;
+    if (ch == 3) kk = (float)kCF * (2.0f / soft - (1.0f + x));
+    else if (ch == 4) kk = (float)kTR * (1.0f - 2.0f * x * omx);
+    else if (ch == 5) kk = (float)kCA * (1.0f / soft + omx / x - 1.0f + x * omx);
+    else kk = (float)kCF * 0.5f * (x + 2.0f * omx / x);
+    isr_pdf_indices(ch, fl_i, num, den_i);
+    x1 = eta / x;
+  }
+  if (type != kFF) {
+    // the densities: the one under the ratio is the end's own where the table
+    // does not depend on Q^2
+    F1 = pdf32(M, S, num, x1, tw);
+    float F0;
+    if (M.q_independent) F0 = tw >= (float)kQ2Min && tw <= (float)kQ2Max ? bn.z : 0.0f;
+    else F0 = pdf32(M, S, den_i, eta, tw);
+    const float B = bch == 0 ? bn.x : bn.y;
+    if (!ini) {
+      const float ratio = F0 > 0.0f ? x * F1 / F0 : 0.0f;
+      w8 = as_ratio * kk / pover * ratio / B;
+    } else {
+      float Fratio = F0 > 0.0f ? F1 / F0 : 0.0f;
+      if (ch == 3 || ch == 4) {
+        const float m2 = S.m2[pdf_index(fl_i)];
+        if (m2 > 0.0f) Fratio *= (tw - m2) / tw;  // heavy-quark measure correction
+      }
+      const float rr = B > 0.0f ? kk * J * x / pover * Fratio / B : 0.0f;
+      w8 = as_ratio * rr / Um;
+      if (ch == 4) { new_fl_i = 21; fl_j = -fl_i; }
+      if (ch == 5) { new_fl_i = 21; fl_j = 21; }
+    }
+  }
+  out.z = z;
+  out.omz = omz;
+  out.w = w8;
+  if (!isfinite(w8)) {
+    out.what = kCycNumeric;
+    return out;
+  }
+  const uint4 o1 = block_of(M.P.seed, id, draw);
+  if (w8 > 1.0f && learned_end) {
+    out.omz = zeta;
+    out.what = kCycViolation | (mbin << 16);
+    return out;
+  }
+  if (!(u24(o1.y) < w8)) return out;
+  if (ch == 2 || ch == 6) {
+    const float Rfl = u24(block_of(M.P.seed, id, draw + 1).y);
+    if (ch == 2) {
+      int f = 1 + (int)floorf(Rfl * M.P.nf);
+      if (f > M.P.nf) f = M.P.nf;
+      new_fl_i = f; fl_j = -f;
+    } else {
+      float target = Rfl * F1, acc = 0.0f;
+      int pick = 10;
+#pragma unroll 1
+      for (int f = 1; f <= 10; ++f) {
+        acc += pdf32(M, S, f, x1, tw);
+        if (target < acc) { pick = f; break; }
+      }
+      int fl = pick <= 5 ? pick : -(pick - 5);
+      new_fl_i = fl; fl_j = fl;
+    }
+  }
+  out.what = (n >= M.P.nmax ? kCycCapacity : kCycAccept) | ((new_fl_i & 0xff) << 8) | ((fl_j & 0xff) << 16);
+  return out;
+}
+
+// the larger kept trial of end q
+__device__ __forceinline__ void keep_max(GSmem& F, const WS& w, int slot, int q, float m) {
+  if (q < kTmx) F.tmx[slot][q] = m;
+  else w.Tmx(q) = m;
+}
+// end q's kept trial of one channel
+__device__ __forceinline__ void keep_channel(const WS& w, int q, int ch, float lt, float rz) {
+  reinterpret_cast<float2*>(&w.Trial(q))[ch] = make_float2(lt, rz);
+}
+
+// the kept trials of end q from block d on
+__device__ __forceinline__ void draw_end(const MixedCtx& M, GSmem& F, const SmemPdf& S, const WS& w, int slot, int q,
+                                         const float4& rec,
+                                         uint64_t id, uint64_t d, float lnT, int row, GCount& cnt) {
+  float4 tr = make_float4(-INFINITY, 0.5f, -INFINITY, 0.5f);
+  if (__float_as_int(rec.w) >= 0) {
+    const float lnTc = S.lnTc[row], lnTmax = fminf(lnT, rec.z);
+    const bool above = lnTmax > lnTc;
+    const float m2 = M.heavy && q < 4 ? end_m2(S, w.Aux(q), q, row) : 0.0f;
+    const bool isr = S.pp[row] != 0 && q < 4;
+#pragma unroll 1
+    for (int c = 0; c < 2; ++c) {
+      const float ic = c == 0 ? rec.x : rec.y;  // 1/c
+      if (ic < 0.0f) continue;                  // channel absent for this emitter
+      const uint64_t dc = d++;
+      if (!(above && ic > 0.0f)) continue;
+      const uint4 o = block_of(M.P.seed, id, dc);
+      const float lt = trial_lnt(lnTmax, ic, __logf(u24(o.y)), m2), rz = u24(o.w);
+      cnt.trials += 1;
+      cnt.isr_trials += isr ? 1 : 0;
+      if (c == 0) { tr.x = lt; tr.y = rz; }
+      else { tr.z = lt; tr.w = rz; }
+    }
+  }
+  w.Trial(q) = tr;
+  keep_max(F, w, slot, q, tr.z > tr.x ? tr.z : tr.x);
+}
+
+// ---- load: eight lanes per slot -------------------------------------------
+// The slot's ended event (if `store`) back into the caller's records.
+__device__ __forceinline__ void store_slot(const MixedCtx& M, GSmem& F, const WS& w, int slot, int gl, GCount& cnt) {
+  const DevEvents& E = M.E;
+  const uint64_t e = F.ev[slot];
+  const int n = F.n[slot];
+  for (int p = gl; p < n; p += 8) {
+    double v[4];
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) v[mu] = w.P(mu, p);
+    const uint32_t t = w.T(p);
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) E.P(mu, p, e) = v[mu];
+    E.F(p, e) = tag_fl(t);
+    E.C(p, e) = tag_col(t);
+    E.A(p, e) = tag_acol(t);
+  }
+  if (gl == 0) {
+    const int st = F.end[slot];
+    E.npart[e] = n;
+    E.n_emit[e] = F.n_emit[slot];
+    E.status[e] = st;
+    E.t[e] = (double)__expf(F.lnT[slot]);
+    E.eta[e] = F.eta0[slot];
+    E.eta[E.cap + e] = F.eta1[slot];
+    E.draw[e] = F.draw[slot];
+    cnt.finished += 1;
+    if (st == GAPS_ERR_CAPACITY) cnt.err_cap += 1;
+    else if (st == GAPS_ERR_ITER_CAP) cnt.err_iter += 1;
+    else if (st == GAPS_ERR_NUMERIC) cnt.err_num += 1;
+  }
+}
+// The launch's next event into the slot; an empty slot when there is none.
+__device__ __forceinline__ void refill_slot(const MixedCtx& M, GSmem& F, const LearnedSmem& ls, const WS& w, int slot,
+                                            int gl, GCount& cnt) {
+  const DevEvents& E = M.E;
+  const unsigned group = 0xffu << (threadIdx.x & 24);
+  __syncwarp(group);  // the slot was read by all eight lanes
+  while (true) {
+    unsigned long long e = 0;
+    if (gl == 0) e = atomicAdd(M.next, 1ull);
+    e = __shfl_sync(group, e, 0, 8);
+    if (e >= M.n) {
+      if (gl == 0) F.live[slot] = 0;
+      return;
+    }
+    int st = E.status[e];
+    const int n = E.npart[e];
+    const float lnT = __logf((float)E.t[e]);
+    const bool bad = st == GAPS_STATUS_ACTIVE && (n < 2 || n > M.P.nmax);
+    if (bad) st = GAPS_ERR_NUMERIC;
+    if (st != GAPS_STATUS_ACTIVE) {
+      // not an event to shower: only its scalars are written, in the
+      // persistent schedule always, in the wavefront if it is refused
+      __syncwarp(group);
+      if (gl == 0) {
+        if (bad || !M.wave) {
+          E.status[e] = st;
+          E.t[e] = (double)__expf(lnT);
+        }
+        cnt.finished += 1;
+        if (bad && M.wave) cnt.err_num += 1;
+      }
+      continue;
+    }
+    for (int p = gl; p < n; p += 8) {
+#pragma unroll
+      for (int mu = 0; mu < 4; ++mu) w.P(mu, p) = E.P(mu, p, e);
+      w.T(p) = pack_tag(E.F(p, e), E.C(p, e), E.A(p, e));
+    }
+    if (gl < 4 && ls.key) ls.keyat(gl, w.lane) = make_float4(-1.0f, -1.0f, -1.0f, 0.0f);
+    if (gl == 0) {
+      F.ev[slot] = e;
+      F.draw[slot] = E.draw[e];
+      F.eta0[slot] = E.eta[e];
+      F.eta1[slot] = E.eta[E.cap + e];
+      F.lnT[slot] = lnT;
+      F.n[slot] = n;
+      F.n_emit[slot] = E.n_emit[e];
+      F.steps[slot] = 0;
+      F.row[slot] = mix_row(M.P, M.first + e);
+      F.live[slot] = 1;
+      F.end[slot] = GAPS_STATUS_ACTIVE;
+      F.table[slot] = 1;
+      F.keep[slot] = 0;
+      F.chg[slot] = -1;
+    }
+    return;
+  }
+}
+
+// ---- touch: eight lanes per slot ------------------------------------------
+// (slot < 0: none for this group; the warp's groups go together)
+__device__ __forceinline__ void phase_touch(GSmem& F, const WS& w, int slot, int gl) {
+  const int what = slot >= 0 ? F.table[slot] : 0;
+  slot = max(slot, 0);
+  const int n = F.n[slot], ne = what == 1 ? 2 * n : 0;
+  const int keep = F.keep[slot], chg = F.chg[slot];
+  const int ci = chg & 0xff, ck = (chg >> 8) & 0xff, T = 99 + n;
+  const uint32_t* tg = &w.T(0);
+  unsigned bits = 0;  // bit r: end 8 r + gl
+  const int scans = __reduce_max_sync(0xffffffffu, (ne + 7) / 8);
+#pragma unroll 4
+  for (int r = 0; r < scans; ++r) {
+    const int q = r * 8 + gl;
+    bool form = q < ne;
+    if (form && chg >= 0 && q < keep) {
+      // an end away from the emitter, the spectator and the new parton whose
+      // partner is neither of them keeps its record (the same bits that a
+      // recomputation gives); one without a partner or with the new tag is
+      // matched again
+      const int i = q >> 1, k = __float_as_int(w.End(q).w);
+      const uint32_t ti = tg[i];
+      const int tag = (q & 1) ? tag_acol(ti) : tag_col(ti);
+      form = !(i != ci && i != ck && k != ci && k != ck && (tag == 0 || (k >= 0 && tag != T)));
+    }
+    bits |= form ? 1u << r : 0u;
+  }
+  const bool one = what == 2;  // a failed map: the winner's end draws again
+  if (one && gl == 0) bits = 1u;
+  const int mine = __popc(bits);
+  int inc = mine;
+#pragma unroll
+  for (int o = 1; o < 8; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, inc, o, 8);
+    if (gl >= o) inc += t;
+  }
+  const int todo = __shfl_sync(0xffffffffu, inc, 7, 8);
+  int base = 0;
+  if (gl == 0 && what) base = atomicAdd(&F.n_ends, todo);
+  base = __shfl_sync(0xffffffffu, base, 0, 8);
+  const bool fits = what && base + todo <= kEndList;
+  if (gl == 0 && what) {
+    if (fits) atomicMax(&F.n_ends_ok, base + todo);
+    F.ready[slot] = fits;
+  }
+  if (what) {
+    F.mk1[slot][gl] = 0;
+    F.mk2[slot][gl] = 0;
+  }
+  if (fits) {
+    int at = base + inc - mine;
+    while (bits) {
+      const int r = __ffs(bits) - 1;
+      bits &= bits - 1;
+      F.ends[at++] = one ? 0x10000u | (slot << 8) | chg : (slot << 8) | (r * 8 + gl);
+    }
+  }
+}
+
+// ---- form: one lane per end -----------------------------------------------
+__device__ __forceinline__ void phase_form(const MixedCtx& M, GSmem& F, const SmemPdf& S, const LearnedSmem& ls,
+                                           int base_lane, int tid, GCount& cnt) {
+  // 8 to 32 ends a warp: a pass is a chain of dependent loads, which the other
+  // warps hide
+  const int total = F.n_ends_ok, per = min(32, max(8, (total + kWorkers / 32 - 1) / (kWorkers / 32)));
+  if ((tid & 31) >= per) return;
+  for (int j = (tid >> 5) * per + (tid & 31); j < total; j += per * (kWorkers / 32)) {
+    const unsigned ent = F.ends[j];
+    const int slot = (ent >> 8) & 0xff, q = ent & 0xff;
+    const WS w{M.W, base_lane + slot, M.P.nmax};
+    const float4 old = w.End(q);  // (on its way while the record is formed)
+    float4 rec;
+    bool marked;
+    if (ent & 0x10000u) {
+      rec = old;
+      marked = true;
+    } else {
+      const int n = F.n[slot], row = F.row[slot], keep = F.keep[slot];
+      const bool pp = S.pp[row] != 0;
+      const uint32_t* tg = &w.T(0);
+      float s, eta;
+      int type;
+      float4 aux, bnd;
+      rec = end_record_impl<true>(M, S, w, tg, nullptr, n, (float)F.eta0[slot], (float)F.eta1[slot], row, q, s, eta, type,
+                                  aux, bnd);
+      w.Aux(q) = aux;
+      if (type >= 0) w.Bnd(q) = bnd;
+      bool anew = q >= keep;
+      if (pp && q < 4) {
+        // an initial-state end: with the learned proposal its record is scaled
+        // by the mean bin height, from the network when its inputs changed
+        const bool valid = type >= 0 && rec.x > 0.0f && rec.y > 0.0f && (type == kIF || type == kII);
+        const int fl_i = tag_fl(tg[q >> 1]);
+        if (valid && M.Lc.learned && F.live[slot] == 1) {
+          const float4 key = ls.keyat(q, w.lane);
+          const float code = (float)(type * 32 + pdf_index(fl_i));
+          if (!(key.x == eta && key.y == s && key.z == code)) {
+            atomicOr(&F.defer[slot], 1u << q);
+            F.q[atomicAdd(&F.n_q, 1)] = (unsigned short)(4 * slot + q);
+            anew = true;
+            cnt.tiles += 1;
+          } else {
+            rec.x = old.x;
+            rec.y = old.y;
+          }
+        } else if (ls.code) {
+          // every other one proposes with height 1 in all bins (the plain bound)
+          for (int c = 0; c < 2; ++c) *reinterpret_cast<uint2*>(ls.at(q, c, w.lane)) = make_uint2(0u, 0u);
+          ls.keyat(q, w.lane) = make_float4(-1.0f, -1.0f, -1.0f, 0.0f);
+        }
+      }
+      // an end whose record is unchanged keeps its trials (set_end's rule)
+      marked = anew;
+      if (!anew) {
+        marked = !(__float_as_uint(old.x) == __float_as_uint(rec.x) && __float_as_uint(old.y) == __float_as_uint(rec.y) &&
+                   __float_as_uint(old.z) == __float_as_uint(rec.z) && __float_as_uint(old.w) == __float_as_uint(rec.w));
+      }
+      if (marked) w.End(q) = rec;
+    }
+    if (marked) {
+      // Philox blocks of this end: one per channel present
+      const int nd = __float_as_int(rec.w) >= 0 ? (rec.x >= 0.0f ? 1 : 0) + (rec.y >= 0.0f ? 1 : 0) : 0;
+      if (nd) {
+        atomicOr(nd == 1 ? &F.mk1[slot][q >> 5] : &F.mk2[slot][q >> 5], 1u << (q & 31));
+        atomicAdd(&F.tot[slot], nd);
+      }
+    }
+    F.ends[j] = (ent & 0xffffu) | (marked ? 0x10000u : 0u);
+  }
+}
+
+// ---- draw: one lane per marked end, and the chain's uniforms --------------
+__device__ __forceinline__ void phase_draw(const MixedCtx& M, GSmem& F, const SmemPdf& S, int base_lane, int tid,
+                                           GCount& cnt) {
+  const int total = F.n_ends_ok, per = min(32, max(8, (total + kWorkers / 32 - 1) / (kWorkers / 32)));
+  for (int j = (tid >> 5) * per + (tid & 31); (tid & 31) < per && j < total; j += per * (kWorkers / 32)) {
+    const unsigned ent = F.ends[j];
+    if (!(ent & 0x10000u)) continue;
+    const int slot = (ent >> 8) & 0xff, q = ent & 0xff;
+    if (q < 4 && ((F.defer[slot] >> q) & 1u)) continue;  // drawn after the network
+    int off = 0;
+    const int wq = q >> 5;
+    for (int k = 0; k < wq; ++k) off += __popc(F.mk1[slot][k]) + 2 * __popc(F.mk2[slot][k]);
+    const unsigned below = (1u << (q & 31)) - 1u;
+    off += __popc(F.mk1[slot][wq] & below) + 2 * __popc(F.mk2[slot][wq] & below);
+    const WS w{M.W, base_lane + slot, M.P.nmax};
+    draw_end(M, F, S, w, slot, q, w.End(q), M.first + F.ev[slot], F.draw[slot] + (uint64_t)off, F.lnT[slot], F.row[slot], cnt);
+  }
+  // block 3 k + 2 below: the next trial of cycle k's winner if it is vetoed
+  for (int i = tid; i < kCyc * kSlots; i += kWorkers) {
+    const int slot = i % kSlots, k = i / kSlots;
+    if (!F.ready[slot]) continue;
+    const uint64_t id = M.first + F.ev[slot], d = F.draw[slot] + (uint64_t)F.tot[slot] + 3 * (uint64_t)k + 2;
+    const uint4 o = block_of(M.P.seed, id, d);
+    F.cyc[k][slot] = GCycle{0, __logf(u24(o.y)), u24(o.w)};
+  }
+}
+
+// ---- net: the network's tiles of the queued ends, four a warp step --------
+__device__ __forceinline__ void phase_net(const MixedCtx& M, GSmem& F, const SmemPdf& S, const LearnedSmem& ls,
+                                          const MlpSmem& mlp, int base_lane, int warp_id, int lane_id, GCount& cnt) {
+  const int nq = F.n_q;
+  for (int g = warp_id; 4 * g < nq; g += kWorkers / 32) {
+    const int j = 4 * g + lane_id;
+    const bool have = lane_id < 4 && j < nq;
+    const int sl = have ? F.q[j] >> 2 : 0, q = have ? F.q[j] & 3 : 0, row = F.row[sl];
+    const WS w{M.W, base_lane + sl, M.P.nmax};
+    float4 ax = make_float4(1.0f, 0.5f, 0.0f, 0.0f), rec = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (have) {
+      ax = w.Aux(q);
+      rec = w.End(q);  // with the plain bound
+    }
+    const unsigned eval = __ballot_sync(0xffffffffu, have) & 0xFu;
+    const int type = __float_as_int(rec.w) < 2 ? kII : kIF;  // (the queued ends have a partner)
+    const float tc = have ? __expf(S.lnTc[row]) : 1.0f;
+    float scale0 = 0.0f, scale1 = 0.0f;
+    learned_heights(M, mlp, ls, F.m.stage[warp_id], F.m.ustage[warp_id], eval, tc, ax.y, ax.x, type,
+                    tag_fl(__float_as_uint(ax.z)), w.lane, q, lane_id, scale0, scale1, true);
+    if (have) {
+      rec.x *= scale0;
+      rec.y *= scale1;
+      w.End(q) = rec;
+      // its trials, at the counter reserved for them (ends 0 .. 3: word 0)
+      const unsigned below = (1u << q) - 1u;
+      const int off = __popc(F.mk1[sl][0] & below) + 2 * __popc(F.mk2[sl][0] & below);
+      draw_end(M, F, S, w, sl, q, rec, M.first + F.ev[sl], F.draw[sl] + (uint64_t)off, F.lnT[sl], row, cnt);
+    }
+    __syncwarp();
+  }
+}
+
+// ---- chain: four lanes per slot -------------------------------------------
+// Lane j holds the largest kept trial of its ends 16 r + 4 j .. + 3 and of every
+// fourth end from kTmx on, with that end's trials and record: the loads for a
+// lane's next candidate are on their way while the other lanes' candidates win.
+// (Holding the two largest, so that no load is waited for, cost more
+// instructions than it saved: 24 500 clocks a round against 16 500.)
+__device__ __forceinline__ void phase_chain(const MixedCtx& M, GSmem& F, const SmemPdf& S, int base_lane, int tid) {
+  const unsigned full = 0xffffffffu;
+  const int slot = tid >> 2, gl = tid & 3, gshift = tid & 28;
+  const bool on = F.ready[slot];
+  const WS w{M.W, base_lane + slot, M.P.nmax};
+  const int ne = on ? 2 * F.n[slot] : 0, row = F.row[slot];
+  const bool pp = S.pp[row] != 0;
+  const float lnTc = S.lnTc[row];
+  if (on && gl == 0) {
+    F.draw[slot] += (uint64_t)F.tot[slot];
+    F.nv[slot] = 0;
+    if (F.table[slot] == 1) F.table[slot] = 3;  // (counted at the commit)
+  }
+  // the largest of each of the lane's four quadruples of ends, of the ends from
+  // kTmx on, and of all; then the (lowest) end that has it
+  float qm[kTmx / 16], om = -INFINITY, m1;
+  auto quad = [&](int r) {
+    const int q = 16 * r + 4 * gl;
+    const float4 v = *reinterpret_cast<const float4*>(&F.tmx[slot][q]);
+    const float a = q < ne ? v.x : -INFINITY, b = q + 1 < ne ? v.y : -INFINITY;
+    const float c = q + 2 < ne ? v.z : -INFINITY, d = q + 3 < ne ? v.w : -INFINITY;
+    return fmaxf(fmaxf(a, b), fmaxf(c, d));
+  };
+  auto rest = [&]() {
+    om = -INFINITY;
+    for (int q = kTmx + gl; q < ne; q += 4) om = fmaxf(om, w.Tmx(q));
+  };
+  auto largest = [&]() {
+    m1 = fmaxf(fmaxf(fmaxf(qm[0], qm[1]), fmaxf(qm[2], qm[3])), om);
+  };
+  auto locate = [&]() -> int {
+    if (!(m1 > -INFINITY)) return -1;
+    const int r = qm[0] == m1 ? 0 : qm[1] == m1 ? 1 : qm[2] == m1 ? 2 : qm[3] == m1 ? 3 : 4;
+    if (r == 4) {
+      int q = kTmx + gl;
+      while (q + 4 < ne && w.Tmx(q) != m1) q += 4;
+      return q;
+    }
+    const int q = 16 * r + 4 * gl;
+    const float4 v = *reinterpret_cast<const float4*>(&F.tmx[slot][q]);
+    return q + (v.x == m1 ? 0 : v.y == m1 ? 1 : v.z == m1 ? 2 : 3);
+  };
+#pragma unroll
+  for (int r = 0; r < kTmx / 16; ++r) qm[r] = quad(r);
+  if (ne > kTmx) rest();
+  largest();
+  int q1 = locate();
+  float4 tr = w.Trial(max(q1, 0)), rec = w.End(max(q1, 0));
+  int len = 0;
+  bool done = false, going = on;
+#pragma unroll 1
+  for (int k = 0; k < kCyc; ++k) {
+    float best = fmaxf(m1, __shfl_xor_sync(full, m1, 1));
+    best = fmaxf(best, __shfl_xor_sync(full, best, 2));
+    bool mine = q1 >= 0 && m1 == best;
+    unsigned own = (__ballot_sync(full, mine) >> gshift) & 0xfu;
+    if (__any_sync(full, (own & (own - 1)) != 0)) {  // equal trials: the lowest end wins
+      int qm = mine ? q1 : 0x7fffffff;
+      qm = min(qm, __shfl_xor_sync(full, qm, 1));
+      qm = min(qm, __shfl_xor_sync(full, qm, 2));
+      mine = mine && q1 == qm;
+      own = (__ballot_sync(full, mine) >> gshift) & 0xfu;
+    }
+    if (going && (own == 0 || best < lnTc)) {
+      done = true;
+      going = false;
+    }
+    if (!__any_sync(full, going)) break;
+    len += going ? 1 : 0;
+    if (going && mine) {
+      const int q = q1, ch = tr.z > tr.x ? 1 : 0;
+      const GCycle rd = F.cyc[k][slot];
+      const float ic = ch == 0 ? rec.x : rec.y;
+      const float lnTmax = fminf(best, rec.z);
+      float lt = -INFINITY, rz = 0.5f;
+      int counted = 0;
+      if (lnTmax > lnTc && ic > 0.0f) {
+        counted = pp && q < 4 ? 3 : 1;
+        const float hq = M.heavy && q < 4 ? end_m2(S, w.Aux(q), q, row) : 0.0f;
+        lt = trial_lnt(lnTmax, ic, rd.best, hq);
+        rz = rd.Rz;
+      }
+      const bool ini = pp && q < 4, ink = pp && __float_as_int(rec.w) < 2;
+      const int type = ini ? (ink ? kII : kIF) : (ink ? kFI : kFF);
+      F.cyc[k][slot] = GCycle{(2 * q + ch) | (counted << 9) | (type << 12), best, ch ? tr.w : tr.y};
+      if (ch == 0) { tr.x = lt; tr.y = rz; } else { tr.z = lt; tr.w = rz; }
+      keep_channel(w, q, ch, lt, rz);
+      keep_max(F, w, slot, q, tr.z > tr.x ? tr.z : tr.x);
+      if (q < kTmx) {
+        const int r = q >> 4;
+        const float m = quad(r);
+#pragma unroll
+        for (int u = 0; u < kTmx / 16; ++u)
+          if (u == r) qm[u] = m;
+      } else {
+        rest();
+      }
+      largest();
+      q1 = locate();
+      if (q1 != q && q1 >= 0) {
+        tr = w.Trial(q1);
+        rec = w.End(q1);
+      }
+    }
+  }
+  if (on && gl == 0) {
+    F.len[slot] = len;
+    F.done[slot] = done;
+  }
+}
+
+// ---- list: the chain's cycles by dipole type, one lane per cycle ----------
+__device__ __forceinline__ void phase_list(GSmem& F, int tid, int lane_id) {
+  int it[2], type[2], base = 0;
+  unsigned m[2][4];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int i = tid + h * kWorkers, slot = i % kSlots, k = i / kSlots;
+    it[h] = 8 * slot + k;
+    type[h] = k < kCyc && F.ready[slot] && k < F.len[slot] ? F.cyc[k][slot].type() : -1;
+#pragma unroll
+    for (int t = 0; t < 4; ++t) m[h][t] = __ballot_sync(0xffffffffu, type[h] == t);
+  }
+  // lane t reserves the warp's places in list t
+#pragma unroll
+  for (int t = 0; t < 4; ++t)
+    if (lane_id == t) base = atomicAdd(&F.n_items[t], __popc(m[0][t]) + __popc(m[1][t]));
+  const unsigned below = (1u << lane_id) - 1u;
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    const int b = __shfl_sync(0xffffffffu, base, t);
+    if (type[0] == t) F.items[t][b + __popc(m[0][t] & below)] = (unsigned short)it[0];
+    if (type[1] == t) F.items[t][b + __popc(m[0][t]) + __popc(m[1][t] & below)] = (unsigned short)it[1];
+  }
+}
+
+// ---- weigh: one lane per cycle, a warp's cycles of one dipole type --------
+__device__ __forceinline__ void phase_weigh(const MixedCtx& M, GSmem& F, const SmemPdf& S, const LearnedSmem& ls,
+                                            int base_lane, int warp_id, int lane_id, GCount& cnt) {
+  int c = warp_id;  // chunk of 32 items, the types one after the other
+#pragma unroll 1
+  for (int t = 0; t < 4; ++t) {
+    const int n = F.n_items[t], chunks = (n + 31) / 32;
+    for (; c < chunks; c += kWorkers / 32) {
+      const int j = 32 * c + lane_id;
+      cnt.warp_steps += 1;
+      if (j < n) {
+        const int it = F.items[t][j], slot = it >> 3, k = it & 7;
+        const WS w{M.W, base_lane + slot, M.P.nmax};
+        const GCycle cy = F.cyc[k][slot];
+        const GWeight r = weigh_cycle(M, S, ls, w, F.n[slot], F.row[slot], F.live[slot] == 1, M.first + F.ev[slot],
+                                      F.draw[slot] + 3 * (uint64_t)k, t, cy);
+        cnt.lane_steps += 1;
+        if ((r.what & 0xff) != kCycVeto) {
+          F.wt[k][slot] = r;
+          atomicOr(&F.nv[slot], 1u << k);
+        }
+      }
+    }
+    c -= chunks;
+  }
+}
+
+// ---- commit: one lane per slot --------------------------------------------
+__device__ __forceinline__ void phase_commit(const MixedCtx& M, GSmem& F, int base_lane, int tid, int par, GCount& cnt) {
+  const int slot = tid;
+  if (slot >= kSlots || !F.ready[slot]) return;
+  const WS w{M.W, base_lane + slot, M.P.nmax};
+  if (F.table[slot]) {
+    cnt.rebuilds += F.table[slot] == 3 ? 1 : 0;
+    F.table[slot] = 0;
+  }
+  const int len = F.len[slot], room = M.P.max_steps - F.steps[slot];
+  int f = F.nv[slot] ? __ffs(F.nv[slot]) - 1 : -1;
+  if (f >= room) f = -1;
+  const int vetoed = f >= 0 ? f : min(len, room);  // committed vetoed cycles
+  float lnT = F.lnT[slot];
+  for (int k = 0; k < vetoed; ++k) {
+    const int c = F.cyc[k][slot].win;
+    cnt.trials += (c >> 9) & 1;
+    cnt.isr_trials += (c >> 10) & 1;
+  }
+  cnt.steps += vetoed;
+  cnt.vetoes += vetoed;
+  if (vetoed > 0) lnT = F.cyc[vetoed - 1][slot].best;
+  // the trials that the cycles from f (or from the cap) on replaced, back, the
+  // latest first (a cycle may replace what an earlier one wrote)
+  // (a winner's trial is its end's larger one)
+  for (int k = len - 1; k >= vetoed; --k) {
+    const GCycle c = F.cyc[k][slot];
+    keep_channel(w, c.end(), c.channel(), c.best, c.Rz);
+    keep_max(F, w, slot, c.end(), c.best);
+  }
+  uint64_t draw = F.draw[slot] + 3 * (uint64_t)vetoed;
+  int steps = F.steps[slot] + vetoed, st = GAPS_STATUS_ACTIVE;
+  if (f >= 0) {
+    const GCycle cy = F.cyc[f][slot];
+    const GWeight r = F.wt[f][slot];
+    const int out = r.what & 0xff;
+    if (out != kCycViolation) lnT = cy.best;
+    draw += 2;
+    steps += 1;
+    cnt.steps += 1;
+    if (r.w > 1.0f && out != kCycNumeric) {
+      cnt.violations += 1;
+      const int q = cy.end();
+      const float4 ax = w.Aux(q);
+      const int row = F.row[slot], fl = tag_fl(__float_as_uint(ax.z));
+      const SmemPdf& S = F.S;
+      const bool pp = S.pp[row] != 0, ini = pp && q < 4, ink = pp && __float_as_int(w.End(q).w) < 2;
+      const int type = ini ? (ink ? kII : kIF) : (ink ? kFI : kFF);
+      const int ch = (ini ? (fl == 21 ? 5 : 3) : (fl == 21 ? 1 : 0)) + cy.channel();
+      const float tw = __expf(cy.best);
+      if (out == kCycViolation) {
+        if (M.Lc.vlog) {
+          const unsigned long long at = atomicAdd(M.Lc.vcount, 1ull);
+          if (at < M.Lc.vcap) {
+            M.Lc.vlog[2 * at] = make_float4(ax.y, ax.x, tw, r.w);
+            M.Lc.vlog[2 * at + 1] = make_float4((float)isr_class(type, ch, fl), (float)(r.what >> 16), r.z, r.omz);
+          }
+        }
+      } else {
+        log_plain_violation(M, ax.y, ax.x, tw, r.w, type, ch, r.z);
+      }
+    }
+    if (out == kCycNumeric) st = GAPS_ERR_NUMERIC;
+    else if (out == kCycCapacity) st = GAPS_ERR_CAPACITY;
+    else if (steps < M.P.max_steps) {
+      F.park[slot] = cy;
+      F.pw[slot] = r;
+      F.parked[par][atomicAdd(&F.n_park[par], 1)] = (unsigned char)slot;
+      F.busy[slot] = 1;
+      // the learned bound failed: the event goes on from the scale before this
+      // cycle with the plain bounds
+      if (out == kCycViolation) F.live[slot] = 3;
+    }
+  } else if (F.done[slot] && vetoed == len && steps < M.P.max_steps) {
+    steps += 1;
+    cnt.steps += 1;
+    st = GAPS_STATUS_DONE;
+  }
+  if (st == GAPS_STATUS_ACTIVE && steps >= M.P.max_steps) st = GAPS_ERR_ITER_CAP;
+  F.lnT[slot] = lnT;
+  F.draw[slot] = draw;
+  F.steps[slot] = steps;
+  F.end[slot] = st;
+  if (st != GAPS_STATUS_ACTIVE) {
+    F.ended[par][atomicAdd(&F.n_ended[par], 1)] = (unsigned char)slot;
+    F.busy[slot] = 1;
+  }
+}
+
+// ---- emit: one lane per parked emission -----------------------------------
+__device__ __forceinline__ void phase_emit(const MixedCtx& M, GSmem& F, const SmemPdf& S, int base_lane, int par, int i,
+                                           GCount& cnt) {
+  const int slot = F.parked[par][i];
+  const WS w{M.W, base_lane + slot, M.P.nmax};
+  const GCycle cy = F.park[slot];
+  const GWeight r = F.pw[slot];
+  int table = 1, keep = 0, chg = -1;
+  if ((r.what & 0xff) == kCycAccept) {
+    const int q = cy.end(), bi = q >> 1, k = __float_as_int(w.End(q).w);
+    const uint32_t ti = __float_as_uint(w.Aux(q).z);
+    const bool pp = S.pp[F.row[slot]] != 0, ini = pp && bi < 2, ink = pp && k < 2;
+    const int type = ini ? (ink ? kII : kIF) : (ink ? kFI : kFF), fl = tag_fl(ti);
+    const int ch = (ini ? (fl == 21 ? 5 : 3) : (fl == 21 ? 1 : 0)) + cy.channel();
+    // the azimuth: words 2 and 3 of the veto's first block
+    const uint64_t id = M.first + F.ev[slot], d = F.draw[slot] - 2;
+    const uint4 o = block_of(M.P.seed, id, d);
+    const Emission em{0, bi, k, q & 1, ch, type, (int)(int8_t)((r.what >> 8) & 0xff), (int)(int8_t)((r.what >> 16) & 0xff),
+                      r.z, r.omz, __expf(cy.best), u01(o.z, o.w), ti};
+    Lane L;
+    L.n = F.n[slot];
+    L.n_emit = F.n_emit[slot];
+    L.eta0 = F.eta0[slot];
+    L.eta1 = F.eta1[slot];
+    if (emit(M, w, L, em)) {
+      cnt.accepts += 1;
+      keep = 2 * (L.n - 1);  // the ends that existed before
+      // an initial-initial emission kicks every final parton: all ends
+      if (type != kII) chg = bi | (k << 8);
+      F.n[slot] = L.n;
+      F.n_emit[slot] = L.n_emit;
+      F.eta0[slot] = L.eta0;
+      F.eta1[slot] = L.eta1;
+    } else {
+      cnt.vetoes += 1;  // the map failed: the winner's end draws again
+      table = 2;
+      chg = q;
+    }
+  }
+  F.table[slot] = table;
+  F.keep[slot] = keep;
+  F.chg[slot] = chg;
+  F.busy[slot] = 2;
+}
+
+// Before the round of parity par: the emitters' results are handed over, the
+// slots with ends to form listed.
+__device__ __forceinline__ void prepare_round(GSmem& F, int tid, int par) {
+  if (tid >= kSlots) return;
+  if (F.busy[tid] == 2) F.busy[tid] = 0;
+  const bool on = F.live[tid] && F.busy[tid] == 0;
+  F.ready[tid] = on;
+  F.tot[tid] = 0;
+  F.defer[tid] = 0;
+  if (on && F.table[tid]) F.tables[par][atomicAdd(&F.n_tables[par], 1)] = (unsigned char)tid;
+}
+
+__global__ void __launch_bounds__(kGThreads, 1) k_shower_groups(const __grid_constant__ MixedCtx M) {
+  extern __shared__ __align__(16) unsigned char group_smem[];
+  GSmem& F = *reinterpret_cast<GSmem*>(group_smem);
+  const SmemPdf& S = F.S;
+  {
+    const unsigned* src = reinterpret_cast<const unsigned*>(M.tables);
+    unsigned* dst = reinterpret_cast<unsigned*>(&F.S);
+    for (int k = threadIdx.x; k < (int)(sizeof(SmemPdf) / 4); k += kGThreads) dst[k] = src[k];
+  }
+  const int tid = threadIdx.x, lane_id = tid & 31, warp_id = tid >> 5, gl = tid & 7;
+  LearnedSmem ls;
+  ls.code = nullptr;
+  ls.key = nullptr;
+  ls.dec = F.dec;
+  if (M.Lc.learned) {
+    ls.code = M.W.lcode;
+    ls.key = M.W.lkey;
+    if (tid < 256) F.dec[tid] = tid < 255 ? exp2f(-(float)tid * 0.0625f) : 0.0f;
+  }
+  const MlpSmem& mlp = *reinterpret_cast<const MlpSmem*>(F.image);
+  if (M.Lc.learned) {
+    const uint4* src = reinterpret_cast<const uint4*>(M.Lc.image);
+    uint4* dst = reinterpret_cast<uint4*>(F.image);
+    for (int k = tid; k < (int)(kMlpSmemBytes / 16); k += kGThreads) dst[k] = src[k];
+  }
+  if (tid < kSlots) {
+    // (an empty slot is read too: the row is an index)
+    F.live[tid] = F.busy[tid] = F.ready[tid] = F.table[tid] = 0;
+    F.row[tid] = F.n[tid] = F.n_emit[tid] = F.steps[tid] = F.keep[tid] = F.tot[tid] = F.len[tid] = F.done[tid] = 0;
+    F.chg[tid] = -1;
+    F.end[tid] = GAPS_STATUS_ACTIVE;
+    F.lnT[tid] = 0.0f;
+    F.ev[tid] = F.draw[tid] = 0;
+    F.eta0[tid] = F.eta1[tid] = 0.0;
+    F.defer[tid] = F.nv[tid] = 0;
+  }
+  if (tid < 2) F.n_tables[tid] = F.n_park[tid] = F.n_ended[tid] = 0;
+  if (tid == 0) F.n_q = F.n_ends = F.n_ends_ok = 0;
+  if (tid < 4) F.n_items[tid] = 0;
+  __syncthreads();
+  const int base_lane = blockIdx.x * kSlots;
+  GCount cnt;
+  // the first events (few: their slots spread over the warps)
+  for (int i = tid >> 3; tid < kWorkers && i < M.slots; i += kWorkers / 8) {
+    const int slot = (i % (4 * kSlots / 32)) * 8 + i / (4 * kSlots / 32);  // eight slots a warp of the chain
+    refill_slot(M, F, ls, WS{M.W, base_lane + slot, M.P.nmax}, slot, gl, cnt);
+  }
+  __syncthreads();
+  prepare_round(F, tid, 0);
+  __syncthreads();
+  if (warp_id >= kWorkers / 32) {
+    // ---- the emitters ----------------------------------------------------
+    for (int par = 0;; par ^= 1) {
+      // the emissions and the ended events of the round before, beside the
+      // workers' round
+      for (int i = tid - kWorkers; i < F.n_park[par ^ 1]; i += kEmitters) phase_emit(M, F, S, base_lane, par ^ 1, i, cnt);
+      __syncwarp();
+      for (int i = (tid - kWorkers) >> 3; i < F.n_ended[par ^ 1]; i += kEmitters / 8) {
+        const int slot = F.ended[par ^ 1][i];
+        const WS w{M.W, base_lane + slot, M.P.nmax};
+        store_slot(M, F, w, slot, gl, cnt);
+        refill_slot(M, F, ls, w, slot, gl, cnt);
+        if (gl == 0) F.busy[slot] = 2;
+      }
+      if (!__syncthreads_or(0)) break;
+      __syncthreads();
+    }
+  } else {
+    // ---- the workers -----------------------------------------------------
+    for (int par = 0;; par ^= 1) {
+      const int n_tables = F.n_tables[par];
+      for (int i = tid >> 3; i - ((tid >> 3) & 3) < n_tables; i += kWorkers / 8) {  // (whole warps)
+        const int slot = i < n_tables ? F.tables[par][i] : -1;
+        phase_touch(F, WS{M.W, base_lane + max(slot, 0), M.P.nmax}, slot, gl);
+      }
+      workers_sync();
+      phase_form(M, F, S, ls, base_lane, tid, cnt);
+      workers_sync();
+      phase_draw(M, F, S, base_lane, tid, cnt);
+      workers_sync();
+      if (M.Lc.learned) {
+        phase_net(M, F, S, ls, mlp, base_lane, warp_id, lane_id, cnt);
+        workers_sync();
+      }
+      if (tid < 4 * kSlots) phase_chain(M, F, S, base_lane, tid);
+      workers_sync();
+      phase_list(F, tid, lane_id);
+      workers_sync();
+      phase_weigh(M, F, S, ls, base_lane, warp_id, lane_id, cnt);
+      workers_sync();
+      phase_commit(M, F, base_lane, tid, par, cnt);
+      // another round while a slot holds an event
+      if (!__syncthreads_or(tid < kSlots && F.live[tid] != 0)) break;
+      // between the two barriers nothing is in flight
+      if (tid == 0) {
+        F.n_park[par ^ 1] = F.n_ended[par ^ 1] = F.n_tables[par] = 0;
+        F.n_ends = F.n_ends_ok = F.n_q = 0;
+      }
+      if (tid < 4) F.n_items[tid] = 0;
+      prepare_round(F, tid, par ^ 1);
+      __syncthreads();
+    }
+  }
+  Counters32 sum;
+  sum.steps = cnt.steps; sum.trials = cnt.trials; sum.isr_trials = cnt.isr_trials;
+  sum.vetoes = cnt.vetoes; sum.accepts = cnt.accepts; sum.violations = cnt.violations;
+  flush_counters(M, sum, cnt.finished, cnt.err_cap, cnt.err_iter, cnt.err_num, cnt.lane_steps, cnt.warp_steps,
+                 cnt.rebuilds, cnt.tiles, lane_id);
+}
 
 // ---------------------------------------------------------------------------
 // Warp-per-event persistent shower (GAPS_SCHED_WARP). Each warp owns one event
@@ -2579,20 +3481,7 @@ __global__ void __launch_bounds__(MAXT, MINB) k_shower_warp(const __grid_constan
     ls.key = reinterpret_cast<float4*>(ls.code + (size_t)nw * 64);
     for (int k = threadIdx.x; k < 256; k += blockDim.x) dec[k] = k < 255 ? exp2f(-(float)k * 0.0625f) : 0.0f;
   }
-  for (int q = threadIdx.x; q < 12 * kSmNX; q += blockDim.x) {
-    int f = q / kSmNX, ix = q % kSmNX;
-    S.umax[f][ix] = (float)M.P.umax[q];
-    S.lmin[f][ix] = (float)M.P.lmin[q];
-    float xf = 0.0f;
-    if (f < 11) xf = M.P.grid[((size_t)f * kNX + ix) * kNQ];
-    else for (int k = 1; k <= 10; ++k) xf += M.P.grid[((size_t)k * kNX + ix) * kNQ];
-    S.xf[f][ix] = xf;
-  }
-  for (int q = threadIdx.x; q < 12 * (kSmNX + 1); q += blockDim.x)
-    S.sufmax[q / (kSmNX + 1)][q % (kSmNX + 1)] = (float)M.P.sufmax[q];
-  for (int q = threadIdx.x; q < 12 * kSmNX; q += blockDim.x) S.first[q / kSmNX][q % kSmNX] = (float)M.P.first[q];
-  if (threadIdx.x < 12) S.m2[threadIdx.x] = (float)M.P.m2[threadIdx.x];
-  load_rows(S, M.P);
+  load_tables(S, M);
   __syncthreads();
 
   Lane L;
@@ -2698,6 +3587,7 @@ void workset_carve(void* base, int lanes, int nmax, WorkSet& W) {
   W.lcode = (unsigned char*)p;
   p += (size_t)lanes * 64;
   W.tag = (uint32_t*)p;
+  W.bnd = nullptr;
 }
 
 
@@ -2806,6 +3696,7 @@ cudaError_t mixed_kernels_init() {
   e = opt_in(k_wave_veto<2>, bytes, e);
   e = opt_in(k_wave_veto<3>, bytes, e);
   e = opt_in(k_wave_veto<4>, bytes, e);
+  e = opt_in(k_shower_groups, (int)sizeof(GSmem), e);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_shower_warp<256, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWarpKernelMaxDyn);
   if (e == cudaSuccess)
@@ -2862,6 +3753,10 @@ MixedCtx mixed_ctx(const DevParams& P, const DevEvents& E, const WorkSet& W, con
   M.V = WaveSet{};
   M.wave_par = 0;
   M.wave_budget = 0;
+  M.slots = M.wave = 0;
+  M.heavy = 0;
+  for (int f = 0; f < 12; ++f) M.heavy = M.heavy || P.m2[f] > 0.0;
+  M.tables = nullptr;
   return M;
 }
 
@@ -2896,6 +3791,47 @@ cudaError_t launch_shower_mixed(const DevParams& P, const DevEvents& E, const Wo
   return cudaGetLastError();
 }
 
+// The kept-trial shower: one block per SM, each with a working set of kSlots
+// events.
+
+int groups_blocks(int sm_count) { return sm_count; }
+int groups_lanes(int blocks) { return blocks * kSlots; }
+size_t groups_bytes(int lanes, int nmax) {
+  return (workset_bytes(lanes, nmax) + 255) / 256 * 256 + (size_t)lanes * 2 * nmax * sizeof(float4);
+}
+void groups_carve(void* base, int lanes, int nmax, WorkSet& W) {
+  workset_carve(base, lanes, nmax, W);
+  W.bnd = (float4*)((char*)base + (workset_bytes(lanes, nmax) + 255) / 256 * 256);
+}
+
+namespace {
+__global__ void k_groups_tables(const __grid_constant__ MixedCtx M, SmemPdf* out) { load_tables(*out, M); }
+}  // namespace
+// the FP32 tables of a context (they depend on its parameters only)
+size_t groups_tables_bytes() { return sizeof(SmemPdf); }
+cudaError_t launch_groups_tables(const DevParams& P, void* out, cudaStream_t stream) {
+  MixedCtx M = mixed_ctx(P, DevEvents{}, WorkSet{}, LearnedCfg{}, 0, 0, 1, 1, 1, nullptr);
+  k_groups_tables<<<1, 256, 0, stream>>>(M, reinterpret_cast<SmemPdf*>(out));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_shower_groups(const DevParams& P, const DevEvents& E, const WorkSet& W, const LearnedCfg& Lc,
+                                 uint64_t first, uint64_t n, int blocks, int wave, int q_independent,
+                                 const void* tables, unsigned long long* next, cudaStream_t stream) {
+  if (n == 0) return cudaSuccess;
+  MixedCtx M = mixed_ctx(P, E, W, Lc, first, n, 1, 1, q_independent, next);
+  M.tables = tables;
+  M.wave = wave;
+  // fewer events than slots: as few in a block as give every event a slot
+  const uint64_t per = (n + blocks - 1) / blocks;
+  M.slots = per < (uint64_t)kSlots ? (int)per : kSlots;
+  const unsigned grid = (unsigned)min((uint64_t)blocks, (n + M.slots - 1) / M.slots);
+  cudaError_t err = cudaMemsetAsync(next, 0, sizeof(unsigned long long), stream);
+  if (err != cudaSuccess) return err;
+  k_shower_groups<<<grid, kGThreads, sizeof(GSmem), stream>>>(M);
+  return cudaGetLastError();
+}
+
 // Per-event state of the wavefront schedule for `cap` events: sizes and
 // carve (every array 256-byte aligned).
 namespace {
@@ -2903,9 +3839,8 @@ size_t al256(size_t b) { return (b + 255) / 256 * 256; }
 }  // namespace
 
 size_t wave_state_bytes(uint64_t cap) {
-  return al256(cap * sizeof(float)) + 7 * al256(cap * sizeof(int)) + al256(2 * cap * sizeof(double)) +
+  return al256(cap * sizeof(float)) + 5 * al256(cap * sizeof(int)) + al256(2 * cap * sizeof(double)) +
          al256(cap * sizeof(uint64_t)) + al256(cap * (size_t)kWavePendBytes) + al256(4 * cap * sizeof(uint32_t)) +
-         al256(12 * cap * sizeof(float4)) + al256(4 * cap * sizeof(uint32_t)) +
          al256(WL_NCTL * sizeof(unsigned long long));
 }
 
@@ -2919,14 +3854,10 @@ void wave_state_carve(void* base, uint64_t cap, WaveSet& V) {
   V.status = (int*)take(cap * sizeof(int));
   V.steps = (int*)take(cap * sizeof(int));
   V.flags = (int*)take(cap * sizeof(int));
-  V.keep = (int*)take(cap * sizeof(int));
-  V.chg = (int*)take(cap * sizeof(int));
   V.eta = (double*)take(2 * cap * sizeof(double));
   V.draw = (uint64_t*)take(cap * sizeof(uint64_t));
   V.pend = (unsigned char*)take(cap * (size_t)kWavePendBytes);
   V.list = (uint32_t*)take(4 * cap * sizeof(uint32_t));
-  V.mlpq = (float4*)take(12 * cap * sizeof(float4));
-  V.mlpi = (uint32_t*)take(4 * cap * sizeof(uint32_t));
   V.ctl = (unsigned long long*)take(WL_NCTL * sizeof(unsigned long long));
 }
 
@@ -2945,13 +3876,9 @@ cudaError_t launch_shower_wave(const DevParams& P, const DevEvents& E, const Wor
   M.wave_budget = budget;
   cudaError_t err = cudaMemsetAsync(V.ctl, 0, WL_NCTL * sizeof(unsigned long long), stream);
   if (err != cudaSuccess) return err;
-  // dynamic shared memory: the rebuild kernel evaluates the network itself
-  // only when it redraws (with kept trials the network pass does), the veto
-  // kernel only decodes heights, the persistent kernel does both
+  // dynamic shared memory: the veto kernel only decodes heights, the others also
+  // evaluate the network
   const bool learned = Lc.learned != 0;
-  const bool keep = P.trial_mode == GAPS_TRIALS_KEEP;
-  const size_t dyn_ends = mixed_dyn_bytes(block_size, P.nmax, learned, !keep) +
-                          (learned && keep ? (size_t)(block_size / 32) * kMlpBuf * sizeof(uint32_t) : 0);
   const size_t dyn_veto = mixed_dyn_bytes(block_size, P.nmax, learned, false);
   const size_t dyn = mixed_dyn_bytes(block_size, P.nmax, learned, true);
   const int tier = mixed_tier(blocks, block_size, sm_count);
@@ -2962,10 +3889,9 @@ cudaError_t launch_shower_wave(const DevParams& P, const DevEvents& E, const Wor
   k_wave_init<<<flat_blocks, 128, 0, stream>>>(M);
   for (int w = 0; w <= passes; ++w) {
     M.wave_par = w & 1;
-    if (tier == 2) k_wave_ends<2><<<blocks, block_size, dyn_ends, stream>>>(M);
-    else if (tier == 3) k_wave_ends<3><<<blocks, block_size, dyn_ends, stream>>>(M);
-    else k_wave_ends<4><<<blocks, block_size, dyn_ends, stream>>>(M);
-    if (Lc.learned) k_wave_mlp<<<sm_count * 2, 256, 0, stream>>>(M);
+    if (tier == 2) k_wave_ends<2><<<blocks, block_size, dyn, stream>>>(M);
+    else if (tier == 3) k_wave_ends<3><<<blocks, block_size, dyn, stream>>>(M);
+    else k_wave_ends<4><<<blocks, block_size, dyn, stream>>>(M);
     if (w == passes) break;  // the last rebuilds, then the persistent kernel
     if (veto_tier == 2) k_wave_veto<2><<<veto_blocks, block_size, dyn_veto, stream>>>(M);
     else if (veto_tier == 3) k_wave_veto<3><<<veto_blocks, block_size, dyn_veto, stream>>>(M);
