@@ -27,7 +27,7 @@ size_t groups_bytes(int lanes, int nmax);
 void groups_carve(void* base, int lanes, int nmax, WorkSet& W);
 size_t groups_tables_bytes();
 cudaError_t launch_groups_tables(const DevParams&, void*, cudaStream_t);
-cudaError_t launch_isr_targets(const DevParams&, int, const float4*, uint64_t, float*, float*, cudaStream_t);
+cudaError_t launch_isr_targets(const DevParams&, int, const float4*, uint64_t, float*, float*, int, cudaStream_t);
 cudaError_t mixed_kernels_init();
 cudaError_t launch_mlp_image(const float* params, void* image, cudaStream_t stream);
 size_t mlp_image_bytes();
@@ -633,7 +633,7 @@ int gaps_isr_targets(gaps_ctx* ctx, const float* states, uint64_t n_states, floa
   if (!ctx || !states || !features || !targets) return GAPS_ERR_INVALID_ARG;
   if (ctx->cfg.n_mix > 0 || ctx->cfg.process == GAPS_EE_QQ) return GAPS_ERR_INVALID_ARG;
   return cuda_fail(launch_isr_targets(ctx->P, ctx->q_independent, reinterpret_cast<const float4*>(states),
-                                      n_states, features, targets, (cudaStream_t)stream));
+                                      n_states, features, targets, ctx->n_sm, (cudaStream_t)stream));
 }
 
 int gaps_set_learned_proposal(gaps_ctx* ctx, const float* params, const float* log_margins) {

@@ -148,8 +148,7 @@ __device__ __forceinline__ bool loc_x(const MixedCtx& M, float x, int& ix, float
   return true;
 }
 
-// out of line: one copy for all call sites (instruction-cache footprint)
-__device__ __noinline__ float pdf32(const MixedCtx& M, const SmemPdf& S, int f, float x, float q2) {
+__device__ __forceinline__ float pdf32_inline(const MixedCtx& M, const SmemPdf& S, int f, float x, float q2) {
   if (f < 0 || f > 11) return 0.0f;
   int ix;
   float fx;
@@ -168,6 +167,10 @@ __device__ __noinline__ float pdf32(const MixedCtx& M, const SmemPdf& S, int f, 
   float lo = (1.0f - fx) * node(ix, iq) + fx * node(ix + 1, iq);
   float hi = (1.0f - fx) * node(ix, iq + 1) + fx * node(ix + 1, iq + 1);
   return lo * (1.0f - fq) + hi * fq;
+}
+// out of line: one copy for all call sites (instruction-cache footprint)
+__device__ __noinline__ float pdf32(const MixedCtx& M, const SmemPdf& S, int f, float x, float q2) {
+  return pdf32_inline(M, S, f, x, q2);
 }
 
 __device__ __noinline__ float bound32(const MixedCtx& M, const SmemPdf& S, int num, int den, float eta) {
@@ -447,8 +450,10 @@ struct IsrEval {
 // Acceptance ratio r = kernel J x / Pover * PDF ratio / bound of an
 // initial-state winner (Appendix B.4/B.5), with (1-z) given directly; the
 // cycle's weight is alpha_s(t)/alpha_s(t_c) * r. ok = false outside the map.
+// HOISTED: the caller has the bound and F(eta), which do not depend on z.
+template <bool HOISTED = false>
 __device__ IsrEval isr_eval32(const MixedCtx& M, const SmemPdf& S, int type, int ch, int fl_i, float eta, float s,
-                              float tw, float z, float omz, float pover) {
+                              float tw, float z, float omz, float pover, float B_ = 0.0f, float F0_ = 0.0f) {
   IsrEval e;
   e.ok = false;
   e.r = 0.0f; e.x = 1.0f; e.omx = 0.0f; e.u = 0.0f; e.omu = 1.0f; e.v = 0.0f; e.sumF = 0.0f;
@@ -482,9 +487,9 @@ __device__ IsrEval isr_eval32(const MixedCtx& M, const SmemPdf& S, int type, int
   else kk = (float)kCF * 0.5f * (x + 2.0f * omx / x);
   int num, den;
   isr_pdf_indices(ch, fl_i, num, den);
-  const float B = bound32(M, S, num, den, eta);
-  const float F0 = pdf32(M, S, den, eta, tw);
-  const float F1 = pdf32(M, S, num, eta / x, tw);
+  const float B = HOISTED ? B_ : bound32(M, S, num, den, eta);
+  const float F0 = HOISTED ? F0_ : pdf32(M, S, den, eta, tw);
+  const float F1 = HOISTED ? pdf32_inline(M, S, num, eta / x, tw) : pdf32(M, S, num, eta / x, tw);
   if (ch == 6) e.sumF = F1;
   float Fratio = F0 > 0.0f ? F1 / F0 : 0.0f;
   if (ch == 3 || ch == 4) {
@@ -2266,10 +2271,11 @@ __global__ void k_wave_final(const __grid_constant__ MixedCtx M) {
 // free until the chain's four lanes per slot leave the worker warps (224). 96
 // and 128 slots are slower, 168 and 200 alike; 168 leaves shared memory for the
 // network image. Measured, one GPU, before (a warp of events, then a pass per
-// phase over all events) and now: 32 768 p p events with matrix-element
-// corrections and the plain bound 47.2 -> 23.9 ms, 65 536 with the learned
-// proposal 116.8 -> 82 ms, 10 240 leading-order p p events 24.4 -> 7.1 ms, 200
-// events 14.4 -> 3.9 ms, 32 768 events of a beam and process mix 58.8 -> 35.3 ms.
+// phase over all events) and now: 262 144 p p events with matrix-element
+// corrections and the plain bound 46.9 -> 24.0 ms, 700 001 with the learned
+// proposal 116.6 -> 81.1 ms, 100 003 leading-order p p events 24.4 -> 7.0 ms,
+// 4096 events 14.5 -> 4.1 ms, 500 000 events of a beam and process mix
+// 58.8 -> 35.2 ms.
 // ---------------------------------------------------------------------------
 constexpr int kSlots = 168;
 constexpr int kWorkers = 896;               // 28 warps
@@ -3597,76 +3603,92 @@ namespace {
 // end, channel and zeta bin, the largest acceptance ratio r over 33 zeta points
 // of the bin and 64 scales t log-spaced over [t_c, t_kin] (both ends), as ln(max(r, 1e-6)),
 // with the network's input features of the row.
-constexpr int kTeacherZ = 32, kTeacherT = 64;
-__global__ void k_isr_targets(const __grid_constant__ MixedCtx M, const float4* states, uint64_t n_states, float* feats, float* targets) {
+//
+// Bound by FP32 issue: 2112 ratios a row. A warp takes `bins` bins of one state
+// and channel, with the scales on its lanes (two a lane), so that the dipole
+// type and the channel are the same for all lanes and everything that does not
+// depend on zeta (scale, limits, F(eta), the bound) is formed once; one lane
+// per zeta point forms z. With one thread per row, 16 rows of two channels and
+// often two dipole types shared a warp and each repeated all of it for every
+// point: 25.7 ms for 50 000 states, 9.3 ms now (issue slots 75 % used; 10.4 ms
+// at the 80 registers the compiler takes on its own, three blocks an SM).
+constexpr int kTeacherZ = 32, kTeacherT = 64, kTeacherWarps = 8, kTeacherBlocks = 4;
+__global__ void __launch_bounds__(kTeacherWarps * 32, kTeacherBlocks)
+    k_isr_targets(const __grid_constant__ MixedCtx M, const float4* states, uint64_t n_states, int bins, float* feats,
+                  float* targets) {
   __shared__ SmemPdf S;
-  for (int q = threadIdx.x; q < 12 * kSmNX; q += blockDim.x) {
-    int f = q / kSmNX, ix = q % kSmNX;
-    S.umax[f][ix] = (float)M.P.umax[q];
-    S.lmin[f][ix] = (float)M.P.lmin[q];
-    float xf = 0.0f;
-    if (f < 11) xf = M.P.grid[((size_t)f * kNX + ix) * kNQ];
-    else for (int k = 1; k <= 10; ++k) xf += M.P.grid[((size_t)k * kNX + ix) * kNQ];
-    S.xf[f][ix] = xf;
-  }
-  for (int q = threadIdx.x; q < 12 * (kSmNX + 1); q += blockDim.x)
-    S.sufmax[q / (kSmNX + 1)][q % (kSmNX + 1)] = (float)M.P.sufmax[q];
-  for (int q = threadIdx.x; q < 12 * kSmNX; q += blockDim.x) S.first[q / kSmNX][q % kSmNX] = (float)M.P.first[q];
-  if (threadIdx.x < 12) S.m2[threadIdx.x] = (float)M.P.m2[threadIdx.x];
+  load_tables(S, M);
   __syncthreads();
-  const uint64_t row = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (row >= n_states * 16) return;
-  const float4 st = states[row / 16];
-  const int c = (int)((row / 8) % 2), m = (int)(row % 8);
-  const float eta = st.x, s = st.y;
-  const int type = (int)st.z, fidx = (int)st.w;
-  const int fl_i = fidx == 0 ? 21 : (fidx <= 5 ? fidx : -(fidx - 5));
-  const int ch = (fl_i == 21 ? 5 : 3) + c;
-  const float tc = __expf(M.lnTc);
-  float f[4];
-  mlp_features(eta, s, tc, m, isr_class(type, ch, fl_i), f);
-  for (int k = 0; k < 4; ++k) feats[4 * row + k] = f[k];
-  int shape;
-  float coefd;
-  channel_over32(ch, type, M.P.nf, shape, coefd);
-  float zm, delta;
-  float best = 0.0f;
-  const float tk = tkin32(type, s, eta);
-  if (tk > tc && zlim32(type, tc, s, eta, zm, delta)) {
-    const float ltc = __logf(tc), ltk = __logf(tk);
-    for (int a = 0; a <= kTeacherZ; ++a) {
-      const float zeta = ((float)m + (float)a * (1.0f / kTeacherZ)) * 0.125f;
-      float z, omz;
-      shape_sample32(shape, zm, delta, fminf(zeta, 0.99999994f), z, omz);
-      const float pover = shape_val32(shape, (float)coefd, z, omz);
-      for (int b = 0; b < kTeacherT; ++b) {
+  constexpr unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const uint64_t items = n_states * (uint64_t)(16 / bins);
+  for (uint64_t it = (uint64_t)blockIdx.x * kTeacherWarps + (threadIdx.x >> 5); it < items;
+       it += (uint64_t)gridDim.x * kTeacherWarps) {
+    const uint64_t row0 = it * bins;
+    const float4 st = states[row0 / 16];
+    const int c = (int)((row0 / 8) % 2), m0 = (int)(row0 % 8);
+    const float eta = st.x, s = st.y;
+    const int type = (int)st.z, fidx = (int)st.w;
+    const int fl_i = fidx == 0 ? 21 : (fidx <= 5 ? fidx : -(fidx - 5));
+    const int ch = (fl_i == 21 ? 5 : 3) + c;
+    const float tc = __expf(M.lnTc);
+    int shape;
+    float coefd;
+    channel_over32(ch, type, M.P.nf, shape, coefd);
+    float zm, delta;
+    const float tk = tkin32(type, s, eta);
+    const bool open = tk > tc && zlim32(type, tc, s, eta, zm, delta);
+    float t[2], zm_t[2], delta_t[2], F0[2], B = 0.0f;
+    bool ok[2];
+    if (open) {
+      int num, den;
+      isr_pdf_indices(ch, fl_i, num, den);
+      B = bound32(M, S, num, den, eta);
+      const float ltc = __logf(tc), ltk = __logf(tk);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
         // log-spaced, both ends included: the ratio is often largest at t_c
-        const float t = __expf(ltc + (ltk - ltc) * (float)b * (1.0f / (kTeacherT - 1)));
-        float zm_t, delta_t;
-        if (!zlim32(type, t, s, eta, zm_t, delta_t) || !(omz > delta_t) || !(z > zm_t)) continue;
-        const IsrEval ev = isr_eval32(M, S, type, ch, fl_i, eta, s, t, z, omz, pover);
-        if (ev.ok) best = fmaxf(best, ev.r);
+        t[h] = __expf(ltc + (ltk - ltc) * (float)(lane + 32 * h) * (1.0f / (kTeacherT - 1)));
+        ok[h] = zlim32(type, t[h], s, eta, zm_t[h], delta_t[h]);
+        F0[h] = pdf32(M, S, den, eta, t[h]);
       }
     }
+    for (int m = m0; m < m0 + bins; ++m) {
+      float best = 0.0f;
+      if (open) {
+        // lane a: zeta point a of the bin; its last point is the same on all
+        float z_l, omz_l, po_l, z_e, omz_e, po_e;
+        shape_sample32(shape, zm, delta, fminf(((float)m + (float)lane * (1.0f / kTeacherZ)) * 0.125f, 0.99999994f), z_l,
+                       omz_l);
+        po_l = shape_val32(shape, (float)coefd, z_l, omz_l);
+        shape_sample32(shape, zm, delta, fminf(((float)m + (float)kTeacherZ * (1.0f / kTeacherZ)) * 0.125f, 0.99999994f),
+                       z_e, omz_e);
+        po_e = shape_val32(shape, (float)coefd, z_e, omz_e);
+#pragma unroll 1
+        for (int a = 0; a <= kTeacherZ; ++a) {
+          float z = __shfl_sync(full, z_l, a & 31), omz = __shfl_sync(full, omz_l, a & 31),
+                pover = __shfl_sync(full, po_l, a & 31);
+          if (a == kTeacherZ) { z = z_e; omz = omz_e; pover = po_e; }
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            if (!ok[h] || !(omz > delta_t[h]) || !(z > zm_t[h])) continue;
+            const IsrEval ev = isr_eval32<true>(M, S, type, ch, fl_i, eta, s, t[h], z, omz, pover, B, F0[h]);
+            if (ev.ok) best = fmaxf(best, ev.r);
+          }
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(full, best, o));
+      const uint64_t row = row0 + (m - m0);
+      float f[4];
+      mlp_features(eta, s, tc, m, isr_class(type, ch, fl_i), f);
+      if (lane < 4) feats[4 * row + lane] = lane == 0 ? f[0] : lane == 1 ? f[1] : lane == 2 ? f[2] : f[3];
+      if (lane == 0) targets[row] = __logf(fmaxf(best, 1e-6f));
+    }
   }
-  targets[row] = __logf(fmaxf(best, 1e-6f));
 }
 
 }  // namespace
-
-cudaError_t launch_isr_targets(const DevParams& P, int q_independent, const float4* states, uint64_t n_states,
-                               float* feats, float* targets, cudaStream_t stream) {
-  if (n_states == 0) return cudaSuccess;
-  MixedCtx M;
-  M.P = P;
-  M.q_independent = q_independent;
-  M.lnTc = (float)gm_log(P.t_cut);
-  M.asOver2pi = (float)(P.as_over / (2.0 * kPi));
-  M.lxminf = (float)P.lxmin; M.dlxf = (float)P.dlx; M.lqminf = (float)P.lqmin; M.dlqf = (float)P.dlq;
-  const uint64_t rows = n_states * 16;
-  k_isr_targets<<<(unsigned)((rows + 127) / 128), 128, 0, stream>>>(M, states, n_states, feats, targets);
-  return cudaGetLastError();
-}
 
 constexpr int kWarpKernelMaxDyn = 200 * 1024;
 
@@ -3773,6 +3795,22 @@ void launch_persistent(const MixedCtx& M, int tier, int blocks, int block_size, 
   else k_shower_mixed<4, WAVE, VMAX><<<blocks, block_size, dyn, stream>>>(M);
 }
 }  // namespace
+
+cudaError_t launch_isr_targets(const DevParams& P, int q_independent, const float4* states, uint64_t n_states,
+                               float* feats, float* targets, int sm_count, cudaStream_t stream) {
+  if (n_states == 0) return cudaSuccess;
+  const MixedCtx M = mixed_ctx(P, DevEvents{}, WorkSet{}, LearnedCfg{}, 0, 0, 1, 1, q_independent, nullptr);
+  // all bins of a state and channel in one warp, which then forms what they
+  // share once (5 % of the work), or one bin where that would give the resident
+  // warps fewer than four items each
+  const uint64_t resident = (uint64_t)max(1, sm_count) * kTeacherBlocks * kTeacherWarps;
+  const int bins = 2 * n_states >= 4 * resident ? 8 : 1;
+  const uint64_t blocks = (n_states * (16 / bins) + kTeacherWarps - 1) / kTeacherWarps;
+  // (three blocks in turn at most: every block loads the tables)
+  const unsigned grid = (unsigned)min(blocks, (uint64_t)max(1, sm_count) * kTeacherBlocks * 3);
+  k_isr_targets<<<grid, kTeacherWarps * 32, 0, stream>>>(M, states, n_states, bins, feats, targets);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_shower_mixed(const DevParams& P, const DevEvents& E, const WorkSet& W, const LearnedCfg& Lc,
                                 uint64_t first, uint64_t n, int blocks, int block_size, int sm_count, int period,
