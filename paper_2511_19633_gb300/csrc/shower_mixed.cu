@@ -876,13 +876,13 @@ struct Emission {
 // (relative error (2^-23)^4 before rounding, i.e. an ulp of FP64), a few
 // instructions each instead of the library's division sequences. For normal
 // arguments within the FP32 range, which every invariant here is.
-__device__ __forceinline__ double rcp64(double x) {
+__device__ __noinline__ double rcp64(double x) {
   double r = (double)__frcp_rn((float)x);
   r = r * fma(-x, r, 2.0);
   r = r * fma(-x, r, 2.0);
   return r;
 }
-__device__ __forceinline__ double rsqrt64(double x) {
+__device__ __noinline__ double rsqrt64(double x) {
   double r = (double)rsqrtf((float)x);
   r = r * fma(-0.5 * x * r, r, 1.5);
   r = r * fma(-0.5 * x * r, r, 1.5);
@@ -1027,6 +1027,7 @@ __device__ __noinline__ bool emit(const MixedCtx& M, const W& w, Lane& L, const 
       KK[mu] = Kp[mu] + Kn[mu];
     }
     const double iKK2 = 2.0 * rcp64(dot4(KK, KK)), iKp2 = 2.0 * rcp64(dot4(Kp, Kp));
+#pragma unroll 1
     for (int m = 2; m < L.n; ++m) {
       double q[4];
 #pragma unroll
@@ -2224,69 +2225,79 @@ __global__ void k_wave_final(const __grid_constant__ MixedCtx M) {
 
 // ---------------------------------------------------------------------------
 // The kept-trial shower (GAPS_TRIALS_KEEP, the persistent and the wavefront
-// schedule): one block per SM holds kSlots events in flight and takes them
-// through the phases of an emission together, each phase's work items spread
-// over the lanes whatever event they belong to.
+// schedule): one block per SM holds kSlots events in flight. Its warps are of
+// four kinds, which work side by side on different slots; a round ends when all
+// have done what the round before listed for them. Within a kind the warps go
+// through phases together, each phase's work items spread over the lanes
+// whatever event they belong to.
 //
-//   touch   lists the ends that the slots' last emissions touched (eight lanes
-//           per slot)
-//   form    one lane per listed end: its record; ends whose record changed are
-//           marked, with the number of Philox blocks that their trials use
-//   draw    one lane per marked end: its trials, at the counter that the marks
-//           below it give (the canonical order); at the same time one lane per
-//           slot and cycle: the uniforms of the next trials of eight cycles
-//   net     the learned proposal's tiles of the changed initial-state ends,
-//           four a warp step, and their trials
-//   chain   four lanes per slot: eight cycles under the assumption of vetoes
-//           (the largest kept trial wins and its channel draws again)
-//   weigh   one lane per cycle, sorted by dipole type: the acceptance weight
-//   commit  one lane per slot: the cycles up to the first that was not vetoed;
-//           the trials that the cycles behind it replaced are put back
-//   emit    four more warps, beside all of the above, on the last round's
-//           results: the FP64 kinematics of its emissions, one lane each; its
-//           ended events are written back and the next ones loaded, eight
-//           lanes per slot
+//   cycles: chain   four lanes per slot: eight cycles under the assumption of
+//                   vetoes (the largest kept trial wins and its channel draws
+//                   again); the cycles are listed by dipole type
+//           weigh   one lane per cycle, a warp's of one type: the acceptance
+//                   weight
+//           commit  one lane per slot: the cycles up to the first that was not
+//                   vetoed; the trials that the cycles behind it replaced are
+//                   put back; an accepted cycle is parked, an ended event listed
+//   emit:           one lane per parked emission, a warp per dipole type: its
+//                   FP64 kinematics and colours
+//   load:           eight lanes per ended event: written back, the next one
+//                   loaded
+//   form:   touch   lists the ends that the slots' last emissions touched (eight
+//                   lanes per slot)
+//           form    one lane per listed end: its record; ends whose record
+//                   changed are marked, with the number of Philox blocks that
+//                   their trials use
+//           draw    one lane per marked end: its trials, at the counter that the
+//                   marks below it give (the canonical order)
+//           net     the learned proposal's tiles of the changed initial-state
+//                   ends, four a warp step, and their trials
 //
 // The chain may run ahead because a vetoed cycle uses exactly three Philox
 // blocks (two of the veto, one of the winner's next trial). Every cycle uses
 // the numbers that one lane per event would use, so the events are the same
 // bits.
 //
-// Why this shape. The bound is instruction fetch and the latency of serial
-// steps, not arithmetic or memory: an event is 32 000 instructions a lane of
+// Why this shape. The bound is the latency of serial steps and instruction
+// fetch, not arithmetic or memory: an event is some 35 000 warp instructions of
 // phases that have little code in common. With one lane per event 7 of 32 lanes
 // were active in the veto cycles and 12 in the rebuilds (53 000 instructions an
 // event), and with independent warps the phases' code (160 KB) evicted itself
-// from the instruction cache (two thirds of the stalls). In lockstep all warps
-// of the SM run one phase's code, and lists keep the lanes full; what is left is
-// a round of 66 000 clocks (touch 7 000, form 18 000, draw 5 000, chain 17 000,
-// list 3 000, weigh 11 000, commit 5 000; net 24 000 where it runs), most of it
-// the latency of one event's chain of loads and trials. The events in flight
-// (about 3 KB each) stay in L2 where a pass over a whole chunk per phase moved
-// 71 KB an event through DRAM. An emission's FP64 runs at 1/64 of the FP32 rate
-// and costs a warp the same for 1 or 32 lanes, so it needs a list of many
-// events, and warps of its own to hide behind the other phases.
+// from the instruction cache (two thirds of the stalls). In lockstep the warps
+// of a kind run one phase's code, and lists keep the lanes full. All kinds in
+// one sequence made a round of 66 000 clocks and 3.5 rounds of an accepted
+// emission; side by side it is 56 000 and 4.5 with all slots in use, but 28 000
+// instead of 37 000 with few, which is how every launch ends (a long event is a
+// chain of rounds). An emission's FP64 runs at 1/64 of the FP32 rate and costs a
+// warp the same for 1 or 32 lanes. The events in flight (about 3 KB each) stay
+// in L2, where a pass over a whole chunk per phase moved 71 KB an event through
+// DRAM.
 //
-// kSlots: a round's time is mostly latency, so more events a round are nearly
-// free until the chain's four lanes per slot leave the worker warps (224). 96
-// and 128 slots are slower, 168 and 200 alike; 168 leaves shared memory for the
-// network image. Measured, one GPU, before (a warp of events, then a pass per
-// phase over all events) and now: 262 144 p p events with matrix-element
-// corrections and the plain bound 46.9 -> 24.0 ms, 700 001 with the learned
-// proposal 116.6 -> 81.1 ms, 100 003 leading-order p p events 24.4 -> 7.0 ms,
-// 4096 events 14.5 -> 4.1 ms, 500 000 events of a beam and process mix
-// 58.8 -> 35.2 ms.
+// kSlots, kTmx, kEndList: more slots hide more latency, but what the shared
+// memory leaves is the L1 cache, in steps: 192 slots with 48 ends each fit the
+// step of 164 KB (196 KB with the network). 168 slots with 64 ends, 4096 listed
+// ends and the network's memory always there: 22.2 instead of 20.4 ms in the
+// second case below. Two blocks of 80 slots an SM, in lockstep: 27.0 against
+// 22.5 ms. Warps per kind: 12 + 14, 16 + 10 and 18 + 8 for cycles and form are
+// slower.
+//
+// Measured, one GPU, before (a warp of events, then a pass per phase over all
+// events) and now: 700 001 p p events with the learned proposal 116.6 -> 70.6
+// ms, 262 144 with the plain bound 46.9 -> 20.4 ms, 100 003 leading-order p p
+// events 24.4 -> 6.1 ms, 4096 events 14.5 -> 3.0 ms, 500 000 events of a beam
+// and process mix 58.8 -> 26.8 ms.
 // ---------------------------------------------------------------------------
-constexpr int kSlots = 168;
-constexpr int kWorkers = 896;               // 28 warps
-constexpr int kEmitters = 128;              // four warps, one per scheduler
-constexpr int kGThreads = kWorkers + kEmitters;
+constexpr int kSlots = 192;
+// the warps of the block, by what they do
+constexpr int kCycleWarps = 14, kFormWarps = 12, kEmitWarps = 4, kLoadWarps = 2;
+constexpr int kGThreads = 32 * (kCycleWarps + kFormWarps + kEmitWarps + kLoadWarps);
 constexpr int kCyc = 8;                     // cycles of a round
-constexpr int kEndList = 4096;              // ends formed in a round (the slots beyond wait for the next)
-constexpr int kTmx = 64;                    // ends whose larger kept trial is in shared memory
-static_assert(4 * kSlots <= kWorkers && 4 * kSlots % 32 == 0 && kSlots <= 256, "the phases' lane mappings");
+constexpr int kEndList = 1024;              // ends formed in a round (the slots beyond wait for the next)
+constexpr int kTmx = 48;                    // ends whose larger kept trial is in shared memory
+static_assert(kEmitWarps == 4, "one per dipole type, and per scheduler");
+static_assert(kSlots <= 256 && kGThreads <= 1024, "bytes, and a block");
 static_assert(kEndList >= 256, "one event always fits");
-static_assert(kCyc * kSlots <= 2 * kWorkers, "two cycles a thread in phase_list");
+static_assert(kCyc == 8, "two cycles a lane of the chain");
 
 // a thread's counters of one launch (32 bits: a lane sees a small share of the
 // launch's events)
@@ -2321,8 +2332,7 @@ struct GSmem {
   int n[kSlots], n_emit[kSlots], steps[kSlots], row[kSlots];
   int live[kSlots];    // the slot holds an event: 1, on the plain bounds after a violation: 3
   int end[kSlots];     // its status once it ended (GAPS_STATUS_ACTIVE before)
-  int busy[kSlots];    // 1: an emission is parked or being built, 2: it is built
-  int ready[kSlots];   // takes part in this round's chain
+  int busy[kSlots];    // 0: takes part in the next round's cycles; 1: an emission, a load or ends to form
   int table[kSlots];   // 1: form the touched ends, 2: only end chg draws again
   int keep[kSlots];    // ends that may keep their trials
   int chg[kSlots];     // emitter | spectator << 8, or -1: every end
@@ -2334,28 +2344,29 @@ struct GSmem {
   GCycle park[kSlots];           // the parked emission: its cycle
   GWeight pw[kSlots];            // and weight
   alignas(16) float tmx[kSlots][kTmx + 4];  // the larger kept trial of ends 0 .. kTmx - 1 (the rest: WS::Tmx)
-  int n_ends, n_ends_ok, n_q, n_items[4], n_tables[2], n_park[2], n_ended[2];
+  int n_ends, n_ends_ok, n_q, n_items[4], n_ready[2], n_tables[2], n_park[2][4], n_ended[2];
   unsigned ends[kEndList];       // slot << 8 | end; bit 16: draw only, then: marked
-  unsigned short q[4 * kSlots];  // 4 slot + end of the network's queue
   unsigned short items[4][kCyc * kSlots];  // 8 slot + cycle, by dipole type
-  // slots with ends to form, with a parked emission, ended; by the round's parity
-  unsigned char tables[2][kSlots], parked[2][kSlots], ended[2][kSlots];
-  float dec[256];
-  alignas(16) unsigned char image[kMlpSmemBytes];  // the network's BF16 image
+  // by the parity of the round that lists them: slots for the next round's
+  // cycles, with ends to form, with a parked emission (by its dipole type), ended
+  unsigned char cycles[2][kSlots], tables[2][kSlots], parked[2][4][kSlots], ended[2][kSlots];
   GCycle cyc[kCyc][kSlots];
-  union {
-    GWeight wt[kCyc][kSlots];
-    struct {
-      alignas(16) float stage[kWorkers / 32][64][4];  // (float4 rows)
-      float ustage[kWorkers / 32][64];
-    } m;
-  };
+  alignas(16) GWeight wt[kCyc][kSlots];
+  // from here only with the learned proposal (left out of the launch's shared
+  // memory without it, which leaves the L1 cache more)
+  alignas(16) unsigned char image[kMlpSmemBytes];  // the network's BF16 image
+  alignas(16) float stage[kFormWarps][64][4];      // (float4 rows)
+  float ustage[kFormWarps][64];
+  float dec[256];
+  unsigned short q[4 * kSlots];  // 4 slot + end of the network's queue
 };
 
 static_assert(sizeof(GSmem) <= 227 * 1024, "one block per SM");
+constexpr size_t kGSmemPlain = offsetof(GSmem, image);
 
-__device__ __forceinline__ void workers_sync() { asm volatile("bar.sync 1, 896;" ::: "memory"); }
-static_assert(kWorkers == 896, "workers_sync");
+// barriers among the warps of one kind
+__device__ __forceinline__ void cycles_sync() { asm volatile("bar.sync 1, %0;" ::"n"(32 * kCycleWarps) : "memory"); }
+__device__ __forceinline__ void forms_sync() { asm volatile("bar.sync 2, %0;" ::"n"(32 * kFormWarps) : "memory"); }
 
 // Philox block d of event id, one copy for all phases
 __device__ __noinline__ uint4 block_of(uint64_t seed, uint64_t id, uint64_t d) {
@@ -2693,7 +2704,7 @@ __device__ __forceinline__ void refill_slot(const MixedCtx& M, GSmem& F, const L
 
 // ---- touch: eight lanes per slot ------------------------------------------
 // (slot < 0: none for this group; the warp's groups go together)
-__device__ __forceinline__ void phase_touch(GSmem& F, const WS& w, int slot, int gl) {
+__device__ __forceinline__ void phase_touch(GSmem& F, const WS& w, int slot, int gl, int par) {
   const int what = slot >= 0 ? F.table[slot] : 0;
   slot = max(slot, 0);
   const int n = F.n[slot], ne = what == 1 ? 2 * n : 0;
@@ -2733,8 +2744,14 @@ __device__ __forceinline__ void phase_touch(GSmem& F, const WS& w, int slot, int
   base = __shfl_sync(0xffffffffu, base, 0, 8);
   const bool fits = what && base + todo <= kEndList;
   if (gl == 0 && what) {
-    if (fits) atomicMax(&F.n_ends_ok, base + todo);
-    F.ready[slot] = fits;
+    F.tot[slot] = 0;
+    F.defer[slot] = 0;
+    if (fits) {
+      atomicMax(&F.n_ends_ok, base + todo);
+      F.busy[slot] = 0;
+    } else {
+      F.tables[par][atomicAdd(&F.n_tables[par], 1)] = (unsigned char)slot;
+    }
   }
   if (what) {
     F.mk1[slot][gl] = 0;
@@ -2755,9 +2772,9 @@ __device__ __forceinline__ void phase_form(const MixedCtx& M, GSmem& F, const Sm
                                            int base_lane, int tid, GCount& cnt) {
   // 8 to 32 ends a warp: a pass is a chain of dependent loads, which the other
   // warps hide
-  const int total = F.n_ends_ok, per = min(32, max(8, (total + kWorkers / 32 - 1) / (kWorkers / 32)));
+  const int total = F.n_ends_ok, per = min(32, max(8, (total + kFormWarps - 1) / kFormWarps));
   if ((tid & 31) >= per) return;
-  for (int j = (tid >> 5) * per + (tid & 31); j < total; j += per * (kWorkers / 32)) {
+  for (int j = (tid >> 5) * per + (tid & 31); j < total; j += per * kFormWarps) {
     const unsigned ent = F.ends[j];
     const int slot = (ent >> 8) & 0xff, q = ent & 0xff;
     const WS w{M.W, base_lane + slot, M.P.nmax};
@@ -2822,11 +2839,11 @@ __device__ __forceinline__ void phase_form(const MixedCtx& M, GSmem& F, const Sm
   }
 }
 
-// ---- draw: one lane per marked end, and the chain's uniforms --------------
+// ---- draw: one lane per marked end ----------------------------------------
 __device__ __forceinline__ void phase_draw(const MixedCtx& M, GSmem& F, const SmemPdf& S, int base_lane, int tid,
                                            GCount& cnt) {
-  const int total = F.n_ends_ok, per = min(32, max(8, (total + kWorkers / 32 - 1) / (kWorkers / 32)));
-  for (int j = (tid >> 5) * per + (tid & 31); (tid & 31) < per && j < total; j += per * (kWorkers / 32)) {
+  const int total = F.n_ends_ok, per = min(32, max(8, (total + kFormWarps - 1) / kFormWarps));
+  for (int j = (tid >> 5) * per + (tid & 31); (tid & 31) < per && j < total; j += per * kFormWarps) {
     const unsigned ent = F.ends[j];
     if (!(ent & 0x10000u)) continue;
     const int slot = (ent >> 8) & 0xff, q = ent & 0xff;
@@ -2839,21 +2856,13 @@ __device__ __forceinline__ void phase_draw(const MixedCtx& M, GSmem& F, const Sm
     const WS w{M.W, base_lane + slot, M.P.nmax};
     draw_end(M, F, S, w, slot, q, w.End(q), M.first + F.ev[slot], F.draw[slot] + (uint64_t)off, F.lnT[slot], F.row[slot], cnt);
   }
-  // block 3 k + 2 below: the next trial of cycle k's winner if it is vetoed
-  for (int i = tid; i < kCyc * kSlots; i += kWorkers) {
-    const int slot = i % kSlots, k = i / kSlots;
-    if (!F.ready[slot]) continue;
-    const uint64_t id = M.first + F.ev[slot], d = F.draw[slot] + (uint64_t)F.tot[slot] + 3 * (uint64_t)k + 2;
-    const uint4 o = block_of(M.P.seed, id, d);
-    F.cyc[k][slot] = GCycle{0, __logf(u24(o.y)), u24(o.w)};
-  }
 }
 
 // ---- net: the network's tiles of the queued ends, four a warp step --------
 __device__ __forceinline__ void phase_net(const MixedCtx& M, GSmem& F, const SmemPdf& S, const LearnedSmem& ls,
                                           const MlpSmem& mlp, int base_lane, int warp_id, int lane_id, GCount& cnt) {
   const int nq = F.n_q;
-  for (int g = warp_id; 4 * g < nq; g += kWorkers / 32) {
+  for (int g = warp_id; 4 * g < nq; g += kFormWarps) {
     const int j = 4 * g + lane_id;
     const bool have = lane_id < 4 && j < nq;
     const int sl = have ? F.q[j] >> 2 : 0, q = have ? F.q[j] & 3 : 0, row = F.row[sl];
@@ -2867,7 +2876,7 @@ __device__ __forceinline__ void phase_net(const MixedCtx& M, GSmem& F, const Sme
     const int type = __float_as_int(rec.w) < 2 ? kII : kIF;  // (the queued ends have a partner)
     const float tc = have ? __expf(S.lnTc[row]) : 1.0f;
     float scale0 = 0.0f, scale1 = 0.0f;
-    learned_heights(M, mlp, ls, F.m.stage[warp_id], F.m.ustage[warp_id], eval, tc, ax.y, ax.x, type,
+    learned_heights(M, mlp, ls, F.stage[warp_id], F.ustage[warp_id], eval, tc, ax.y, ax.x, type,
                     tag_fl(__float_as_uint(ax.z)), w.lane, q, lane_id, scale0, scale1, true);
     if (have) {
       rec.x *= scale0;
@@ -2888,20 +2897,34 @@ __device__ __forceinline__ void phase_net(const MixedCtx& M, GSmem& F, const Sme
 // lane's next candidate are on their way while the other lanes' candidates win.
 // (Holding the two largest, so that no load is waited for, cost more
 // instructions than it saved: 24 500 clocks a round against 16 500.)
-__device__ __forceinline__ void phase_chain(const MixedCtx& M, GSmem& F, const SmemPdf& S, int base_lane, int tid) {
+// (the warp's groups go together; slot < 0: none for this group)
+__device__ __forceinline__ void phase_chain(const MixedCtx& M, GSmem& F, const SmemPdf& S, int base_lane, int slot,
+                                            int lane_id) {
   const unsigned full = 0xffffffffu;
-  const int slot = tid >> 2, gl = tid & 3, gshift = tid & 28;
-  const bool on = F.ready[slot];
+  const int gl = lane_id & 3, gshift = lane_id & 28;
+  const bool on = slot >= 0;
+  slot = max(slot, 0);
   const WS w{M.W, base_lane + slot, M.P.nmax};
   const int ne = on ? 2 * F.n[slot] : 0, row = F.row[slot];
   const bool pp = S.pp[row] != 0;
   const float lnTc = S.lnTc[row];
-  if (on && gl == 0) {
-    F.draw[slot] += (uint64_t)F.tot[slot];
-    F.nv[slot] = 0;
-    if (F.table[slot] == 1) F.table[slot] = 3;  // (counted at the commit)
+  if (on) {
+    // block 3 k + 2 from here: the next trial of cycle k's winner if it is vetoed
+    const uint64_t id = M.first + F.ev[slot], d = F.draw[slot] + (uint64_t)F.tot[slot];
+#pragma unroll 1
+    for (int k = gl; k < kCyc; k += 4) {
+      const uint4 o = block_of(M.P.seed, id, d + 3 * (uint64_t)k + 2);
+      F.cyc[k][slot] = GCycle{0, __logf(u24(o.y)), u24(o.w)};
+    }
+    __syncwarp(0xfu << gshift);
+    if (gl == 0) {
+      F.draw[slot] = d;
+      F.tot[slot] = 0;
+      F.nv[slot] = 0;
+      if (F.table[slot] == 1) F.table[slot] = 3;  // (counted at the commit)
+    }
   }
-  // the largest of each of the lane's four quadruples of ends, of the ends from
+  // the largest of each of the lane's quadruples of ends, of the ends from
   // kTmx on, and of all; then the (lowest) end that has it
   float qm[kTmx / 16], om = -INFINITY, m1;
   auto quad = [&](int r) {
@@ -2913,16 +2936,23 @@ __device__ __forceinline__ void phase_chain(const MixedCtx& M, GSmem& F, const S
   };
   auto rest = [&]() {
     om = -INFINITY;
+#pragma unroll 1
     for (int q = kTmx + gl; q < ne; q += 4) om = fmaxf(om, w.Tmx(q));
   };
   auto largest = [&]() {
-    m1 = fmaxf(fmaxf(fmaxf(qm[0], qm[1]), fmaxf(qm[2], qm[3])), om);
+    m1 = om;
+#pragma unroll
+    for (int u = 0; u < kTmx / 16; ++u) m1 = fmaxf(m1, qm[u]);
   };
   auto locate = [&]() -> int {
     if (!(m1 > -INFINITY)) return -1;
-    const int r = qm[0] == m1 ? 0 : qm[1] == m1 ? 1 : qm[2] == m1 ? 2 : qm[3] == m1 ? 3 : 4;
-    if (r == 4) {
+    int r = kTmx / 16;
+#pragma unroll
+    for (int u = kTmx / 16 - 1; u >= 0; --u)
+      if (qm[u] == m1) r = u;
+    if (r == kTmx / 16) {
       int q = kTmx + gl;
+#pragma unroll 1
       while (q + 4 < ne && w.Tmx(q) != m1) q += 4;
       return q;
     }
@@ -2997,30 +3027,28 @@ __device__ __forceinline__ void phase_chain(const MixedCtx& M, GSmem& F, const S
     F.len[slot] = len;
     F.done[slot] = done;
   }
-}
-
-// ---- list: the chain's cycles by dipole type, one lane per cycle ----------
-__device__ __forceinline__ void phase_list(GSmem& F, int tid, int lane_id) {
-  int it[2], type[2], base = 0;
+  __syncwarp();
+  // the cycles by dipole type, two a lane; lane t reserves the warp's places in
+  // list t
+  int type[2], base = 0;
   unsigned m[2][4];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    const int i = tid + h * kWorkers, slot = i % kSlots, k = i / kSlots;
-    it[h] = 8 * slot + k;
-    type[h] = k < kCyc && F.ready[slot] && k < F.len[slot] ? F.cyc[k][slot].type() : -1;
+    type[h] = on && gl + 4 * h < len ? F.cyc[gl + 4 * h][slot].type() : -1;
 #pragma unroll
-    for (int t = 0; t < 4; ++t) m[h][t] = __ballot_sync(0xffffffffu, type[h] == t);
+    for (int t = 0; t < 4; ++t) m[h][t] = __ballot_sync(full, type[h] == t);
   }
-  // lane t reserves the warp's places in list t
 #pragma unroll
   for (int t = 0; t < 4; ++t)
     if (lane_id == t) base = atomicAdd(&F.n_items[t], __popc(m[0][t]) + __popc(m[1][t]));
   const unsigned below = (1u << lane_id) - 1u;
 #pragma unroll
   for (int t = 0; t < 4; ++t) {
-    const int b = __shfl_sync(0xffffffffu, base, t);
-    if (type[0] == t) F.items[t][b + __popc(m[0][t] & below)] = (unsigned short)it[0];
-    if (type[1] == t) F.items[t][b + __popc(m[0][t]) + __popc(m[1][t] & below)] = (unsigned short)it[1];
+    const int b = __shfl_sync(full, base, t);
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (type[h] == t)
+        F.items[t][b + (h ? __popc(m[0][t]) : 0) + __popc(m[h][t] & below)] = (unsigned short)(8 * slot + gl + 4 * h);
   }
 }
 
@@ -3031,7 +3059,7 @@ __device__ __forceinline__ void phase_weigh(const MixedCtx& M, GSmem& F, const S
 #pragma unroll 1
   for (int t = 0; t < 4; ++t) {
     const int n = F.n_items[t], chunks = (n + 31) / 32;
-    for (; c < chunks; c += kWorkers / 32) {
+    for (; c < chunks; c += kCycleWarps) {
       const int j = 32 * c + lane_id;
       cnt.warp_steps += 1;
       if (j < n) {
@@ -3052,9 +3080,7 @@ __device__ __forceinline__ void phase_weigh(const MixedCtx& M, GSmem& F, const S
 }
 
 // ---- commit: one lane per slot --------------------------------------------
-__device__ __forceinline__ void phase_commit(const MixedCtx& M, GSmem& F, int base_lane, int tid, int par, GCount& cnt) {
-  const int slot = tid;
-  if (slot >= kSlots || !F.ready[slot]) return;
+__device__ __forceinline__ void phase_commit(const MixedCtx& M, GSmem& F, int base_lane, int slot, int par, GCount& cnt) {
   const WS w{M.W, base_lane + slot, M.P.nmax};
   if (F.table[slot]) {
     cnt.rebuilds += F.table[slot] == 3 ? 1 : 0;
@@ -3118,7 +3144,7 @@ __device__ __forceinline__ void phase_commit(const MixedCtx& M, GSmem& F, int ba
     else if (steps < M.P.max_steps) {
       F.park[slot] = cy;
       F.pw[slot] = r;
-      F.parked[par][atomicAdd(&F.n_park[par], 1)] = (unsigned char)slot;
+      F.parked[par][cy.type()][atomicAdd(&F.n_park[par][cy.type()], 1)] = (unsigned char)slot;
       F.busy[slot] = 1;
       // the learned bound failed: the event goes on from the scale before this
       // cycle with the plain bounds
@@ -3141,9 +3167,8 @@ __device__ __forceinline__ void phase_commit(const MixedCtx& M, GSmem& F, int ba
 }
 
 // ---- emit: one lane per parked emission -----------------------------------
-__device__ __forceinline__ void phase_emit(const MixedCtx& M, GSmem& F, const SmemPdf& S, int base_lane, int par, int i,
-                                           GCount& cnt) {
-  const int slot = F.parked[par][i];
+__device__ __forceinline__ void phase_emit(const MixedCtx& M, GSmem& F, const SmemPdf& S, int base_lane, int slot,
+                                           int par, GCount& cnt) {
   const WS w{M.W, base_lane + slot, M.P.nmax};
   const GCycle cy = F.park[slot];
   const GWeight r = F.pw[slot];
@@ -3182,19 +3207,25 @@ __device__ __forceinline__ void phase_emit(const MixedCtx& M, GSmem& F, const Sm
   F.table[slot] = table;
   F.keep[slot] = keep;
   F.chg[slot] = chg;
-  F.busy[slot] = 2;
+  F.tables[par][atomicAdd(&F.n_tables[par], 1)] = (unsigned char)slot;
 }
 
-// Before the round of parity par: the emitters' results are handed over, the
-// slots with ends to form listed.
+// Between two rounds: the slots whose events go on with the next round's
+// cycles, and what this round has used up (par: its parity).
 __device__ __forceinline__ void prepare_round(GSmem& F, int tid, int par) {
-  if (tid >= kSlots) return;
-  if (F.busy[tid] == 2) F.busy[tid] = 0;
-  const bool on = F.live[tid] && F.busy[tid] == 0;
-  F.ready[tid] = on;
-  F.tot[tid] = 0;
-  F.defer[tid] = 0;
-  if (on && F.table[tid]) F.tables[par][atomicAdd(&F.n_tables[par], 1)] = (unsigned char)tid;
+  if (tid < (kSlots + 31) / 32 * 32) {
+    const bool on = tid < kSlots && F.live[tid] && F.busy[tid] == 0;
+    const unsigned m = __ballot_sync(0xffffffffu, on);
+    int base = 0;
+    if ((tid & 31) == 0) base = atomicAdd(&F.n_ready[par], __popc(m));
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (on) F.cycles[par][base + __popc(m & ((1u << (tid & 31)) - 1u))] = (unsigned char)tid;
+  }
+  if (tid < 4) F.n_items[tid] = F.n_park[par ^ 1][tid] = 0;
+  if (tid == 0) {
+    F.n_ready[par ^ 1] = F.n_tables[par ^ 1] = F.n_ended[par ^ 1] = 0;
+    F.n_ends = F.n_ends_ok = F.n_q = 0;
+  }
 }
 
 __global__ void __launch_bounds__(kGThreads, 1) k_shower_groups(const __grid_constant__ MixedCtx M) {
@@ -3224,7 +3255,8 @@ __global__ void __launch_bounds__(kGThreads, 1) k_shower_groups(const __grid_con
   }
   if (tid < kSlots) {
     // (an empty slot is read too: the row is an index)
-    F.live[tid] = F.busy[tid] = F.ready[tid] = F.table[tid] = 0;
+    F.live[tid] = F.table[tid] = 0;
+    F.busy[tid] = 1;
     F.row[tid] = F.n[tid] = F.n_emit[tid] = F.steps[tid] = F.keep[tid] = F.tot[tid] = F.len[tid] = F.done[tid] = 0;
     F.chg[tid] = -1;
     F.end[tid] = GAPS_STATUS_ACTIVE;
@@ -3233,72 +3265,64 @@ __global__ void __launch_bounds__(kGThreads, 1) k_shower_groups(const __grid_con
     F.eta0[tid] = F.eta1[tid] = 0.0;
     F.defer[tid] = F.nv[tid] = 0;
   }
-  if (tid < 2) F.n_tables[tid] = F.n_park[tid] = F.n_ended[tid] = 0;
+  if (tid < 2) F.n_ready[tid] = F.n_tables[tid] = F.n_ended[tid] = 0;
+  if (tid < 8) F.n_park[tid & 1][tid >> 1] = 0;
   if (tid == 0) F.n_q = F.n_ends = F.n_ends_ok = 0;
   if (tid < 4) F.n_items[tid] = 0;
   __syncthreads();
   const int base_lane = blockIdx.x * kSlots;
   GCount cnt;
-  // the first events (few: their slots spread over the warps)
-  for (int i = tid >> 3; tid < kWorkers && i < M.slots; i += kWorkers / 8) {
-    const int slot = (i % (4 * kSlots / 32)) * 8 + i / (4 * kSlots / 32);  // eight slots a warp of the chain
+  // the first events
+  for (int slot = tid >> 3; slot < M.slots; slot += kGThreads / 8) {
     refill_slot(M, F, ls, WS{M.W, base_lane + slot, M.P.nmax}, slot, gl, cnt);
+    if (gl == 0 && F.live[slot]) F.tables[1][atomicAdd(&F.n_tables[1], 1)] = (unsigned char)slot;
   }
   __syncthreads();
-  prepare_round(F, tid, 0);
-  __syncthreads();
-  if (warp_id >= kWorkers / 32) {
-    // ---- the emitters ----------------------------------------------------
-    for (int par = 0;; par ^= 1) {
-      // the emissions and the ended events of the round before, beside the
-      // workers' round
-      for (int i = tid - kWorkers; i < F.n_park[par ^ 1]; i += kEmitters) phase_emit(M, F, S, base_lane, par ^ 1, i, cnt);
-      __syncwarp();
-      for (int i = (tid - kWorkers) >> 3; i < F.n_ended[par ^ 1]; i += kEmitters / 8) {
-        const int slot = F.ended[par ^ 1][i];
+  // Every round each kind of warp works on what the round before has listed for
+  // it. Another round while a slot holds an event.
+  for (int par = 0;; par ^= 1) {
+    const int was = par ^ 1;
+    if (warp_id < kCycleWarps) {
+      const int n = F.n_ready[was];
+      for (int i0 = 0; i0 < n; i0 += 8 * kCycleWarps) {  // (few slots are spread over the warps)
+        const int i = i0 + warp_id + kCycleWarps * (lane_id >> 2);
+        phase_chain(M, F, S, base_lane, i < n ? F.cycles[was][i] : -1, lane_id);
+      }
+      cycles_sync();
+      phase_weigh(M, F, S, ls, base_lane, warp_id, lane_id, cnt);
+      cycles_sync();
+      for (int i = tid; i < n; i += 32 * kCycleWarps) phase_commit(M, F, base_lane, F.cycles[was][i], par, cnt);
+    } else if (warp_id < kCycleWarps + kFormWarps) {
+      const int ftid = tid - 32 * kCycleWarps, n = F.n_tables[was];
+      for (int i = ftid >> 3; i - ((ftid >> 3) & 3) < n; i += 4 * kFormWarps) {  // (whole warps)
+        const int slot = i < n ? F.tables[was][i] : -1;
+        phase_touch(F, WS{M.W, base_lane + max(slot, 0), M.P.nmax}, slot, gl, par);
+      }
+      forms_sync();
+      phase_form(M, F, S, ls, base_lane, ftid, cnt);
+      forms_sync();
+      phase_draw(M, F, S, base_lane, ftid, cnt);
+      if (M.Lc.learned) {  // (other ends than the draws')
+        phase_net(M, F, S, ls, mlp, base_lane, ftid >> 5, lane_id, cnt);
+      }
+    } else if (warp_id < kCycleWarps + kFormWarps + kEmitWarps) {
+      const int t = warp_id - kCycleWarps - kFormWarps;
+      for (int i = lane_id; i < F.n_park[was][t]; i += 32)
+        phase_emit(M, F, S, base_lane, F.parked[was][t][i], par, cnt);
+    } else {
+      const int ltid = tid - 32 * (kCycleWarps + kFormWarps + kEmitWarps);
+      for (int i = ltid >> 3; i < F.n_ended[was]; i += 4 * kLoadWarps) {
+        const int slot = F.ended[was][i];
         const WS w{M.W, base_lane + slot, M.P.nmax};
         store_slot(M, F, w, slot, gl, cnt);
         refill_slot(M, F, ls, w, slot, gl, cnt);
-        if (gl == 0) F.busy[slot] = 2;
+        if (gl == 0 && F.live[slot]) F.tables[par][atomicAdd(&F.n_tables[par], 1)] = (unsigned char)slot;
       }
-      if (!__syncthreads_or(0)) break;
-      __syncthreads();
     }
-  } else {
-    // ---- the workers -----------------------------------------------------
-    for (int par = 0;; par ^= 1) {
-      const int n_tables = F.n_tables[par];
-      for (int i = tid >> 3; i - ((tid >> 3) & 3) < n_tables; i += kWorkers / 8) {  // (whole warps)
-        const int slot = i < n_tables ? F.tables[par][i] : -1;
-        phase_touch(F, WS{M.W, base_lane + max(slot, 0), M.P.nmax}, slot, gl);
-      }
-      workers_sync();
-      phase_form(M, F, S, ls, base_lane, tid, cnt);
-      workers_sync();
-      phase_draw(M, F, S, base_lane, tid, cnt);
-      workers_sync();
-      if (M.Lc.learned) {
-        phase_net(M, F, S, ls, mlp, base_lane, warp_id, lane_id, cnt);
-        workers_sync();
-      }
-      if (tid < 4 * kSlots) phase_chain(M, F, S, base_lane, tid);
-      workers_sync();
-      phase_list(F, tid, lane_id);
-      workers_sync();
-      phase_weigh(M, F, S, ls, base_lane, warp_id, lane_id, cnt);
-      workers_sync();
-      phase_commit(M, F, base_lane, tid, par, cnt);
-      // another round while a slot holds an event
-      if (!__syncthreads_or(tid < kSlots && F.live[tid] != 0)) break;
-      // between the two barriers nothing is in flight
-      if (tid == 0) {
-        F.n_park[par ^ 1] = F.n_ended[par ^ 1] = F.n_tables[par] = 0;
-        F.n_ends = F.n_ends_ok = F.n_q = 0;
-      }
-      if (tid < 4) F.n_items[tid] = 0;
-      prepare_round(F, tid, par ^ 1);
-      __syncthreads();
-    }
+    if (!__syncthreads_or(tid < kSlots && F.live[tid] != 0)) break;
+    // between the two barriers nothing is in flight
+    prepare_round(F, tid, par);
+    __syncthreads();
   }
   Counters32 sum;
   sum.steps = cnt.steps; sum.trials = cnt.trials; sum.isr_trials = cnt.isr_trials;
@@ -3866,7 +3890,7 @@ cudaError_t launch_shower_groups(const DevParams& P, const DevEvents& E, const W
   const unsigned grid = (unsigned)min((uint64_t)blocks, (n + M.slots - 1) / M.slots);
   cudaError_t err = cudaMemsetAsync(next, 0, sizeof(unsigned long long), stream);
   if (err != cudaSuccess) return err;
-  k_shower_groups<<<grid, kGThreads, sizeof(GSmem), stream>>>(M);
+  k_shower_groups<<<grid, kGThreads, Lc.learned ? sizeof(GSmem) : kGSmemPlain, stream>>>(M);
   return cudaGetLastError();
 }
 

@@ -11,7 +11,7 @@ from tests.gpu_common import gaps
 
 pytestmark = pytest.mark.gpu
 
-SLOTS = 168  # events in flight per SM
+SLOTS = 192  # events in flight per SM
 
 
 @pytest.fixture(scope="module")
