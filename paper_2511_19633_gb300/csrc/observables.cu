@@ -103,24 +103,38 @@ __device__ __forceinline__ uint32_t above(int i, int w) {
   return kFull << (i - lo + 1);
 }
 
+// |p| of the event's momenta (kept in nnd) and, in FP32, their directions, which
+// the pair distances below use
+template <typename R, int N>
+__device__ __forceinline__ void keep_norm(ObsEvent<R, N>& W, int i) {
+  const R n = norm3(W.ps[i]);
+  W.nnd[i] = n;
+  if constexpr (sizeof(R) == 4) {
+    W.ipt2[i] = W.ps[i][1] / n;
+    W.y[i] = W.ps[i][2] / n;
+    W.phi[i] = W.ps[i][3] / n;
+  }
+}
+
 // thrust: all 2^(n-1) subsets for n <= 12 (total momentum is zero), otherwise
 // the exact construction from candidate axes p_i x p_j with the four sign
 // choices of i and j; the lanes share the candidates, the maximum is exact
 template <int GW, typename R, int N>
 __device__ __forceinline__ R thrust(const ObsTeam<GW>& T, const ObsEvent<R, N>& W, int n) {
   R sum = 0;
-  for (int i = 0; i < n; ++i) sum += norm3(W.ps[i]);
-  if (n < 2 || !(sum > R(0))) return R(1);
+  for (int i = 0; i < n; ++i) sum += W.nnd[i];
+  const bool any = n >= 2 && sum > R(0);
   R best = 0;
   if (n <= 12) {
-    for (uint32_t m = T.lane; m < (1u << (n - 1)); m += GW) {
+    const uint32_t subsets = any ? 1u << (n - 1) : 0u;
+    for (uint32_t m = T.lane; m < subsets; m += GW) {
       R v0 = 0, v1 = 0, v2 = 0;
       for (int i = 0; i < n; ++i)
         if ((m >> i) & 1u) { v0 += W.ps[i][1]; v1 += W.ps[i][2]; v2 += W.ps[i][3]; }
       R l = sqrt(v0 * v0 + v1 * v1 + v2 * v2);
       best = fmax(best, l);
     }
-  } else {
+  } else if (any) {
     for (int i = 0; i < n; ++i) {
       for (int j = i + 1 + T.lane; j < n; j += GW) {
         const R* pi = W.ps[i];
@@ -147,60 +161,73 @@ __device__ __forceinline__ R thrust(const ObsTeam<GW>& T, const ObsEvent<R, N>& 
     }
   }
   best = team_fmax(T, best);
-  return R(2) * best / sum;
+  return any ? R(2) * best / sum : R(1);
+}
+
+// y_ij of the Durham algorithm from the kept norms and directions
+template <typename R, int N>
+__device__ __forceinline__ R durham_yij(const ObsEvent<R, N>& W, int i, int j, R evis2) {
+  R omc;  // 1 - cos(theta_ij)
+  if constexpr (sizeof(R) == 8) {
+    omc = R(1) -
+          (W.ps[i][1] * W.ps[j][1] + W.ps[i][2] * W.ps[j][2] + W.ps[i][3] * W.ps[j][3]) / (W.nnd[i] * W.nnd[j]);
+  } else {
+    // |n_i - n_j|^2 / 2 keeps the relative precision for collinear pairs
+    R d0 = W.ipt2[i] - W.ipt2[j], d1 = W.y[i] - W.y[j], d2 = W.phi[i] - W.phi[j];
+    omc = R(0.5) * (d0 * d0 + d1 * d1 + d2 * d2);
+  }
+  R emin = fmin(W.ps[i][0], W.ps[j][0]);
+  return R(2) * emin * emin * omc / evis2;
 }
 
 // Durham clustering, E-scheme; y23, y34 = smallest y_ij when 3 -> 2, 4 -> 3.
 // Each step takes the smallest y_ij over the remaining pairs in row-major
 // order of the pair (lowest i, then lowest j, on ties); a merged pair keeps
-// the slot of i, and j leaves.
+// the slot of i, and j leaves. The lanes share the pairs of the remaining ones,
+// which nnj lists in ascending order.
 template <int GW, typename R, int N>
 __device__ __forceinline__ void durham(const ObsTeam<GW>& T, ObsEvent<R, N>& W, int m, R& y23, R& y34) {
-  constexpr int kWords = ObsEvent<R, N>::kWords;
-  const int lane = T.lane, last = m;
+  const int lane = T.lane;
   R evis = 0;
   for (int i = 0; i < m; ++i) evis += W.ps[i][0];
+  const R evis2 = evis * evis;
   y23 = 0; y34 = 0;
-  if (lane < kWords)
-    W.am[lane] = m >= 32 * (lane + 1) ? kFull : (m > 32 * lane ? (1u << (m - 32 * lane)) - 1u : 0u);
+  for (int i = lane; i < m; i += GW) W.nnj[i] = i;
   __syncwarp();
-  while (__any_sync(kFull, m > 1)) {
+  while (__any_sync(kFull, m > 2)) {
     R ymin = R(INFINITY);
     int key = INT_MAX;
-    for (int i = m > 1 ? lane : last; i < last; i += GW) {
-      if (!((W.am[i >> 5] >> (i & 31)) & 1u)) continue;
-      const R ni = norm3(W.ps[i]);
-      for (int w = i >> 5; w < kWords; ++w) {
-        uint32_t bits = W.am[w] & above(i, w);
-        while (bits) {
-          const int j = 32 * w + __ffs(bits) - 1;
-          bits &= bits - 1;
-          R nj = norm3(W.ps[j]);
-          R omc;  // 1 - cos(theta_ij)
-          if constexpr (sizeof(R) == 8) {
-            omc = R(1) - (W.ps[i][1] * W.ps[j][1] + W.ps[i][2] * W.ps[j][2] + W.ps[i][3] * W.ps[j][3]) / (ni * nj);
-          } else {
-            // |n_i - n_j|^2 / 2 keeps the relative precision for collinear pairs
-            R d0 = W.ps[i][1] / ni - W.ps[j][1] / nj, d1 = W.ps[i][2] / ni - W.ps[j][2] / nj,
-              d2 = W.ps[i][3] / ni - W.ps[j][3] / nj;
-            omc = R(0.5) * (d0 * d0 + d1 * d1 + d2 * d2);
-          }
-          R emin = fmin(W.ps[i][0], W.ps[j][0]);
-          R yij = R(2) * emin * emin * omc / (evis * evis);
-          if (yij < ymin) { ymin = yij; key = i * kMaxFinal + j; }
-        }
-      }
+    const int pairs = m > 2 ? m * (m - 1) / 2 : 0;
+    for (int p = lane; p < pairs; p += GW) {
+      // the pair a < b with p = b (b - 1) / 2 + a
+      int b = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)p)) * 0.5f);
+      if (b * (b - 1) / 2 > p) --b;
+      const int a = p - b * (b - 1) / 2, i = W.nnj[a], j = W.nnj[b];
+      const R yij = durham_yij(W, i, j, evis2);
+      const int k = i * kMaxFinal + j;
+      if (yij < ymin || (yij == ymin && key != INT_MAX && k < key)) { ymin = yij; key = k; }
     }
     team_argmin(T, ymin, key);
     if (key == INT_MAX) m = 0;  // no finite y_ij (degenerate momenta)
-    if (m > 1) {
-      const int bi = key / kMaxFinal, bj = key % kMaxFinal;
+    const bool on = m > 2;
+    const int bi = on ? key / kMaxFinal : 0, bj = on ? key % kMaxFinal : 0;
+    if (on) {
       if (m == 3) y23 = ymin;
       if (m == 4) y34 = ymin;
       if (lane < 4) W.ps[bi][lane] += W.ps[bj][lane];
-      if (lane == 0) W.am[bj >> 5] &= ~(1u << (bj & 31));
-      m -= 1;
     }
+    __syncwarp();
+    // bi's norm, and bj out of the list
+    if (on && lane == 0) keep_norm(W, bi);
+    for (int i0 = 0; __any_sync(kFull, on && i0 < m - 1); i0 += GW) {
+      const int i = i0 + lane;
+      const bool in = on && i < m - 1;
+      const int here = in ? W.nnj[i] : 0, next = in ? W.nnj[i + 1] : 0;
+      __syncwarp();
+      if (in && here >= bj) W.nnj[i] = next;
+      __syncwarp();
+    }
+    m -= 1;
     __syncwarp();
   }
 }
@@ -514,7 +541,11 @@ __global__ void __launch_bounds__(kObsThreads, sizeof(R) == 4 ? 4 : 2)
         const int m = load_event(T, E, g0 + k, s_np[k], ppk, W.one);
         R a = 0, b = 0, c = 0;
         int jets = 0;
-        if (!ppk) a = thrust(T, W.one, m);
+        if (!ppk) {
+          for (int i = lane; i < m; i += 32) keep_norm(W.one, i);
+          __syncwarp();
+          a = thrust(T, W.one, m);
+        }
         cluster(T, W.one, m, ppk, a, b, c, jets);
         if (lane == 0) { s_a[k] = a; s_b[k] = b; s_c[k] = c; s_jets[k] = jets; }
       } else {
@@ -527,13 +558,24 @@ __global__ void __launch_bounds__(kObsThreads, sizeof(R) == 4 ? 4 : 2)
         const int m = load_event(T, E, g0 + k, mine ? s_np[k] : 0, ppk, V);
         R a = ppk ? 0 : 1, b = 0, c = 0;  // (thrust 1: no momenta)
         int jets = 0;
-        // thrust: its candidates grow fast with the size, so the whole warp
-        // takes the events in turn
-        for (int g = 0; g < kObsGroups; ++g) {
-          const int mg = __shfl_sync(kFull, ppk ? 0 : m, g * kObsLanes);
-          if (mg == 0) continue;
-          const R tg = thrust(ObsTeam<32>(lane), W.four[g], mg);
-          if (lane / kObsLanes == g) a = tg;
+        const int mt = ppk ? 0 : m;
+        if (__any_sync(kFull, mt > 0)) {
+          for (int i = T.lane; i < mt; i += kObsLanes) keep_norm(V, i);
+          __syncwarp();
+          // thrust: of small events together; its candidates grow fast with the
+          // size, so that the whole warp takes larger ones in turn (up to four
+          // subsets a lane against one a lane of each event in turn)
+          if (__all_sync(kFull, mt <= 6)) {
+            const R t = thrust(T, V, mt);
+            if (!ppk) a = t;
+          } else {
+            for (int g = 0; g < kObsGroups; ++g) {
+              const int mg = __shfl_sync(kFull, mt, g * kObsLanes);
+              if (mg == 0) continue;
+              const R tg = thrust(ObsTeam<32>(lane), W.four[g], mg);
+              if (lane / kObsLanes == g) a = tg;
+            }
+          }
         }
         __syncwarp();
         cluster(T, V, m, ppk, a, b, c, jets);
