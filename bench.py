@@ -35,7 +35,7 @@ WORKLOADS = {
     "pp_nlo_1e7": (2, 13600.0, 10_000_000, 1 << 22, 1, None,
                    "NLO-matched pp -> Z at 13.6 TeV, synthetic 100x50 PDF, 1e7 events per step in "
                    "chunks of 2^22, FP32 trials/PDF + FP64 kinematics, learned initial-state proposal, "
-                   "wavefront shower over live-event lists, one CUDA graph per step"),
+                   "kept-trial shower in step over the events of an SM, one CUDA graph per step"),
     "pp_lo_1e6_fp64": (1, 13600.0, 1_000_000, 1_000_000, 0, None,
                        "pp -> Z at 13.6 TeV, LO + initial/final-state shower, synthetic 100x50 PDF, "
                        "1e6 events, FP64 (per-event oracle parity)"),
@@ -52,7 +52,7 @@ WORKLOADS = {
 }
 DEFAULT_WORKLOAD = "pp_nlo_1e7"
 # the kernel that dominates a step of the mixed-precision path
-SHOWER_KERNEL = "k_shower_mixed"
+SHOWER_KERNEL = "k_shower_groups"
 
 # Algorithmic work per unit, as the scope of the measurement defines it: a
 # dipole trial is a log, an exp, a log for the z sample and about 25 FMA
@@ -81,9 +81,8 @@ OPS_PER_ACCEPT = 1200.0
 # 128 FP32 lanes x 2.07 GHz, and 1.25 TFLOP/s FP64 (dense).
 LANE_PEAK_TOPS_NOMINAL = 152 * 128 * 2.07e9 / 1e12
 FP64_PEAK_TFLOPS_NOMINAL = 1.25
-# DRAM bytes (read + write) per event of the shower phase (every kernel of the
-# wavefront between the hard process and the observables), from one ncu
-# capture of the current kernels on a 262 144-event case of the same workload
+# DRAM bytes (read + write) per event of the shower kernel, from one ncu
+# capture of it on a 262 144-event case of the same workload
 # (the traffic grows with the events showered); scaled to a chunk by its
 # events. Workloads and variants without a capture report null.
 SHOWER_DRAM_BYTES_PER_EVENT = {
@@ -399,7 +398,7 @@ def run_ours(args, ws, rank, local):
                         "fit_rmse": res["fit_rmse"], "pipeline": "gaps_train_learned_proposal (one C-ABI call)"}
 
     # mixed precision: the wavefront schedule (default) or the persistent one;
-    # FP64: persistent or one thread per event
+    # FP64: persistent or per event (one kernel)
     if mixed:
         schedule = G.GAPS_SCHED_WAVE if args.schedule == 3 else G.GAPS_SCHED_PERSISTENT
     else:
@@ -408,13 +407,6 @@ def run_ours(args, ws, rank, local):
              "emit_batch": args.emit_batch}
     if schedule == G.GAPS_SCHED_WAVE:
         shape.update(wave_passes=args.passes, wave_cycles=args.cycles, wave_veto_blocks_per_sm=args.veto_bps)
-    tuning = None
-    if mixed and not args.no_autotune:
-        from paper_2511_19633_gb300 import autotune
-        tuning = autotune.autotune(process, sqrt_s, pdf, n_events=1 << 21, mix=mix, learned=learned,
-                                   schedule=schedule)
-        shape = tuning["best"]
-
     def config(pdf_ptr=None, trial_mode=None, sched=None):
         sh = dict(shape)
         if sched is not None and sched != schedule:  # another schedule: its own defaults
@@ -468,14 +460,9 @@ def run_ours(args, ws, rank, local):
         from paper_2511_19633_gb300.sharding import max_over_ranks
         ms = max_over_ranks(ms, dist, device="cuda")
     value = total * args.steps * ws / (ms / 1e3)
-    G.gaps_destroy(ctx)  # its memory (two wavefront slots) goes back before the end-to-end contexts
-    # kernels per chunk: hard process, the shower's kernels, observables
-    if schedule == G.GAPS_SCHED_WAVE:
-        P = shape.get("wave_passes", 24)
-        shower_kernels = 1 + (P + 1) * (2 if learned is not None else 1) + 2 * P + 2
-    else:
-        shower_kernels = 1
-    launches = (2 + shower_kernels) * n_chunks * args.steps
+    G.gaps_destroy(ctx)  # its memory (two slots) goes back before the end-to-end contexts
+    # kernels per chunk: hard process, shower, observables
+    launches = 3 * n_chunks * args.steps
 
     # end to end through the C ABI with host buffers: a fresh context per step
     # (PDF grid and network from host memory), the full path as one graph,
@@ -503,16 +490,15 @@ def run_ours(args, ws, rank, local):
     d2h = obs_host.numel() * 8 + h_host.numel() * 8
 
     # comparisons on samples of the same workload: the plain GPU veto
-    # algorithm (FP64, one thread per event, no compaction, plain bound: the
-    # paper's layout) and the compacted mixed-precision shower without the
-    # learned proposal
+    # algorithm (FP64, every trial redrawn, plain bound: the paper's arithmetic)
+    # and the mixed-precision shower without the learned proposal
     plain = mixed_plain = trial_modes = persistent = None
     if not args.no_plain:
         n_plain = min(total, 1 << 19)
         cfgp = G.make_config(process, sqrt_s, pdf_grid=pdf if uses_pdf else None, nmax=nmax, seed=1,
                              precision=G.GAPS_FP64, schedule=G.GAPS_SCHED_PER_EVENT, mix=mix)
         plain = _time_variant(G, cfgp, ev, 1 << 51, n_plain, chunk, stream)
-        plain["mode"] = "FP64, one thread per event, no compaction, plain bound (the paper's layout)"
+        plain["mode"] = "FP64, every trial redrawn, plain bound, eight lanes per event"
         if mixed and learned is not None:
             n_mp = min(total, chunk)
             mixed_plain = _time_variant(G, config(), ev, (1 << 51) + (1 << 24), n_mp, chunk, stream)
@@ -568,17 +554,15 @@ def run_ours(args, ws, rank, local):
         achieved = ops / busy_s / 1e12
         impl = implementation_ops_mixed(stats) / busy_s / 1e12
         bpe = SHOWER_DRAM_BYTES_PER_EVENT.get((name, learned is not None))
-        kname = SHOWER_KERNEL if schedule != G.GAPS_SCHED_WAVE else (
-            "the shower phase: k_wave_veto, k_wave_ends, k_wave_mlp, k_wave_emit, k_wave_init/final and the "
-            "k_shower_mixed tail, timed together" + (
-                "; chunks run on two streams, so the time is the whole timed region (hard process and "
-                "observables included)" if overlapped else ""))
+        kname = SHOWER_KERNEL + (
+            "; chunks run on two streams, so the time is the whole timed region (hard process and "
+            "observables included)" if overlapped else "")
         roof = {"bound": "alu", "kernel": kname, "achieved": achieved, "peak": lane_peak,
                 "unit": "Tops/s (operations of the scope's work units per second)",
                 "frac": achieved / lane_peak,
                 "traffic": None if bpe is None else bpe * per_launch_events,
-                "traffic_unit": "bytes per chunk's shower phase (ncu DRAM read + write of its kernels on "
-                                "262 144 events, scaled by events)",
+                "traffic_unit": "bytes per chunk's shower (ncu DRAM read + write on 262 144 events, "
+                                "scaled by events)",
                 "peak_source": ("measured: FP32 FMA lane throughput of this GPU (gaps_alu_peak, "
                                 "median SM clock %s MHz)" % alu["clocks"].get("sm_mhz"))
                 if "error" not in alu else "nominal 152 x 128 lanes x 2.07 GHz (microbenchmark failed)",
@@ -597,7 +581,7 @@ def run_ours(args, ws, rank, local):
                 "shower_ms_per_launch": mean_shower_ms, "events_per_launch": per_launch_events,
                 "flop_per_event": flops / max(1, stats["events"])}
     if plain is not None and plain.get("shower_ms"):
-        # the FP64 paper-layout kernel against the measured FP64 pipe
+        # the FP64 kernel against the measured FP64 pipe
         f = fp64_flops(plain["stats"]) / (plain["shower_ms"] / 1e3) / 1e12
         plain["roofline"] = {"bound": "alu", "kernel": "k_shower_fp64", "achieved": f, "peak": fp64_peak,
                              "unit": "TFLOP/s", "frac": f / fp64_peak,
@@ -610,10 +594,8 @@ def run_ours(args, ws, rank, local):
         "data": "synthetic",
         "config": {"workload": name, "description": desc, "events_per_step": total, "chunk": chunk,
                    "parallelism": "independent event ranges per GPU" if ws > 1 else "single GPU",
-                   "schedule": {G.GAPS_SCHED_WAVE: "wavefront passes (rebuild, network, veto, emission kernels "
-                                                   "over live-event lists), persistent kernel for the last events",
-                                G.GAPS_SCHED_PERSISTENT: "persistent, live-event refill",
-                                G.GAPS_SCHED_PER_EVENT: "one thread per event"}[schedule],
+                   "schedule": ("kept trials: cycles, emissions, loads and end records of 192 events per SM "
+                                "side by side" if mixed else "eight lanes per event, finished events replaced"),
                    "launch_shape": shape, "learned_proposal": learned is not None,
                    "cuda_graph": "one graph per step (all chunks), parameters updated in place",
                    "l2": "event records of %.1f GB per chunk rewritten every chunk (> 129 MB L2)"
@@ -641,9 +623,6 @@ def run_ours(args, ws, rank, local):
         "hbm_gbs_measured": peaks.get("hbm_gbs"),
         "alu_peaks": alu,
     }
-    if tuning is not None:
-        line["autotune"] = {"best": tuning["best"], "sample_events": tuning["sample_events"],
-                            "candidates": len(tuning["table"])}
     if rank == 0 and not args.no_cpu_baseline:
         line["cpu_baseline"] = cpu_baseline(process, sqrt_s, mix)
     if rank == 0:
@@ -669,7 +648,8 @@ def main():
     ap.add_argument("--cycles", type=int, default=64)
     ap.add_argument("--period", type=int, default=1)
     ap.add_argument("--emit-batch", type=int, default=16)
-    ap.add_argument("--no-autotune", action="store_true")
+    ap.add_argument("--no-autotune", action="store_true",
+                    help="accepted; kept trials leave nothing to tune")
     ap.add_argument("--no-plain", action="store_true")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-learned", action="store_true")

@@ -31,10 +31,12 @@
  *     scratch of the events in flight (allocated by gaps_init: 208 B x nmax per
  *     event, 64 events per SM, 259 MB for 128 slots; calls on several streams
  *     share it), for GAPS_MIXED, a
- *     working set of nmax partons per resident thread (allocated by the
- *     first mixed gaps_shower call; about 132 B x nmax x resident threads),
- *     or with GAPS_SCHED_WAVE one per event of ev->capacity (about
- *     132 B x nmax + 160 B per event).
+ *     working set allocated by the first mixed gaps_shower call: with kept
+ *     trials (the default) of the events in flight, 192 per SM (about 170 B x
+ *     nmax each, 0.6 GB for 128 slots, whatever ev->capacity); with the other
+ *     trial schemes nmax partons per resident thread (about 132 B x nmax x
+ *     resident threads), or with GAPS_SCHED_WAVE one per event of ev->capacity
+ *     (about 132 B x nmax + 160 B per event).
  */
 #ifndef GAPS_H
 #define GAPS_H
@@ -69,8 +71,12 @@ extern "C" {
 #define GAPS_FP64        0   /* all FP64; matches the reference per event */
 #define GAPS_MIXED       1   /* FP32 trials, PDF and bounds; FP64 kinematics */
 
-/* launch schedules of the shower (GAPS_FP64 runs one kernel, eight lanes per
- * event, for both of the first two) */
+/* launch schedules of the shower. GAPS_FP64 runs one kernel, eight lanes per
+ * event, for both of the first two. GAPS_MIXED with kept trials runs one kernel
+ * for GAPS_SCHED_PERSISTENT and GAPS_SCHED_WAVE (phases in step over the events
+ * of an SM, without the fields below that shape a launch); what differs is the
+ * handling of records that are not to be showered and, for GAPS_SCHED_WAVE, the
+ * largest ev->capacity and gaps_process's second slot */
 #define GAPS_SCHED_PER_EVENT  0   /* GAPS_MIXED: the same as GAPS_SCHED_PERSISTENT */
 #define GAPS_SCHED_PERSISTENT 1   /* persistent grid, finished lanes take the next event */
 #define GAPS_SCHED_WARP       2   /* GAPS_MIXED only: persistent grid, one event per warp
@@ -78,7 +84,8 @@ extern "C" {
 #define GAPS_SCHED_WAVE       3   /* GAPS_MIXED only: wavefront passes, one kernel per phase
                                      (end tables, veto cycles, emissions) over lists of
                                      live events, then the persistent grid for the events
-                                     still live; identical events to GAPS_SCHED_PERSISTENT */
+                                     still live; identical events to GAPS_SCHED_PERSISTENT
+                                     (one kernel with kept trials, as said above) */
 
 /* per-event status values; negative values are the error codes above */
 #define GAPS_STATUS_ACTIVE 0
@@ -129,7 +136,9 @@ typedef struct {
     double p_s;           /* probability of an S event in GAPS_PP_Z_NLO, in (0,1) */
     uint64_t seed;        /* Philox key */
     const float* pdf_grid;/* host pointer to the PDF grid (pp processes), copied */
-    int block_size;       /* GAPS_MIXED: threads per block for the shower, 0 = library default */
+    int block_size;       /* GAPS_MIXED: threads per block for the shower, 0 = library default
+                             (this field, the three after schedule and the wave_* ones
+                             below are checked but not used with GAPS_TRIALS_KEEP) */
     int schedule;         /* GAPS_SCHED_PER_EVENT, GAPS_SCHED_PERSISTENT or GAPS_SCHED_WARP */
     int blocks_per_sm;    /* GAPS_MIXED: resident blocks per SM, 0 = default */
     int refill_period;    /* GAPS_MIXED: idle lanes take new events at most every
@@ -247,8 +256,8 @@ int gaps_generate_hard(gaps_ctx* ctx, uint64_t first_event, uint64_t n,
  * read and written in place; first_event must be the value given to
  * gaps_generate_hard (it keys the random streams). GAPS_FP64 reproduces the
  * FP64 reference evaluation bit for bit; GAPS_MIXED runs the trials, PDF and
- * acceptance in FP32 with FP64 kinematics on a persistent grid with live-event
- * refill, and agrees with it in distribution. Returns GAPS_ERR_CUDA if the
+ * acceptance in FP32 with FP64 kinematics on a persistent grid whose finished
+ * events are replaced, and agrees with it in distribution. Returns GAPS_ERR_CUDA if the
  * working set cannot be allocated. */
 int gaps_shower(gaps_ctx* ctx, uint64_t first_event, uint64_t n,
                 const gaps_events* ev, void* stream);
@@ -468,7 +477,8 @@ int gaps_observables(gaps_ctx* ctx, uint64_t first_event, uint64_t n, const gaps
  * called while `stream` or the context's other calls are being captured.
  * With GAPS_MIXED and GAPS_SCHED_WAVE and two or more chunks the context
  * allocates a second slot (records and observables like `ev` and obs_dev, and
- * a second wavefront working set, about 100 GB for 2^22 events of 128 slots)
+ * a second working set: about 24 GB for 2^22 events of 128 slots with kept
+ * trials, about 100 GB with the others)
  * and the graph runs the odd chunks there on a second stream, concurrently
  * with the even ones in `ev`; obs_host and the histograms are the same, but
  * after the call `ev` and obs_dev hold only the even chunks' records and
