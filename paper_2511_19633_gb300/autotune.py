@@ -1,5 +1,8 @@
 """Launch-shape autotuner for the mixed-precision shower.
 
+Kept trials (make_config's default) do not use these fields: the sweep is for the
+other trial schemes.
+
 Sweeps, on a sample of the workload, threads per block x resident blocks per
 SM x refill (compaction) period x emission batch for the persistent schedule,
 or block shape x wavefront passes x veto cycles per pass for the wavefront

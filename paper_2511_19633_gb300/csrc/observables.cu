@@ -17,9 +17,11 @@
 // instructions of those steps, and warps that take events by size stay in step
 // and end together; the minimum over candidates of the few pseudo-jets whose
 // neighbour changed is shared by an event's lanes (all of them scanned by one
-// lane each: 1.49 ms for 150 001 p p events, 1.04 ms shared, 0.60 ms with the
-// events by size). One event a warp, 32 events a warp in turn: 1.54 ms, 1.24 ms
-// for 4096 p p events (0.17 now), 8.6 ms for 30 000 p p events in FP64 (1.8).
+// lane each: 1.49 ms for 150 001 p p events, 1.04 ms shared, 0.58 ms with the
+// events by size). One event a warp, 32 events a warp in turn: 1.55 ms, 1.24 ms
+// for 4096 p p events (0.17 now), 8.6 ms for 30 000 p p events in FP64 (1.8). The
+// division by R^2 in the distance is needed in place: comparing the dividends
+// and dividing only on near ties took 0.69 ms (a branch in the scans).
 #include "physics_fp64.cuh"
 
 namespace gaps {
@@ -498,7 +500,7 @@ __global__ void __launch_bounds__(kObsThreads, sizeof(R) == 4 ? 4 : 2)
           ++mc;
         }
       }
-      s_np[me] = (unsigned char)np;
+      s_np[me] = (unsigned char)min(max(np, 0), 255);
       s_kind[me] = pp;
     }
     // their order: the events too large for a quarter of a warp (all, if every

@@ -9,8 +9,12 @@
 // generate-select draw fewer blocks. In every mode the histograms agree with
 // the FP64 ones within statistics.
 //
-// Layout: every lane of the persistent grid owns a lane-major working set in
-// global memory (each event contiguous, so a lane walks its own cache lines):
+// Kept trials run in k_shower_groups (phases over the events of an SM), the
+// other schemes in the persistent lane kernel or the wavefront's passes.
+//
+// Layout: every lane of the persistent grid (every slot of k_shower_groups) owns a
+// lane-major working set in global memory (each event contiguous, so a lane walks
+// its own cache lines):
 //   p      f64 [L][nmax][4]     momenta
 //   tag    u32 [L][nmax]        flavour | colour << 8 | anticolour << 16
 //   end    f32x4 [L][2 nmax]    the event's colour ends in canonical order
