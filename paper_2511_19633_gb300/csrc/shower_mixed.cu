@@ -2286,10 +2286,10 @@ __global__ void k_wave_final(const __grid_constant__ MixedCtx M) {
 // slower.
 //
 // Measured, one GPU, before (a warp of events, then a pass per phase over all
-// events) and now: 700 001 p p events with the learned proposal 116.6 -> 70.6
-// ms, 262 144 with the plain bound 46.9 -> 20.4 ms, 100 003 leading-order p p
-// events 24.4 -> 6.1 ms, 4096 events 14.5 -> 3.0 ms, 500 000 events of a beam
-// and process mix 58.8 -> 26.8 ms.
+// events) and now: 700 001 p p events with the learned proposal 116.6 -> 69.8
+// ms, 262 144 with the plain bound 46.9 -> 18.9 ms, 100 003 leading-order p p
+// events 24.4 -> 5.8 ms, 4096 events 14.5 -> 3.0 ms, 500 000 events of a beam
+// and process mix 58.8 -> 25.2 ms.
 // ---------------------------------------------------------------------------
 constexpr int kSlots = 192;
 // the warps of the block, by what they do
@@ -2648,7 +2648,7 @@ __device__ __forceinline__ void store_slot(const MixedCtx& M, GSmem& F, const WS
   }
 }
 // The launch's next event into the slot; an empty slot when there is none.
-__device__ __forceinline__ void refill_slot(const MixedCtx& M, GSmem& F, const LearnedSmem& ls, const WS& w, int slot,
+__device__ __noinline__ void refill_slot(const MixedCtx& M, GSmem& F, const LearnedSmem& ls, const WS& w, int slot,
                                             int gl, GCount& cnt) {
   const DevEvents& E = M.E;
   const unsigned group = 0xffu << (threadIdx.x & 24);
@@ -2863,7 +2863,10 @@ __device__ __forceinline__ void phase_draw(const MixedCtx& M, GSmem& F, const Sm
 }
 
 // ---- net: the network's tiles of the queued ends, four a warp step --------
-__device__ __forceinline__ void phase_net(const MixedCtx& M, GSmem& F, const SmemPdf& S, const LearnedSmem& ls,
+// (out of line, like the load: what few warps run, or only with the learned
+// proposal, then neither lies between the other phases' code nor takes their
+// registers: 456 -> 204 bytes of spills, 262 144 events 19.9 -> 18.9 ms)
+__device__ __noinline__ void phase_net(const MixedCtx& M, GSmem& F, const SmemPdf& S, const LearnedSmem& ls,
                                           const MlpSmem& mlp, int base_lane, int warp_id, int lane_id, GCount& cnt) {
   const int nq = F.n_q;
   for (int g = warp_id; 4 * g < nq; g += kFormWarps) {
