@@ -86,7 +86,7 @@ FP64_PEAK_TFLOPS_NOMINAL = 1.25
 # (the traffic grows with the events showered); scaled to a chunk by its
 # events. Workloads and variants without a capture report null.
 SHOWER_DRAM_BYTES_PER_EVENT = {
-    ("pp_nlo_1e7", True): (3881.5e6 + 5541.6e6) / 262144,   # learned proposal
+    ("pp_nlo_1e7", True): (4347.4e6 + 6358.5e6) / 262144,   # learned proposal
 }
 
 
