@@ -31,9 +31,9 @@
 // copy of each it is 154 KB and half the time. An FP64 instruction in the
 // screening loop, even a comparison, waits behind the other warps' FP64 work.
 // Whole path (hard events, shower, observables), one thread per event and now:
-// 30 000 LO pp -> Z events at 13.6 TeV 1128 and 26 ms, 3001 NLO events with
-// heavy-quark thresholds 1093 and 17 ms (the longest event's chain of cycles),
-// 10 000 e+e- events at 91.2 GeV 35.0 and 1.9 ms, 500 of them 22.2 and 0.7 ms.
+// 30 000 LO pp -> Z events at 13.6 TeV 1138 and 24 ms, 3001 NLO events with
+// heavy-quark thresholds 1093 and 16 ms (the longest event's chain of cycles),
+// 10 000 e+e- events at 91.2 GeV 34.0 and 1.5 ms, 500 of them 21 and 0.64 ms.
 #define GAPS_GM_OUT_OF_LINE
 #include "physics_fp64.cuh"
 
