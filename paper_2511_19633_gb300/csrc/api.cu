@@ -437,9 +437,12 @@ int gaps_init(gaps_ctx** out, const gaps_config* cfg) {
   set_bound_tables(P, ctx->d_tables, c.pdf_grid);
   P.counters = ctx->d_counters;
   for (int r = 0; r < P.n_rows; ++r) set_hist_defs(P.rows[r].process, ctx->H.h[r]);
-  if (c.precision == GAPS_MIXED &&
-      (cudaMalloc(&ctx->d_tables32, groups_tables_bytes()) != cudaSuccess ||
-       launch_groups_tables(P, ctx->d_tables32, nullptr) != cudaSuccess || cudaStreamSynchronize(nullptr) != cudaSuccess)) {
+  // the fills and the tables above are ordered with the legacy stream only, and
+  // the first call may come on a stream that does not wait for it: an FP64 shower
+  // would read the flags of its scratch before they are cleared
+  if ((c.precision == GAPS_MIXED && (cudaMalloc(&ctx->d_tables32, groups_tables_bytes()) != cudaSuccess ||
+                                     launch_groups_tables(P, ctx->d_tables32, nullptr) != cudaSuccess)) ||
+      cudaStreamSynchronize(nullptr) != cudaSuccess) {
     cudaGetLastError();
     gaps_destroy(ctx);
     return GAPS_ERR_CUDA;
