@@ -1169,4 +1169,13 @@ void gaps_destroy(gaps_ctx* ctx) {
   delete ctx;
 }
 
+// ---- for the tests; not part of the interface (gaps.h does not declare them) --
+
+// takes every part of the FP64 scratch, or gives them back (none may be in use)
+int gaps_test_hold_scratch(gaps_ctx* ctx, int hold) {
+  if (!ctx || !ctx->d_pool) return GAPS_ERR_INVALID_ARG;
+  const int rc = cuda_fail(cudaMemset(ctx->d_pool, hold ? 1 : 0, ctx->pool_flag_bytes));
+  return rc != GAPS_OK ? rc : cuda_fail(cudaStreamSynchronize(nullptr));
+}
+
 }  // extern "C"

@@ -899,13 +899,23 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
     __threadfence();
   }
   __syncthreads();
-  if (s_region < 0) return;  // cannot happen: see above (the events stay active)
-  const size_t slot = (size_t)s_region * kGroups + tid / kG;
-  Scratch w = scratch_of(pool + slot * (size_t)P.nmax * kSlotBytesPerParton, P.nmax);
   const uint64_t block0 = (uint64_t)blockIdx.x * per_block;
   const unsigned block_n = (unsigned)(n_events - block0 < per_block ? n_events - block0 : per_block);
 
   Counters cnt;
+  if (s_region < 0) {
+    // not expected, see above; should it happen, its events end with an error
+    for (unsigned j = tid; j < block_n; j += kThreads) {
+      cnt.finished += 1;
+      if (E.status[block0 + j] != GAPS_STATUS_ACTIVE) continue;
+      E.status[block0 + j] = GAPS_ERR_NUMERIC;
+      cnt.err_num += 1;
+    }
+    flush_counters(P, cnt);
+    return;
+  }
+  const size_t slot = (size_t)s_region * kGroups + tid / kG;
+  Scratch w = scratch_of(pool + slot * (size_t)P.nmax * kSlotBytesPerParton, P.nmax);
   Event S;
   Group g{kG};
   bool exhausted = false, first_take = true;
