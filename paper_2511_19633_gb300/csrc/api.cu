@@ -578,20 +578,26 @@ int shower_mixed(gaps_ctx* ctx, uint64_t first_event, uint64_t n, const gaps_eve
 }  // namespace
 
 namespace {
+// the context's learned proposal as a shower takes it
+LearnedCfg learned_cfg(const gaps_ctx* ctx) {
+  LearnedCfg Lc{};
+  bool any_pp = false;
+  for (int r = 0; r < ctx->P.n_rows; ++r) any_pp = any_pp || ctx->P.rows[r].process != GAPS_EE_QQ;
+  // veto-max runs every channel's veto with the plain bounds
+  Lc.learned = ctx->learned && ctx->d_mlp && any_pp && ctx->cfg.trial_mode != GAPS_TRIALS_VETOMAX;
+  Lc.mlp = ctx->d_mlp;
+  Lc.image = ctx->d_mlp_image;
+  Lc.vlog = reinterpret_cast<float4*>(ctx->vlog);
+  Lc.vcount = reinterpret_cast<unsigned long long*>(ctx->vcount);
+  Lc.vcap = ctx->vcap;
+  return Lc;
+}
+
 // gaps_shower; slot 1: the second wavefront slot of gaps_process
 int shower_impl(gaps_ctx* ctx, uint64_t first_event, uint64_t n, const gaps_events* ev, void* stream, int slot) {
   const gaps_config& c = ctx->cfg;
   if (c.precision == GAPS_MIXED) {
-    LearnedCfg Lc{};
-    bool any_pp = false;
-    for (int r = 0; r < ctx->P.n_rows; ++r) any_pp = any_pp || ctx->P.rows[r].process != GAPS_EE_QQ;
-    // veto-max runs every channel's veto with the plain bounds
-    Lc.learned = ctx->learned && ctx->d_mlp && any_pp && c.trial_mode != GAPS_TRIALS_VETOMAX;
-    Lc.mlp = ctx->d_mlp;
-    Lc.image = ctx->d_mlp_image;
-    Lc.vlog = reinterpret_cast<float4*>(ctx->vlog);
-    Lc.vcount = reinterpret_cast<unsigned long long*>(ctx->vcount);
-    Lc.vcap = ctx->vcap;
+    const LearnedCfg Lc = learned_cfg(ctx);
     if (c.schedule == GAPS_SCHED_WARP) {
       const int bs = c.block_size > 0 ? c.block_size : 128;
       const int per_sm = c.blocks_per_sm > 0 ? c.blocks_per_sm : 2;
@@ -1170,6 +1176,13 @@ void gaps_destroy(gaps_ctx* ctx) {
 }
 
 // ---- for the tests; not part of the interface (gaps.h does not declare them) --
+
+// gaps_shower of a GAPS_MIXED context in the lane kernel (one event a lane, phases
+// and code apart from the kept-trial kernel's): that kernel's reference
+int gaps_test_shower_lanes(gaps_ctx* ctx, uint64_t first_event, uint64_t n, const gaps_events* ev, void* stream) {
+  if (!ctx || !events_ok(ctx, ev, n) || ctx->cfg.precision != GAPS_MIXED) return GAPS_ERR_INVALID_ARG;
+  return shower_mixed(ctx, first_event, n, ev, learned_cfg(ctx), stream);
+}
 
 // takes every part of the FP64 scratch, or gives them back (none may be in use)
 int gaps_test_hold_scratch(gaps_ctx* ctx, int hold) {
