@@ -229,8 +229,10 @@ typedef struct {
     uint64_t accepts;     /* accepted emissions */
     uint64_t violations;  /* acceptance weights above one (overestimate failures) */
     uint64_t err_capacity, err_iter_cap, err_numeric;
-    uint64_t lane_steps;  /* active lanes summed over warp steps (divergence) */
-    uint64_t warp_steps;  /* warp steps x 32 */
+    uint64_t lane_steps;  /* active lanes summed over warp steps (divergence); kept trials:
+                             the cycles evaluated there, without those evaluated ahead
+                             and then dropped */
+    uint64_t warp_steps;  /* warp steps x 32 (kept trials: of the cycles' acceptance only) */
     uint64_t rebuilds;    /* GAPS_MIXED: warp-cooperative colour-end table rebuilds */
     uint64_t mlp_tiles;   /* GAPS_MIXED: 16-row network evaluations of the learned proposal */
 } gaps_stats;

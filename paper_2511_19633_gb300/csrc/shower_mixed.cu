@@ -2307,7 +2307,7 @@ static_assert(kCyc == 8, "two cycles a lane of the chain");
 // launch's events)
 struct GCount {
   unsigned steps = 0, trials = 0, isr_trials = 0, vetoes = 0, accepts = 0, violations = 0, rebuilds = 0, tiles = 0;
-  unsigned lane_steps = 0, warp_steps = 0;  // lanes that weighed a cycle, lanes of their warps
+  unsigned lane_steps = 0, warp_steps = 0;  // weighed cycles that were committed, lanes of the weighing warps
   unsigned finished = 0, err_cap = 0, err_iter = 0, err_num = 0;
 };
 
@@ -3075,7 +3075,6 @@ __device__ __forceinline__ void phase_weigh(const MixedCtx& M, GSmem& F, const S
         const GCycle cy = F.cyc[k][slot];
         const GWeight r = weigh_cycle(M, S, ls, w, F.n[slot], F.row[slot], F.live[slot] == 1, M.first + F.ev[slot],
                                       F.draw[slot] + 3 * (uint64_t)k, t, cy);
-        cnt.lane_steps += 1;
         if ((r.what & 0xff) != kCycVeto) {
           F.wt[k][slot] = r;
           atomicOr(&F.nv[slot], 1u << k);
@@ -3105,6 +3104,7 @@ __device__ __forceinline__ void phase_commit(const MixedCtx& M, GSmem& F, int ba
   }
   cnt.steps += vetoed;
   cnt.vetoes += vetoed;
+  cnt.lane_steps += vetoed + (f >= 0 ? 1 : 0);
   if (vetoed > 0) lnT = F.cyc[vetoed - 1][slot].best;
   // the trials that the cycles from f (or from the cap) on replaced, back, the
   // latest first (a cycle may replace what an earlier one wrote)
