@@ -880,26 +880,43 @@ struct Emission {
 // (relative error (2^-23)^4 before rounding, i.e. an ulp of FP64), a few
 // instructions each instead of the library's division sequences. For normal
 // arguments within the FP32 range, which every invariant here is.
-__device__ __noinline__ double rcp64(double x) {
-  double r = (double)__frcp_rn((float)x);
-  r = r * fma(-x, r, 2.0);
-  r = r * fma(-x, r, 2.0);
-  return r;
-}
-__device__ __noinline__ double rsqrt64(double x) {
-  double r = (double)rsqrtf((float)x);
-  r = r * fma(-0.5 * x * r, r, 1.5);
-  r = r * fma(-0.5 * x * r, r, 1.5);
-  return r;
-}
+struct InlineMath {
+  static constexpr bool kInline = true;
+  static __device__ __forceinline__ double rcp(double x) {
+    double r = (double)__frcp_rn((float)x);
+    r = r * fma(-x, r, 2.0);
+    r = r * fma(-x, r, 2.0);
+    return r;
+  }
+  static __device__ __forceinline__ double rsqrt(double x) {
+    double r = (double)rsqrtf((float)x);
+    r = r * fma(-0.5 * x * r, r, 1.5);
+    r = r * fma(-0.5 * x * r, r, 1.5);
+    return r;
+  }
+};
+__device__ __noinline__ double rcp64(double x) { return InlineMath::rcp(x); }
+__device__ __noinline__ double rsqrt64(double x) { return InlineMath::rsqrt(x); }
+// One copy of each. Which is faster depends on the kernel around it (2^20 NLO
+// events, called and inline): with 128 registers a thread the lane kernel takes 335
+// and 353 ms redrawing, 307 and 324 ms with generate-select, 314 and 329 ms with
+// veto-max; with 80 registers 285 and 269, 229 and 238, 311 and 278 ms; with 64
+// registers (256 threads x 4) 247 and 255, 212 and 202, 276 and 256 ms. The warp
+// kernel takes 1019 and 1059 ms for half of them, the wavefront's passes are level,
+// and the kept-trial kernel, which its instruction fetches bound, calls them.
+struct CalledMath {
+  static constexpr bool kInline = false;
+  static __device__ __forceinline__ double rcp(double x) { return rcp64(x); }
+  static __device__ __forceinline__ double rsqrt(double x) { return rsqrt64(x); }
+};
 
 // Transverse basis of a dipole (as in physics_fp64.cuh) with one reciprocal
 // per divisor: the mixed-precision kernel needs FP64 accuracy here, not the
 // FP64 kernel's operation-for-operation agreement with the reference, and
 // every FP64 division is a long instruction sequence.
-__device__ __noinline__ void transverse_basis_mixed(const double P[4], const double K[4], double e1[4],
-                                                    double e2[4]) {
-  const double iPK = rcp64(dot4(P, K));
+template <class F>
+__device__ __forceinline__ void transverse_basis_body(const double P[4], const double K[4], double e1[4], double e2[4]) {
+  const double iPK = F::rcp(dot4(P, K));
   const double N1 = 1.0 + 2.0 * P[1] * K[1] * iPK;
   const double N2 = 1.0 + 2.0 * P[2] * K[2] * iPK;
   const double N3 = 1.0 + 2.0 * P[3] * K[3] * iPK;
@@ -911,7 +928,7 @@ __device__ __noinline__ void transverse_basis_mixed(const double P[4], const dou
   if (a == 1) b = (N3 > N2) ? 3 : 2;
   else if (a == 2) b = (N3 > N1) ? 3 : 1;
   else b = (N2 > N1) ? 2 : 1;
-  const double ina = rsqrt64(Na);
+  const double ina = F::rsqrt(Na);
   const double ka = K[a] * iPK, pa = P[a] * iPK, kb = K[b] * iPK, pb = P[b] * iPK;
   double e2p[4];
 #pragma unroll
@@ -919,40 +936,50 @@ __device__ __noinline__ void transverse_basis_mixed(const double P[4], const dou
   const double e1b = e1[b];
 #pragma unroll
   for (int mu = 0; mu < 4; ++mu) e2p[mu] = (mu == b ? 1.0 : 0.0) + kb * P[mu] + pb * K[mu] - e1b * e1[mu];
-  const double in2 = rsqrt64(-dot4(e2p, e2p));
+  const double in2 = F::rsqrt(-dot4(e2p, e2p));
 #pragma unroll
   for (int mu = 0; mu < 4; ++mu) e2[mu] = e2p[mu] * in2;
 }
 
+__device__ __noinline__ void transverse_basis_mixed(const double P[4], const double K[4], double e1[4],
+                                                    double e2[4]) {
+  transverse_basis_body<CalledMath>(P, K, e1, e2);
+}
+__device__ __noinline__ void transverse_basis_inline(const double P[4], const double K[4], double e1[4],
+                                                     double e2[4]) {
+  transverse_basis_body<InlineMath>(P, K, e1, e2);
+}
+
 // Appendix B.4 and B.5 maps as in physics_fp64.cuh, with one reciprocal per
 // divisor (FP64 accuracy without the FP64 kernel's operation order)
+template <class F>
 __device__ __forceinline__ bool if_map_mixed(double r, double z, double omz, double& x, double& omx, double& u,
                                              double& omu) {
-  const double iq = rcp64(omz + r);
+  const double iq = F::rcp(omz + r);
   const double disc = 1.0 - 4.0 * r * z * omz * iq * iq;
   if (!(disc >= 0.0)) return false;
-  const double sq = disc > 0.0 ? disc * rsqrt64(disc) : 0.0;
-  x = 2.0 * z * omz * iq * rcp64(1.0 + sq);
-  u = x * r * rcp64(omz);
+  const double sq = disc > 0.0 ? disc * F::rsqrt(disc) : 0.0;
+  x = 2.0 * z * omz * iq * F::rcp(1.0 + sq);
+  u = x * r * F::rcp(omz);
   omu = 1.0 - u;
   if (!(omu > 0.0)) return false;
-  omx = omz * rcp64(omu);
+  omx = omz * F::rcp(omu);
   return true;
 }
 
+template <class F>
 __device__ __forceinline__ bool ii_map_mixed(double r, double z, double omz, double& x, double& omx, double& v) {
-  const double iq = rcp64(omz + r);
+  const double iq = F::rcp(omz + r);
   x = z * omz * iq;
   omx = (omz * omz + r) * iq;
-  v = x * r * rcp64(omz);
+  v = x * r * F::rcp(omz);
   return omx - v > 0.0;
 }
 
 // Accepted emission: FP64 kinematics (Appendix B maps, II Lorentz kick) and
 // colour update; the warp then rebuilds the event's end table cooperatively.
-// Kept out of line: it runs on the parked lanes of a warp only.
-template <class W>
-__device__ __noinline__ bool emit(const MixedCtx& M, const W& w, Lane& L, const Emission& em) {
+template <class F, class W>
+__device__ __forceinline__ bool emit_body(const MixedCtx& M, const W& w, Lane& L, const Emission& em) {
   const int bi = em.bi, k = em.k, bside = em.bside, ch = em.ch, type = em.type;
   const int new_fl_i = em.new_fl_i, fl_j = em.fl_j;
   const float z = em.z, omz = em.omz, tw = em.tw;
@@ -969,10 +996,11 @@ __device__ __noinline__ bool emit(const MixedCtx& M, const W& w, Lane& L, const 
   const double zd = omz < 0.5f ? 1.0 - (double)omz : (double)z;
   const double omzd = omz < 0.5f ? (double)omz : 1.0 - (double)z;
   double e1v[4], e2v[4];
-  transverse_basis_mixed(Pm, K, e1v, e2v);
+  if constexpr (F::kInline) transverse_basis_inline(Pm, K, e1v, e2v);
+  else transverse_basis_mixed(Pm, K, e1v, e2v);
   double cph, sph;
   gm_sincos2pi(Rphi, cph, sph);
-  const double st = t * rsqrt64(t);
+  const double st = t * F::rsqrt(t);
   double kt[4];
 #pragma unroll
   for (int mu = 0; mu < 4; ++mu) kt[mu] = st * (cph * e1v[mu] + sph * e2v[mu]);
@@ -983,9 +1011,9 @@ __device__ __noinline__ bool emit(const MixedCtx& M, const W& w, Lane& L, const 
   double eta_f = 1.0;  // factor of eta of the incoming slot `eta_slot`
   int eta_slot = -1;
   double xd = 1.0, omxd = 0.0, vd = 0.0;
-  const double isd = rcp64(sd);
+  const double isd = F::rcp(sd);
   if (type == kFF || type == kFI) {
-    const double yd = t * rcp64(zd * omzd * sd);  // y (FF) or rho (FI)
+    const double yd = t * F::rcp(zd * omzd * sd);  // y (FF) or rho (FI)
     a1 = zd; b1 = yd * omzd; c1 = 1.0;
     a3 = omzd; b3 = yd * zd; c3 = -1.0;
     a2 = 0.0; c2 = 0.0;
@@ -998,16 +1026,16 @@ __device__ __noinline__ bool emit(const MixedCtx& M, const W& w, Lane& L, const 
     }
   } else if (type == kIF) {
     double ud, omud;
-    if (!if_map_mixed(t * isd, zd, omzd, xd, omxd, ud, omud)) return false;
-    const double ixd = rcp64(xd);
+    if (!if_map_mixed<F>(t * isd, zd, omzd, xd, omxd, ud, omud)) return false;
+    const double ixd = F::rcp(xd);
     a1 = ixd; b1 = 0.0; c1 = 0.0;
     a3 = omud * omxd * ixd; b3 = ud; c3 = -1.0;
     a2 = ud * omxd * ixd; b2 = omud; c2 = 1.0;
     eta_slot = bi;
     eta_f = ixd;
   } else {
-    if (!ii_map_mixed(t * isd, zd, omzd, xd, omxd, vd)) return false;
-    const double ixd = rcp64(xd);
+    if (!ii_map_mixed<F>(t * isd, zd, omzd, xd, omxd, vd)) return false;
+    const double ixd = F::rcp(xd);
     a1 = ixd; b1 = 0.0; c1 = 0.0;
     a3 = (omxd - vd) * ixd; b3 = vd; c3 = -1.0;
     a2 = 0.0; b2 = 1.0; c2 = 0.0;
@@ -1030,7 +1058,7 @@ __device__ __noinline__ bool emit(const MixedCtx& M, const W& w, Lane& L, const 
       Kn[mu] = (pi2[mu] + K[mu]) - pj[mu];
       KK[mu] = Kp[mu] + Kn[mu];
     }
-    const double iKK2 = 2.0 * rcp64(dot4(KK, KK)), iKp2 = 2.0 * rcp64(dot4(Kp, Kp));
+    const double iKK2 = 2.0 * F::rcp(dot4(KK, KK)), iKp2 = 2.0 * F::rcp(dot4(Kp, Kp));
 #pragma unroll 1
     for (int m = 2; m < L.n; ++m) {
       double q[4];
@@ -1071,6 +1099,15 @@ __device__ __noinline__ bool emit(const MixedCtx& M, const W& w, Lane& L, const 
   L.n += 1;
   L.n_emit += 1;
   return true;
+}
+// Kept out of line: it runs on the parked lanes of a warp only.
+template <class W>
+__device__ __noinline__ bool emit(const MixedCtx& M, const W& w, Lane& L, const Emission& em) {
+  return emit_body<CalledMath>(M, w, L, em);
+}
+template <class W>
+__device__ __noinline__ bool emit_inline(const MixedCtx& M, const W& w, Lane& L, const Emission& em) {
+  return emit_body<InlineMath>(M, w, L, em);
 }
 
 static_assert(sizeof(Emission) <= kWavePendBytes, "parked emission exceeds its slot");
@@ -1778,7 +1815,8 @@ __device__ __forceinline__ void flush_counters(const MixedCtx& M, const Counters
 // WAVE = true: the wavefront schedule's final pass; the lanes take the events
 // of the live list, whose working-set lanes and end tables the wavefront
 // passes left ready, and write their state back to the WaveSet arrays.
-template <int MINB, bool WAVE, bool VMAX = false>
+// INL: emissions with InlineMath.
+template <int MINB, bool WAVE, bool VMAX = false, bool INL = VMAX && MINB != 2>
 __global__ void __launch_bounds__(256, MINB) k_shower_mixed(const __grid_constant__ MixedCtx M) {
   __shared__ SmemPdf S;
   extern __shared__ __align__(16) unsigned char dyn_lane_smem[];
@@ -1882,7 +1920,8 @@ __global__ void __launch_bounds__(256, MINB) k_shower_mixed(const __grid_constan
           done_emit = true;
           keep = cache ? 0 : -1;
         } else {
-          done_emit = emit(M, WS{M.W, L.slot, M.P.nmax}, L, pend);
+          done_emit = INL ? emit_inline(M, WS{M.W, L.slot, M.P.nmax}, L, pend)
+                          : emit(M, WS{M.W, L.slot, M.P.nmax}, L, pend);
           if (done_emit) {
             cnt.accepts += 1;
             keep = cache ? 2 * (L.n - 1) : -1;  // the ends that existed before
@@ -3742,6 +3781,8 @@ cudaError_t mixed_kernels_init() {
   cudaError_t e = cudaSuccess;
   e = opt_in(k_shower_mixed<2, false>, bytes, e);
   e = opt_in(k_shower_mixed<3, false>, bytes, e);
+  e = opt_in(k_shower_mixed<3, false, false, true>, bytes, e);
+  e = opt_in(k_shower_mixed<4, false, false, true>, bytes, e);
   e = opt_in(k_shower_mixed<4, false>, bytes, e);
   e = opt_in(k_shower_mixed<2, true>, bytes, e);
   e = opt_in(k_shower_mixed<3, true>, bytes, e);
@@ -3825,8 +3866,20 @@ int mixed_tier(int blocks, int block_size, int sm_count) {
   return threads_per_sm <= 512 ? 2 : (threads_per_sm <= 768 ? 3 : 4);
 }
 
+// (the faster of called and inline reciprocals in emissions, as measured at CalledMath)
 template <bool WAVE, bool VMAX = false>
 void launch_persistent(const MixedCtx& M, int tier, int blocks, int block_size, size_t dyn, cudaStream_t stream) {
+  if constexpr (!WAVE && !VMAX) {
+    const bool redraw = M.P.trial_mode == GAPS_TRIALS_REDRAW;
+    if (tier == 3 && redraw) {
+      k_shower_mixed<3, false, false, true><<<blocks, block_size, dyn, stream>>>(M);
+      return;
+    }
+    if (tier == 4 && !redraw) {
+      k_shower_mixed<4, false, false, true><<<blocks, block_size, dyn, stream>>>(M);
+      return;
+    }
+  }
   if (tier == 2) k_shower_mixed<2, WAVE, VMAX><<<blocks, block_size, dyn, stream>>>(M);
   else if (tier == 3) k_shower_mixed<3, WAVE, VMAX><<<blocks, block_size, dyn, stream>>>(M);
   else k_shower_mixed<4, WAVE, VMAX><<<blocks, block_size, dyn, stream>>>(M);
