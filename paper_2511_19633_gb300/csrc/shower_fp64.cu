@@ -855,7 +855,7 @@ __device__ __forceinline__ void batch(const Group g, int K, const DevParams& P, 
     }
     if (gl == 0) {
       E.npart[S.e] = S.n;
-      E.t[S.e] = S.t;
+      if (S.t < INFINITY) E.t[S.e] = S.t;  // (else no cycle had a trial)
       E.eta[S.e] = S.eta0;
       E.eta[E.cap + S.e] = S.eta1;
       E.n_emit[S.e] = S.n_emit;
@@ -948,7 +948,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
         for (int mu = 0; mu < 4; ++mu) w.p[4 * s + mu] = E.P(mu, s, e);
         w.tag[s] = Tag{E.F(s, e), E.C(s, e), E.A(s, e), 0};
       }
-      S.t = E.t[e];
+      // (a record without a scale, NaN, begins at its dipoles' largest ones)
+      S.t = isnan(E.t[e]) ? INFINITY : E.t[e];
       S.eta0 = E.eta[e];
       S.eta1 = E.eta[E.cap + e];
       S.n_emit = E.n_emit[e];
