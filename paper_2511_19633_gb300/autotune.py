@@ -1,7 +1,8 @@
 """Launch-shape autotuner for the mixed-precision shower.
 
-Kept trials (make_config's default) do not use these fields: the sweep is for the
-other trial schemes.
+Kept trials (make_config's default for GAPS_MIXED) and GAPS_FP64 have one launch
+shape, which these fields do not reach: autotune times it once. The sweep is for
+the other trial schemes (trial_mode=GAPS_TRIALS_REDRAW, _SELECT or _VETOMAX).
 
 Sweeps, on a sample of the workload, threads per block x resident blocks per
 SM x refill (compaction) period x emission batch for the persistent schedule,
@@ -40,12 +41,12 @@ WAVE_GRID = {
 
 def time_shape(process, sqrt_s, pdf, shape: dict, n_events: int, precision=G.GAPS_MIXED,
                first: int = 1 << 44, reps: int = 1, mix=None, learned=None,
-               schedule=G.GAPS_SCHED_PERSISTENT) -> dict:
+               schedule=G.GAPS_SCHED_PERSISTENT, trial_mode=None) -> dict:
     """Shower time of one launch shape; mix: rows of a mixed batch; learned:
-    (params, log_margins) of the learned proposal."""
+    (params, log_margins) of the learned proposal; trial_mode: as make_config's."""
     uses_pdf = process or (mix and any(r[0] for r in mix))
     cfg = G.make_config(process, sqrt_s, pdf_grid=pdf if uses_pdf else None, nmax=128,
-                        precision=precision, schedule=schedule, mix=mix, **shape)
+                        precision=precision, schedule=schedule, mix=mix, trial_mode=trial_mode, **shape)
     ctx = G.gaps_init(cfg)
     try:
         if learned is not None:
@@ -74,8 +75,17 @@ def time_shape(process, sqrt_s, pdf, shape: dict, n_events: int, precision=G.GAP
             "lane_efficiency": st["lane_steps"] / max(1, st["warp_steps"])}
 
 
+def has_launch_shape(precision, schedule, trial_mode=None) -> bool:
+    """Whether a context's showers use the fields that the grids sweep."""
+    mode = G.make_config(G.GAPS_EE_QQ, 91.2, precision=precision, schedule=schedule, trial_mode=trial_mode).trial_mode
+    return precision == G.GAPS_MIXED and mode != G.GAPS_TRIALS_KEEP
+
+
 def autotune(process, sqrt_s, pdf, n_events: int = 1 << 21, grid: dict | None = None,
-             precision=G.GAPS_MIXED, mix=None, learned=None, schedule=G.GAPS_SCHED_PERSISTENT) -> dict:
+             precision=G.GAPS_MIXED, mix=None, learned=None, schedule=G.GAPS_SCHED_PERSISTENT,
+             trial_mode=None) -> dict:
+    """The fastest launch shape of `grid` and the table of all. With one launch
+    shape (has_launch_shape) the first of the grid, timed once, stands for all."""
     grid = grid or (WAVE_GRID if schedule == G.GAPS_SCHED_WAVE else DEFAULT_GRID)
     keys = list(grid)
     table = []
@@ -84,7 +94,9 @@ def autotune(process, sqrt_s, pdf, n_events: int = 1 << 21, grid: dict | None = 
         if shape.get("block_size", 128) * shape.get("blocks_per_sm", 1) > 2048:
             continue  # more threads than an SM holds
         table.append(time_shape(process, sqrt_s, pdf, shape, n_events, precision, mix=mix, learned=learned,
-                                schedule=schedule))
+                                schedule=schedule, trial_mode=trial_mode))
+        if not has_launch_shape(precision, schedule, trial_mode):
+            break
     best = min(table, key=lambda r: r["ms"])
     return {"best": {k: best[k] for k in keys}, "best_events_per_s": best["events_per_s"],
             "sample_events": n_events, "table": table}
