@@ -90,6 +90,23 @@ SHOWER_DRAM_BYTES_PER_EVENT = {
 }
 
 
+# launch-shape options of the command line: they reach the kernels of the other
+# trial schemes in the comparisons, the timed kernels have one shape
+SHAPE_OPTIONS = {"block": 256, "bps": 4, "passes": 24, "veto_bps": 2, "cycles": 64, "period": 1, "emit_batch": 16}
+
+
+def timed_launch_shape(mixed: bool) -> dict:
+    """The launch shape of the timed region's shower kernel (one for all options)."""
+    if mixed:
+        return {"blocks_per_sm": 1, "threads_per_block": 1024, "events_in_flight_per_sm": 192}
+    return {"blocks_per_sm": 4, "threads_per_block": 128, "events_in_flight_per_sm": 64}
+
+
+def shape_options_given(args) -> list:
+    """The launch-shape options that differ from their defaults."""
+    return ["--" + k.replace("_", "-") for k, v in SHAPE_OPTIONS.items() if getattr(args, k) != v]
+
+
 def fp64_flops(stats: dict) -> float:
     return (stats["trials"] * FLOP_PER_TRIAL + stats["isr_trials"] * FLOP_PER_ISR_TRIAL
             + stats["steps"] * FLOP_PER_STEP + stats["accepts"] * FLOP_PER_ACCEPT)
@@ -362,6 +379,9 @@ def run_ours(args, ws, rank, local):
         dist.init_process_group("nccl", device_id=torch.device("cuda", local))
     name = args.workload
     process, sqrt_s, total, chunk, precision, mix, desc = WORKLOADS[name]
+    if shape_options_given(args) and rank == 0:
+        print("the timed kernel has one launch shape, which %s do not change"
+              % ", ".join(shape_options_given(args)), file=sys.stderr)
     if args.events:
         total = args.events
         chunk = min(chunk, total)
@@ -517,11 +537,11 @@ def run_ours(args, ws, rank, local):
                 fitted["gain_vs_certified"] = fitted["value"] / mixed_plain["value"]
                 mixed_plain["fitted_pdf_bound"] = fitted
         if mixed and schedule == G.GAPS_SCHED_WAVE:
-            # the persistent schedule (one kernel, lanes refilled) on the same events
+            # the persistent schedule on the same events: the same kernel with kept trials
             n_mp = min(total, chunk)
             persistent = _time_variant(G, config(sched=G.GAPS_SCHED_PERSISTENT), ev, (1 << 51) + (1 << 24), n_mp,
                                        chunk, stream, learned)
-            persistent["mode"] = "persistent schedule, 256 x 4 per SM, same events and proposal"
+            persistent["mode"] = "persistent schedule (the same kernel), same events and proposal"
         if mixed:
             # the trial schemes on the same events, persistent schedule: max-veto
             # redrawing every channel, max-veto keeping the losing trials,
@@ -596,7 +616,7 @@ def run_ours(args, ws, rank, local):
                    "parallelism": "independent event ranges per GPU" if ws > 1 else "single GPU",
                    "schedule": ("kept trials: cycles, emissions, loads and end records of 192 events per SM "
                                 "side by side" if mixed else "eight lanes per event, finished events replaced"),
-                   "launch_shape": shape, "learned_proposal": learned is not None,
+                   "launch_shape": timed_launch_shape(mixed), "learned_proposal": learned is not None,
                    "cuda_graph": "one graph per step (all chunks), parameters updated in place",
                    "l2": "event records of %.1f GB per chunk rewritten every chunk (> 129 MB L2)"
                          % (chunk * nmax * 44 / 1e9)},
@@ -641,15 +661,11 @@ def main():
     ap.add_argument("--events", type=int, default=0, help="override events per step")
     ap.add_argument("--schedule", type=int, default=3,
                     help="mixed precision: 3 wavefront, 1 persistent; FP64: 1 persistent, 0 per event")
-    ap.add_argument("--block", type=int, default=256)
-    ap.add_argument("--bps", type=int, default=4)
-    ap.add_argument("--passes", type=int, default=24)
-    ap.add_argument("--veto-bps", type=int, default=2)
-    ap.add_argument("--cycles", type=int, default=64)
-    ap.add_argument("--period", type=int, default=1)
-    ap.add_argument("--emit-batch", type=int, default=16)
+    for opt, default in SHAPE_OPTIONS.items():
+        ap.add_argument("--" + opt.replace("_", "-"), type=int, default=default,
+                        help="launch shape in the comparisons; the timed kernels have one")
     ap.add_argument("--no-autotune", action="store_true",
-                    help="accepted; kept trials leave nothing to tune")
+                    help="accepted and without effect: the timed kernels have one launch shape")
     ap.add_argument("--no-plain", action="store_true")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-learned", action="store_true")
