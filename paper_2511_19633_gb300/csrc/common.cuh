@@ -102,12 +102,12 @@ struct WaveSet {
   double* eta;              // [2][cap] momentum fractions of slots 0 and 1
   uint64_t* draw;           // [cap] next Philox block of the event's stream
   unsigned char* pend;      // [cap][kWavePendBytes] the parked emission of the pass
-  uint32_t* list;           // [4][cap] live events of even / odd passes, (unused), rebuilds
+  uint32_t* list;           // [3][cap] live events of even / odd passes, rebuilds
   unsigned long long* ctl;  // [8] lengths of the lists, work counter of the veto pass
   uint64_t cap;
 };
 constexpr int kWavePendBytes = 64;
-enum WaveList { WL_LIVE0 = 0, WL_LIVE1 = 1, WL_REBUILD = 3, WL_GRAB = 4, WL_NCTL = 8 };
+enum WaveList { WL_LIVE0 = 0, WL_LIVE1 = 1, WL_REBUILD = 2, WL_GRAB = 3, WL_NCTL = 8 };
 // WaveSet::flags bits
 constexpr int kWaveParked = 8;
 // events of the live list a veto warp takes with one atomic on the work counter

@@ -399,16 +399,6 @@ __device__ __forceinline__ int partner_from_table(const unsigned char* own, int 
   return (m == 0xff || m == i) ? -1 : m;
 }
 
-template <class W>
-__device__ __forceinline__ int find_partner(const W& w, int n, int i, int side, int tag) {
-  for (int m = 0; m < n; ++m) {
-    if (m == i) continue;
-    uint32_t t = w.T(m);
-    if (side == 0 ? (tag_acol(t) == tag) : (tag_col(t) == tag)) return m;
-  }
-  return -1;
-}
-
 // class of an initial-state end and channel for the learned bound: 22 per
 // dipole type (IF, II): q<-q and g<-q for each quark table index, g<-g, q<-g
 __device__ __forceinline__ int isr_class(int type, int ch, int fl_emitter) {
@@ -1549,14 +1539,16 @@ __device__ __forceinline__ void select_trial(const WS& w, int ne, float lnT, flo
 // only the ends marked by the last rebuild draw, and after a veto only the
 // winner's channel: every channel's trials are a Poisson process in ln t, so
 // when the winner at t_w is vetoed, each other channel's trial is the first
-// point of its process below t_w.
+// point of its process below t_w. (KEEPS = false: the wavefront's passes, which no
+// kept trials reach.)
+template <bool KEEPS>
 __device__ int step_mixed(const MixedCtx& M, const SmemPdf& S, const LearnedSmem& ls, const WS& w, Lane& L,
                           uint64_t id, Counters32& cnt, Emission& pend, bool& parked) {
   const bool pp = S.pp[L.row] != 0;
   const float lnTc = S.lnTc[L.row];
   const uint32_t k0 = (uint32_t)M.P.seed, k1 = (uint32_t)(M.P.seed >> 32);
   const uint32_t e0 = (uint32_t)id, e1 = (uint32_t)(id >> 32);
-  const bool cache = M.P.trial_mode == GAPS_TRIALS_KEEP;
+  const bool cache = KEEPS && M.P.trial_mode == GAPS_TRIALS_KEEP;
   float best = -INFINITY;
   int bq = -1, bch = 0;
   float bRz = 0.5f;
@@ -1852,7 +1844,7 @@ __global__ void __launch_bounds__(256, MINB) k_shower_mixed(const __grid_constan
   int since_flush = 0;
   // ends keep their trials (max-veto) or accepted points (veto-max) while
   // their records are unchanged
-  const bool cache = M.P.trial_mode == GAPS_TRIALS_KEEP || VMAX;
+  const bool cache = (!WAVE && M.P.trial_mode == GAPS_TRIALS_KEEP) || VMAX;
   while (true) {
     // warp-aggregated refill of idle lanes
     unsigned idle = __ballot_sync(0xffffffffu, !active);
@@ -1954,8 +1946,7 @@ __global__ void __launch_bounds__(256, MINB) k_shower_mixed(const __grid_constan
     warp_steps += 32;
     if (active && !parked) {
       int st = VMAX ? step_vetomax(M, S, WS{M.W, L.slot, M.P.nmax}, L, M.first + L.ev, cnt, pend, parked)
-                    : step_mixed(M, S, ls, WS{M.W, L.slot, M.P.nmax}, L, M.first + L.ev, cnt,
-                                                     pend, parked);
+                    : step_mixed<!WAVE>(M, S, ls, WS{M.W, L.slot, M.P.nmax}, L, M.first + L.ev, cnt, pend, parked);
       if (++L.steps >= M.P.max_steps && st == GAPS_STATUS_ACTIVE) st = GAPS_ERR_ITER_CAP;
       if (st != GAPS_STATUS_ACTIVE) {
         L.status = st;
@@ -2179,8 +2170,7 @@ __global__ void __launch_bounds__(256, MINB) k_wave_veto(const __grid_constant__
     warp_steps += 32;
     bool to_next = false;
     if (active) {
-      int st = step_mixed(M, S, ls, WS{M.W, L.slot, M.P.nmax}, L, M.first + L.ev, cnt, pend,
-                                              parked);
+      int st = step_mixed<false>(M, S, ls, WS{M.W, L.slot, M.P.nmax}, L, M.first + L.ev, cnt, pend, parked);
       if (++L.steps >= M.P.max_steps && st == GAPS_STATUS_ACTIVE) st = GAPS_ERR_ITER_CAP;
       ++cycles;
       if (st != GAPS_STATUS_ACTIVE) {
@@ -3968,7 +3958,7 @@ size_t al256(size_t b) { return (b + 255) / 256 * 256; }
 
 size_t wave_state_bytes(uint64_t cap) {
   return al256(cap * sizeof(float)) + 5 * al256(cap * sizeof(int)) + al256(2 * cap * sizeof(double)) +
-         al256(cap * sizeof(uint64_t)) + al256(cap * (size_t)kWavePendBytes) + al256(4 * cap * sizeof(uint32_t)) +
+         al256(cap * sizeof(uint64_t)) + al256(cap * (size_t)kWavePendBytes) + al256(3 * cap * sizeof(uint32_t)) +
          al256(WL_NCTL * sizeof(unsigned long long));
 }
 
@@ -3985,7 +3975,7 @@ void wave_state_carve(void* base, uint64_t cap, WaveSet& V) {
   V.eta = (double*)take(2 * cap * sizeof(double));
   V.draw = (uint64_t*)take(cap * sizeof(uint64_t));
   V.pend = (unsigned char*)take(cap * (size_t)kWavePendBytes);
-  V.list = (uint32_t*)take(4 * cap * sizeof(uint32_t));
+  V.list = (uint32_t*)take(3 * cap * sizeof(uint32_t));
   V.ctl = (unsigned long long*)take(WL_NCTL * sizeof(unsigned long long));
 }
 
