@@ -84,8 +84,9 @@ extern "C" {
 #define GAPS_SCHED_WAVE       3   /* GAPS_MIXED only: wavefront passes, one kernel per phase
                                      (end tables, veto cycles, emissions) over lists of
                                      live events, then the persistent grid for the events
-                                     still live; identical events to GAPS_SCHED_PERSISTENT
-                                     (one kernel with kept trials, as said above) */
+                                     still live; the events of GAPS_SCHED_PERSISTENT, but
+                                     for the last bit of a weight (one kernel with kept
+                                     trials, as said above) */
 
 /* per-event status values; negative values are the error codes above */
 #define GAPS_STATUS_ACTIVE 0

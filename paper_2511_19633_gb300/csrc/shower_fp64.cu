@@ -52,8 +52,9 @@ __device__ __noinline__ uint4 block_of(uint64_t event, uint64_t draw, uint32_t k
 // cycles), and the about eight ends that an emission touches in one step
 constexpr int kG = 8;
 // cycles of a batch when a warp has one event left and gives it all its lanes
-// (3001 NLO events: 33 ms with 8 lanes to the end, 28 ms with 32; 8, 16 or 32
-// cycles a batch made no difference beyond the runs' spread)
+// (shower of 3001 NLO events with heavy-quark thresholds: 15.6 ms with 8 lanes to
+// the end, 13.8 ms with 32; 8, 16 or 32 cycles a batch, 14.3, 13.8 and 13.1 ms, are
+// within the spread of single launches, 11 to 19 ms)
 constexpr int kWideBatch = 16;
 constexpr int kThreads = 128;
 constexpr int kGroups = kThreads / kG;  // events a block holds

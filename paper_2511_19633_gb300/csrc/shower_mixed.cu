@@ -9,8 +9,11 @@
 // generate-select draw fewer blocks. In every mode the histograms agree with
 // the FP64 ones within statistics.
 //
-// Kept trials run in k_shower_groups (phases over the events of an SM), the
-// other schemes in the persistent lane kernel or the wavefront's passes.
+// gaps_shower and gaps_process run kept trials in k_shower_groups (phases over the
+// events of an SM), the other schemes in the persistent lane kernel or the
+// wavefront's passes. The lane kernel also takes kept trials, for the calls that log
+// samples (gaps_collect_isr_states, gaps_collect_pdf_ratios) and for
+// gaps_shower_static.
 //
 // Layout: every lane of the persistent grid (every slot of k_shower_groups) owns a
 // lane-major working set in global memory (each event contiguous, so a lane walks
@@ -1984,7 +1987,8 @@ __global__ void __launch_bounds__(256, MINB) k_shower_mixed(const __grid_constan
 // After the fixed number of passes the remaining live events finish in the
 // persistent kernel above (WAVE = true). Every event takes the same steps
 // with the same random numbers as in the persistent kernel, so the two
-// schedules give identical events. The working set has one lane per event of
+// schedules give the same events (but for the last bit of a weight, see
+// k_shower_groups). The working set has one lane per event of
 // the chunk (lane = event index), so no state moves between the kernels.
 // ---------------------------------------------------------------------------
 
@@ -2288,8 +2292,12 @@ __global__ void k_wave_final(const __grid_constant__ MixedCtx M) {
 //
 // The chain may run ahead because a vetoed cycle uses exactly three Philox
 // blocks (two of the veto, one of the winner's next trial). Every cycle uses
-// the numbers that one lane per event would use, so the events are the same
-// bits.
+// the numbers that one lane per event would use, so the events are the lane
+// kernel's. Kernels differ at most in the last bit of a weight, where the compiler
+// contracts a product differently: of 2 10^8 NLO events with the learned proposal
+// three took another history than in the earlier pass-per-phase kernels, each at one
+// accept decision, and one of the three also differed between those and the lane
+// kernel.
 //
 // Why this shape. The bound is the latency of serial steps and instruction
 // fetch, not arithmetic or memory: an event is some 35 000 warp instructions of
@@ -2308,13 +2316,13 @@ __global__ void k_wave_final(const __grid_constant__ MixedCtx M) {
 //
 // kSlots, kTmx, kEndList: more slots hide more latency, but what the shared
 // memory leaves is the L1 cache, in steps: 192 slots with 48 ends each fit the
-// step of 164 KB (196 KB with the network). 168 slots with 64 ends, 4096 listed
-// ends and the network's memory always there: 22.2 instead of 20.4 ms in the
-// second case below. Two blocks of 80 slots an SM, in lockstep: 27.0 against
-// 22.5 ms. Warps per kind: 12 + 14, 16 + 10 and 18 + 8 for cycles and form are
-// slower.
+// step of 164 KB (196 KB with the network). Shower of 262 144 events with the plain
+// bound 17.5 ms, of 2^20 with the learned proposal 88.4; with 168 slots, 64 ends
+// each and 4096 listed ends 18.9 and 98.8, with 160 slots 19.0 and 93.8. When the
+// first of these took 22.5 ms, two blocks of 80 slots an SM, in lockstep, took 27.0,
+// and 12 + 14, 16 + 10 or 18 + 8 warps for cycles and form were slower too.
 //
-// Measured, one GPU, before (a warp of events, then a pass per phase over all
+// Measured, one GPU, whole passes (hard events, shower, observables), before (a warp of events, then a pass per phase over all
 // events) and now: 700 001 p p events with the learned proposal 116.6 -> 69.8
 // ms, 262 144 with the plain bound 46.9 -> 18.9 ms, 100 003 leading-order p p
 // events 24.4 -> 5.8 ms, 4096 events 14.5 -> 3.0 ms, 500 000 events of a beam
