@@ -2372,6 +2372,7 @@ struct GSmem {
   float lnT[kSlots];
   int n[kSlots], n_emit[kSlots], steps[kSlots], row[kSlots];
   int live[kSlots];    // the slot holds an event: 1, on the plain bounds after a violation: 3
+  int held[kSlots];    // live between the rounds (it changes during one)
   int end[kSlots];     // its status once it ended (GAPS_STATUS_ACTIVE before)
   int busy[kSlots];    // 0: takes part in the next round's cycles; 1: an emission, a load or ends to form
   int table[kSlots];   // 1: form the touched ends, 2: only end chg draws again
@@ -2385,7 +2386,7 @@ struct GSmem {
   GCycle park[kSlots];           // the parked emission: its cycle
   GWeight pw[kSlots];            // and weight
   alignas(16) float tmx[kSlots][kTmx + 4];  // the larger kept trial of ends 0 .. kTmx - 1 (the rest: WS::Tmx)
-  int n_ends, n_ends_ok, n_q, n_items[4], n_ready[2], n_tables[2], n_park[2][4], n_ended[2], n_live[2];
+  int n_ends, n_ends_ok, n_q, n_items[4], n_ready[2], n_tables[2], n_park[2][4], n_ended[2];
   unsigned ends[kEndList];       // slot << 8 | end; bit 16: draw only, then: marked
   unsigned short items[4][kCyc * kSlots];  // 8 slot + cycle, by dipole type
   // by the parity of the round that lists them: slots for the next round's
@@ -3259,19 +3260,17 @@ __device__ __forceinline__ void phase_emit(const MixedCtx& M, GSmem& F, const Sm
 // (par: its parity).
 __device__ __forceinline__ void prepare_round(GSmem& F, int tid, int par) {
   if (tid < (kSlots + 31) / 32 * 32) {
-    const bool live = tid < kSlots && F.live[tid], on = live && F.busy[tid] == 0;
-    const unsigned m = __ballot_sync(0xffffffffu, on), held = __ballot_sync(0xffffffffu, live);
+    const bool on = tid < kSlots && F.live[tid] && F.busy[tid] == 0;
+    const unsigned m = __ballot_sync(0xffffffffu, on);
     int base = 0;
-    if ((tid & 31) == 0) {
-      base = atomicAdd(&F.n_ready[par], __popc(m));
-      atomicAdd(&F.n_live[par], __popc(held));
-    }
+    if ((tid & 31) == 0) base = atomicAdd(&F.n_ready[par], __popc(m));
     base = __shfl_sync(0xffffffffu, base, 0);
     if (on) F.cycles[par][base + __popc(m & ((1u << (tid & 31)) - 1u))] = (unsigned char)tid;
   }
+  if (tid < kSlots) F.held[tid] = F.live[tid];
   if (tid < 4) F.n_items[tid] = F.n_park[par ^ 1][tid] = 0;
   if (tid == 0) {
-    F.n_ready[par ^ 1] = F.n_tables[par ^ 1] = F.n_ended[par ^ 1] = F.n_live[par ^ 1] = 0;
+    F.n_ready[par ^ 1] = F.n_tables[par ^ 1] = F.n_ended[par ^ 1] = 0;
     F.n_ends = F.n_ends_ok = F.n_q = 0;
   }
 }
@@ -3304,7 +3303,7 @@ __global__ void __launch_bounds__(kGThreads, 1) k_shower_groups(const __grid_con
   if (tid < kSlots) {
     // (an empty slot is read too: the row is an index)
     F.live[tid] = F.table[tid] = 0;
-    F.busy[tid] = 1;
+    F.busy[tid] = F.held[tid] = 1;
     F.row[tid] = F.n[tid] = F.n_emit[tid] = F.steps[tid] = F.keep[tid] = F.tot[tid] = F.len[tid] = F.done[tid] = 0;
     F.chg[tid] = -1;
     F.end[tid] = GAPS_STATUS_ACTIVE;
@@ -3313,7 +3312,7 @@ __global__ void __launch_bounds__(kGThreads, 1) k_shower_groups(const __grid_con
     F.eta0[tid] = F.eta1[tid] = 0.0;
     F.defer[tid] = F.nv[tid] = 0;
   }
-  if (tid < 2) F.n_ready[tid] = F.n_tables[tid] = F.n_ended[tid] = F.n_live[tid] = 0;
+  if (tid < 2) F.n_ready[tid] = F.n_tables[tid] = F.n_ended[tid] = 0;
   if (tid < 8) F.n_park[tid & 1][tid >> 1] = 0;
   if (tid == 0) F.n_q = F.n_ends = F.n_ends_ok = 0;
   if (tid < 4) F.n_items[tid] = 0;
@@ -3327,7 +3326,8 @@ __global__ void __launch_bounds__(kGThreads, 1) k_shower_groups(const __grid_con
   }
   __syncthreads();
   // Every round each kind of warp works on what the round before has listed for
-  // it. Another round while a slot holds an event.
+  // it. Another round while a slot held an event before this one (the load warps
+  // fill the slots until they reach the barrier, so that the last round is idle).
   for (int par = 0;; par ^= 1) {
     const int was = par ^ 1;
     if (warp_id < kCycleWarps) {
@@ -3367,12 +3367,10 @@ __global__ void __launch_bounds__(kGThreads, 1) k_shower_groups(const __grid_con
         if (gl == 0 && F.live[slot]) F.tables[par][atomicAdd(&F.n_tables[par], 1)] = (unsigned char)slot;
       }
     }
-    // between the two barriers nothing is in flight (the slots are counted there
-    // and not in the first barrier: the load warps fill them until they reach it)
-    __syncthreads();
+    if (!__syncthreads_or(tid < kSlots && F.held[tid] != 0)) break;
+    // between the two barriers nothing is in flight
     prepare_round(F, tid, par);
     __syncthreads();
-    if (F.n_live[par] == 0) break;
   }
   Counters32 sum;
   sum.steps = cnt.steps; sum.trials = cnt.trials; sum.isr_trials = cnt.isr_trials;
