@@ -2317,8 +2317,8 @@ __global__ void k_wave_final(const __grid_constant__ MixedCtx M) {
 // kSlots, kTmx, kEndList: more slots hide more latency, but what the shared
 // memory leaves is the L1 cache, in steps: 192 slots with 48 ends each fit the
 // step of 164 KB (196 KB with the network). Shower of 262 144 events with the plain
-// bound 17.5 ms, of 2^20 with the learned proposal 88.4; with 168 slots, 64 ends
-// each and 4096 listed ends 18.9 and 98.8, with 160 slots 19.0 and 93.8. When the
+// bound 17.4 ms, of 2^20 with the learned proposal 86.8; with 168 slots, 64 ends
+// each and 4096 listed ends 18.5 and 96.8, with 160 slots 18.8 and 92.2. When the
 // first of these took 22.5 ms, two blocks of 80 slots an SM, in lockstep, took 27.0,
 // and 12 + 14, 16 + 10 or 18 + 8 warps for cycles and form were slower too.
 //
